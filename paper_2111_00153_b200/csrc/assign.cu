@@ -2,150 +2,376 @@
 // assignment block) and the packed buffer's metadata built from it, so that a layer can be quantized and
 // packed from nothing but its fp32 weights and the ratio.
 //
-//   row_stats_kernel   per row: population variance in double by two plain passes in reduction order (the
-//                      definition's order of additions, so that the ranking agrees with it bit for bit) and
-//                      max |w|.  32 rows per warp-sized tile: the tile is read coalesced and walked row-wise
-//                      from shared memory.
-//   rank_kernel        rank of every row under the key (variance, row index): the number of rows that come
-//                      before it.  M^2 / 2 comparisons, tiled through shared memory.
-//   build_meta_kernel  one block: the kind of every row from its rank (the n8 highest ranks Fixed-8, the nP
-//                      lowest PoT-4, the rest Fixed-4), the stable grouping by prefix sums over the rows in
-//                      original order, and every metadata section of the packed buffer.
+// The ranking key is (population variance in double, summed in reduction order; row index).  Adding in
+// reduction order is one dependent chain of 2 K double additions per row (55 us at K = 576, 450 us at K = 4608
+// when every row walked its own), but the assignment needs no more than who is below the two cuts of the
+// ranking.  So:
+//   row_stats_kernel   one block per row, one pass over the weights: the variance summed in parallel, a bound
+//                      on how far it can be from the definition's value, and max |w|.
+//   assign_kernel      one block: finds the two cuts by a radix selection over the parallel variances; a row
+//                      whose interval reaches across a cut (in practice: rows that are copies of one another)
+//                      is undecided, gets the definition's chain of additions, and the undecided rows are
+//                      ordered by the exact key.  Then the kind of every row, the stable grouping by prefix
+//                      sums in original order, and every metadata section of the packed buffer.
+// The result is the definition's in every case.
 #include "common.cuh"
 
 namespace rmsmp {
 
 namespace {
 
-constexpr int kStatRows = 32;
+constexpr int kStatThreads = 128;
+constexpr int kAssignThreads = 1024;
+constexpr int kAssignMaxBlocks = 65536 / kBlockRows;      // the entry point takes at most 65536 rows
+constexpr int kAssignSmemRows = 2048;                     // rows whose statistics are kept in shared memory
 
-__global__ void __launch_bounds__(256) row_stats_kernel(const float* __restrict__ W, int M, int K, double* __restrict__ var,
-                                                        float* __restrict__ amax)
+struct RowStats {             // scratch, 16 bytes per row
+    double* var;              // parallel variance; the exact one once an undecided row has been resolved
+    float* err;               // |var - definition's variance| <= err; 0: var is exact
+    float* amax;              // max |w|, 1 for an all-zero row
+};
+
+// One pass with the row's first weight as the origin: x = w - c, s1 = sum x, s2 = sum x^2, variance
+// (s2 - s1^2 / K) / K.  With u = 2^-53 and q = s2 / K, any order of additions leaves |error| <= 4 (K + 8) u q
+// (|s1| sum|x| <= K s2), and the definition's own two passes are off by at most (K + 4) u var + 2 ((K + 1) u A)^2
+// with A = mean |w|, A^2 <= 2 (c^2 + q); G = 2 (K + 16) u below leaves a factor of more than two.
+__global__ void __launch_bounds__(kStatThreads) row_stats_kernel(const float* __restrict__ W, int K, RowStats out)
 {
-    // 8 warps: each loads 4 rows x 32 columns of a 32 x 32 tile; thread r < 32 then walks row r of the tile
-    __shared__ float tile[kStatRows][33];
-    const int row0 = blockIdx.x * kStatRows;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int my_row = row0 + threadIdx.x;
-    double sum = 0.0;
+    __shared__ double s_red[2][kStatThreads / 32];
+    __shared__ float s_max[kStatThreads / 32];
+    const int row = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float* w = W + (size_t)row * K;
+    const double c = (double)__ldg(w);
+    double s1 = 0.0, s2 = 0.0;
     float mx = 0.0f;
-    for (int pass = 0; pass < 2; ++pass) {
-        const double mean = (pass == 1) ? sum / (double)K : 0.0;
-        double ss = 0.0;
-        for (int k0 = 0; k0 < K; k0 += 32) {
-            __syncthreads();
-            for (int r = warp; r < kStatRows; r += 8) {
-                const int row = row0 + r, k = k0 + lane;
-                tile[r][lane] = (row < M && k < K) ? W[(size_t)row * K + k] : 0.0f;
-            }
-            __syncthreads();
-            if (threadIdx.x < kStatRows && my_row < M) {
-                const int kn = min(32, K - k0);
-                for (int j = 0; j < kn; ++j) {
-                    const float w = tile[threadIdx.x][j];
-                    if (pass == 0) {
-                        sum = __dadd_rn(sum, (double)w);
-                        mx = fmaxf(mx, fabsf(w));
-                    } else {
-                        const double d = __dsub_rn((double)w, mean);
-                        ss = __dadd_rn(ss, __dmul_rn(d, d));
-                    }
-                }
-            }
+    auto add = [&](float v) {
+        const double x = (double)v - c;
+        s1 += x;
+        s2 = __fma_rn(x, x, s2);
+        mx = fmaxf(mx, fabsf(v));
+    };
+    if ((K & 3) == 0) {
+        const int n4 = K >> 2;
+        for (int i = threadIdx.x; i < n4; i += 4 * kStatThreads) {
+            float4 v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (i + j * kStatThreads < n4) v[j] = __ldg(reinterpret_cast<const float4*>(w) + i + j * kStatThreads);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (i + j * kStatThreads < n4) { add(v[j].x); add(v[j].y); add(v[j].z); add(v[j].w); }
         }
-        if (pass == 1 && threadIdx.x < kStatRows && my_row < M) {
-            var[my_row] = ss / (double)K;
-            amax[my_row] = (mx == 0.0f) ? 1.0f : mx;
-        }
+    } else {
+        for (int i = threadIdx.x; i < K; i += kStatThreads) add(__ldg(w + i));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if (lane == 0) { s_red[0][warp] = s1; s_red[1][warp] = s2; s_max[warp] = mx; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kStatThreads / 32; ++i) { s1 += s_red[0][i]; s2 += s_red[1][i]; mx = fmaxf(mx, s_max[i]); }
+        const double q = s2 / (double)K, G = (double)(K + 16) * 2.220446049250313e-16;      // 2^-52
+        double v = fabs(fmax((s2 - s1 * s1 / (double)K) / (double)K, 0.0));
+        float e = __double2float_ru(6.0 * G * q + 4.0 * G * G * (c * c + q));
+        if (mx == 0.0f) { v = 0.0; e = 0.0f; }                     // an all-zero row's variance is exactly zero
+        if (!(v <= 1e300) || !(e <= 3e38f)) { v = __longlong_as_double(0x7FF0000000000000ll); e = 0.0f; }     // not finite: last, by row index
+        out.var[row] = v;
+        out.err[row] = e;
+        out.amax[row] = (mx == 0.0f) ? 1.0f : mx;
     }
 }
 
-__global__ void __launch_bounds__(256) rank_kernel(const double* __restrict__ var, int M, int32_t* __restrict__ rank)
+// The definition's variance: two plain passes in reduction order, every operation rounded on its own.
+__device__ double exact_variance(const float* __restrict__ w, int K)
 {
-    __shared__ double s_var[256];
-    const int r = blockIdx.x * 256 + threadIdx.x;
-    const double mine = (r < M) ? var[r] : 0.0;
-    int before = 0;
-    for (int j0 = 0; j0 < M; j0 += 256) {
-        __syncthreads();
-        s_var[threadIdx.x] = (j0 + threadIdx.x < M) ? var[j0 + threadIdx.x] : 0.0;
-        __syncthreads();
-        const int jn = min(256, M - j0);
-        for (int j = 0; j < jn; ++j) {
-            const double v = s_var[j];
-            before += (v < mine || (v == mine && j0 + j < r)) ? 1 : 0;
+    double mean = 0.0, acc = 0.0;
+    for (int pass = 0; pass < 2; ++pass) {
+        acc = 0.0;
+        auto add = [&](float v) {
+            if (pass == 0) {
+                acc = __dadd_rn(acc, (double)v);
+            } else {
+                const double d = __dsub_rn((double)v, mean);
+                acc = __dadd_rn(acc, __dmul_rn(d, d));
+            }
+        };
+        if ((K & 3) == 0) {
+            const float4* w4 = reinterpret_cast<const float4*>(w);
+            float4 v = __ldg(w4);
+            for (int i = 0; i < (K >> 2); ++i) {
+                const float4 nx = __ldg(w4 + min(i + 1, (K >> 2) - 1));
+                add(v.x); add(v.y); add(v.z); add(v.w);
+                v = nx;
+            }
+        } else {
+            for (int i = 0; i < K; ++i) add(__ldg(w + i));
         }
+        if (pass == 0) mean = acc / (double)K;
     }
-    if (r < M) rank[r] = before;
+    return acc / (double)K;
 }
 
 struct MetaArgs {
+    const float* W;
     uint8_t* blob;
-    const int32_t* rank;
+    RowStats st;
     const float* alpha;       // per row: the caller's, or the max |w| found by row_stats_kernel
     uint8_t* scheme_out;      // optional
     uint8_t* bits_out;        // optional
     uint64_t off_perm, off_slot, off_wstep, off_alpha, off_kind, off_blocks;
-    int M, Cin, kh, kw, Cp, Kp, nP, nF4, n8, nblocks, pot_mode;
+    int M, K, Cin, kh, kw, Cp, Kp, nP, nF4, n8, nblocks, pot_mode;
 };
 
-__global__ void __launch_bounds__(1024, 1) build_meta_kernel(MetaArgs a)
+// N values reduced over the block, for every thread (s: N * 32 entries).
+template <int N, typename T, typename Op>
+__device__ __forceinline__ void block_reduce(T (&v)[N], Op op, T* s)
 {
-    __shared__ int s_cnt[3][1024];      // rows of each kind in this thread's chunk of rows, then exclusive prefix
-    const int t = threadIdx.x, nt = blockDim.x;
-    const int per = (a.M + nt - 1) / nt;                  // consecutive rows per thread: the grouping stays stable
-    const int r0 = t * per, r1 = min(a.M, r0 + per);
-    auto kind_of = [&](int r) -> int {
-        const int rk = a.rank[r];
-        return rk < a.nP ? kPoT4 : (rk < a.M - a.n8 ? kFixed4 : kFixed8);
-    };
-    int c[3] = {0, 0, 0};
-    for (int r = r0; r < r1; ++r) ++c[kind_of(r)];
-    for (int k = 0; k < 3; ++k) s_cnt[k][t] = c[k];
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[i] = op(v[i], __shfl_xor_sync(0xffffffffu, v[i], o));
+    __syncthreads();                                      // the previous use of `s` is over
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int i = 0; i < N; ++i) s[32 * i + (threadIdx.x >> 5)] = v[i];
     __syncthreads();
-    if (t < 3) {                                          // three serial scans of 1024 entries: negligible
-        int run = 0;
-        for (int i = 0; i < nt; ++i) { const int v = s_cnt[t][i]; s_cnt[t][i] = run; run += v; }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        v[i] = s[32 * i + (threadIdx.x & 31)];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[i] = op(v[i], __shfl_xor_sync(0xffffffffu, v[i], o));
     }
-    __syncthreads();
+}
+
+// One block: everything here is latency (a few barriers per step), so the statistics are copied to shared memory
+// first and the selection starts at the first bit in which the variances differ at all (their exponents mostly
+// agree): two or three digits for random weights instead of eight.
+__global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
+{
+    __shared__ int s_hist[2][256];
+    __shared__ unsigned long long s_prefix[2];
+    __shared__ int s_left[2], s_same[2];
+    __shared__ double s_dbl[4 * 32];
+    __shared__ unsigned long long s_u64[32];
+    __shared__ int s_int[2 * 32];
+    __shared__ int s_undecided;
+    __shared__ int s_warp[3][32];
+    __shared__ int s_start[3][kAssignMaxBlocks + 1];      // rows of each kind in front of every 128-row block
+    __shared__ double s_var[kAssignSmemRows];
+    __shared__ float s_err[kAssignSmemRows];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int M = a.M;
+    const bool local = M <= kAssignSmemRows;
+    double* const var = local ? s_var : a.st.var;
+    float* const err = local ? s_err : a.st.err;
+    uint8_t* kind = a.blob + a.off_kind;
     int32_t* perm = reinterpret_cast<int32_t*>(a.blob + a.off_perm);
     int32_t* slot = reinterpret_cast<int32_t*>(a.blob + a.off_slot);
+    const int cut[2] = {a.nP, M - a.n8};                  // rows in front of each cut of the ranking
+    bool need[2];
+    for (int c = 0; c < 2; ++c) need[c] = cut[c] > 0 && cut[c] < M && (c == 0 || cut[1] != cut[0]);
+
+    // ---- the statistics, and the bits in which the keys differ (a non-negative double orders like its bits)
+    const unsigned long long key0 = (unsigned long long)__double_as_longlong(a.st.var[0]);
+    unsigned long long diff[1] = {0ull};
+    for (int r = t; r < M; r += kAssignThreads) {
+        const double v = a.st.var[r];
+        if (local) { s_var[r] = v; s_err[r] = a.st.err[r]; }
+        diff[0] |= (unsigned long long)__double_as_longlong(v) ^ key0;
+    }
+    if (t < 256) { s_hist[0][t] = 0; s_hist[1][t] = 0; }
+    if (t == 0) s_undecided = 0;
+    block_reduce<1>(diff, [](unsigned long long x, unsigned long long y) { return x | y; }, s_u64);
+    int top = 64 - __clzll((long long)diff[0]);           // bits from `top` up are common to all keys
+    if (t < 2) { s_prefix[t] = top < 64 ? key0 & (~0ull << top) : 0ull; s_left[t] = cut[t]; s_same[t] = M; }
+    __syncthreads();
+
+    // ---- the largest key in front of each cut, up to eight bits at a time
+    while (top > 0) {
+        const int shift = max(top - 8, 0);
+        const unsigned long long above = top < 64 ? ~0ull << top : 0ull;
+        const unsigned long long pre0 = s_prefix[0], pre1 = s_prefix[1];
+        const bool one = pre0 == pre1 && need[0] && need[1];       // both cuts still in the same bin: one histogram
+        for (int r = t; r < M; r += kAssignThreads) {
+            const unsigned long long key = (unsigned long long)__double_as_longlong(var[r]);
+            const int d = (int)((key & ~above) >> shift);
+            if (need[0] && (key & above) == pre0) atomicAdd(&s_hist[0][d], 1);
+            if (need[1] && !one && (key & above) == pre1) atomicAdd(&s_hist[1][d], 1);
+        }
+        __syncthreads();
+        if (warp < 2 && need[warp]) {
+            // the digit in which the cut's last row lies: a warp scans the 256 counters, eight to a lane
+            const int* h = s_hist[one ? 0 : warp];
+            int n[8], sum = 0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { n[j] = h[8 * lane + j]; sum += n[j]; }
+            int incl = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+            int before = incl - sum;
+            const int left = s_left[warp];
+            __syncwarp();
+            if (before < left && left <= incl) {
+                int j = 0;
+                while (before + n[j] < left) before += n[j++];
+                s_left[warp] = left - before;
+                s_same[warp] = n[j];
+                s_prefix[warp] |= (unsigned long long)(8 * lane + j) << shift;
+            }
+        }
+        __syncthreads();
+        top = shift;
+        if (top > 0 && (!need[0] || s_same[0] == 1) && (!need[1] || s_same[1] == 1)) {
+            // one row left at each cut: its key is the rest of the digits
+            const unsigned long long known = ~0ull << shift, k0 = s_prefix[0], k1 = s_prefix[1];
+            __syncthreads();
+            for (int r = t; r < M; r += kAssignThreads) {
+                const unsigned long long key = (unsigned long long)__double_as_longlong(var[r]);
+                if (need[0] && (key & known) == k0) s_prefix[0] = key;
+                if (need[1] && (key & known) == k1) s_prefix[1] = key;
+            }
+            __syncthreads();
+            break;
+        }
+        if (t < 256) { s_hist[0][t] = 0; s_hist[1][t] = 0; }
+        __syncthreads();
+    }
+    if (cut[1] == cut[0] && t == 0) { s_prefix[1] = s_prefix[0]; s_left[1] = s_left[0]; s_same[1] = s_same[0]; }
+    __syncthreads();
+
+    // ---- which side of each cut: rows that may lie on either are listed (in the slot section, free until the end)
+    double key_at[2], edge[4];
+    bool tie[2];
+    for (int c = 0; c < 2; ++c) {
+        key_at[c] = __longlong_as_double((long long)s_prefix[c]);
+        tie[c] = s_same[c] > s_left[c];                   // more rows share the last key than fit in front of the cut
+        double lo = -1.0, hi = -__longlong_as_double(0x7FF0000000000000ll);
+        if (cut[c] > 0 && cut[c] < M) {
+            for (int r = t; r < M; r += kAssignThreads) {
+                const double v = var[r], e = (double)err[r];
+                if (v <= key_at[c]) lo = fmax(lo, v + e);
+                if (v > key_at[c] || (tie[c] && v == key_at[c])) hi = fmax(hi, e - v);
+            }
+        }
+        edge[2 * c] = lo; edge[2 * c + 1] = hi;
+    }
+    block_reduce<4>(edge, [](double x, double y) { return fmax(x, y); }, s_dbl);
+    // 0: in front of the cut, 1: behind it, 2: undecided
+    auto side = [&](int c, double v, double e) -> int {
+        if (cut[c] <= 0) return 1;
+        if (cut[c] >= M) return 0;
+        const double hi_edge = edge[2 * c], lo_edge = -edge[2 * c + 1];      // the rows in front reach up to, the rows behind down to here
+        const bool clear = !tie[c] && hi_edge < lo_edge;
+        if (v <= key_at[c]) return (clear || (!(tie[c] && v == key_at[c]) && v + e < lo_edge)) ? 0 : 2;
+        return (clear || v - e > hi_edge) ? 1 : 2;
+    };
+    int in_front[2] = {0, 0};
+    for (int r = t; r < M; r += kAssignThreads) {
+        const double v = var[r], e = (double)err[r];
+        const int s0 = side(0, v, e), s1 = side(1, v, e);
+        in_front[0] += s0 == 0; in_front[1] += s1 == 0;
+        kind[r] = (uint8_t)(s0 | s1 << 2);                // the two sides; turned into the kind below
+        if (s0 == 2 || s1 == 2) slot[atomicAdd(&s_undecided, 1)] = r;
+    }
+    __syncthreads();
+    const int nu = s_undecided;
+    if (nu > 0) {
+        block_reduce<2>(in_front, [](int x, int y) { return x + y; }, s_int);
+        const int want0 = cut[0] - in_front[0], want1 = cut[1] - in_front[1];
+        for (int i = t; i < nu; i += kAssignThreads) {
+            const int r = slot[i];
+            if (err[r] != 0.0f) { var[r] = exact_variance(a.W + (size_t)r * a.K, a.K); err[r] = 0.0f; }
+        }
+        __syncthreads();
+        for (int i = t; i < nu; i += kAssignThreads) {
+            const int r = slot[i];
+            const double v = var[r];
+            const int sides = kind[r];
+            int before0 = 0, before1 = 0;                 // undecided rows of the same cut that come first
+            for (int j = 0; j < nu; ++j) {
+                const int r2 = slot[j];
+                const double v2 = var[r2];
+                if (!(v2 < v || (v2 == v && r2 < r))) continue;
+                // (bits 4-7 keep a row's result apart from its sides, which other threads still read)
+                before0 += (kind[r2] & 3) == 2; before1 += ((kind[r2] >> 2) & 3) == 2;
+            }
+            int res = sides;
+            if ((sides & 3) == 2) res |= (before0 < want0 ? 0 : 1) << 4;
+            if (((sides >> 2) & 3) == 2) res |= (before1 < want1 ? 0 : 1) << 5;
+            kind[r] = (uint8_t)res;
+        }
+        __syncthreads();
+    }
+
+    // ---- stable grouping: consecutive rows per thread, prefix sums over the threads
+    const int per = (M + kAssignThreads - 1) / kAssignThreads;
+    const int r0 = min(M, t * per), r1 = min(M, r0 + per);
+    int cnt[3] = {0, 0, 0};
+    for (int r = r0; r < r1; ++r) {
+        const int s = kind[r];
+        const int s0 = (s & 3) == 2 ? (s >> 4) & 1 : s & 3, s1 = ((s >> 2) & 3) == 2 ? (s >> 5) & 1 : (s >> 2) & 3;
+        const int k = s0 == 0 ? kPoT4 : (s1 == 0 ? kFixed4 : kFixed8);
+        kind[r] = (uint8_t)k;
+        cnt[0] += k == 0; cnt[1] += k == 1; cnt[2] += k == 2;
+    }
+    int next[3];                                          // position inside each group
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        int incl = cnt[k];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+        if (lane == 31) s_warp[k][warp] = incl;
+        next[k] = incl - cnt[k];
+    }
+    __syncthreads();
+    if (warp < 3) {
+        const int v = s_warp[warp][lane];
+        int incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int u = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += u; }
+        s_warp[warp][lane] = incl - v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 3; ++k) next[k] += s_warp[k][warp];
+
     float* wstep = reinterpret_cast<float*>(a.blob + a.off_wstep);
     float* alpha = reinterpret_cast<float*>(a.blob + a.off_alpha);
-    uint8_t* kind = a.blob + a.off_kind;
-    int32_t* blocks = reinterpret_cast<int32_t*>(a.blob + a.off_blocks);
     const int base[3] = {0, a.nP, a.nP + a.nF4};
-    int next[3] = {s_cnt[0][t], s_cnt[1][t], s_cnt[2][t]};       // position inside each group
     for (int r = r0; r < r1; ++r) {
-        const int k = kind_of(r);
-        const int p = base[k] + next[k];
+        if ((r & (kBlockRows - 1)) == 0)
+            for (int k = 0; k < 3; ++k) s_start[k][r / kBlockRows] = next[k];
+        const int k = kind[r];
+        const int p = (k == 0 ? base[0] + next[0]++ : (k == 1 ? base[1] + next[1]++ : base[2] + next[2]++));
         perm[p] = r;
         slot[r] = p;
-        kind[r] = (uint8_t)k;
         const float al = a.alpha[r];
         alpha[r] = al;
         wstep[r] = __fdiv_rn(al, k == kPoT4 ? 64.0f : (k == kFixed4 ? 7.0f : 127.0f));
         if (a.scheme_out) a.scheme_out[r] = (k == kPoT4) ? RMSMP_SCHEME_POT : RMSMP_SCHEME_FIXED;
         if (a.bits_out) a.bits_out[r] = (k == kFixed8) ? 8 : 4;
-        ++next[k];
     }
+    if (t == 0) { s_start[0][a.nblocks] = a.nP; s_start[1][a.nblocks] = a.nF4; s_start[2][a.nblocks] = a.n8; }
     __syncthreads();
     // block table: first position (inside its group) and count of each kind among the block's 128 rows
-    for (int b = t; b < a.nblocks; b += nt) {
-        int cnt[3] = {0, 0, 0}, first[3] = {0, 0, 0};
-        const int rb = b * kBlockRows, re = min(a.M, rb + kBlockRows);
-        for (int r = rb; r < re; ++r) {
-            const int k = kind[r];
-            if (cnt[k] == 0) first[k] = slot[r] - base[k];
-            ++cnt[k];
+    int32_t* blocks = reinterpret_cast<int32_t*>(a.blob + a.off_blocks);
+    for (int i = t; i < 8 * a.nblocks; i += kAssignThreads) {
+        const int b = i >> 3, j = i & 7, k = j >> 1;
+        int v = 0;
+        if (k < 3) {
+            const int n = s_start[k][b + 1] - s_start[k][b];
+            v = (j & 1) ? n : (n ? s_start[k][b] : 0);
         }
-        int32_t* be = blocks + 8 * b;
-        be[0] = first[0]; be[1] = cnt[0]; be[2] = first[1]; be[3] = cnt[1]; be[4] = first[2]; be[5] = cnt[2]; be[6] = 0; be[7] = 0;
+        blocks[i] = v;
     }
     if (t == 0) {
         BlobHeader* H = reinterpret_cast<BlobHeader*>(a.blob);
         H->magic = kLayerMagic; H->version = kBlobVersion;
-        H->M = a.M; H->Cin = a.Cin; H->kh = a.kh; H->kw = a.kw; H->Cp = a.Cp; H->Kp = a.Kp;
+        H->M = M; H->Cin = a.Cin; H->kh = a.kh; H->kw = a.kw; H->Cp = a.Cp; H->Kp = a.Kp;
         H->nP = a.nP; H->nF4 = a.nF4; H->n8 = a.n8; H->nblocks = a.nblocks; H->pot_mode = a.pot_mode;
         H->pad0[0] = H->pad0[1] = H->pad0[2] = 0;
         H->status = 0;
@@ -160,18 +386,19 @@ cudaError_t launch_assign_meta(const float* dW, const rmsmp_layer& L, const floa
                                void* d_scratch, uint8_t* d_scheme, uint8_t* d_bits, cudaStream_t st)
 {
     const int M = L.M, K = L.Cin * L.kh * L.kw;
-    double* var = static_cast<double*>(d_scratch);
-    int32_t* rank = reinterpret_cast<int32_t*>(var + M);
-    float* amax = reinterpret_cast<float*>(rank + M);
-    row_stats_kernel<<<(M + kStatRows - 1) / kStatRows, 256, 0, st>>>(dW, M, K, var, amax);
-    rank_kernel<<<(M + 255) / 256, 256, 0, st>>>(var, M, rank);
+    RowStats rs;
+    rs.var = static_cast<double*>(d_scratch);
+    rs.err = reinterpret_cast<float*>(rs.var + M);
+    rs.amax = rs.err + M;
+    row_stats_kernel<<<M, kStatThreads, 0, st>>>(dW, K, rs);
     MetaArgs a;
-    a.blob = blob; a.rank = rank; a.alpha = d_alpha ? d_alpha : amax; a.scheme_out = d_scheme; a.bits_out = d_bits;
+    a.W = dW; a.K = K; a.st = rs;
+    a.blob = blob; a.alpha = d_alpha ? d_alpha : rs.amax; a.scheme_out = d_scheme; a.bits_out = d_bits;
     a.off_perm = L.off_perm; a.off_slot = L.off_slot; a.off_wstep = L.off_wstep; a.off_alpha = L.off_alpha;
     a.off_kind = L.off_kind; a.off_blocks = L.off_blocks;
     a.M = M; a.Cin = L.Cin; a.kh = L.kh; a.kw = L.kw; a.Cp = L.Cp; a.Kp = L.Kp;
     a.nP = L.nP; a.nF4 = L.nF4; a.n8 = L.n8; a.nblocks = L.nblocks; a.pot_mode = pot_mode;
-    build_meta_kernel<<<1, 1024, 0, st>>>(a);
+    assign_kernel<<<1, kAssignThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -574,6 +574,51 @@ def test_assignment_on_the_device_matches_oracle(shape, ratio):
             assert np.array_equal(acc, O.matmul(v_ref, act))
 
 
+def _rows_at_the_cuts(name, g, M, K):
+    """Weights whose ranking the parallel variances cannot decide by themselves, or only just."""
+    W = synth.weights_normal(g, (M, K))
+    if name == "copies":                                # four different rows, each many times: ties at both cuts
+        W = W[g.integers(0, min(4, M), size=M)]
+    elif name == "all_equal":
+        W[:] = W[0]
+    elif name == "constant":                            # true variance zero, the definition's is rounding noise
+        W[:] = g.uniform(0.1, 0.9, size=(M, 1)).astype(np.float32)
+    elif name == "zero_rows":                           # pruned rows, more than fit in front of the first cut
+        W[g.permutation(M)[: M * 7 // 10]] = 0.0
+    elif name == "offset":                              # mean 2^12 times the spread: the parallel sums cancel
+        W += np.float32(80.0)
+    elif name == "permuted":                            # the same weights in another order: sums differ in the last bits only
+        for r in range(1, M):
+            W[r] = W[0][g.permutation(K)]
+    return np.ascontiguousarray(W)
+
+
+@pytest.mark.parametrize("name", ["normal", "copies", "all_equal", "constant", "zero_rows", "offset", "permuted"])
+@pytest.mark.parametrize("M,K,ratio", [(1, 5, (60, 35, 5)), (33, 31, (60, 35, 5)), (257, 100, (50, 40, 10)),
+                                       (1100, 36, (60, 35, 5)), (2500, 64, (65, 30, 5)), (300, 64, (95, 0, 5))])
+def test_assignment_at_the_cuts_of_the_ranking(M, K, ratio, name):
+    """Whole-number result (which row gets which scheme), so no tolerance: it is the oracle's for rows whose
+    variances tie, or differ by less than the summation error, at a cut; fewer and more rows than threads, and more
+    than the statistics in shared memory."""
+    import torch
+    Wt = _rows_at_the_cuts(name, synth.rng(86, M + K), M, K)
+    layer = R.rmsmp_layer_init_ratio(M, K, 1, 1, ratio)
+    d_packed = torch.empty(layer.packed_bytes, dtype=torch.uint8, device="cuda")
+    scratch = torch.full((R.rmsmp_assign_scratch_bytes(M),), 0xA5, dtype=torch.uint8, device="cuda")
+    d_scheme, d_bits = (torch.empty(M, dtype=torch.uint8, device="cuda") for _ in range(2))
+    R.rmsmp_assign_quantize_pack(torch.from_numpy(Wt).cuda(), R.W_LINEAR, layer, ratio, None, R.POT_NEAREST, d_packed, scratch,
+                                 d_scheme, d_bits)
+    scheme, bits = O.assign_rows(Wt, ratio)
+    assert np.array_equal(d_scheme.cpu().numpy(), scheme) and np.array_equal(d_bits.cpu().numpy(), bits)
+    vals, perm, ws = Hn.unpack(layer, d_packed)
+    assert np.array_equal(perm, O.group_rows(scheme, bits))
+    # the metadata that the host route writes for this map: header, permutation, scales, kinds, block table
+    ref_layer, ref = Hn.pack_layer(Wt, scheme, bits, synth.alpha_rows(Wt))
+    for off, n in ((0, 68), (layer.off_perm, 4 * M), (layer.off_slot, 4 * M), (layer.off_wstep, 4 * M), (layer.off_alpha, 4 * M),
+                   (layer.off_kind, M), (layer.off_blocks, 32 * layer.nblocks)):
+        assert torch.equal(d_packed[off:off + n], ref[off:off + n])
+
+
 # ------------------------------------------------------------------ depthwise convolution
 
 @pytest.mark.parametrize("C,k,stride,pad,B,H,W,kind", [
