@@ -1,13 +1,19 @@
 // Depthwise convolution (one input channel per filter, as in MobileNet-v2's 3x3 layers): every channel c
 // has its own filter row with its own scheme and precision (Figure 2), y[b][ho][wo][c] = sum over the
 // taps of value[c][i][j] * a[b][ho*s+i-p][wo*s+j-p][c].  There is no reduction over channels, hence no
-// matrix product: the layer is bound by its output write, and the work is one integer multiply-add per
-// tap on the CUDA cores.  A block expands the layer's codes once into shared memory, one word per tap and
-// channel quad (channel 4q+j in byte j).  An activation word of a quad is split into four words that keep
-// one channel's byte each, and a 4-way byte dot product of such a word with the weight word is exactly
-// that channel's product.  For 3 x 3 filters of stride 1 or 2 a thread owns one quad, keeps its nine
-// weight words in registers and computes a run of four neighbouring outputs of a row, so that every
-// loaded and split activation word serves all the taps that touch it.
+// matrix product: the layer is bound by its output write, and the work is integer multiply-adds on the
+// CUDA cores.  A block expands the layer's codes once into shared memory, one word per tap and channel
+// quad (channel 4q+j in byte j).
+//
+// 3 x 3 filters of stride 1 or 2: what bounds a straightforward kernel is the integer pipe, because
+// channels-last words put four CHANNELS into a word while the 4-way dot product wants four TAPS (splitting
+// every word into one-channel words spent three of four products on zeros: 42 instructions per output,
+// 74 us for 56 x 56 x 192 at batch 64).  So the words of four neighbouring columns are transposed (4 x 4
+// bytes, eight permutes), which makes the three taps of a kernel row one dot product; a thread owns a
+// channel quad and four neighbouring columns and walks down a strip of rows, so that every input row is
+// loaded and transposed once for the three output rows that it touches, and the next row's loads are in
+// flight meanwhile (46 us).
+// Other filters: a word is split into four one-channel words, one output per work item.
 #include <algorithm>
 #include "common.cuh"
 
@@ -16,7 +22,58 @@ namespace rmsmp {
 namespace {
 
 constexpr int kDwThreads = 256;
-constexpr int kDwRun = 4;                                  // outputs of one row per thread (3 x 3 path)
+constexpr int kDwCols = 4;                                 // output columns per thread (3 x 3 path)
+// Sums start from the bits of 1.5 * 2^23: a nine-tap sum of int8 products is below 2^18, so the finished word IS the
+// float 1.5 * 2^23 + sum and one subtraction gives float(sum) exactly.
+constexpr int kDwMagicBits = 0x4B400000;
+constexpr float kDwMagic = 12582912.0f;
+
+__device__ __forceinline__ uint32_t dw_prmt(uint32_t a, uint32_t b, uint32_t sel)
+{
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+    return d;
+}
+
+// Byte c of the words w0..w3 (columns) to bytes 0..3 of t[c]: channels-last words to one word per channel.
+__device__ __forceinline__ void dw_transpose(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t (&t)[4])
+{
+    const uint32_t a = dw_prmt(w0, w1, 0x5140u), b = dw_prmt(w2, w3, 0x5140u);      // channels 0 and 1
+    const uint32_t c = dw_prmt(w0, w1, 0x7362u), d = dw_prmt(w2, w3, 0x7362u);      // channels 2 and 3
+    t[0] = dw_prmt(a, b, 0x5410u); t[1] = dw_prmt(a, b, 0x7632u);
+    t[2] = dw_prmt(c, d, 0x5410u); t[3] = dw_prmt(c, d, 0x7632u);
+}
+
+// One input row of a thread's strip, ready for the dot products: for every channel the words whose bytes 0..2
+// are the three columns under a kernel row.
+struct DwRow { uint32_t w[4][kDwCols]; };      // [channel][output column]
+
+template <int kS>
+__device__ __forceinline__ void dw_arrange(const uint32_t (&a)[3 * kS + 3], DwRow& r)
+{
+    uint32_t g[4];
+    dw_transpose(a[0], a[1], a[2], a[3], g);
+    if constexpr (kS == 1) {
+        const uint32_t lo = dw_prmt(a[4], a[5], 0x5140u), hi = dw_prmt(a[4], a[5], 0x7362u);      // columns 4, 5: channels 0, 1 / 2, 3
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            r.w[c][0] = g[c];                                                               // columns 0 1 2
+            r.w[c][1] = g[c] >> 8;                                                          // columns 1 2 3
+            r.w[c][2] = dw_prmt(g[c], c < 2 ? lo : hi, (c & 1) ? 0x6632u : 0x4432u);        // columns 2 3 4
+            r.w[c][3] = dw_prmt(g[c], c < 2 ? lo : hi, (c & 1) ? 0x7763u : 0x5543u);        // columns 3 4 5
+        }
+    } else {
+        uint32_t h[4];
+        dw_transpose(a[4], a[5], a[6], a[7], h);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            r.w[c][0] = g[c];                                                               // columns 0 1 2
+            r.w[c][1] = dw_prmt(g[c], h[c], 0x4432u);                                       // columns 2 3 4
+            r.w[c][2] = h[c];                                                               // columns 4 5 6
+            r.w[c][3] = dw_prmt(h[c], a[8], 0x0032u | (uint32_t)(4 + c) << 8 | (uint32_t)(4 + c) << 12);      // columns 6 7 8
+        }
+    }
+}
 
 __device__ __forceinline__ void dw_store(const Problem& p, uint32_t n, int q, const int* acc)
 {
@@ -30,9 +87,9 @@ __device__ __forceinline__ void dw_store(const Problem& p, uint32_t n, int q, co
     if (p.acc) reinterpret_cast<int4*>(p.acc + (size_t)n * p.ld_out)[q] = make_int4(acc[0], acc[1], acc[2], acc[3]);
 }
 
-// kS = 1, 2: 3 x 3 filters of that stride, runs of kDwRun outputs; kS = 0: any filter, one output per item.
+// kS = 1, 2: 3 x 3 filters of that stride, strips of `strip` output rows; kS = 0: any filter, one output per item.
 template <int kS>
-__global__ void __launch_bounds__(kDwThreads, 4) depthwise_kernel(const Problem p)
+__global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const Problem p, const int strip)
 {
     extern __shared__ uint32_t s_w[];                     // [tap][quad]: channel 4q+j in byte j
     const int taps = p.kh * p.kw, C = p.M;
@@ -56,58 +113,98 @@ __global__ void __launch_bounds__(kDwThreads, 4) depthwise_kernel(const Problem 
     const int my_i = threadIdx.x / lanes_q, my_q0 = threadIdx.x - my_i * lanes_q;
     if (my_i >= ipg) return;
     if constexpr (kS != 0) {
-        const uint32_t rpr = (uint32_t)(p.Wo + kDwRun - 1) / kDwRun;   // runs per output row
-        const uint32_t n_runs = (uint32_t)(p.N / p.Wo) * rpr;
-        constexpr int kXW = (kDwRun - 1) * kS + 3;                     // input columns a run touches
+        const uint32_t ncol = (uint32_t)(p.Wo + kDwCols - 1) / kDwCols, nstrip = (uint32_t)(p.Ho + strip - 1) / (uint32_t)strip;
+        const uint32_t n_items = (uint32_t)p.B * nstrip * ncol;
+        constexpr int kXW = 3 * kS + 3;                                // input columns under four outputs
         for (int qi = 0; qi < qpt; ++qi) {
             const int q = my_q0 + qi * lanes_q;
             if (q >= quads) break;
-            uint32_t w9[9];
+            uint32_t f[3][4];                                          // kernel row, channel: taps in bytes 0..2
 #pragma unroll
-            for (int t = 0; t < 9; ++t) w9[t] = s_w[t * quads + q];
-            for (uint32_t run = blockIdx.x * (uint32_t)ipg + my_i; run < n_runs; run += gridDim.x * (uint32_t)ipg) {
-                const uint32_t bh = run / rpr;                         // image * Ho + output row
-                const int wo0 = (int)(run - bh * rpr) * kDwRun;
-                const uint32_t b = bh / (uint32_t)p.Ho;
-                const int ho = (int)(bh - b * (uint32_t)p.Ho);
-                const int8_t* img = p.act + (size_t)b * p.H * p.W * p.pix_pitch;
-                int acc[kDwRun][4];
+            for (int i = 0; i < 3; ++i) dw_transpose(s_w[(3 * i) * quads + q], s_w[(3 * i + 1) * quads + q], s_w[(3 * i + 2) * quads + q], 0u, f[i]);
+            const float4 ws = __ldg(reinterpret_cast<const float4*>(p.wstep) + q);
+            const float sc[4] = {__fmul_rn(ws.x, p.act_step), __fmul_rn(ws.y, p.act_step), __fmul_rn(ws.z, p.act_step), __fmul_rn(ws.w, p.act_step)};
+            for (uint32_t item = blockIdx.x * (uint32_t)ipg + my_i; item < n_items; item += gridDim.x * (uint32_t)ipg) {
+                const uint32_t sb = item / ncol;                       // image * strips + strip
+                const int wo0 = (int)(item - sb * ncol) * kDwCols;
+                const uint32_t b = sb / nstrip;
+                const int ho0 = (int)(sb - b * nstrip) * strip;
+                const int rows = min(strip, p.Ho - ho0), cols = min(kDwCols, p.Wo - wo0);
+                const int x0 = wo0 * kS - p.pad;
+                const int8_t* src = p.act + (size_t)b * p.H * p.W * p.pix_pitch + (int64_t)x0 * p.pix_pitch + 4 * q;
+                const uint32_t pitch = (uint32_t)p.pix_pitch;
+                const int64_t row_pitch = (int64_t)p.W * p.pix_pitch;
+                uint32_t in_x = 0;                                     // which of the columns lie inside the image
 #pragma unroll
-                for (int r = 0; r < kDwRun; ++r) acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0;
-                // all loads of the run first (rows and columns outside the image read as zero), then the arithmetic
-                uint32_t a[3][kXW];
+                for (int x = 0; x < kXW; ++x) in_x |= ((unsigned)(x0 + x) < (unsigned)p.W ? 1u : 0u) << x;
+                auto load = [&](int y, uint32_t (&a)[kXW]) {           // rows and columns outside the image read as zero
+                    const int8_t* r = src + (int64_t)y * row_pitch;
+                    if ((unsigned)y >= (unsigned)p.H) {
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const int y = ho * kS + i - p.pad;
-                    const bool yin = y >= 0 && y < p.H;
-                    const int8_t* rowp = img + (size_t)(yin ? y : 0) * p.W * p.pix_pitch;
+                        for (int x = 0; x < kXW; ++x) a[x] = 0u;
+                    } else if (in_x == (1u << kXW) - 1u) {             // the usual case, without a predicate per column
 #pragma unroll
-                    for (int xx = 0; xx < kXW; ++xx) {
-                        const int x = wo0 * kS + xx - p.pad;
-                        a[i][xx] = (yin && x >= 0 && x < p.W) ? __ldg(reinterpret_cast<const uint32_t*>(rowp + (size_t)x * p.pix_pitch) + q) : 0u;
+                        for (int x = 0; x < kXW; ++x) a[x] = __ldg(reinterpret_cast<const uint32_t*>(r + (uint32_t)x * pitch));
+                    } else {
+#pragma unroll
+                        for (int x = 0; x < kXW; ++x) a[x] = ((in_x >> x) & 1u) ? __ldg(reinterpret_cast<const uint32_t*>(r + (uint32_t)x * pitch)) : 0u;
                     }
-                }
+                };
+                float* out = p.out + ((size_t)b * p.Ho * p.Wo + (size_t)ho0 * p.Wo + wo0) * p.ld_out + 4 * q;
+                int32_t* acc_out = p.acc ? p.acc + (out - p.out) : nullptr;
+                const uint32_t ld = (uint32_t)p.ld_out;
+                const size_t row_out = (size_t)p.Wo * p.ld_out;
+                // one output row from the three arranged input rows under it
+                auto emit = [&](int h, const DwRow& r0, const DwRow& r1, const DwRow& r2) {
+                    float* o = out + (size_t)h * row_out;
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
+                    for (int j = 0; j < kDwCols; ++j) {
+                        int acc[4];
 #pragma unroll
-                    for (int xx = 0; xx < kXW; ++xx) {
-                        const int a0 = (int)(a[i][xx] & 0x000000FFu), a1 = (int)(a[i][xx] & 0x0000FF00u);
-                        const int a2 = (int)(a[i][xx] & 0x00FF0000u), a3 = (int)(a[i][xx] & 0xFF000000u);
-#pragma unroll
-                        for (int j = 0; j < 3; ++j) {
-                            if ((xx - j) % kS != 0 || xx - j < 0 || (xx - j) / kS >= kDwRun) continue;
-                            const int r = (xx - j) / kS;
-                            const int w = (int)w9[i * 3 + j];
-                            acc[r][0] = __dp4a(a0, w, acc[r][0]);
-                            acc[r][1] = __dp4a(a1, w, acc[r][1]);
-                            acc[r][2] = __dp4a(a2, w, acc[r][2]);
-                            acc[r][3] = __dp4a(a3, w, acc[r][3]);
+                        for (int c = 0; c < 4; ++c)
+                            acc[c] = __dp4a((int)r2.w[c][j], (int)f[2][c], __dp4a((int)r1.w[c][j], (int)f[1][c], __dp4a((int)r0.w[c][j], (int)f[0][c], kDwMagicBits)));
+                        if (j < cols) {
+                            *reinterpret_cast<float4*>(o + (uint32_t)j * ld) =
+                                make_float4(__fmul_rn(__fsub_rn(__int_as_float(acc[0]), kDwMagic), sc[0]), __fmul_rn(__fsub_rn(__int_as_float(acc[1]), kDwMagic), sc[1]),
+                                            __fmul_rn(__fsub_rn(__int_as_float(acc[2]), kDwMagic), sc[2]), __fmul_rn(__fsub_rn(__int_as_float(acc[3]), kDwMagic), sc[3]));
+                            if (acc_out)
+                                *reinterpret_cast<int4*>(acc_out + (size_t)h * row_out + (uint32_t)j * ld) =
+                                    make_int4(acc[0] - kDwMagicBits, acc[1] - kDwMagicBits, acc[2] - kDwMagicBits, acc[3] - kDwMagicBits);
                         }
                     }
-                }
+                };
+                DwRow r[3];
+                uint32_t a[kXW], nx[kXW];
+                int y = ho0 * kS - p.pad;                              // the input row to arrange next
+                if constexpr (kS == 1) {
+                    load(y, a);
+                    load(y + 1, nx);
+                    dw_arrange<1>(a, r[0]);
+                    load(y + 2, a);
+                    dw_arrange<1>(nx, r[1]);
+                    y += 3;
+                    for (int h = 0; h < rows; h += 3) {
+                        // three output rows a turn, so that the rows' places in r[] are fixed; a row's words are
+                        // loaded while the row in front of it is worked on
+                        load(y, nx); dw_arrange<1>(a, r[2]); emit(h, r[0], r[1], r[2]);
+                        if (h + 1 < rows) { load(y + 1, a); dw_arrange<1>(nx, r[0]); emit(h + 1, r[1], r[2], r[0]); }
+                        if (h + 2 < rows) { load(y + 2, nx); dw_arrange<1>(a, r[1]); emit(h + 2, r[2], r[0], r[1]); }
 #pragma unroll
-                for (int r = 0; r < kDwRun; ++r)
-                    if (wo0 + r < p.Wo) dw_store(p, bh * (uint32_t)p.Wo + (uint32_t)(wo0 + r), q, acc[r]);
+                        for (int x = 0; x < kXW; ++x) a[x] = nx[x];
+                        y += 3;
+                    }
+                } else {
+                    load(y, a);
+                    load(y + 1, nx);
+                    dw_arrange<2>(a, r[0]);
+                    load(y + 2, a);
+                    y += 3;
+                    for (int h = 0; h < rows; h += 2) {                // r[0] and r[2] take turns as the shared row
+                        dw_arrange<2>(nx, r[1]); load(y, nx); dw_arrange<2>(a, r[2]); load(y + 1, a); emit(h, r[0], r[1], r[2]);
+                        if (h + 1 < rows) { dw_arrange<2>(nx, r[1]); load(y + 2, nx); dw_arrange<2>(a, r[0]); load(y + 3, a); emit(h + 1, r[2], r[1], r[0]); }
+                        y += 4;
+                    }
+                }
             }
         }
         return;
@@ -165,15 +262,30 @@ cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
     if (per_sm < 1) per_sm = 1;
     const int quads = p.M >> 2;
     const int ipg = kDwThreads / std::min(quads, kDwThreads);          // items a block takes per pass
-    const int64_t items = variant ? (p.N / p.Wo) * ((p.Wo + kDwRun - 1) / kDwRun) : p.N;
-    // at least four passes per block, so that expanding the filter table stays a small part of its work
-    int64_t blocks = ((items + ipg - 1) / ipg + 3) / 4;
     const int64_t cap = (int64_t)sm_count() * per_sm;
+    int strip = 1;
+    int64_t blocks;
+    if (variant) {
+        // Height of a strip: a tall one arranges fewer input rows twice, a short one gives more strips to share out
+        // (an item costs about its rows plus one row's worth of start-up and rows shared with its neighbours).
+        const int64_t per_row = (int64_t)p.B * ((p.Wo + kDwCols - 1) / kDwCols);
+        int64_t best = INT64_MAX;
+        for (int n = 1; n <= p.Ho; n += 1 + n / 4) {
+            const int s = (p.Ho + n - 1) / n;
+            const int64_t groups = (per_row * ((p.Ho + s - 1) / s) + ipg - 1) / ipg;
+            const int64_t cost = ((groups + cap - 1) / cap) * (2 * s + 3);
+            if (cost < best) { best = cost; strip = s; }
+        }
+        blocks = (per_row * ((p.Ho + strip - 1) / strip) + ipg - 1) / ipg;
+    } else {
+        // at least four passes per block, so that expanding the filter table stays a small part of its work
+        blocks = ((p.N + ipg - 1) / ipg + 3) / 4;
+    }
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    if (variant == 1) depthwise_kernel<1><<<(unsigned)blocks, kDwThreads, smem, st>>>(p);
-    else if (variant == 2) depthwise_kernel<2><<<(unsigned)blocks, kDwThreads, smem, st>>>(p);
-    else depthwise_kernel<0><<<(unsigned)blocks, kDwThreads, smem, st>>>(p);
+    if (variant == 1) depthwise_kernel<1><<<(unsigned)blocks, kDwThreads, smem, st>>>(p, strip);
+    else if (variant == 2) depthwise_kernel<2><<<(unsigned)blocks, kDwThreads, smem, st>>>(p, strip);
+    else depthwise_kernel<0><<<(unsigned)blocks, kDwThreads, smem, st>>>(p, strip);
     return cudaGetLastError();
 }
 

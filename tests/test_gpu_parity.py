@@ -651,6 +651,35 @@ def test_depthwise_conv_matches_oracle(C, k, stride, pad, B, H, W, kind):
     assert np.array_equal(y.cpu().numpy().view(np.uint32), y_ref.view(np.uint32))
 
 
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("C,pad,B,H,W", [
+    (4, 0, 1, 3, 3),                           # one output
+    (4, 1, 1, 1, 1), (8, 2, 1, 1, 4),          # images smaller than the filter, outputs made of padding only
+    (12, 1, 3, 19, 5), (20, 1, 1, 8, 10),      # columns left over in the last group of four
+    (1028, 1, 1, 9, 6),                        # more channel quads than threads of a block
+    (96, 1, 40, 9, 9),                         # strips of several heights
+])
+def test_depthwise_strips_on_the_whole_code_range(C, pad, B, H, W, stride):
+    """Integer sums of any int8 activation code (not only the 4-bit ones), exact: no tolerance."""
+    import torch
+    g = synth.rng(87, C + H + W)
+    Wt = synth.weights_kaiming(g, C, 1, 3, 3)
+    scheme, bits = O.assign_rows(Wt, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    codes = g.integers(-128, 128, size=(B, H, W, C), dtype=np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    v_ref, wstep = O.quantize_rows(Wt.reshape(C, -1), scheme, bits, alpha)
+    acc_ref = O.conv_depthwise(v_ref.reshape(C, 3, 3), codes, stride, pad)
+    for with_acc in (True, False):
+        y = torch.full(acc_ref.shape, float("nan"), dtype=torch.float32, device="cuda")
+        acc = torch.full(acc_ref.shape, -5, dtype=torch.int32, device="cuda")
+        R.rmsmp_conv_depthwise(layer, d_packed, torch.from_numpy(codes).cuda(), B, H, W, stride, pad, 0.5, y, acc if with_acc else None)
+        torch.cuda.synchronize()
+        if with_acc:
+            assert np.array_equal(acc.cpu().numpy(), acc_ref)
+        assert np.array_equal(y.cpu().numpy().view(np.uint32), O.epilogue(acc_ref, wstep, np.float32(0.5)).view(np.uint32))
+
+
 def test_depthwise_conv_rejects_what_it_cannot_run():
     import torch
     g = synth.rng(86, 1)
