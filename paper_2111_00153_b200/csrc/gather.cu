@@ -64,52 +64,131 @@ __global__ void __launch_bounds__(kGatherThreads) im2col_kernel(const GatherArgs
     }
 }
 
-// The same through shared memory, one output row (b, ho) per block pass: the kh input rows it touches are copied
-// in first, channels packed and the horizontal padding as zeros, so that a thread's 16 source offsets are fixed
-// for all pixels of all rows and its loop has no bounds checks.  s_rows[kh][rowb].
-__global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(const GatherArgs a, const int Wx, const int rowb)
+// The same through shared memory, one output row (b, ho) per block pass.  The kh input rows it touches are copied
+// in first, channels packed, zeros around them (the padding).  A row of the patch matrix is then kh runs of kw * C
+// consecutive bytes, one from each input row, so sixteen output bytes are one to three unaligned 16-byte pieces of
+// shared memory: five words and four funnel shifts each.  A warp builds the same sixteen columns for 32 neighbouring
+// pixels: which runs they come from is uniform, and lanes that are stride * C bytes apart hit the banks at most two
+// deep (a byte at a time with the columns spread over the lanes, conflicts made the layer 96 us at 64 x 224 x 224 x 3,
+// four times what writing the matrix takes; 53 us this way).  The finished rows are assembled in shared memory and
+// leave as one bulk copy: they are consecutive in memory.
+struct RowsArgs {
+    int zero_left, rowb;      // bytes of zeros in front of a staged row (a multiple of 16, at least 16 + pad * C), bytes per staged row
+    int tile;                 // pixels assembled at a time
+};
+// One run's share of a unit (sixteen columns): which input row, the byte that would be the unit's column 0 relative to
+// the pixel's first byte in that row, and the columns that are this run's.
+struct alignas(32) Piece { uint32_t keep[4]; int row, off, last, pad; };      // last: 1 on a unit's last piece
+
+__global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(const GatherArgs a, const RowsArgs ra)
 {
-    extern __shared__ uint8_t s_rows[];
-    const int upr = a.units;
-    const int ppg = kGatherThreads / upr;
-    const int my_p = threadIdx.x / upr, k0 = (threadIdx.x - my_p * upr) << 4;
-    int off[16];
-    uint32_t keep[4] = {0u, 0u, 0u, 0u};                  // byte masks: columns beyond the reduction stay zero
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        const int k = k0 + e;
-        const int tap = k / a.C, c = k - tap * a.C;
-        const int i = tap / a.kw, j = tap - i * a.kw;
-        const bool valid = k < a.K;
-        off[e] = valid ? i * rowb + j * a.C + c : 0;      // offsets are relative to the pixel's first byte: 0 is always inside
-        if (valid) keep[e >> 2] |= 0xFFu << (8 * (e & 3));
-    }
-    const int64_t row_pitch = (int64_t)a.W * a.pix_pitch;
+    extern __shared__ __align__(32) uint8_t s_mem[];
+    uint8_t* const s_out = s_mem;                                          // [tile][ld_cols]
+    uint8_t* const s_rows = s_mem + (size_t)ra.tile * a.ld_cols;           // [kh][rowb]
+    Piece* const s_piece = reinterpret_cast<Piece*>(s_mem + ((size_t)ra.tile * a.ld_cols + (size_t)a.kh * ra.rowb + 31) / 32 * 32);      // in the order of the columns
+    __shared__ int s_base[16];                                             // per input row: where its column -pad starts in s_rows
+    __shared__ int s_first[kGatherThreads];                                // per unit: its first piece, -1 for zero columns
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int run = a.kw * a.C;
+    const int row_bytes = a.W * a.C;                                       // a staged row's own bytes
+    const int chunks = ra.rowb >> 4;
+    const bool dense = a.pix_pitch == a.C;
     const int rows_total = a.B * a.Ho;
+    if (tid < a.units) {
+        // a unit's pieces; in front of it lie as many pieces as whole units, and one more for every run that ended inside one
+        int k = 16 * tid, i = k / run, o = k - i * run;
+        int n = tid + min(i, a.kh - 1);
+        for (int j = 1; j <= min(i, a.kh - 1); ++j) n -= (j * run) % 16 == 0 ? 1 : 0;
+        s_first[tid] = i < a.kh ? n : -1;
+        for (int e = 0; e < 16 && i < a.kh; ++i, o = 0, ++n) {
+            const int len = min(run - o, 16 - e);
+            for (int j = 0; j < 4; ++j) {
+                const int lo = max(e - 4 * j, 0), hi = min(e + len - 4 * j, 4);
+                s_piece[n].keep[j] = hi > lo ? (0xFFFFFFFFu >> (8 * (4 - hi + lo))) << (8 * lo) : 0u;
+            }
+            s_piece[n].row = i; s_piece[n].off = o - e;
+            e += len;
+            s_piece[n].last = (e == 16 || i + 1 == a.kh) ? 1 : 0;
+        }
+    }
     for (int r = blockIdx.x; r < rows_total; r += gridDim.x) {
         const int b = r / a.Ho, ho = r - b * a.Ho;
         const int y0 = ho * a.stride - a.pad;
-        __syncthreads();                                  // the previous row's readers are done
-        for (int q = threadIdx.x; q < a.kh * Wx; q += kGatherThreads) {
-            const int i = q / Wx, xp = q - i * Wx;
-            const int y = y0 + i, x = xp - a.pad;
-            const bool in = (unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W;
-            const int8_t* src = a.act + (int64_t)b * a.H * row_pitch + (int64_t)y * row_pitch + (int64_t)x * a.pix_pitch;
-            uint8_t* dst = s_rows + i * rowb + xp * a.C;
-            for (int c = 0; c < a.C; ++c) dst[c] = in ? (uint8_t)__ldg(src + c) : (uint8_t)0;
+        __syncthreads();                                                   // the previous row's readers are done
+        if (dense) {
+            // rows of packed pixels: 16-byte granules of global memory to the same place inside a granule of shared memory
+            for (int q = tid; q < a.kh * chunks; q += kGatherThreads) {
+                const int i = q / chunks, j = q - i * chunks;
+                const int y = y0 + i;
+                const bool in_y = (unsigned)y < (unsigned)a.H;
+                const int8_t* row = a.act + (int64_t)(b * a.H + (in_y ? y : 0)) * row_bytes;
+                const int lead = (int)(reinterpret_cast<uintptr_t>(row) & 15);
+                const int first = 16 * j - ra.zero_left - lead;            // the granule's first byte, relative to the row
+                uint32_t v[4] = {0u, 0u, 0u, 0u};
+                if (in_y && first > -16 && first < row_bytes) {
+                    if (first >= 0 && first + 16 <= row_bytes) {
+                        const uint4 w = __ldg(reinterpret_cast<const uint4*>(row + first));
+                        v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
+                    } else {
+                        for (int e = 0; e < 16; ++e)
+                            if ((unsigned)(first + e) < (unsigned)row_bytes)
+                                v[e >> 2] |= (uint32_t)(uint8_t)__ldg(row + first + e) << (8 * (e & 3));
+                    }
+                }
+                *reinterpret_cast<uint4*>(s_rows + i * ra.rowb + 16 * j) = make_uint4(v[0], v[1], v[2], v[3]);
+                if (j == 0) s_base[i] = i * ra.rowb + ra.zero_left + lead - a.pad * a.C;
+            }
+        } else {
+            for (int q = tid; q < a.kh * ra.rowb; q += kGatherThreads) {
+                const int i = q / ra.rowb, at = q - i * ra.rowb - ra.zero_left;
+                const int y = y0 + i;
+                uint8_t v = 0;
+                if ((unsigned)y < (unsigned)a.H && (unsigned)at < (unsigned)row_bytes) {
+                    const int x = at / a.C;
+                    v = (uint8_t)__ldg(a.act + ((int64_t)(b * a.H + y) * a.W + x) * a.pix_pitch + (at - x * a.C));
+                }
+                s_rows[q] = v;
+                if (at == -ra.zero_left) s_base[i] = i * ra.rowb + ra.zero_left - a.pad * a.C;
+            }
         }
-        __syncthreads();
-        if (my_p < ppg) {
-            for (int wo = my_p; wo < a.Wo; wo += ppg) {
-                const uint8_t* base = s_rows + wo * a.stride * a.C;
+        for (int p0 = 0; p0 < a.Wo; p0 += ra.tile) {
+            const int np = min(ra.tile, a.Wo - p0);
+            const int groups = (np + 31) >> 5;
+            if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");       // the previous tile has left
+            __syncthreads();
+            int u = warp, g = 0;                                           // unit, group of 32 pixels
+            while (u >= a.units) { u -= a.units; ++g; }
+            while (g < groups) {
+                const int p = g * 32 + lane;
+                const int xoff = (p0 + min(p, np - 1)) * a.stride * a.C;
                 uint32_t out[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-                for (int e = 0; e < 16; ++e) out[e >> 2] |= (uint32_t)base[off[e]] << (8 * (e & 3));
-                *reinterpret_cast<uint4*>(a.cols + ((int64_t)r * a.Wo + wo) * a.ld_cols + k0) =
-                    make_uint4(out[0] & keep[0], out[1] & keep[1], out[2] & keep[2], out[3] & keep[3]);
+                for (int i = s_first[u]; i >= 0;) {                        // the same pieces for the whole warp
+                    const uint4 keep = *reinterpret_cast<const uint4*>(s_piece[i].keep);
+                    const int4 d = *reinterpret_cast<const int4*>(&s_piece[i].row);
+                    const int at = s_base[d.x] + d.y + xoff;
+                    const uint32_t* w = reinterpret_cast<const uint32_t*>(s_rows + (at & ~3));
+                    const uint32_t sh = (uint32_t)at * 8u;                 // (the shift counts modulo 32)
+                    out[0] |= __funnelshift_r(w[0], w[1], sh) & keep.x;
+                    out[1] |= __funnelshift_r(w[1], w[2], sh) & keep.y;
+                    out[2] |= __funnelshift_r(w[2], w[3], sh) & keep.z;
+                    out[3] |= __funnelshift_r(w[3], w[4], sh) & keep.w;
+                    i = d.z ? -1 : i + 1;
+                }
+                if (p < np) *reinterpret_cast<uint4*>(s_out + (size_t)p * a.ld_cols + 16 * u) = make_uint4(out[0], out[1], out[2], out[3]);
+                u += kGatherThreads / 32;
+                while (u >= a.units) { u -= a.units; ++g; }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncthreads();
+            if (tid == 0) {
+                const int8_t* dst = a.cols + ((int64_t)r * a.Wo + p0) * a.ld_cols;
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                             ::"l"(dst), "r"((uint32_t)__cvta_generic_to_shared(s_out)), "r"((uint32_t)(np * (int)a.ld_cols)) : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
         }
     }
+    if (tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 }  // namespace
@@ -125,13 +204,18 @@ cudaError_t launch_im2col(const int8_t* act, int B, int H, int W, int C, int64_t
     a.units = (int)(ld_cols >> 4);
     if (a.N == 0) return cudaSuccess;
     if (a.units > kGatherThreads) return cudaErrorInvalidValue;
-    // input rows in shared memory when they fit without opting in to more
-    const int Wx = (Wo - 1) * stride + kw;
-    const int rowb = (Wx * C + 15) & ~15;
-    const size_t smem = (size_t)kh * rowb + 16;
-    if (smem <= 48 * 1024) {
-        const int64_t blocks = std::min<int64_t>((int64_t)B * Ho, (int64_t)sm_count() * 8);
-        im2col_rows_kernel<<<(unsigned)blocks, kGatherThreads, smem, st>>>(a, Wx, rowb);
+    // input rows in shared memory when they fit without opting in to more, beside the tile that is assembled
+    RowsArgs ra;
+    auto up16 = [](int n) { return (n + 15) & ~15; };
+    ra.zero_left = up16(pad * C) + 16;
+    ra.rowb = ra.zero_left + 16 + up16(std::max(W, (Wo - 1) * stride + kw - pad) * C) + up16(pad * C) + 32;
+    ra.tile = (int)std::min<int64_t>(Wo, std::max<int64_t>(1, 20 * 1024 / ld_cols));
+    if (ra.tile < Wo && ra.tile >= 32) ra.tile &= ~31;
+    const size_t smem = ((size_t)ra.tile * ld_cols + (size_t)kh * ra.rowb + 31) / 32 * 32 + 32 + sizeof(Piece) * (size_t)(a.units + kh);
+    if (smem <= 46 * 1024) {
+        const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, 200 * 1024 / smem));
+        const int64_t blocks = std::min<int64_t>((int64_t)B * Ho, (int64_t)sm_count() * per_sm);
+        im2col_rows_kernel<<<(unsigned)blocks, kGatherThreads, smem, st>>>(a, ra);
         return cudaGetLastError();
     }
     const int ppg = kGatherThreads / a.units;

@@ -741,6 +741,32 @@ def test_first_layer_patch_matrix_and_gemm_match_oracle_conv(M, Cin, k, stride, 
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("C,kh,kw,stride,pad,B,H,W,ld,offset", [
+    (3, 7, 7, 2, 3, 1, 21, 70, 160, 0),        # more than one group of 32 pixels, the last one ragged
+    (3, 7, 7, 2, 3, 2, 9, 11, 160, 5),         # input that does not start on a 16-byte boundary
+    (1, 3, 3, 1, 1, 1, 6, 5, 16, 3),           # six runs of three bytes in a row's sixteen columns
+    (1, 2, 1, 1, 0, 1, 4, 4, 48, 0),           # runs of one byte, zero columns beyond a whole unit
+    (5, 3, 3, 3, 4, 1, 8, 300, 4096, 1),       # a tile of five pixels, padding wider than the image needs
+    (2, 16, 16, 8, 16, 1, 3, 3, 512, 0),       # the largest filter: mostly padding
+    (64, 3, 3, 1, 1, 1, 3, 33, 576, 0),        # runs longer than a unit
+])
+def test_patch_matrix_pieces(C, kh, kw, stride, pad, B, H, W, ld, offset):
+    """Bytes are copied, so they must be the oracle's; the bytes around the matrix stay as they were."""
+    import torch
+    g = synth.rng(92, C + H + W)
+    act = g.integers(-128, 128, size=(B, H, W, C), dtype=np.int8)
+    raw = torch.full((offset + act.size + 64,), 77, dtype=torch.int8, device="cuda")
+    raw[offset:offset + act.size] = torch.from_numpy(act.reshape(-1)).cuda()
+    ref = O.im2col(act, kh, kw, stride, pad, ld)
+    out = torch.full((ref.size + 256,), 99, dtype=torch.int8, device="cuda")
+    R.rmsmp_im2col_codes(raw.data_ptr() + offset, B, H, W, C, C, kh, kw, stride, pad, out[128:], ld)
+    torch.cuda.synchronize()
+    got = out.cpu().numpy()
+    assert np.array_equal(got[128:-128].reshape(ref.shape), ref)
+    assert (got[:128] == 99).all() and (got[-128:] == 99).all()
+
+
+@pytest.mark.gpu
 def test_patch_matrix_rejects_bad_arguments():
     import torch
     a = torch.zeros((1, 4, 4, 3), dtype=torch.int8, device="cuda")
