@@ -137,25 +137,40 @@ def lib() -> C.CDLL:
 
 
 def _dp(t):
-    """Device pointer of a torch tensor, or pass an int / None through."""
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return C.c_void_p(t)
-    return C.c_void_p(t.data_ptr())
+    """Device pointer of a torch tensor, or pass an int / None through (the argtypes make it a pointer)."""
+    if t is None or isinstance(t, int):
+        return t
+    return t.data_ptr()
 
 
 def _hp(a: np.ndarray):
-    return C.c_void_p(a.ctypes.data)
+    return a.ctypes.data
+
+
+_current_raw_stream = None
 
 
 def _stream(stream):
     if stream is None:
-        import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return _current_raw_stream() if _current_raw_stream is not None else _first_stream()
     if isinstance(stream, int):
-        return C.c_void_p(stream)
-    return C.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
+
+
+def _first_stream():
+    """The current stream through torch's public call, which also starts CUDA up.  From then on its handle is read
+    directly where this torch has the accessor: the public call builds a Stream object (3.4 us, a third of a small
+    layer's call; the accessor 0.2 us)."""
+    global _current_raw_stream
+    import torch
+    handle = torch.cuda.current_stream().cuda_stream
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw is not None and device is not None:
+        _current_raw_stream = lambda: raw(device())
+    else:
+        _current_raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+    return handle
 
 
 def _check(st: int, where: str):
