@@ -37,6 +37,9 @@ struct RowStats {             // scratch, 16 bytes per row
 // with A = mean |w|, A^2 <= 2 (c^2 + q); G = 2 (K + 16) u below leaves a factor of more than two.
 __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(const float* __restrict__ W, int K, RowStats out)
 {
+    pdl_wait();
+    pdl_trigger();
+    W = pdl_ordered(W);
     __shared__ double s_red[2][kStatThreads / 32];
     __shared__ float s_max[kStatThreads / 32];
     const int row = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -166,6 +169,8 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int M = a.M;
     const bool local = M <= kAssignSmemRows;
+    pdl_wait();
+    pdl_trigger();
     double* const var = local ? s_var : a.st.var;
     float* const err = local ? s_err : a.st.err;
     uint8_t* kind = a.blob + a.off_kind;
@@ -390,7 +395,8 @@ cudaError_t launch_assign_meta(const float* dW, const rmsmp_layer& L, const floa
     rs.var = static_cast<double*>(d_scratch);
     rs.err = reinterpret_cast<float*>(rs.var + M);
     rs.amax = rs.err + M;
-    row_stats_kernel<<<M, kStatThreads, 0, st>>>(dW, K, rs);
+    cudaError_t e = launch_dependent(row_stats_kernel, (unsigned)M, kStatThreads, 0, st, dW, K, rs);
+    if (e != cudaSuccess) return e;
     MetaArgs a;
     a.W = dW; a.K = K; a.st = rs;
     a.blob = blob; a.alpha = d_alpha ? d_alpha : rs.amax; a.scheme_out = d_scheme; a.bits_out = d_bits;
@@ -398,8 +404,7 @@ cudaError_t launch_assign_meta(const float* dW, const rmsmp_layer& L, const floa
     a.off_kind = L.off_kind; a.off_blocks = L.off_blocks;
     a.M = M; a.Cin = L.Cin; a.kh = L.kh; a.kw = L.kw; a.Cp = L.Cp; a.Kp = L.Kp;
     a.nP = L.nP; a.nF4 = L.nF4; a.n8 = L.n8; a.nblocks = L.nblocks; a.pot_mode = pot_mode;
-    assign_kernel<<<1, kAssignThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(assign_kernel, 1, kAssignThreads, 0, st, a);
 }
 
 }  // namespace rmsmp

@@ -93,6 +93,8 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
 {
     extern __shared__ uint32_t s_w[];                     // [tap][quad]: channel 4q+j in byte j
     const int taps = p.kh * p.kw, C = p.M;
+    pdl_wait();
+    pdl_trigger();
     {
         uint8_t* s_b = reinterpret_cast<uint8_t*>(s_w);
         for (int c = threadIdx.x; c < C; c += kDwThreads) {
@@ -283,10 +285,8 @@ cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
     }
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    if (variant == 1) depthwise_kernel<1><<<(unsigned)blocks, kDwThreads, smem, st>>>(p, strip);
-    else if (variant == 2) depthwise_kernel<2><<<(unsigned)blocks, kDwThreads, smem, st>>>(p, strip);
-    else depthwise_kernel<0><<<(unsigned)blocks, kDwThreads, smem, st>>>(p, strip);
-    return cudaGetLastError();
+    return launch_dependent(variant == 1 ? depthwise_kernel<1> : variant == 2 ? depthwise_kernel<2> : depthwise_kernel<0>, (unsigned)blocks,
+                            kDwThreads, smem, st, p, strip);
 }
 
 }  // namespace rmsmp

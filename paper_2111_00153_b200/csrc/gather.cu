@@ -26,6 +26,8 @@ __global__ void __launch_bounds__(kGatherThreads) im2col_kernel(const GatherArgs
 {
     // thread <-> (pixel of the block's current group, 16-byte piece of its row): fixed per thread; the pixel index
     // advances by whole groups; 32-bit index arithmetic (the host checks the counts)
+    pdl_wait();
+    pdl_trigger();
     const int upr = a.units;
     const int ppg = kGatherThreads / upr;                 // pixels per group (units <= kGatherThreads is checked by the host)
     const int my_p = threadIdx.x / upr, k0 = (threadIdx.x - my_p * upr) << 4;
@@ -111,6 +113,8 @@ __global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(const Gathe
             s_piece[n].last = (e == 16 || i + 1 == a.kh) ? 1 : 0;
         }
     }
+    pdl_wait();
+    pdl_trigger();
     for (int r = blockIdx.x; r < rows_total; r += gridDim.x) {
         const int b = r / a.Ho, ho = r - b * a.Ho;
         const int y0 = ho * a.stride - a.pad;
@@ -215,13 +219,11 @@ cudaError_t launch_im2col(const int8_t* act, int B, int H, int W, int C, int64_t
     if (smem <= 46 * 1024) {
         const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, 200 * 1024 / smem));
         const int64_t blocks = std::min<int64_t>((int64_t)B * Ho, (int64_t)sm_count() * per_sm);
-        im2col_rows_kernel<<<(unsigned)blocks, kGatherThreads, smem, st>>>(a, ra);
-        return cudaGetLastError();
+        return launch_dependent(im2col_rows_kernel, (unsigned)blocks, kGatherThreads, smem, st, a, ra);
     }
     const int ppg = kGatherThreads / a.units;
     const int64_t blocks = std::min<int64_t>((a.N + ppg - 1) / ppg, (int64_t)sm_count() * 16);
-    im2col_kernel<<<(unsigned)blocks, kGatherThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(im2col_kernel, (unsigned)blocks, kGatherThreads, 0, st, a);
 }
 
 }  // namespace rmsmp

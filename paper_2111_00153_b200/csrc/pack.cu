@@ -67,6 +67,7 @@ struct PackArgs {
 __global__ void __launch_bounds__(256) pack_kernel(PackArgs a)
 {
     extern __shared__ __align__(16) uint8_t s_code[];
+    pdl_wait();                                              // and no trigger: see launch_dependent
     const int p = blockIdx.x;
     const int r = reinterpret_cast<const int32_t*>(a.blob + a.off_perm)[p];
     const float alpha = reinterpret_cast<const float*>(a.blob + a.off_alpha)[r];
@@ -159,8 +160,7 @@ cudaError_t launch_pack(const float* dW, int conv_oihw, const rmsmp_layer& L, in
         cudaError_t e = cudaFuncSetAttribute(pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    pack_kernel<<<L.M, 256, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(pack_kernel, (unsigned)L.M, 256, smem, st, a);
 }
 
 // ------------------------------------------------------------------ metadata fetch
@@ -170,6 +170,8 @@ cudaError_t launch_pack(const float* dW, int conv_oihw, const rmsmp_layer& L, in
 __global__ void __launch_bounds__(256) fetch_mapped_kernel(uint8_t* __restrict__ dst, const uint8_t* __restrict__ src,
                                                            size_t bytes)
 {
+    pdl_wait();
+    pdl_trigger();
     const size_t n16 = bytes / 16;
     const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nthr = (size_t)gridDim.x * blockDim.x;
     // host memory: loads that bypass the caches, so that a reused slot is never read stale
@@ -183,8 +185,7 @@ cudaError_t launch_fetch_mapped(void* d_dst, const void* mapped_src, size_t byte
     size_t blocks = (bytes / 16 + 255) / 256;
     if (blocks > 64) blocks = 64;
     if (blocks == 0) blocks = 1;
-    fetch_mapped_kernel<<<(unsigned)blocks, 256, 0, st>>>(static_cast<uint8_t*>(d_dst), static_cast<const uint8_t*>(mapped_src), bytes);
-    return cudaGetLastError();
+    return launch_dependent(fetch_mapped_kernel, (unsigned)blocks, 256, 0, st, static_cast<uint8_t*>(d_dst), static_cast<const uint8_t*>(mapped_src), bytes);
 }
 
 // ------------------------------------------------------------------ unpack (parity/debug)
@@ -232,6 +233,9 @@ cudaError_t launch_unpack(const rmsmp_layer& L, const uint8_t* blob, int8_t* val
 __global__ void __launch_bounds__(256) expand_kernel(const uint8_t* __restrict__ blob, rmsmp_layer L,
                                                      int8_t* __restrict__ wexp)
 {
+    pdl_wait();
+    pdl_trigger();
+    blob = pdl_ordered(blob);
     const int chunks = L.Kp >> 5;
     const int64_t total = (int64_t)L.M * chunks;
     const int32_t* slot = reinterpret_cast<const int32_t*>(blob + L.off_slot);
@@ -273,8 +277,7 @@ cudaError_t launch_expand(const rmsmp_layer& L, const uint8_t* blob, int8_t* wex
     const int64_t total = (int64_t)L.M * (L.Kp >> 5);
     int64_t blocks = (total + 255) / 256;
     if (blocks > (int64_t)sm_count() * 8) blocks = (int64_t)sm_count() * 8;
-    expand_kernel<<<(unsigned)blocks, 256, 0, st>>>(blob, L, wexp);
-    return cudaGetLastError();
+    return launch_dependent(expand_kernel, (unsigned)blocks, 256, 0, st, blob, L, wexp);
 }
 
 // ------------------------------------------------------------------ activation quantizer
@@ -303,6 +306,9 @@ __global__ void __launch_bounds__(256) quantize_act_kernel(const float* __restri
 {
     const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     const size_t nthr = (size_t)gridDim.x * blockDim.x;
+    pdl_wait();
+    pdl_trigger();
+    x = pdl_ordered(x);
     if (vec) {
         // A warp takes 1024 consecutive values per step: eight 128-bit loads per lane, each
         // instruction covering 512 contiguous bytes, then eight 32-bit stores of 128 contiguous
@@ -349,8 +355,7 @@ cudaError_t launch_quantize_act(const float* x, size_t count, float alpha, int k
     const size_t cap = (size_t)sm_count() * 32;
     if (blocks > cap) blocks = cap;
     if (blocks == 0) blocks = 1;
-    quantize_act_kernel<<<(unsigned)blocks, 256, 0, st>>>(x, count, alpha, kind, codes, vec);
-    return cudaGetLastError();
+    return launch_dependent(quantize_act_kernel, (unsigned)blocks, 256, 0, st, x, count, alpha, kind, codes, vec);
 }
 
 }  // namespace rmsmp

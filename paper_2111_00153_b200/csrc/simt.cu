@@ -97,6 +97,8 @@ __device__ __forceinline__ int shiftadd32(const uint4& c, const uint32_t a[8], i
 template <bool SHIFTADD>
 __global__ void __launch_bounds__(256) rowwarp_kernel(Problem p)
 {
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -190,9 +192,7 @@ cudaError_t launch_simt(const Problem& p, bool shiftadd, cudaStream_t st)
     int64_t warps = ngroups * p.M;
     int64_t blocks = (warps + 7) / 8;
     if (blocks > (int64_t)sm_count() * 8) blocks = (int64_t)sm_count() * 8;
-    if (shiftadd) rowwarp_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(p);
-    else rowwarp_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(shiftadd ? rowwarp_kernel<true> : rowwarp_kernel<false>, (unsigned)blocks, 256, 0, st, p);
 }
 
 // ------------------------------------------------------------------ grouped small-batch launch
@@ -329,6 +329,9 @@ template <int NT>
 __global__ void __launch_bounds__(256, 2) grouped_kernel(const uint8_t* __restrict__ gtable, int use_smem)
 {
     extern __shared__ __align__(16) uint8_t s_table[];
+    pdl_wait();
+    pdl_trigger();
+    gtable = pdl_ordered(gtable);
     const uint8_t* table = gtable;
     if (use_smem) {
         const int n16 = reinterpret_cast<const GroupedTable*>(gtable)->bytes >> 4;
@@ -521,6 +524,9 @@ __device__ __forceinline__ void stream_finish(const StreamItem& it, int lane, in
 __global__ void __launch_bounds__(256, 2) grouped_stream_kernel(const uint8_t* __restrict__ gtable, int use_smem)
 {
     extern __shared__ __align__(16) uint8_t s_table[];
+    pdl_wait();
+    pdl_trigger();
+    gtable = pdl_ordered(gtable);
     const uint8_t* table = gtable;
     if (use_smem) {
         const int n16 = reinterpret_cast<const GroupedTable*>(gtable)->bytes >> 4;
@@ -616,9 +622,7 @@ cudaError_t launch_grouped(const uint8_t* d_table, size_t table_bytes, int64_t t
         if (e != cudaSuccess) return e;
         attr_done[dev] = true;
     }
-    if (nt == 1) grouped_stream_kernel<<<(unsigned)blocks, 256, smem, st>>>(d_table, use_smem);
-    else grouped_kernel<kTok><<<(unsigned)blocks, 256, smem, st>>>(d_table, use_smem);
-    return cudaGetLastError();
+    return launch_dependent(nt == 1 ? grouped_stream_kernel : grouped_kernel<kTok>, (unsigned)blocks, 256, smem, st, d_table, use_smem);
 }
 
 }  // namespace rmsmp

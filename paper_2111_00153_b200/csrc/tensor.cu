@@ -275,6 +275,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait();                                           // and no trigger: see launch_dependent
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
 
@@ -1124,8 +1125,10 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
     static bool attr_set[4][2][3][kMaxDevices] = {};
     if (!ensure_smem_attr(reinterpret_cast<const void*>(fn), kSmemLimit, attr_set[mode][i2][io])) return RMSMP_ERR_CUDA;
     const int grid = (int)std::min<int64_t>(c.ntiles, sm_count());
-    fn<<<grid, kThreads, c.smem_bytes, st>>>(p, c, mp);
-    if (cudaGetLastError() != cudaSuccess) return RMSMP_ERR_CUDA;
+    if (launch_dependent(fn, (unsigned)grid, kThreads, c.smem_bytes, st, p, c, mp) != cudaSuccess) {
+        cudaGetLastError();
+        return RMSMP_ERR_CUDA;
+    }
     return RMSMP_OK;
 }
 

@@ -230,6 +230,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     __syncthreads();
     cluster_sync_all();                                   // both CTAs' barriers exist before anyone signals the peer
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    pdl_wait();                                           // and no trigger: see launch_dependent
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
 
@@ -502,11 +503,13 @@ rmsmp_status launch_pair(const Problem& p, cudaStream_t st)
     lc.blockDim = dim3(kThreads2, 1, 1);
     lc.dynamicSmemBytes = c.smem_bytes;
     lc.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // as launch_dependent
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
-    lc.numAttrs = 1;
+    lc.numAttrs = 2;
     if (cudaLaunchKernelEx(&lc, pair_kernel, p, c, mp) != cudaSuccess) {
         cudaGetLastError();
         return RMSMP_ERR_CUDA;

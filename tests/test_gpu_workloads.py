@@ -462,3 +462,68 @@ def test_grouped_tensor_launches_in_a_row_see_the_inputs_of_their_turn():
         for k, ((acc_ref, y_ref), y) in enumerate(zip(refs, outs[t])):
             want = np.roll(y_ref, t, axis=0)
             assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32)), (t, k)
+
+
+@pytest.mark.parametrize("M,K,N", [(128, 256, 8), (300, 1024, 100), (512, 2304, 128)])
+def test_calls_in_a_row_on_the_same_buffers_are_ordered(M, K, N):
+    """Kernels are launched as programmatic dependents: a call may be placed while the one in front still runs, so
+    every call of a chain that keeps rewriting the same buffers must still see what the calls in front of it wrote
+    (weights packed on both routes, expanded, activations quantized, both tensor paths, the re-quantizing epilogue).
+    Codes and sums are integers and an output is one multiply: the chain must equal the synchronised calls bit for bit."""
+    import torch
+    g = synth.rng(95, M)
+    sets = []
+    for _ in range(2):
+        W = synth.weights_normal(g, (M, K))
+        scheme, bits = O.assign_rows(W, (60, 35, 5))
+        x = synth.act_halfnormal(g, (N, K))
+        sets.append((W, scheme, bits, synth.alpha_rows(W), torch.from_numpy(W).cuda(), torch.from_numpy(x).cuda()))
+    layer = R.rmsmp_layer_init_ratio(M, K, 1, 1, (60, 35, 5))
+    packed = torch.zeros(layer.packed_bytes, dtype=torch.uint8, device="cuda")
+    scratch = torch.zeros(R.rmsmp_assign_scratch_bytes(M), dtype=torch.uint8, device="cuda")
+    ws = torch.zeros(R.rmsmp_workspace_bytes(layer), dtype=torch.int8, device="cuda")
+    codes = torch.zeros((N, K), dtype=torch.int8, device="cuda")
+    rq = torch.zeros((N, (M + 15) // 16 * 16), dtype=torch.int8, device="cuda")
+    y = torch.zeros((N, M), dtype=torch.float32, device="cuda")
+    arr = R.make_gemm_items([(layer, packed, codes, N, K, float(np.float32(3.0) / np.float32(15.0)), y, M, None, 1)])
+    table = torch.empty(R.rmsmp_grouped_plan_bytes(arr), dtype=torch.uint8, device="cuda")
+    plan = R.rmsmp_gemm_grouped_prepare(arr, R.OUT_NM, table)
+
+    def chain(i, wait):
+        out = []
+        _, scheme, bits, alpha, dW, dx = sets[i & 1]
+        if i & 2:
+            ref_layer = R.rmsmp_layer_init(M, K, 1, 1, scheme, bits)
+            R.rmsmp_quantize_pack(dW, R.W_LINEAR, ref_layer, scheme, bits, alpha, R.POT_NEAREST, packed)
+        else:
+            R.rmsmp_assign_quantize_pack(dW, R.W_LINEAR, layer, (60, 35, 5), None, R.POT_NEAREST, packed, scratch)
+        wait()
+        step = R.rmsmp_quantize_act(dx, N * K, 3.0, R.ACT_U4, codes)
+        wait()
+        R.rmsmp_gemm_grouped_launch(plan)
+        wait()
+        out.append(y.clone())
+        R.rmsmp_expand_weights(layer, packed, ws)
+        wait()
+        R.rmsmp_gemm_workspace(layer, packed, ws, codes, N, K, step, y, M)
+        wait()
+        out.append(y.clone())
+        R.rmsmp_gemm(layer, packed, codes, N, K, step, y, M)
+        wait()
+        out.append(y.clone())
+        R.rmsmp_gemm_workspace_requant(layer, packed, ws, codes, N, K, step, 0.5, R.ACT_U4, rq, rq.shape[1])
+        wait()
+        out.append(rq.clone())
+        return out
+    want = [chain(i, torch.cuda.synchronize) for i in range(4)]
+    for i in range(4):
+        W, scheme, bits, alpha, _, dx = sets[i & 1]
+        c_ref, st_ref = O.quantize_act(dx.cpu().numpy(), 3.0, O.ACT_U4)
+        y_ref = O.layer_linear(W, scheme, bits, alpha, c_ref, st_ref)[-1]
+        for k in range(3):
+            assert np.array_equal(want[i][k].cpu().numpy().view(np.uint32), np.asarray(y_ref).reshape(N, M).view(np.uint32))
+    torch.cuda.synchronize()
+    got = [(i & 3, chain(i & 3, lambda: None)) for i in range(24)]
+    torch.cuda.synchronize()
+    for i, out in got:
+        assert all(torch.equal(a, b) for a, b in zip(out, want[i]))
