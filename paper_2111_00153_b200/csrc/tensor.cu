@@ -217,6 +217,31 @@ __device__ __forceinline__ void fill_resident_weights(const Problem& p, const Te
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the MMAs read these bytes through the async proxy
 }
 
+// ------------------------------------------------------------------ re-quantizing epilogue
+
+constexpr float kRqMagic = 12582912.0f;          // 1.5 * 2^23: adding it rounds to an integer, half to even
+
+// Two fp32 values per instruction.
+__device__ __forceinline__ uint64_t f32x2(float a, float b)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ void f32x2_split(uint64_t d, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d)); }
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// Four accumulator columns of the warp's 32 lanes.
+__device__ __forceinline__ void tmem_ld_four(uint32_t taddr, uint32_t (&v)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n\ttcgen05.wait::ld.sync.aligned;"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr) : "memory");
+}
+
 // ------------------------------------------------------------------ the kernel
 
 // kM2: a tile covers two row blocks (TensorCfg::m2), compiled separately so that the common form keeps its registers.
@@ -702,33 +727,52 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                         const bool tail = cfg.tail_rows && (c == (cfg.npix >> 5));
                         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                         __syncwarp();
-                        // pass 1, branch-free so that the 32 dependent chains interleave: the division-free
-                        // code of every value, and one bit per value whose code the division must decide
-                        // (scaled value u = acc * g with g = scale / alpha * Q folded into one factor: a few
-                        // ulps from the defining chain of roundings, far inside the 1e-4 guard band)
-                        uint32_t undecided = rq_fast.ok ? 0u : 0xffffffffu;
-                        const float g = __fmul_rn(__fmul_rn(scale, rq_fast.r), rq_fast.q);
-                        const float u_lo = __fmul_rn(rq_fast.lo, rq_fast.q), u_hi = rq_fast.q;
+                        // t = the clipped value on 0..1 from one saturating fused operation, u = t * range + low; adding
+                        // 1.5 * 2^23 in the same operation as that product rounds u, and the same product again with the
+                        // rounded value taken off says how far u was from it.  The defining chain and this one are a
+                        // handful of roundings of relative size 2^-24 of at most 15 apart (< 8e-6), so a value at least
+                        // 1e-5 away from every boundary k + 1/2 has the same code.  The largest remainder of a lane's
+                        // values decides about the second pass (one chunk of 32 x 32 in fifty has a value to decide again).
+                        const float range = p.rq_kind == RMSMP_ACT_U4 ? 15.0f : 14.0f, low = p.rq_kind == RMSMP_ACT_U4 ? 0.0f : -7.0f;
+                        const float bias = p.rq_kind == RMSMP_ACT_U4 ? 0.0f : 0.5f;
+                        const float g = __fmul_rn(__fmul_rn(scale, rq_fast.r), p.rq_kind == RMSMP_ACT_U4 ? 1.0f : 0.5f);
+                        const bool fast = rq_fast.ok && fabsf(g) <= 1e20f;
+                        const uint64_t range2 = f32x2(range, range), magic2 = f32x2(kRqMagic + low, kRqMagic + low), minus2 = f32x2(-1.0f, -1.0f);
+                        uint32_t again = fast ? 0u : 0xFFu;              // bit i: a value of columns 4i .. 4i + 3 has to be decided again
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const float kMagic = 12582912.0f;
-                            float u = __fmul_rn(__int2float_rn((int)v[j] >> shift), g);
-                            u = fminf(fmaxf(u, u_lo), u_hi);
-                            const float sgm = __fadd_rn(u, kMagic);
-                            const float dev = __fsub_rn(u, __fsub_rn(sgm, kMagic));
-                            undecided |= (fabsf(dev) <= 0.4999f ? 0u : 1u) << j;
-                            asm volatile("st.shared.u8 [%0], %1;" ::"r"(my_stage + j * 32 + lane), "r"(__float_as_uint(sgm)) : "memory");
+                        for (int i = 0; i < 8; ++i) {
+                            float far = 0.0f;
+#pragma unroll
+                            for (int j = 4 * i; j < 4 * i + 4; j += 2) {
+                                const uint64_t t2 = f32x2(__saturatef(__fmaf_rn(__int2float_rn((int)v[j] >> shift), g, bias)),
+                                                          __saturatef(__fmaf_rn(__int2float_rn((int)v[j + 1] >> shift), g, bias)));
+                                const uint64_t s2 = fma_f32x2(t2, range2, magic2);
+                                const uint64_t d2 = fma_f32x2(t2, range2, fma_f32x2(s2, minus2, magic2));
+                                float s0, s1, d0, d1;
+                                f32x2_split(s2, s0, s1);
+                                f32x2_split(d2, d0, d1);
+                                asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(far) : "f"(d0), "f"(d1));
+                                asm volatile("st.shared.u8 [%0], %1;" ::"r"(my_stage + j * 32 + lane), "r"(__float_as_uint(s0)) : "memory");
+                                asm volatile("st.shared.u8 [%0], %1;" ::"r"(my_stage + j * 32 + 32 + lane), "r"(__float_as_uint(s1)) : "memory");
+                            }
+                            again |= far > 0.49999f ? 1u << i : 0u;
                         }
-                        // pass 2, rare: those values again by the definition
-                        while (undecided) {
-                            const int j = __ffs(undecided) - 1;
-                            undecided &= undecided - 1;
-                            uint32_t a = 0;
-#pragma unroll
-                            for (int jj = 0; jj < 32; ++jj) a = (jj == j) ? v[jj] : a;     // registers cannot be indexed
-                            const float y = __fmul_rn(__int2float_rn((int)a >> shift), scale);
-                            const uint32_t code = (uint32_t)act_code(y, p.rq_alpha, p.rq_kind);
-                            asm volatile("st.shared.u8 [%0], %1;" ::"r"(my_stage + j * 32 + lane), "r"(code) : "memory");
+                        // Those columns again by the definition, from tensor memory (the whole warp takes every step: the
+                        // load is a warp-wide instruction).  This code is small and touches none of the registers above,
+                        // so that its mere presence costs nothing.
+                        again = __reduce_or_sync(0xffffffffu, again);
+                        while (again) {
+                            const int j0 = 4 * (__ffs(again) - 1);
+                            again &= again - 1;
+                            uint32_t w[4];
+                            tmem_ld_four(taddr + c * 32 + j0, w);
+#pragma unroll 1
+                            for (int j = j0; j < j0 + 4; ++j) {
+                                const float y = __fmul_rn(__int2float_rn((int)w[0] >> shift), scale);
+                                asm volatile("st.shared.u8 [%0], %1;" ::"r"(my_stage + j * 32 + lane), "r"((uint32_t)act_code(y, p.rq_alpha, p.rq_kind)) : "memory");
+                                w[0] = w[1]; w[1] = w[2]; w[2] = w[3];
+                            }
+                            __syncwarp();
                         }
                         fence_proxy_async_smem();
                         __syncwarp();
@@ -822,13 +866,16 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             for (int c = cfirst; c < nchunks; c += 2 * cstride) {
                 const int c1 = c + cstride, c2 = c + 2 * cstride;
                 const bool more1 = c1 < nchunks;
-                if (more1) tmem_ld_issue(taddr + c1 * 32, vb); else release_tmem();
+                // (a re-quantizing chunk may read its accumulators again: the buffer is handed back after it)
+                if (more1) tmem_ld_issue(taddr + c1 * 32, vb); else if (!kRQ) release_tmem();
                 emit(va, c);
+                if (!more1 && kRQ) release_tmem();
                 if (more1) {
                     tmem_ld_wait(vb);
                     const bool more2 = c2 < nchunks;
-                    if (more2) tmem_ld_issue(taddr + c2 * 32, va); else release_tmem();
+                    if (more2) tmem_ld_issue(taddr + c2 * 32, va); else if (!kRQ) release_tmem();
                     emit(vb, c1);
+                    if (!more2 && kRQ) release_tmem();
                     if (more2) tmem_ld_wait(va);
                 }
             }
