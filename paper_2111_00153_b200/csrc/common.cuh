@@ -150,6 +150,9 @@ bool encode_act_maps_4(const Problem& p, int bk, int th, int tb, void* maps4);
 // two-CTA form of the workspace mode (tensor2.cu): false if it cannot, or should not, run this problem
 bool pair_supported(const Problem& p);
 rmsmp_status launch_pair(const Problem& p, cudaStream_t st);
+// problems that do not fill the chip: narrow tiles, the reduction shared by a cluster (split.cu)
+bool split_supported(const Problem& p);
+rmsmp_status launch_split(const Problem& p, cudaStream_t st);
 
 // ---- activation boxes of the tensor-core kernels ----
 // A stride-2 convolution reads, for one filter tap, every second pixel of every second input row.

@@ -1,0 +1,484 @@
+// Tensor-core contraction for problems that do not fill the chip: few pixels or tokens, a few row blocks, often a
+// long reduction (a network's late layers for one image, a small linear layer).  The persistent kernel gives such a
+// problem two to sixty tiles, one CTA each, and every CTA walks the whole reduction alone (18 k-blocks: 12 us, 36:
+// 16.6 us, with 2 and 4 of 148 SMs busy).  Here the tiles are narrow (128 rows x 16 to 128 pixels) and the reduction
+// of a tile is shared by the CTAs of a cluster (1, 2, 4 or 8): each multiplies its k-blocks into its own tensor
+// memory, sends every eight columns of its int32 sums to the CTA that owns them through distributed shared memory,
+// and the owner adds the parts and writes the output.  Integer sums: the order does not matter.
+//
+// Warp roles (448 threads): warp 0 fetches the activation boxes (TMA, filter taps as in the persistent kernel); warp 1
+// allocates tensor memory and issues the MMAs; warps 2-13 make the A operand -- with a workspace, warp 2 fetches the
+// expanded rows by TMA; without one, three groups of four warps take the k-blocks in turn, a thread per row, and
+// expand the codes into the swizzled stage -- and are the
+// epilogue afterwards, three warps per tensor-memory quarter.  The ring is as deep as the CTA's share of the
+// reduction where that fits, so that all copies are in flight at once.
+// Every mbarrier wait is bounded; when one runs out RMSMP_ERR_TIMEOUT is recorded, the roles leave their loops, and
+// the cluster barriers are still met by every thread.  No load uses cluster multicast.
+#include <cuda.h>
+#include <algorithm>
+#include <cstring>
+#include "common.cuh"
+#include "decode.cuh"
+#include "actq.cuh"
+#include "ptx.cuh"
+#include "tmap.cuh"
+
+namespace rmsmp {
+
+namespace {
+
+constexpr int kSplitThreads = 448;
+constexpr int kSplitFirst = 2;                   // first of the twelve working warps
+constexpr int kSplitRing = 8;
+constexpr int kSplitSmem = 200 * 1024;
+
+struct SplitCfg {
+    int tb, th, npix;        // images / output rows / pixels per tile (the last tile of an image or batch may have fewer)
+    int n_pad;               // npix rounded up to 16: accumulator columns
+    int tiles_per_image;     // > 0: a tile is th rows of one image
+    int ntn;                 // pixel tiles
+    int cpt, nkb;            // bk-channel chunks per tap, k-blocks
+    int last_ksteps;         // 32-code steps in the last chunk of a tap
+    int S;                   // CTAs that share a tile's reduction
+    int bk, a_bytes, b_bytes, nst;
+    int tmem_cols;
+    int cpo;                 // groups of eight columns per owner
+    int pre;                 // 1: the A operand comes expanded from a workspace
+    uint32_t idesc, tx_b, smem_bytes;
+};
+
+struct SplitMaps { CUtensorMap act[4], wexp; };
+
+__device__ __forceinline__ uint32_t split_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t split_map(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void split_ld8(uint32_t taddr, uint32_t (&v)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\ttcgen05.wait::ld.sync.aligned;"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void split_sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
+// kRQ: the epilogue writes the next layer's activation codes.  kPre: the A operand comes expanded from a workspace
+// (registers for two CTAs per SM, so that the next launch's set-up fits beside this one).
+template <int kRQ, int kPre>
+__global__ void __launch_bounds__(kSplitThreads, kPre ? 2 : 1)
+split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitMaps maps)
+{
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t sA = smem_base, sB = sA + cfg.nst * cfg.a_bytes;
+    const uint32_t sRed = sB + cfg.nst * cfg.b_bytes;            // S > 1: [source CTA][column][128 rows] int32
+    __shared__ __align__(8) uint64_t s_full[kSplitRing], s_empty[kSplitRing], s_tfull;
+    __shared__ uint32_t s_tmem_base;
+    __shared__ int s_abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cfg.S > 1 ? split_rank() : 0u;
+    const uint32_t tile = blockIdx.x / (uint32_t)cfg.S;
+    const int nt = (int)(tile / (uint32_t)p.nblocks), blk = (int)(tile - (uint32_t)nt * (uint32_t)p.nblocks);
+    const int kb0 = (int)rank * cfg.nkb / cfg.S, n_kb = ((int)rank + 1) * cfg.nkb / cfg.S - kb0;      // this CTA's k-blocks
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < cfg.nst; ++s) {
+            mbar_init(smem_u32(&s_full[s]), kPre ? 2 : 5);     // activation producer, and weight producer or the four warps of a group
+            mbar_init(smem_u32(&s_empty[s]), 1);
+        }
+        mbar_init(smem_u32(&s_tfull), 1);
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(cfg.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (cfg.S > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");      // this CTA runs: its shared memory may be written
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t tmem_base = s_tmem_base;
+    volatile int* abort_flag = &s_abort;
+
+    int b0, h0;
+    if (cfg.tiles_per_image) { b0 = nt / cfg.tiles_per_image; h0 = (nt - b0 * cfg.tiles_per_image) * cfg.th; }
+    else { b0 = nt * cfg.tb; h0 = 0; }
+    auto full = [&](int s) { return smem_u32(&s_full[s]); };
+    auto empty = [&](int s) { return smem_u32(&s_empty[s]); };
+
+    if (warp == 0 || (warp == kSplitFirst && kPre)) {
+        // ---------------------------------------------------------- TMA producers
+        if (lane == 0) {
+            int tap = kb0 / cfg.cpt, cc = kb0 - tap * cfg.cpt;
+            int ti = tap / p.kw, tj = tap - ti * p.kw;
+            int s = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int i = 0; i < n_kb; ++i) {
+                if (i >= cfg.nst && !mbar_wait(empty(s), ph ^ 1, abort_flag)) { ok = false; break; }
+                if (warp == 0) {
+                    mbar_arrive_expect_tx(full(s), cfg.tx_b);
+                    const TapBox t = tap_box(p, h0, ti, tj);
+                    tma_load_4d(sB + s * cfg.b_bytes, &maps.act[t.map], full(s), cc * cfg.bk, t.x, t.y, b0);
+                } else {
+                    mbar_arrive_expect_tx(full(s), (uint32_t)cfg.a_bytes);
+                    tma_load_2d(sA + s * cfg.a_bytes, &maps.wexp, full(s), tap * p.Cp + cc * cfg.bk, blk * kBlockRows);
+                }
+                if (++s == cfg.nst) { s = 0; ph ^= 1; }
+                if (++cc == cfg.cpt) { cc = 0; ++tap; if (++tj == p.kw) { tj = 0; ++ti; } }
+            }
+            if (!ok)
+                for (int i = 0; i < 200; ++i) __nanosleep(1000);   // let copies in flight land
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ---------------------------------------------------------- MMA issuer
+        if (lane == 0) {
+            const uint64_t da = smem_desc_kmajor(sA, cfg.bk), db = smem_desc_kmajor(sB, cfg.bk);
+            const uint32_t hi = (uint32_t)(da >> 32), a_step = (uint32_t)cfg.a_bytes >> 4, b_step = (uint32_t)cfg.b_bytes >> 4;
+            int s = 0, cc = kb0 % cfg.cpt;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int i = 0; i < n_kb; ++i) {
+                if (!mbar_wait(full(s), ph, abort_flag)) { ok = false; break; }
+                tc_fence_after();
+                const int ksteps = cc == cfg.cpt - 1 ? cfg.last_ksteps : cfg.bk >> 5;
+                const uint32_t a_lo = (uint32_t)da + s * a_step, b_lo = (uint32_t)db + s * b_step;
+                for (int k = 0; k < ksteps; ++k)
+                    mma_i8_halves(tmem_base, a_lo + 2 * k, b_lo + 2 * k, hi, cfg.idesc, (i | k) ? 1u : 0u);
+                mma_commit(empty(s));
+                if (++s == cfg.nst) { s = 0; ph ^= 1; }
+                if (++cc == cfg.cpt) cc = 0;
+            }
+            if (ok) mma_commit(smem_u32(&s_tfull));
+        }
+        __syncwarp();
+    } else if (!kPre) {
+        // ---------------------------------------------------------- expanders
+        const int grp = (warp - kSplitFirst) >> 2;
+        // A thread expands one row, in original order: eight neighbouring lanes store to eight different swizzle phases.
+        // (In packed order a warp decodes one kind only, but its lanes' rows collide in the banks; 2 % slower.  Against
+        // the workspace form this costs about 2.3 us a launch, the way from the row's place to its first codes to the
+        // first stage, and 0.1 to 0.2 us a k-block.)
+        const int row = ((warp - kSplitFirst) & 3) * 32 + lane, m_row = blk * kBlockRows + row;
+        int kind = -1;
+        const uint8_t* src = p.q4;
+        if (m_row < p.M) {
+            kind = p.kind[m_row];
+            const int packed = __ldg(p.slot + m_row);
+            src = kind == kFixed8 ? p.q8 + (size_t)(packed - p.nP - p.nF4) * p.Kp : p.q4 + (size_t)packed * (p.Kp >> 1);
+        }
+        const uint32_t swz = cfg.bk == 128 ? (uint32_t)(row & 7) : (uint32_t)((row >> 1) & 3);
+        const uint32_t row_off = (uint32_t)row * (uint32_t)cfg.bk;
+        // The codes of a k-block are in registers before its turn comes: the next one's are loaded as soon as this one's
+        // are expanded, so that the trip to L2 passes during the other groups' turns.
+        const bool eight = kind == kFixed8;
+        uint4 raw[8];
+        auto fetch_pos = [&](int i, int& ksteps) -> const uint4* {
+            const int kb = kb0 + i, tap = kb / cfg.cpt, cc = kb - tap * cfg.cpt;
+            const int koff = tap * p.Cp + cc * cfg.bk;
+            ksteps = i >= n_kb ? 0 : (cc == cfg.cpt - 1 ? cfg.last_ksteps : cfg.bk >> 5);
+            return reinterpret_cast<const uint4*>(src + (eight ? koff : koff >> 1));
+        };
+        auto pieces_of = [&](int ksteps) { return kind < 0 ? 0 : (eight ? 2 * ksteps : ksteps); };      // 16-byte pieces of a row
+        int ksteps;
+        {
+            const uint4* q = fetch_pos(grp, ksteps);
+            const int pieces = pieces_of(ksteps);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) raw[u] = u < pieces ? __ldg(q + u) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        for (int i = grp; i < n_kb; i += 3) {
+            const int s = i % cfg.nst;
+            int next_ksteps;
+            const uint4* q = fetch_pos(i + 3, next_ksteps);
+            const int next_pieces = pieces_of(next_ksteps);
+            if (i >= cfg.nst && !mbar_wait_warp(empty(s), ((i / cfg.nst) & 1) ^ 1, abort_flag)) break;
+            const uint32_t dst = sA + s * cfg.a_bytes + row_off;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (u < ksteps) {
+                    uint32_t w[8];
+                    if (kind == kPoT4) {
+                        expand_pot_chunk(raw[u], w);
+                    } else if (kind == kFixed4) {
+                        expand_fixed4_chunk_x16(raw[u], w);
+                    } else {
+                        w[0] = raw[2 * u].x; w[1] = raw[2 * u].y; w[2] = raw[2 * u].z; w[3] = raw[2 * u].w;
+                        w[4] = raw[2 * u + 1].x; w[5] = raw[2 * u + 1].y; w[6] = raw[2 * u + 1].z; w[7] = raw[2 * u + 1].w;
+                    }
+                    __syncwarp();
+                    split_sts128(dst + (((uint32_t)(2 * u) ^ swz) << 4), w[0], w[1], w[2], w[3]);
+                    split_sts128(dst + (((uint32_t)(2 * u + 1) ^ swz) << 4), w[4], w[5], w[6], w[7]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (u < next_pieces) raw[u] = __ldg(q + u);
+            ksteps = next_ksteps;
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full(s));
+        }
+        __syncwarp();
+    }
+
+    // -------------------------------------------------------------- epilogue
+    const int quarter = warp & 3, rank3 = (warp - kSplitFirst) >> 2;       // tensor-memory lanes; which of the quarter's three warps
+    const int m = blk * kBlockRows + quarter * 32 + lane;
+    const bool worker = warp >= kSplitFirst, row_ok = worker && m < p.M;
+    int64_t n0;
+    int nvalid;
+    if (cfg.tiles_per_image) {
+        n0 = ((int64_t)b0 * p.Ho + h0) * p.Wo;
+        nvalid = min(cfg.th, p.Ho - h0) * p.Wo;
+    } else {
+        n0 = (int64_t)nt * cfg.npix;
+        nvalid = (int)min((int64_t)cfg.npix, p.N - n0);
+    }
+    float scale = 0.0f;
+    int shift = 0;
+    if (row_ok) {
+        scale = __fmul_rn(__ldg(p.wstep + m), p.act_step);
+        shift = (!kPre && __ldg(p.kind + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
+    }
+    const ActFast rq = act_fast_setup(kRQ ? p.rq_alpha : 1.0f, kRQ ? p.rq_kind : 0);
+    // the finished sum of this lane's row at column j of the tile
+    auto put = [&](int j, int sum) {
+        const int a = sum >> shift;
+        const float y = __fmul_rn(__int2float_rn(a), scale);
+        const int64_t n = n0 + j;
+        if (kRQ) {
+            p.rq_codes[n * p.ld_codes + m] = (int8_t)act_code_exact(y, p.rq_alpha, p.rq_kind, rq);
+        } else {
+            const int64_t o = p.out_mn ? (int64_t)m * p.ld_out + n : n * p.ld_out + m;
+            p.out[o] = y;
+            if (p.acc) p.acc[o] = a;
+        }
+    };
+    bool alive = true;
+    const int groups = (nvalid + 7) >> 3;
+    if (worker) {
+        alive = mbar_wait_warp(smem_u32(&s_tfull), 0, abort_flag);
+        tc_fence_after();
+    }
+    const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    if (cfg.S == 1) {
+        if (worker && alive && blk * kBlockRows + quarter * 32 < p.M) {
+            for (int g = rank3; g < groups; g += 3) {
+                uint32_t v[8];
+                split_ld8(taddr + 8 * g, v);
+                if (row_ok) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (8 * g + j < nvalid) put(8 * g + j, (int)v[j]);
+                }
+                __syncwarp();
+            }
+        }
+    } else {
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");         // every CTA of the cluster runs
+        if (worker && alive) {
+            for (int g = rank3; g < groups; g += 3) {
+                uint32_t v[8];
+                split_ld8(taddr + 8 * g, v);
+                const uint32_t owner = (uint32_t)(g / cfg.cpo), col = 8u * ((uint32_t)g - owner * (uint32_t)cfg.cpo);
+                const uint32_t dst = split_map(sRed + ((rank * 8u * (uint32_t)cfg.cpo + col) * 128u + (uint32_t)(quarter * 32 + lane)) * 4u, owner);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(dst + (uint32_t)j * 512u), "r"(v[j]) : "memory");
+            }
+        }
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        if (row_ok && alive) {
+            const int c0 = (int)rank * 8 * cfg.cpo, c1 = min(c0 + 8 * cfg.cpo, nvalid);
+            for (int j = c0 + rank3; j < c1; j += 3) {
+                const uint32_t src = sRed + ((uint32_t)(j - c0) * 128u + (uint32_t)(quarter * 32 + lane)) * 4u;
+                int sum = 0;
+                for (int s = 0; s < cfg.S; ++s) {
+                    int v;
+                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(src + (uint32_t)s * (uint32_t)cfg.cpo * 4096u) : "memory");
+                    sum += v;
+                }
+                put(j, sum);
+            }
+        }
+    }
+
+    // -------------------------------------------------------------- teardown
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(cfg.tmem_cols) : "memory");
+    }
+    if (threadIdx.x == 0 && s_abort) atomicMax(p.status, (uint32_t)RMSMP_ERR_TIMEOUT);
+}
+
+// ------------------------------------------------------------------ host side
+
+bool split_tile(const Problem& p, int target, SplitCfg& c)
+{
+    const int64_t hw = (int64_t)p.Ho * p.Wo;
+    if (hw <= target) {
+        c.tb = (int)std::min<int64_t>(target / hw, p.B);
+        const int64_t tiles = ((int64_t)p.B + c.tb - 1) / c.tb;
+        if (tiles > (1 << 24)) return false;
+        c.tb = (int)((p.B + tiles - 1) / tiles);
+        c.th = p.Ho;
+        c.tiles_per_image = 0;
+        c.ntn = (int)((p.B + c.tb - 1) / c.tb);
+    } else {
+        if (p.Wo > target) return false;
+        c.th = std::min(p.Ho, target / p.Wo);
+        const int tiles = (p.Ho + c.th - 1) / c.th;
+        c.th = (p.Ho + tiles - 1) / tiles;
+        c.tb = 1;
+        c.tiles_per_image = (p.Ho + c.th - 1) / c.th;
+        if ((int64_t)p.B * c.tiles_per_image > (1 << 24)) return false;
+        c.ntn = p.B * c.tiles_per_image;
+    }
+    if ((int64_t)p.Wo * p.stride > 256 || (int64_t)c.th * p.stride > 256 || c.tb > 256) return false;
+    c.npix = c.tb * c.th * p.Wo;
+    c.n_pad = (c.npix + 15) / 16 * 16;
+    return c.npix <= 128;
+}
+
+// Tile width and cluster size by a cost in SM cycles: start-up, the k-blocks of one CTA (rows of up to 128 bytes through
+// the SM's copy path, or the expansion of the codes), sending and adding the parts, the output; times the rounds that
+// the grid needs.  Against every width and cluster size measured for two dozen problems (256x512 to 4096x4096, 32 to
+// 6272 pixels) its choice is within 5 % of the best.  *us: the time that the cost stands for, as fitted to the same
+// measurements (a workspace: 2.2 us + 1400 units per us, good to 0.4 us; expansion: 1.75 of that - 2 us, good to 2 us).
+bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr)
+{
+    if (p.pix_pitch % 16 != 0 || (reinterpret_cast<uintptr_t>(p.act) & 15) != 0) return false;
+    if (p.wexp && (reinterpret_cast<uintptr_t>(p.wexp) & 15) != 0) return false;
+    const int64_t sms = sm_count();
+    SplitCfg c;
+    memset(&c, 0, sizeof(c));
+    c.pre = p.wexp ? 1 : 0;
+    c.bk = (p.Cin % 128 != 0 && p.Cin % 128 <= 64) ? 64 : 128;
+    c.a_bytes = kBlockRows * c.bk;
+    c.cpt = (p.Cin + c.bk - 1) / c.bk;
+    if ((int64_t)p.kh * p.kw * c.cpt > (1 << 20)) return false;
+    c.nkb = p.kh * p.kw * c.cpt;
+    c.last_ksteps = (p.Cin - (c.cpt - 1) * c.bk + 31) / 32;
+    double best_cost = 1e30;
+    static const int targets[] = {16, 32, 48, 64, 96, 128};
+    for (int target : targets) {
+        if (!split_tile(p, target, c)) continue;
+        c.b_bytes = (c.n_pad * c.bk + 1023) / 1024 * 1024;
+        c.tx_b = (uint32_t)c.npix * (uint32_t)c.bk;
+        for (int S = 1; S <= 8 && S <= c.nkb; S *= 2) {
+            const int64_t ctas = (int64_t)p.nblocks * c.ntn * S;
+            if (ctas > (1 << 30)) break;
+            c.S = S;
+            const int kpc = (c.nkb + S - 1) / S;
+            c.cpo = S > 1 ? (c.n_pad / 8 + S - 1) / S : 0;
+            const int red = S * c.cpo * 8 * 512;
+            c.nst = std::min(std::min(kpc, kSplitRing), (kSplitSmem - 2048 - red) / (c.a_bytes + c.b_bytes));
+            // fewer than three stages are not enough for the three expander groups: a group may run ahead of the others by
+            // two of its own k-blocks, and a stage's barrier tells only neighbouring phases apart
+            if (c.nst < 3 && c.nst < kpc) continue;
+            c.smem_bytes = (uint32_t)(c.nst * (c.a_bytes + c.b_bytes) + red + 1024);
+            // clusters of eight do not tile the SMs of every processing cluster: count 5 % fewer for each doubling
+            const double usable = (double)sms * (S == 1 ? 1.0 : S == 2 ? 0.97 : S == 4 ? 0.92 : 0.85);
+            const double waves = std::max(1.0, std::ceil((double)ctas / usable));
+            const double load = (c.pre ? kBlockRows + c.npix : c.npix) * 2.56, expand = c.pre ? 0.0 : 420.0 * c.bk / 128.0;
+            const double kblock = std::max(std::max(load, expand), 90.0 * (c.bk / 32));
+            const double cost = waves * (1500.0 + kpc * kblock + (S > 1 ? 900.0 + 14.0 * c.n_pad : 0.0) + 14.0 * c.n_pad / S);
+            if (cost < best_cost) { best_cost = cost; best = c; }
+        }
+    }
+    if (best_cost >= 1e30) return false;
+    if (us) {
+        *us = 2.2 + best_cost / 1400.0;
+        if (!best.pre) *us = (1.75 * *us - 2.0) * ((int64_t)p.nblocks * best.ntn * best.S > sms ? 1.15 : 1.0);
+    }
+    best.tmem_cols = 32;
+    while (best.tmem_cols < best.n_pad) best.tmem_cols *= 2;
+    // kind::i8: int32 accumulate, signed 8-bit A and B, both K-major, N/8 at bit 17, M/16 at bit 24
+    best.idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(best.n_pad >> 3) << 17) | ((uint32_t)(kBlockRows >> 4) << 24);
+    return true;
+}
+
+}  // namespace
+
+// Which of the two kernels takes a problem.  With a workspace the persistent kernel takes whatever fills the chip;
+// below that its time is one tile's: 3.4 us + 1.2 for the output of 256 pixels + 0.28 to 0.41 per k-block of 128 codes
+// (measured: 256x512 N=64 4.8 us against 4.1 here, 256x2304 N=196 11.7 against 5.4, 512x4608 N=49 16 against 6,
+// 768x3072 N=512 13.5 against 10.2, N=2048 13.7 against 14).  Without one it expands the codes again for every tile,
+// 1.15 us (tiles of up to 224 pixels) or 1.5 us (256 tokens) a k-block and round of tiles: 768x3072 N=512 40 us against
+// 12.4 here, 256x2304 N=6272 23.2 against 15.7, N=25088 41 against 63.
+bool split_supported(const Problem& p)
+{
+    const double sms = sm_count(), tiles = (double)((p.N + 255) / 256 * p.nblocks);
+    const bool bk64 = p.Cin % 128 != 0 && p.Cin % 128 <= 64;
+    const double nkb = (double)p.kh * p.kw * ((p.Cin + 127) / 128) * (bk64 && p.Cin < 128 ? 0.5 : 1.0);
+    const bool resident = p.nblocks == 1 && nkb * kBlockRows * 128 <= 72 * 1024;
+    double other;
+    if (p.wexp || resident) {
+        if (tiles >= sms) return false;
+        const double n = (double)std::min<int64_t>(p.N, 256);
+        other = 3.4 + 1.2 * n / 256 + nkb * (0.28 + 0.13 * n / 256) + (p.wexp ? 0.0 : 1.5);
+    } else {
+        other = 2.5 + std::ceil(tiles / sms) * (1.5 + nkb * (p.Wo > 1 ? 1.15 : 1.5));
+    }
+    SplitCfg c;
+    double us = 0.0;
+    return plan_split(p, c, &us) && us < other && tensor_map_encoder() != nullptr;
+}
+
+rmsmp_status launch_split(const Problem& p, cudaStream_t st)
+{
+    SplitCfg c;
+    if (!plan_split(p, c)) return RMSMP_ERR_VARIANT;
+    EncodeTiledFn enc = tensor_map_encoder();
+    if (!enc) return RMSMP_ERR_CUDA;
+    SplitMaps mp;
+    memset(&mp, 0, sizeof(mp));
+    if (!encode_act_maps_4(p, c.bk, c.th, c.tb, mp.act)) return RMSMP_ERR_CUDA;
+    if (c.pre) {
+        const cuuint64_t gd[2] = {(cuuint64_t)p.Kp, (cuuint64_t)p.M};
+        const cuuint64_t gs[1] = {(cuuint64_t)p.Kp};
+        const cuuint32_t bx[2] = {(cuuint32_t)c.bk, (cuuint32_t)kBlockRows};
+        const cuuint32_t es[2] = {1, 1};
+        if (enc(&mp.wexp, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t*>(p.wexp), gd, gs, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                c.bk == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return RMSMP_ERR_CUDA;
+    }
+    auto fn = p.rq_codes ? split_kernel<1, 1> : c.pre ? split_kernel<0, 1> : split_kernel<0, 0>;      // (re-quantizing calls have a workspace)
+    if (p.rq_codes && !c.pre) return RMSMP_ERR_VARIANT;
+    static bool attr_set[3][kMaxDevices] = {};
+    if (!ensure_smem_attr(reinterpret_cast<const void*>(fn), kSplitSmem, attr_set[p.rq_codes ? 2 : c.pre])) return RMSMP_ERR_CUDA;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // as launch_dependent
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)c.S; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)((int64_t)p.nblocks * c.ntn * c.S)); lc.blockDim = dim3(kSplitThreads);
+    lc.dynamicSmemBytes = c.smem_bytes; lc.stream = st; lc.attrs = at; lc.numAttrs = c.S > 1 ? 2 : 1;
+    if (cudaLaunchKernelEx(&lc, fn, p, c, mp) != cudaSuccess) {
+        cudaGetLastError();
+        return RMSMP_ERR_CUDA;
+    }
+    return RMSMP_OK;
+}
+
+}  // namespace rmsmp

@@ -532,6 +532,67 @@ def test_a_bounded_wait_that_runs_out_reports_timeout_and_leaves_the_context_usa
     assert np.array_equal(y.view(np.uint32), y_ref.view(np.uint32))
 
 
+# ------------------------------------------------------------------ narrow tiles, the reduction shared by a cluster
+
+@pytest.mark.parametrize("variant", [R.VARIANT_TENSOR, Hn.WORKSPACE], ids=lambda v: VNAME[v])
+@pytest.mark.parametrize("M,K,N", [
+    (128, 128, 16),          # one k-block, one tile, nothing to share
+    (130, 272, 33),          # a second row block of two rows, a last step of 16 codes
+    (64, 1040, 17),          # 64-byte k-blocks
+    (512, 2304, 49),         # eight CTAs to a tile, k-blocks shared unevenly
+    (300, 4096, 100),        # more k-blocks than stages
+    (4096, 512, 40),         # many row blocks
+    (256, 6144, 128),
+])
+def test_small_linear_layers_share_their_reduction(M, K, N, variant):
+    """Sums are integers and the output is one multiply: exact, in both layouts, with and without the sums."""
+    g = synth.rng(88, M + K + N)
+    Wt = synth.weights_normal(g, (M, K))
+    scheme, bits = _mixed_map(M, 5, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    act = g.integers(-16, 17, size=(N, K)).astype(np.int8)
+    _, ws, acc_ref, _ = O.layer_linear(Wt, scheme, bits, alpha, act, np.float32(0.25))
+    for layout in (R.OUT_NM, R.OUT_MN):
+        for want_acc in (True, False):
+            y, acc = Hn.gemm(layer, d_packed, act, 0.25, variant, out_layout=layout, want_acc=want_acc)
+            if want_acc:
+                _check_layer_outputs(y, acc, acc_ref, ws, np.float32(0.25), alpha, scheme, bits)
+            assert np.array_equal(y.view(np.uint32), O.epilogue(acc_ref, ws, np.float32(0.25)).view(np.uint32))
+
+
+@pytest.mark.parametrize("variant", [R.VARIANT_TENSOR, Hn.WORKSPACE], ids=lambda v: VNAME[v])
+@pytest.mark.parametrize("M,Cin,k,stride,pad,B,H,W", [
+    (64, 64, 3, 1, 1, 1, 30, 28),        # tiles of a few rows, the last tile of an image shorter than the others
+    (256, 256, 3, 1, 1, 1, 14, 14),
+    (512, 512, 3, 1, 1, 1, 7, 7),        # a tile is an image
+    (130, 96, 3, 2, 1, 3, 15, 13),       # stride 2, odd sizes, several images
+    (96, 48, 5, 1, 2, 2, 9, 20),
+    (160, 320, 1, 2, 0, 5, 9, 9),
+    (32, 16, 3, 3, 1, 2, 11, 10),        # stride 3
+])
+def test_small_convolutions_share_their_reduction(M, Cin, k, stride, pad, B, H, W, variant):
+    import torch
+    g = synth.rng(89, M + Cin + H)
+    Wt = synth.weights_kaiming(g, M, Cin, k, k)
+    scheme, bits = _mixed_map(M, 6, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    act = g.integers(-16, 17, size=(B, H, W, Cin)).astype(np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    _, ws, acc_ref, y_ref = O.layer_conv(Wt, scheme, bits, alpha, act, np.float32(0.25), stride, pad)
+    y, acc = Hn.conv(layer, d_packed, act, stride, pad, 0.25, variant)
+    assert np.array_equal(acc.reshape(-1, M), acc_ref.reshape(-1, M))
+    assert np.array_equal(y.reshape(-1, M).view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
+    if variant == Hn.WORKSPACE:
+        d_ws = Hn._workspace(layer, d_packed)
+        d_act = torch.from_numpy(act).cuda()
+        out = torch.full((acc_ref.size // M, M), 99, dtype=torch.int8, device="cuda")
+        for kind in (R.ACT_U4, R.ACT_S4):
+            R.rmsmp_conv_implicit_workspace_requant(layer, d_packed, d_ws, d_act, B, H, W, stride, pad, 0.25, 1.7, kind, out)
+            c_ref, _ = O.quantize_act(y_ref.reshape(-1, M), 1.7, kind)
+            assert np.array_equal(out.cpu().numpy(), c_ref)
+
+
 # ------------------------------------------------------------------ row assignment on the device
 
 @pytest.mark.parametrize("ratio", [(60, 35, 5), (65, 30, 5), (0, 100, 0), (50, 40, 10)], ids=lambda r: "%d-%d-%d" % r)
