@@ -1,4 +1,5 @@
-"""Thin ctypes binding of librmsmp.so: same names as include/rmsmp.h, argument marshalling only.
+"""Thin binding of librmsmp.so: same names as include/rmsmp.h, argument marshalling only (ctypes; an extension
+module for the calls made per layer and pass).
 
 Device buffers are torch CUDA tensors (or raw integer device pointers); torch is used for
 memory and streams, every step of the computation runs in the library's kernels.  There is no
@@ -147,35 +148,78 @@ def _hp(a: np.ndarray):
     return a.ctypes.data
 
 
-_current_raw_stream = None
+def _current_stream():
+    """Handle of the current torch stream."""
+    return _raw_stream() if _raw_stream is not None else _first_stream()
 
 
 def _stream(stream):
     if stream is None:
-        return _current_raw_stream() if _current_raw_stream is not None else _first_stream()
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+_raw_stream = None
 
 
 def _first_stream():
     """The current stream through torch's public call, which also starts CUDA up.  From then on its handle is read
     directly where this torch has the accessor: the public call builds a Stream object (3.4 us, a third of a small
     layer's call; the accessor 0.2 us)."""
-    global _current_raw_stream
+    global _raw_stream
     import torch
     handle = torch.cuda.current_stream().cuda_stream
     raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
     if raw is not None and device is not None:
-        _current_raw_stream = lambda: raw(device())
+        _raw_stream = lambda: raw(device())
     else:
-        _current_raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+        _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
     return handle
 
 
 def _check(st: int, where: str):
     if st != OK:
         raise RmsmpError(st, where)
+
+
+# The calls that a program makes per layer and pass are marshalled by the extension module (csrc/marshal.cpp); it is
+# loaded with the library on the first use of one of them.
+_NATIVE = (
+    "rmsmp_quantize_act",
+    "rmsmp_gemm",
+    "rmsmp_gemm_variant",
+    "rmsmp_gemm_workspace",
+    "rmsmp_gemm_workspace_requant",
+    "rmsmp_conv_implicit",
+    "rmsmp_conv_implicit_variant",
+    "rmsmp_conv_implicit_workspace",
+    "rmsmp_conv_implicit_workspace_requant",
+    "rmsmp_conv_depthwise",
+    "rmsmp_im2col_codes",
+    "rmsmp_expand_weights",
+    "rmsmp_assign_quantize_pack",
+    "rmsmp_gemm_grouped_launch",
+)
+
+
+def _raise(status: int, where: str):
+    raise RmsmpError(status, where)
+
+
+def __getattr__(name):
+    if name not in _NATIVE:
+        raise AttributeError(f"module {__name__!r} has no attribute {name!r}")
+    L = lib()
+    try:
+        from . import _marshal
+    except ImportError as e:
+        raise RuntimeError(f"the extension module _marshal is missing: build it with `python -m {__package__}.build`") from e
+    _marshal.setup({n: C.cast(getattr(L, n), C.c_void_p).value for n in _NATIVE}, _current_stream, _raise)
+    for n in _NATIVE:
+        globals()[n] = getattr(_marshal, n)
+    return globals()[name]
 
 
 def rmsmp_status_string(status: int) -> str:
@@ -224,91 +268,10 @@ def rmsmp_unpack_codes(layer: rmsmp_layer, d_packed, d_values, d_perm=None, d_ws
                                     _dp(d_wstep), _stream(stream)), "rmsmp_unpack_codes")
 
 
-def rmsmp_quantize_act(d_X, count: int, alpha_a: float, kind: int, d_codes, stream=None) -> float:
-    """Returns the activation step (alpha_a/15 or alpha_a/7) as a Python float (fp32 value)."""
-    step = C.c_float(0.0)
-    _check(lib().rmsmp_quantize_act(_dp(d_X), count, alpha_a, kind, _dp(d_codes), C.byref(step),
-                                    _stream(stream)), "rmsmp_quantize_act")
-    return step.value
-
-
-def rmsmp_gemm(layer, d_packed, d_act, N: int, ld_act: int, act_step: float, d_out, ld_out: int,
-               out_layout: int = OUT_NM, d_acc=None, stream=None):
-    _check(lib().rmsmp_gemm(C.byref(layer), _dp(d_packed), _dp(d_act), N, ld_act, act_step,
-                            _dp(d_out), ld_out, out_layout, _dp(d_acc), _stream(stream)),
-           "rmsmp_gemm")
-
-
-def rmsmp_gemm_variant(layer, d_packed, d_act, N: int, ld_act: int, act_step: float, d_out,
-                       ld_out: int, out_layout: int, d_acc, variant: int, stream=None):
-    _check(lib().rmsmp_gemm_variant(C.byref(layer), _dp(d_packed), _dp(d_act), N, ld_act, act_step,
-                                    _dp(d_out), ld_out, out_layout, _dp(d_acc), variant,
-                                    _stream(stream)), "rmsmp_gemm_variant")
-
-
-def rmsmp_conv_implicit(layer, d_packed, d_act, B: int, H: int, W: int, stride: int, pad: int,
-                        act_step: float, d_out, out_layout: int = OUT_NM, d_acc=None, stream=None):
-    _check(lib().rmsmp_conv_implicit(C.byref(layer), _dp(d_packed), _dp(d_act), B, H, W, stride,
-                                     pad, act_step, _dp(d_out), out_layout, _dp(d_acc),
-                                     _stream(stream)), "rmsmp_conv_implicit")
-
-
-def rmsmp_conv_implicit_variant(layer, d_packed, d_act, B: int, H: int, W: int, stride: int,
-                                pad: int, act_step: float, d_out, out_layout: int, d_acc,
-                                variant: int, stream=None):
-    _check(lib().rmsmp_conv_implicit_variant(C.byref(layer), _dp(d_packed), _dp(d_act), B, H, W,
-                                             stride, pad, act_step, _dp(d_out), out_layout,
-                                             _dp(d_acc), variant, _stream(stream)),
-           "rmsmp_conv_implicit_variant")
-
-
-def rmsmp_gemm_workspace_requant(layer, d_packed, d_workspace, d_act, N: int, ld_act: int, act_step: float,
-                                 next_alpha: float, next_kind: int, d_next_codes, ld_codes: int, stream=None) -> float:
-    """Linear layer whose epilogue writes the next layer's 4-bit activation codes; returns their step."""
-    step = C.c_float(0.0)
-    _check(lib().rmsmp_gemm_workspace_requant(C.byref(layer), _dp(d_packed), _dp(d_workspace), _dp(d_act), N, ld_act,
-                                              act_step, next_alpha, next_kind, _dp(d_next_codes), ld_codes,
-                                              C.byref(step), _stream(stream)), "rmsmp_gemm_workspace_requant")
-    return step.value
-
-
-def rmsmp_conv_implicit_workspace_requant(layer, d_packed, d_workspace, d_act, B: int, H: int, W: int, stride: int,
-                                          pad: int, act_step: float, next_alpha: float, next_kind: int,
-                                          d_next_codes, stream=None) -> float:
-    step = C.c_float(0.0)
-    _check(lib().rmsmp_conv_implicit_workspace_requant(C.byref(layer), _dp(d_packed), _dp(d_workspace), _dp(d_act),
-                                                       B, H, W, stride, pad, act_step, next_alpha, next_kind,
-                                                       _dp(d_next_codes), C.byref(step), _stream(stream)),
-           "rmsmp_conv_implicit_workspace_requant")
-    return step.value
-
-
 def rmsmp_workspace_bytes(layer) -> int:
     n = C.c_size_t(0)
     _check(lib().rmsmp_workspace_bytes(C.byref(layer), C.byref(n)), "rmsmp_workspace_bytes")
     return n.value
-
-
-def rmsmp_expand_weights(layer, d_packed, d_workspace, workspace_bytes: int | None = None, stream=None):
-    if workspace_bytes is None:
-        workspace_bytes = d_workspace.numel() * d_workspace.element_size()
-    _check(lib().rmsmp_expand_weights(C.byref(layer), _dp(d_packed), _dp(d_workspace), workspace_bytes,
-                                      _stream(stream)), "rmsmp_expand_weights")
-
-
-def rmsmp_gemm_workspace(layer, d_packed, d_workspace, d_act, N: int, ld_act: int, act_step: float,
-                         d_out, ld_out: int, out_layout: int = OUT_NM, d_acc=None, stream=None):
-    _check(lib().rmsmp_gemm_workspace(C.byref(layer), _dp(d_packed), _dp(d_workspace), _dp(d_act), N,
-                                      ld_act, act_step, _dp(d_out), ld_out, out_layout, _dp(d_acc),
-                                      _stream(stream)), "rmsmp_gemm_workspace")
-
-
-def rmsmp_conv_implicit_workspace(layer, d_packed, d_workspace, d_act, B: int, H: int, W: int,
-                                  stride: int, pad: int, act_step: float, d_out,
-                                  out_layout: int = OUT_NM, d_acc=None, stream=None):
-    _check(lib().rmsmp_conv_implicit_workspace(C.byref(layer), _dp(d_packed), _dp(d_workspace), _dp(d_act),
-                                               B, H, W, stride, pad, act_step, _dp(d_out), out_layout,
-                                               _dp(d_acc), _stream(stream)), "rmsmp_conv_implicit_workspace")
 
 
 def rmsmp_gemm_builtin_scratch(layer, d_packed, d_act, N: int, ld_act: int, act_step: float, d_out,
@@ -365,24 +328,8 @@ def rmsmp_gemm_grouped_prepare(items_array, out_layout: int, d_table, table_byte
     return plan
 
 
-def rmsmp_gemm_grouped_launch(plan, stream=None):
-    _check(lib().rmsmp_gemm_grouped_launch(C.byref(plan), _stream(stream)), "rmsmp_gemm_grouped_launch")
-
-
 def rmsmp_last_device_status(d_packed, stream=None) -> int:
     return lib().rmsmp_last_device_status(_dp(d_packed), _stream(stream))
-
-
-def rmsmp_conv_depthwise(layer, d_packed, d_act, B: int, H: int, W: int, stride: int, pad: int, act_step: float,
-                         d_out, d_acc=None, stream=None):
-    _check(lib().rmsmp_conv_depthwise(C.byref(layer), _dp(d_packed), _dp(d_act), B, H, W, stride, pad, act_step,
-                                      _dp(d_out), _dp(d_acc), _stream(stream)), "rmsmp_conv_depthwise")
-
-
-def rmsmp_im2col_codes(d_act, B: int, H: int, W: int, Cc: int, pix_pitch: int, kh: int, kw: int, stride: int, pad: int,
-                       d_cols, ld_cols: int, stream=None):
-    _check(lib().rmsmp_im2col_codes(_dp(d_act), B, H, W, Cc, pix_pitch, kh, kw, stride, pad, _dp(d_cols), ld_cols,
-                                    _stream(stream)), "rmsmp_im2col_codes")
 
 
 def rmsmp_layer_init_ratio(M: int, Cin: int, kh: int, kw: int, ratio) -> rmsmp_layer:
@@ -396,15 +343,6 @@ def rmsmp_assign_scratch_bytes(M: int) -> int:
     n = C.c_size_t(0)
     _check(lib().rmsmp_assign_scratch_bytes(M, C.byref(n)), "rmsmp_assign_scratch_bytes")
     return n.value
-
-
-def rmsmp_assign_quantize_pack(d_W, w_layout: int, layer, ratio, d_alpha, pot_mode: int, d_packed, d_scratch,
-                               d_scheme=None, d_bits=None, stream=None):
-    """Row assignment on the device + quantize + pack, from the ratio alone."""
-    _check(lib().rmsmp_assign_quantize_pack(_dp(d_W), w_layout, C.byref(layer), int(ratio[0]), int(ratio[1]), int(ratio[2]),
-                                            _dp(d_alpha), pot_mode, _dp(d_packed), d_packed.numel() * d_packed.element_size(),
-                                            _dp(d_scratch), d_scratch.numel() * d_scratch.element_size(), _dp(d_scheme),
-                                            _dp(d_bits), _stream(stream)), "rmsmp_assign_quantize_pack")
 
 
 def rmsmp_selftest_bounded_wait(limit_cycles: int, d_status_word, stream=None):

@@ -147,3 +147,34 @@ def test_no_gpu_means_loud_failure_not_fallback():
     step = C.c_float()
     st = lib.rmsmp_quantize_act(C.c_void_p(0x10000), 16, 1.0, 0, C.c_void_p(0x20000), C.byref(step), None)
     assert st in (R.ERR_CUDA, R.ERR_ARCH)
+
+
+def test_marshalled_calls_take_the_python_signatures_and_raise_like_them():
+    """The calls of the extension module without a GPU: positional and keyword arguments, defaults, argument errors as
+    TypeError, the library's own refusals as RmsmpError with their status."""
+    good = R.rmsmp_layer_init(4, 16, 1, 1, np.zeros(4, np.uint8), np.full(4, 4, np.uint8))
+    args = (good, 256, 256, 1, 16, 0.5, 256, 4)
+    for bad_call, status in (
+            (lambda: R.rmsmp_gemm(good, None, 256, 1, 16, 0.5, 256, 4, stream=0), R.ERR_NULL),
+            (lambda: R.rmsmp_gemm(R.rmsmp_layer(), *args[1:], stream=0), R.ERR_BAD_LAYER),
+            (lambda: R.rmsmp_gemm(layer=good, d_packed=256, d_act=256, N=1, ld_act=8, act_step=0.5, d_out=256, ld_out=4, stream=0), R.ERR_SHAPE),
+            (lambda: R.rmsmp_gemm(*args, 7, None, 0), R.ERR_SHAPE),
+            (lambda: R.rmsmp_gemm(good, 256, 257, *args[3:], stream=0), R.ERR_ALIGN),
+            (lambda: R.rmsmp_gemm(*args[:5], float("inf"), 256, 4, stream=0), R.ERR_SCALE),
+            (lambda: R.rmsmp_gemm_workspace(good, 256, None, *args[2:], stream=0), R.ERR_NULL),
+            (lambda: R.rmsmp_expand_weights(good, 256, 256, 1, stream=0), R.ERR_BUFFER_TOO_SMALL),
+            (lambda: R.rmsmp_quantize_act(256, 0, 3.0, R.ACT_U4, 256, stream=0), R.ERR_SHAPE),
+            (lambda: R.rmsmp_quantize_act(256, 4, -3.0, R.ACT_U4, 256, stream=0), R.ERR_SCALE),
+            (lambda: R.rmsmp_conv_implicit(good, 256, 256, 1, 4, 4, 0, 0, 0.5, 256, stream=0), R.ERR_SHAPE),
+            (lambda: R.rmsmp_im2col_codes(256, 1, 4, 4, 3, 2, 3, 3, 1, 1, 256, 32, stream=0), R.ERR_SHAPE),
+            (lambda: R.rmsmp_gemm_grouped_launch(R.rmsmp_grouped_plan(), stream=0), R.ERR_BAD_LAYER)):
+        with pytest.raises(R.RmsmpError) as e:
+            bad_call()
+        assert e.value.status == status
+    for bad_call in (lambda: R.rmsmp_gemm(good), lambda: R.rmsmp_gemm(*args, nonsense=1), lambda: R.rmsmp_gemm(*args, d_out=1),
+                     lambda: R.rmsmp_gemm(1, *args[1:], stream=0), lambda: R.rmsmp_gemm(R.rmsmp_grouped_plan(), *args[1:], stream=0),
+                     lambda: R.rmsmp_gemm(*args[:3], 1.5, *args[4:], stream=0), lambda: R.rmsmp_gemm(*args, 0, None, 0, 0)):
+        with pytest.raises(TypeError):
+            bad_call()
+    with pytest.raises(OverflowError):
+        R.rmsmp_conv_implicit(good, 256, 256, 1 << 40, 4, 4, 1, 0, 0.5, 256, stream=0)
