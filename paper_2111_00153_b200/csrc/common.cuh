@@ -43,6 +43,8 @@ struct Problem {
     int B, H, W, Ho, Wo, stride, pad;
     int64_t pix_pitch;
     int64_t N;                // B*Ho*Wo
+    int ragged_k;             // linear layer under AUTO: a K that is not a multiple of 16 may take the tensor path (rows are
+                              // 16-byte aligned all the same; the copy engine fills up with zeros)
     int act_nonneg;           // grouped tensor-core launch: every activation code is within 0..15
     // outputs
     float act_step;

@@ -929,7 +929,7 @@ bool encode_act_maps(EncodeTiledFn enc, const Problem& p, int bk, int th, int tb
 
 bool plan(const Problem& p, TensorCfg& c)
 {
-    if (p.pix_pitch % 16 != 0 || p.Cin % 16 != 0) return false;
+    if (p.pix_pitch % 16 != 0 || (p.Cin % 16 != 0 && !p.ragged_k)) return false;
     if ((reinterpret_cast<uintptr_t>(p.act) & 15) != 0) return false;
     if (!p.wexp && p.raw_stage_bytes <= 0) return false;
     if (p.wexp && (reinterpret_cast<uintptr_t>(p.wexp) & 15) != 0) return false;

@@ -561,6 +561,28 @@ def test_small_linear_layers_share_their_reduction(M, K, N, variant):
             assert np.array_equal(y.view(np.uint32), O.epilogue(acc_ref, ws, np.float32(0.25)).view(np.uint32))
 
 
+@pytest.mark.parametrize("N", [1, 2, 31, 33, 300])
+@pytest.mark.parametrize("M,K", [(96, 1), (130, 17), (200, 127), (64, 200), (1000, 513), (20000, 72)])
+def test_linear_layers_of_any_length_under_auto(M, K, N):
+    """K that is no multiple of 16, from one token up, with other bytes behind every row: exact as always."""
+    g = synth.rng(90, M + K + N)
+    Wt = synth.weights_normal(g, (M, K))
+    scheme, bits = _mixed_map(M, 7, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    act = g.integers(-128, 128, size=(N, K)).astype(np.int8)
+    ld = (K + 15) // 16 * 16 + 16
+    import torch
+    a = torch.full((N, ld), 55, dtype=torch.int8, device="cuda")
+    a[:, :K] = torch.from_numpy(act).cuda()
+    y = torch.full((N, M), float("nan"), dtype=torch.float32, device="cuda")
+    acc = torch.full((N, M), -9, dtype=torch.int32, device="cuda")
+    R.rmsmp_gemm(layer, d_packed, a, N, ld, 0.25, y, M, R.OUT_NM, acc)
+    _, ws, acc_ref, _ = O.layer_linear(Wt, scheme, bits, alpha, act, np.float32(0.25))
+    _check_layer_outputs(y.cpu().numpy(), acc.cpu().numpy(), acc_ref, ws, np.float32(0.25), alpha, scheme, bits)
+    assert R.rmsmp_last_device_status(d_packed) == R.OK
+
+
 @pytest.mark.parametrize("variant", [R.VARIANT_TENSOR, Hn.WORKSPACE], ids=lambda v: VNAME[v])
 @pytest.mark.parametrize("M,Cin,k,stride,pad,B,H,W", [
     (64, 64, 3, 1, 1, 1, 30, 28),        # tiles of a few rows, the last tile of an image shorter than the others
