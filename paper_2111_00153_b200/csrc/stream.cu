@@ -601,25 +601,24 @@ stream_kernel(const uint8_t* __restrict__ table)
         const int slot = quarter * 32 + lane;
         uint32_t n = 0;
         bool alive = true;
-        // this lane's row of an item: original index, scale and Fixed-4 shift, fetched ahead of the accumulator
-        auto row_info = [&](int it, float& scale, int& shift, int& m) {
-            scale = 0.f; shift = 0; m = -1;
+        // this lane's row of an item: original index and scale, fetched ahead of the accumulator
+        auto row_info = [&](int it, float& scale, int& m) {
+            scale = 0.f; m = -1;
             if (it >= it1) return;
             const ItemView v = view(it);
             if (slot < v.rows) {
                 m = __ldg(v.P->perm + v.packed0 + slot);
                 scale = __fmul_rn(__ldg(v.P->wstep + m), v.P->act_step);
-                shift = (v.kind == kFixed4) ? 4 : 0;     // expanders store Fixed-4 codes as 16 * value
             }
         };
-        float scale, scale_n; int shift, shift_n, m, m_n;
-        row_info(it0, scale, shift, m);
+        float scale, scale_n; int m, m_n;
+        row_info(it0, scale, m);
         asm volatile("griddepcontrol.wait;" ::: "memory");      // the launch in front of this one may still be writing the same outputs
         for (int it = it0; it < it1 && alive; ++it, ++n) {
             const ItemView vi = view(it);
             const StreamProblem* P = vi.P;
             last_status = P->status;
-            row_info(it + 1, scale_n, shift_n, m_n);
+            row_info(it + 1, scale_n, m_n);
             const uint32_t ab = n & (nAcc - 1u);
             if (!mbar_wait_parked_warp(bar_tfull + 8 * ab, (n >> acc_shift) & 1, abort_flag)) { alive = false; break; }
             tc_fence_after();
@@ -630,15 +629,10 @@ stream_kernel(const uint8_t* __restrict__ table)
             int32_t* const acc = P->acc;
             const int64_t ld = P->ld_out;
             const bool out_mn = P->out_mn != 0;
-            // one value of this lane's row: undo the x16 of Fixed-4 rows, scale, store (and the raw sum if asked for)
-            // this lane's row: where its value of token nn goes
+            // Where this lane's values go: token nn at o_row + nn * o_tok.  A finished sum times `unit` is the integer
+            // sum, exactly (Fixed-4: 1/16 of float(16 * sum), a power of two; PoT: fp32 units, below 2^24), so an output
+            // is two multiplies whatever the kind and the integer itself is formed only where the caller asked for it.
             const int64_t o_row = out_mn ? (int64_t)m * ld : (int64_t)m, o_tok = out_mn ? 1 : ld;
-            auto put = [&](int nn, uint32_t raw) {
-                const int a = (int)raw >> shift;
-                const int64_t o = o_row + (int64_t)nn * o_tok;
-                out[o] = __fmul_rn(__int2float_rn(a), scale);
-                if (acc) acc[o] = a;
-            };
             auto release_tmem = [&]() {
                 // every accumulator of this item is in registers: hand the buffer back
                 tc_fence_before();
@@ -648,7 +642,7 @@ stream_kernel(const uint8_t* __restrict__ table)
             // 16 tokens at a time; with few tokens the 32-code steps went to nch accumulator chains in turn: add them
             const int n16 = (N + 15) >> 4;
             const bool fp = vi.kind == kPoT4;            // fp32 sums: add the chains (exactly), then the integer number of units
-            const float fp_unit = P->fp_unit;
+            const float unit = fp ? P->fp_unit : (vi.kind == kFixed4 ? 0.0625f : 1.0f);
             for (int ch = 0; ch < n16; ++ch) {
                 uint32_t v[16];
                 tmem_ld16(taddr + ch * 16, v);
@@ -663,18 +657,34 @@ stream_kernel(const uint8_t* __restrict__ table)
                         for (int j = 0; j < 16; ++j) v[j] += u[j];
                     }
                 }
-                if (fp) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] = (uint32_t)__float2int_rn(__fmul_rn(__uint_as_float(v[j]), fp_unit));
-                }
                 if (ch == n16 - 1) release_tmem();
                 if (m < 0) continue;
                 const int jmax = min(16, N - ch * 16);
+                const int64_t o0 = o_row + (int64_t)(ch * 16) * o_tok;
+                if (acc) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    if (j < jmax) put(ch * 16 + j, v[j]);
+                    for (int j = 0; j < 16; ++j)
+                        if (j < jmax)
+                            acc[o0 + j * o_tok] = fp ? __float2int_rn(__fmul_rn(__uint_as_float(v[j]), unit)) : (int)v[j] >> (vi.kind == kFixed4 ? 4 : 0);
+                }
+                if (!fp) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__int2float_rn((int)v[j]));
+                }
+                float* o = out + o0;
+                if (jmax == 16) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        *o = __fmul_rn(__fmaf_rn(__uint_as_float(v[j]), unit, 0.0f), scale);      // + 0: a sum of -0 becomes +0
+                        o += o_tok;
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (j < jmax) o[j * o_tok] = __fmul_rn(__fmaf_rn(__uint_as_float(v[j]), unit, 0.0f), scale);
+                }
             }
-            scale = scale_n; shift = shift_n; m = m_n;
+            scale = scale_n; m = m_n;
         }
     }
 
