@@ -239,33 +239,54 @@ __device__ __forceinline__ void tensormap_prefetch(const CUtensorMap* m)
     asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
 }
 // E4M3 copies of the activation codes of every layer with PoT rows: [N][Kp], zeros beyond the layer's
-// reduction length.  blockIdx.y = layer; layers whose bytes can be read as they are have no copy.
+// reduction length.  blockIdx.y = layer; layers whose bytes can be read as they are have no copy.  The launch behind
+// waits for this kernel, so it is all latency: the table is read ahead of the wait for the launch in front, a thread
+// has its four units in flight together, and there are few blocks (the streaming kernel in front holds every register
+// of an SM until it leaves).
+constexpr int kConvUnits = 4;                             // 16-byte units per thread and step
 __global__ void __launch_bounds__(256) act_e4m3_kernel(const uint8_t* __restrict__ table)
 {
     // Programmatic dependent launch on both sides: the streaming kernel behind this one may start at once, and
     // this kernel may have started before the launch in front of it (which may still read the copies) is over.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const StreamHeader* H = reinterpret_cast<const StreamHeader*>(table);
     const StreamProblem& P = reinterpret_cast<const StreamProblem*>(table + H->off_probs)[blockIdx.y];
-    if (!P.act_fp_dst) return;
-    const int upr = P.Kp >> 4;                            // 16-byte units per row
+    uint8_t* const dst = P.act_fp_dst;
+    const int8_t* const codes = P.act_src;
+    const int upr = P.Kp >> 4, Cin = P.Cin, Kp = P.Kp;    // 16-byte units per row
     const int units = P.N * upr;
-    for (int u = blockIdx.x * 256 + threadIdx.x; u < units; u += gridDim.x * 256) {
-        const int n = u / upr, k0 = (u - n * upr) << 4;
-        const int8_t* src = P.act_src + (int64_t)n * P.pix_pitch + k0;
-        uint4 v;
-        if (k0 + 16 <= P.Cin) {
-            v = *reinterpret_cast<const uint4*>(src);
-        } else {
-            uint32_t w[4] = {0u, 0u, 0u, 0u};
-            for (int b = 0; b < 16 && k0 + b < P.Cin; ++b) w[b >> 2] |= (uint32_t)(uint8_t)src[b] << (8 * (b & 3));
-            v = make_uint4(w[0], w[1], w[2], w[3]);
+    const int64_t pitch = P.pix_pitch;
+    if (!dst) return;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int u0 = blockIdx.x * (256 * kConvUnits) + threadIdx.x; u0 < units; u0 += gridDim.x * (256 * kConvUnits)) {
+        uint4 v[kConvUnits];
+#pragma unroll
+        for (int i = 0; i < kConvUnits; ++i) {
+            const int u = u0 + 256 * i;
+            const int n = u / upr, k0 = (u - n * upr) << 4;
+            const int8_t* src = codes + (int64_t)n * pitch + k0;
+            v[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (u < units) {
+                if (k0 + 16 <= Cin) {
+                    v[i] = *reinterpret_cast<const uint4*>(src);
+                } else {
+                    uint32_t w[4] = {0u, 0u, 0u, 0u};
+                    for (int b = 0; b < 16 && k0 + b < Cin; ++b) w[b >> 2] |= (uint32_t)(uint8_t)src[b] << (8 * (b & 3));
+                    v[i] = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
         }
-        uint4 o;
-        o.x = e4m3x4_of_s8x4(v.x); o.y = e4m3x4_of_s8x4(v.y);
-        o.z = e4m3x4_of_s8x4(v.z); o.w = e4m3x4_of_s8x4(v.w);
-        *reinterpret_cast<uint4*>(P.act_fp_dst + (int64_t)n * P.Kp + k0) = o;
+#pragma unroll
+        for (int i = 0; i < kConvUnits; ++i) {
+            const int u = u0 + 256 * i;
+            if (u < units) {
+                uint4 o;
+                o.x = e4m3x4_of_s8x4(v[i].x); o.y = e4m3x4_of_s8x4(v[i].y);
+                o.z = e4m3x4_of_s8x4(v[i].z); o.w = e4m3x4_of_s8x4(v[i].w);
+                const int n = u / upr;
+                *reinterpret_cast<uint4*>(dst + (int64_t)n * Kp + ((u - n * upr) << 4)) = o;
+            }
+        }
     }
 }
 
@@ -868,7 +889,7 @@ bool stream_build_table(const Problem* probs, int count, int sms, uint8_t* h_tab
         q.nkb = p.Kp / 128; q.out_mn = p.out_mn;
     }
 
-    H->conv_grid_x = (uint32_t)std::max<int64_t>(1, std::min<int64_t>(64, (max_units + 255) / 256));
+    H->conv_grid_x = (uint32_t)std::max<int64_t>(1, std::min<int64_t>(64, (max_units + 256 * kConvUnits - 1) / (256 * kConvUnits)));
 
     // work items: every tile of every layer, handed to the CTAs longest first onto the least loaded one; an
     // item's cost is its stages, weighted by kind and box height, plus a constant for start-up and output
