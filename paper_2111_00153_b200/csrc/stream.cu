@@ -679,31 +679,33 @@ stream_kernel(const uint8_t* __restrict__ table)
                     }
                 }
                 if (ch == n16 - 1) release_tmem();
-                if (m < 0) continue;
-                const int jmax = min(16, N - ch * 16);
-                const int64_t o0 = o_row + (int64_t)(ch * 16) * o_tok;
-                if (acc) {
+                if (m >= 0) {
+                    const int jmax = min(16, N - ch * 16);
+                    const int64_t o0 = o_row + (int64_t)(ch * 16) * o_tok;
+                    if (acc) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (j < jmax)
-                            acc[o0 + j * o_tok] = fp ? __float2int_rn(__fmul_rn(__uint_as_float(v[j]), unit)) : (int)v[j] >> (vi.kind == kFixed4 ? 4 : 0);
-                }
-                if (!fp) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__int2float_rn((int)v[j]));
-                }
-                float* o = out + o0;
-                if (jmax == 16) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        *o = __fmul_rn(__fmaf_rn(__uint_as_float(v[j]), unit, 0.0f), scale);      // + 0: a sum of -0 becomes +0
-                        o += o_tok;
+                        for (int j = 0; j < 16; ++j)
+                            if (j < jmax)
+                                acc[o0 + j * o_tok] = fp ? __float2int_rn(__fmul_rn(__uint_as_float(v[j]), unit)) : (int)v[j] >> (vi.kind == kFixed4 ? 4 : 0);
                     }
-                } else {
+                    if (!fp) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (j < jmax) o[j * o_tok] = __fmul_rn(__fmaf_rn(__uint_as_float(v[j]), unit, 0.0f), scale);
+                        for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__int2float_rn((int)v[j]));
+                    }
+                    float* o = out + o0;
+                    if (jmax == 16) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            *o = __fmul_rn(__fmaf_rn(__uint_as_float(v[j]), unit, 0.0f), scale);      // + 0: a sum of -0 becomes +0
+                            o += o_tok;
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (j < jmax) o[j * o_tok] = __fmul_rn(__fmaf_rn(__uint_as_float(v[j]), unit, 0.0f), scale);
+                    }
                 }
+                __syncwarp();                            // the next load is a warp-wide instruction: lanes without a row wait here
             }
             scale = scale_n; m = m_n;
         }

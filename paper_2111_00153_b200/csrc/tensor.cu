@@ -860,6 +860,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 }
             };
             // two register sets: the load of this warp's next chunk is in flight while the current one is emitted
+            // (tensor-memory loads and their waits are warp-wide: every chunk ends with the warp together again)
             uint32_t va[32], vb[32];
             tmem_ld_issue(taddr + cfirst * 32, va);
             tmem_ld_wait(va);
@@ -869,12 +870,14 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 // (a re-quantizing chunk may read its accumulators again: the buffer is handed back after it)
                 if (more1) tmem_ld_issue(taddr + c1 * 32, vb); else if (!kRQ) release_tmem();
                 emit(va, c);
+                __syncwarp();
                 if (!more1 && kRQ) release_tmem();
                 if (more1) {
                     tmem_ld_wait(vb);
                     const bool more2 = c2 < nchunks;
                     if (more2) tmem_ld_issue(taddr + c2 * 32, va); else if (!kRQ) release_tmem();
                     emit(vb, c1);
+                    __syncwarp();
                     if (!more2 && kRQ) release_tmem();
                     if (more2) tmem_ld_wait(va);
                 }
