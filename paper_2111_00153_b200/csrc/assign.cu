@@ -13,6 +13,10 @@
 //                      is undecided, gets the definition's chain of additions, and the undecided rows are
 //                      ordered by the exact key.  Then the kind of every row, the stable grouping by prefix
 //                      sums in original order, and every metadata section of the packed buffer.
+//   assign_small_kernel  the same for up to 4096 rows that the parallel variances decide, up to eight rows a thread: each cut
+//                      is a threshold found by bisection, one counting barrier a step, and nothing goes through
+//                      memory between the statistics and the metadata (64 to 512 rows 9 us -> 4).  Otherwise it leaves the
+//                      layer to assign_kernel's code.
 // The result is the definition's in every case.
 #include "common.cuh"
 
@@ -22,6 +26,7 @@ namespace {
 
 constexpr int kStatThreads = 128;
 constexpr int kAssignThreads = 1024;
+constexpr int kSmallThreads = 512;                        // assign_small_kernel's most
 constexpr int kAssignMaxBlocks = 65536 / kBlockRows;      // the entry point takes at most 65536 rows
 constexpr int kAssignSmemRows = 2048;                     // rows whose statistics are kept in shared memory
 
@@ -129,9 +134,19 @@ struct MetaArgs {
     int M, K, Cin, kh, kw, Cp, Kp, nP, nF4, n8, nblocks, pot_mode;
 };
 
-// N values reduced over the block, for every thread (s: N * 32 entries).
+__device__ __forceinline__ void write_header(const MetaArgs& a)
+{
+    BlobHeader* H = reinterpret_cast<BlobHeader*>(a.blob);
+    H->magic = kLayerMagic; H->version = kBlobVersion;
+    H->M = a.M; H->Cin = a.Cin; H->kh = a.kh; H->kw = a.kw; H->Cp = a.Cp; H->Kp = a.Kp;
+    H->nP = a.nP; H->nF4 = a.nF4; H->n8 = a.n8; H->nblocks = a.nblocks; H->pot_mode = a.pot_mode;
+    H->pad0[0] = H->pad0[1] = H->pad0[2] = 0;
+    H->status = 0;
+}
+
+// N values reduced over the block, for every thread (s: N * 32 entries; id: the operation's identity).
 template <int N, typename T, typename Op>
-__device__ __forceinline__ void block_reduce(T (&v)[N], Op op, T* s)
+__device__ __forceinline__ void block_reduce(T (&v)[N], Op op, T* s, T id)
 {
 #pragma unroll
     for (int i = 0; i < N; ++i)
@@ -144,7 +159,7 @@ __device__ __forceinline__ void block_reduce(T (&v)[N], Op op, T* s)
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-        v[i] = s[32 * i + (threadIdx.x & 31)];
+        v[i] = (threadIdx.x & 31) < (blockDim.x >> 5) ? s[32 * i + (threadIdx.x & 31)] : id;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v[i] = op(v[i], __shfl_xor_sync(0xffffffffu, v[i], o));
     }
@@ -153,7 +168,7 @@ __device__ __forceinline__ void block_reduce(T (&v)[N], Op op, T* s)
 // One block: everything here is latency (a few barriers per step), so the statistics are copied to shared memory
 // first and the selection starts at the first bit in which the variances differ at all (their exponents mostly
 // agree): two or three digits for random weights instead of eight.
-__global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
+__device__ __forceinline__ void assign_rows_block(const MetaArgs& a)
 {
     __shared__ int s_hist[2][256];
     __shared__ unsigned long long s_prefix[2];
@@ -166,11 +181,9 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
     __shared__ int s_start[3][kAssignMaxBlocks + 1];      // rows of each kind in front of every 128-row block
     __shared__ double s_var[kAssignSmemRows];
     __shared__ float s_err[kAssignSmemRows];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, warp = t >> 5;      // (128 threads or more)
     const int M = a.M;
     const bool local = M <= kAssignSmemRows;
-    pdl_wait();
-    pdl_trigger();
     double* const var = local ? s_var : a.st.var;
     float* const err = local ? s_err : a.st.err;
     uint8_t* kind = a.blob + a.off_kind;
@@ -183,14 +196,14 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
     // ---- the statistics, and the bits in which the keys differ (a non-negative double orders like its bits)
     const unsigned long long key0 = (unsigned long long)__double_as_longlong(a.st.var[0]);
     unsigned long long diff[1] = {0ull};
-    for (int r = t; r < M; r += kAssignThreads) {
+    for (int r = t; r < M; r += nt) {
         const double v = a.st.var[r];
         if (local) { s_var[r] = v; s_err[r] = a.st.err[r]; }
         diff[0] |= (unsigned long long)__double_as_longlong(v) ^ key0;
     }
-    if (t < 256) { s_hist[0][t] = 0; s_hist[1][t] = 0; }
+    for (int i = t; i < 256; i += nt) { s_hist[0][i] = 0; s_hist[1][i] = 0; }
     if (t == 0) s_undecided = 0;
-    block_reduce<1>(diff, [](unsigned long long x, unsigned long long y) { return x | y; }, s_u64);
+    block_reduce<1>(diff, [](unsigned long long x, unsigned long long y) { return x | y; }, s_u64, 0ull);
     int top = 64 - __clzll((long long)diff[0]);           // bits from `top` up are common to all keys
     if (t < 2) { s_prefix[t] = top < 64 ? key0 & (~0ull << top) : 0ull; s_left[t] = cut[t]; s_same[t] = M; }
     __syncthreads();
@@ -201,7 +214,7 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
         const unsigned long long above = top < 64 ? ~0ull << top : 0ull;
         const unsigned long long pre0 = s_prefix[0], pre1 = s_prefix[1];
         const bool one = pre0 == pre1 && need[0] && need[1];       // both cuts still in the same bin: one histogram
-        for (int r = t; r < M; r += kAssignThreads) {
+        for (int r = t; r < M; r += nt) {
             const unsigned long long key = (unsigned long long)__double_as_longlong(var[r]);
             const int d = (int)((key & ~above) >> shift);
             if (need[0] && (key & above) == pre0) atomicAdd(&s_hist[0][d], 1);
@@ -234,7 +247,7 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
             // one row left at each cut: its key is the rest of the digits
             const unsigned long long known = ~0ull << shift, k0 = s_prefix[0], k1 = s_prefix[1];
             __syncthreads();
-            for (int r = t; r < M; r += kAssignThreads) {
+            for (int r = t; r < M; r += nt) {
                 const unsigned long long key = (unsigned long long)__double_as_longlong(var[r]);
                 if (need[0] && (key & known) == k0) s_prefix[0] = key;
                 if (need[1] && (key & known) == k1) s_prefix[1] = key;
@@ -242,7 +255,7 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
             __syncthreads();
             break;
         }
-        if (t < 256) { s_hist[0][t] = 0; s_hist[1][t] = 0; }
+        for (int i = t; i < 256; i += nt) { s_hist[0][i] = 0; s_hist[1][i] = 0; }
         __syncthreads();
     }
     if (cut[1] == cut[0] && t == 0) { s_prefix[1] = s_prefix[0]; s_left[1] = s_left[0]; s_same[1] = s_same[0]; }
@@ -256,7 +269,7 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
         tie[c] = s_same[c] > s_left[c];                   // more rows share the last key than fit in front of the cut
         double lo = -1.0, hi = -__longlong_as_double(0x7FF0000000000000ll);
         if (cut[c] > 0 && cut[c] < M) {
-            for (int r = t; r < M; r += kAssignThreads) {
+            for (int r = t; r < M; r += nt) {
                 const double v = var[r], e = (double)err[r];
                 if (v <= key_at[c]) lo = fmax(lo, v + e);
                 if (v > key_at[c] || (tie[c] && v == key_at[c])) hi = fmax(hi, e - v);
@@ -264,7 +277,7 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
         }
         edge[2 * c] = lo; edge[2 * c + 1] = hi;
     }
-    block_reduce<4>(edge, [](double x, double y) { return fmax(x, y); }, s_dbl);
+    block_reduce<4>(edge, [](double x, double y) { return fmax(x, y); }, s_dbl, -__longlong_as_double(0x7FF0000000000000ll));
     // 0: in front of the cut, 1: behind it, 2: undecided
     auto side = [&](int c, double v, double e) -> int {
         if (cut[c] <= 0) return 1;
@@ -275,7 +288,7 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
         return (clear || v - e > hi_edge) ? 1 : 2;
     };
     int in_front[2] = {0, 0};
-    for (int r = t; r < M; r += kAssignThreads) {
+    for (int r = t; r < M; r += nt) {
         const double v = var[r], e = (double)err[r];
         const int s0 = side(0, v, e), s1 = side(1, v, e);
         in_front[0] += s0 == 0; in_front[1] += s1 == 0;
@@ -285,14 +298,14 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
     __syncthreads();
     const int nu = s_undecided;
     if (nu > 0) {
-        block_reduce<2>(in_front, [](int x, int y) { return x + y; }, s_int);
+        block_reduce<2>(in_front, [](int x, int y) { return x + y; }, s_int, 0);
         const int want0 = cut[0] - in_front[0], want1 = cut[1] - in_front[1];
-        for (int i = t; i < nu; i += kAssignThreads) {
+        for (int i = t; i < nu; i += nt) {
             const int r = slot[i];
             if (err[r] != 0.0f) { var[r] = exact_variance(a.W + (size_t)r * a.K, a.K); err[r] = 0.0f; }
         }
         __syncthreads();
-        for (int i = t; i < nu; i += kAssignThreads) {
+        for (int i = t; i < nu; i += nt) {
             const int r = slot[i];
             const double v = var[r];
             const int sides = kind[r];
@@ -313,7 +326,7 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
     }
 
     // ---- stable grouping: consecutive rows per thread, prefix sums over the threads
-    const int per = (M + kAssignThreads - 1) / kAssignThreads;
+    const int per = (M + nt - 1) / nt;
     const int r0 = min(M, t * per), r1 = min(M, r0 + per);
     int cnt[3] = {0, 0, 0};
     for (int r = r0; r < r1; ++r) {
@@ -334,7 +347,7 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
     }
     __syncthreads();
     if (warp < 3) {
-        const int v = s_warp[warp][lane];
+        const int v = lane < (nt >> 5) ? s_warp[warp][lane] : 0;
         int incl = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) { const int u = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += u; }
@@ -364,7 +377,7 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
     __syncthreads();
     // block table: first position (inside its group) and count of each kind among the block's 128 rows
     int32_t* blocks = reinterpret_cast<int32_t*>(a.blob + a.off_blocks);
-    for (int i = t; i < 8 * a.nblocks; i += kAssignThreads) {
+    for (int i = t; i < 8 * a.nblocks; i += nt) {
         const int b = i >> 3, j = i & 7, k = j >> 1;
         int v = 0;
         if (k < 3) {
@@ -373,14 +386,182 @@ __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
         }
         blocks[i] = v;
     }
-    if (t == 0) {
-        BlobHeader* H = reinterpret_cast<BlobHeader*>(a.blob);
-        H->magic = kLayerMagic; H->version = kBlobVersion;
-        H->M = M; H->Cin = a.Cin; H->kh = a.kh; H->kw = a.kw; H->Cp = a.Cp; H->Kp = a.Kp;
-        H->nP = a.nP; H->nF4 = a.nF4; H->n8 = a.n8; H->nblocks = a.nblocks; H->pot_mode = a.pot_mode;
-        H->pad0[0] = H->pad0[1] = H->pad0[2] = 0;
-        H->status = 0;
+    if (t == 0) write_header(a);
+}
+
+__global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
+{
+    pdl_wait();
+    pdl_trigger();
+    assign_rows_block(a);
+}
+
+// Up to kSmallThreads * R rows, R of them per thread (row i * threads + t); 128 threads or more, so that the other form can take over.
+template <int R>
+__global__ void __launch_bounds__(kSmallThreads) assign_small_kernel(MetaArgs a)
+{
+    __shared__ uint32_t s_red[4][32];
+    __shared__ uint32_t s_sum[3];
+    __shared__ int s_cnt[3][16 * R + 1];                  // rows of each kind in every 32 rows, then in front of them
+    const int t = threadIdx.x, nt = blockDim.x, lane = t & 31, warp = t >> 5, warps = nt >> 5;
+    const int M = a.M;
+    const int cut[2] = {a.nP, M - a.n8};
+    pdl_wait();
+    pdl_trigger();
+    bool row[R];
+    double v[R];
+    float err[R], al[R];
+    unsigned long long key[R];                            // a non-negative double orders like its bits
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int r = i * nt + t;
+        row[i] = r < M;
+        v[i] = row[i] ? a.st.var[r] : 0.0;
+        err[i] = row[i] ? a.st.err[r] : 0.0f;
+        al[i] = row[i] ? a.alpha[r] : 1.0f;
+        key[i] = row[i] ? (unsigned long long)__double_as_longlong(v[i]) : ~0ull;      // (never below a threshold)
     }
+    // four values reduced over the block (maxima; a minimum is the maximum of the complement)
+    auto block_max4 = [&](uint32_t (&x)[4]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = __reduce_max_sync(0xffffffffu, x[i]);
+        __syncthreads();
+        if (lane == 0)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s_red[i][warp] = x[i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = __reduce_max_sync(0xffffffffu, lane < warps ? s_red[i][lane] : 0u);
+    };
+    uint32_t range[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+        if (row[i]) { range[0] = max(range[0], (uint32_t)(key[i] >> 32)); range[1] = max(range[1], ~(uint32_t)(key[i] >> 32)); }
+    block_max4(range);
+    const unsigned long long key_lo = (unsigned long long)(~range[1]) << 32, key_hi = ((unsigned long long)range[0] + 1ull) << 32;
+
+    // ---- a threshold for each cut with exactly the rows in front of it below (rows of equal variance at a cut: none)
+    unsigned long long lo[2], hi[2], th[2];
+    bool found[2];
+    for (int c = 0; c < 2; ++c) {
+        lo[c] = key_lo; hi[c] = key_hi;
+        th[c] = cut[c] <= 0 ? 0ull : key_hi;
+        found[c] = cut[c] <= 0 || cut[c] >= M;
+    }
+    // One barrier a step for both cuts: the two counts travel in one word that the warps add to (ballots and a shared
+    // atomic: a warp-wide sum instruction takes as long as the rest of the step).  Three words take turns: a step adds to
+    // one, the one in front of it is being read, the one behind is cleared.
+    if (t < 3) s_sum[t] = 0u;
+    __syncthreads();
+    for (int step = 0;; step = step == 2 ? 0 : step + 1) {
+        bool open[2];
+        unsigned long long mid[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            open[c] = !found[c] && hi[c] - lo[c] > 1;
+            mid[c] = lo[c] + ((hi[c] - lo[c]) >> 1);
+        }
+        if (!open[0] && !open[1]) break;                  // (the same for every thread)
+        uint32_t n = 0;
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+            n += (uint32_t)__popc(__ballot_sync(0xffffffffu, key[i] < mid[0])) + ((uint32_t)__popc(__ballot_sync(0xffffffffu, key[i] < mid[1])) << 16);
+        if (lane == 0 && n) atomicAdd(&s_sum[step], n);
+        if (t == 0) s_sum[step == 2 ? 0 : step + 1] = 0u;
+        __syncthreads();
+        n = *reinterpret_cast<volatile uint32_t*>(&s_sum[step]);
+        const int below[2] = {(int)(n & 0xFFFFu), (int)(n >> 16)};
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            if (!open[c]) continue;
+            if (below[c] == cut[c]) { found[c] = true; th[c] = mid[c]; }
+            else if (below[c] < cut[c]) lo[c] = mid[c];
+            else hi[c] = mid[c];
+        }
+    }
+    // ---- do the variances' error bounds leave both cuts clear?  (in fp32, rounded outwards)
+    uint32_t edge[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        if (!row[i]) continue;
+        const uint32_t up = __float_as_uint(__double2float_ru(v[i] + (double)err[i]));
+        const uint32_t down = ~__float_as_uint(__double2float_rd(fmax(v[i] - (double)err[i], 0.0)));
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            if (key[i] < th[c]) edge[2 * c] = max(edge[2 * c], up); else edge[2 * c + 1] = max(edge[2 * c + 1], down);
+        }
+    }
+    __syncwarp();
+    block_max4(edge);
+    const bool clear0 = cut[0] <= 0 || cut[0] >= M || (found[0] && edge[0] < ~edge[1]);
+    const bool clear1 = cut[1] <= 0 || cut[1] >= M || (found[1] && edge[2] < ~edge[3]);
+    if (!clear0 || !clear1) {
+        assign_rows_block(a);
+        return;
+    }
+
+    // ---- kinds, stable grouping, metadata
+    int kind[R];
+    uint32_t mask[R][3];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        kind[i] = key[i] < th[0] ? kPoT4 : (key[i] < th[1] ? kFixed4 : kFixed8);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            mask[i][k] = __ballot_sync(0xffffffffu, row[i] && kind[i] == k);
+            if (lane == 0) s_cnt[k][i * warps + warp] = __popc(mask[i][k]);
+        }
+    }
+    __syncthreads();
+    const int groups = (M + 31) >> 5;                     // of 32 rows
+    if (warp < 3) {
+        // counts to exclusive prefix sums: a warp per kind, R / 2 (or one) consecutive groups a lane
+        constexpr int kPer = (16 * R + 31) / 32;
+        int n[kPer], sum = 0;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int g = lane * kPer + j;
+            n[j] = g < groups ? s_cnt[warp][g] : 0;
+            sum += n[j];
+        }
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int u = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += u; }
+        int before = incl - sum;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int g = lane * kPer + j;
+            if (g <= groups && g <= 16 * R) s_cnt[warp][g] = before;
+            before += n[j];
+        }
+        if (lane == 31 && groups == 32 * kPer) s_cnt[warp][groups] = before;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int g = i * warps + warp, r = i * nt + t, k = kind[i];
+        if (!row[i]) continue;
+        const int p = s_cnt[k][g] + (k == 0 ? 0 : (k == 1 ? a.nP : a.nP + a.nF4)) +
+                      __popc((k == 0 ? mask[i][0] : (k == 1 ? mask[i][1] : mask[i][2])) & ((1u << lane) - 1u));
+        reinterpret_cast<int32_t*>(a.blob + a.off_perm)[p] = r;
+        reinterpret_cast<int32_t*>(a.blob + a.off_slot)[r] = p;
+        (a.blob + a.off_kind)[r] = (uint8_t)k;
+        reinterpret_cast<float*>(a.blob + a.off_alpha)[r] = al[i];
+        reinterpret_cast<float*>(a.blob + a.off_wstep)[r] = __fdiv_rn(al[i], k == kPoT4 ? 64.0f : (k == kFixed4 ? 7.0f : 127.0f));
+        if (a.scheme_out) a.scheme_out[r] = (k == kPoT4) ? RMSMP_SCHEME_POT : RMSMP_SCHEME_FIXED;
+        if (a.bits_out) a.bits_out[r] = (k == kFixed8) ? 8 : 4;
+    }
+    // block table: first position (inside its group) and count of each kind among the block's 128 rows
+    for (int i = t; i < 8 * a.nblocks; i += nt) {
+        const int g = (i >> 3) * 4, j = i & 7, k = j >> 1;
+        int out = 0;
+        if (k < 3) {
+            const int first = s_cnt[k][g], n = s_cnt[k][min(g + 4, groups)] - first;
+            out = (j & 1) ? n : (n ? first : 0);
+        }
+        reinterpret_cast<int32_t*>(a.blob + a.off_blocks)[i] = out;
+    }
+    if (t == 0) write_header(a);
 }
 
 }  // namespace
@@ -404,7 +585,11 @@ cudaError_t launch_assign_meta(const float* dW, const rmsmp_layer& L, const floa
     a.off_kind = L.off_kind; a.off_blocks = L.off_blocks;
     a.M = M; a.Cin = L.Cin; a.kh = L.kh; a.kw = L.kw; a.Cp = L.Cp; a.Kp = L.Kp;
     a.nP = L.nP; a.nF4 = L.nF4; a.n8 = L.n8; a.nblocks = L.nblocks; a.pot_mode = pot_mode;
-    return launch_dependent(assign_kernel, 1, kAssignThreads, 0, st, a);
+    // few warps: cheap barriers, and a block that finds room on an SM while the statistics still run
+    if (M > 8 * kSmallThreads) return launch_dependent(assign_kernel, 1, kAssignThreads, 0, st, a);
+    if (M > 2 * kSmallThreads) return launch_dependent(assign_small_kernel<8>, 1, kSmallThreads, 0, st, a);
+    if (M > kSmallThreads) return launch_dependent(assign_small_kernel<2>, 1, kSmallThreads, 0, st, a);
+    return launch_dependent(assign_small_kernel<1>, 1, (unsigned)(M <= 128 ? 128 : (M + 31) / 32 * 32), 0, st, a);
 }
 
 }  // namespace rmsmp

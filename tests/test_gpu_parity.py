@@ -678,7 +678,8 @@ def _rows_at_the_cuts(name, g, M, K):
 
 @pytest.mark.parametrize("name", ["normal", "copies", "all_equal", "constant", "zero_rows", "offset", "permuted"])
 @pytest.mark.parametrize("M,K,ratio", [(1, 5, (60, 35, 5)), (33, 31, (60, 35, 5)), (257, 100, (50, 40, 10)),
-                                       (1100, 36, (60, 35, 5)), (2500, 64, (65, 30, 5)), (300, 64, (95, 0, 5))])
+                                       (1024, 36, (60, 35, 5)), (1100, 36, (60, 35, 5)), (2500, 64, (65, 30, 5)),
+                                       (4100, 20, (60, 35, 5)), (300, 64, (95, 0, 5)), (128, 16, (0, 100, 0))])
 def test_assignment_at_the_cuts_of_the_ranking(M, K, ratio, name):
     """Whole-number result (which row gets which scheme), so no tolerance: it is the oracle's for rows whose
     variances tie, or differ by less than the summation error, at a cut; fewer and more rows than threads, and more
