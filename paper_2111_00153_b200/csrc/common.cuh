@@ -154,7 +154,9 @@ bool pair_supported(const Problem& p);
 rmsmp_status launch_pair(const Problem& p, cudaStream_t st);
 // problems that do not fill the chip: narrow tiles, the reduction shared by a cluster (split.cu)
 bool split_supported(const Problem& p);
-rmsmp_status launch_split(const Problem& p, cudaStream_t st);
+rmsmp_status launch_split(const Problem& p, cudaStream_t st, bool gather = false);
+// the same kernel with activations gathered by threads, for what the copy engine cannot address
+bool gather_supported(const Problem& p);
 
 // ---- activation boxes of the tensor-core kernels ----
 // A stride-2 convolution reads, for one filter tap, every second pixel of every second input row.

@@ -133,10 +133,11 @@ rmsmp_status dispatch(Problem& p, rmsmp_variant variant, cudaStream_t st)
 {
     if (variant == RMSMP_VARIANT_AUTO) {
         // The tensor path from one token up (M x K, N; CUDA cores against it: 1000x512 1 5.7 / 4.5 us, 4096x4096 1 15.8 / 9.4,
-        // 16384x1024 16 92 / 8.8, 30000x1024 8 85 / 17.2, 109x1333 3076 272 / 9.9); CUDA cores take what the copy engine
-        // cannot address.
+        // 16384x1024 16 92 / 8.8, 30000x1024 8 85 / 17.2, 109x1333 3076 272 / 9.9); what the copy engine
+        // cannot address goes to the tensor cores through gathered tiles.
         p.ragged_k = p.kh == 1 && p.kw == 1 && p.H == 1 && p.W == 1;
         if (tensor_supported(p)) variant = RMSMP_VARIANT_TENSOR;
+        else if (gather_supported(p)) return launch_split(p, st, true);
         else variant = RMSMP_VARIANT_SIMT;
     }
     cudaError_t e = cudaSuccess;

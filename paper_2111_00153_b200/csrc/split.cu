@@ -12,6 +12,10 @@
 // expand the codes into the swizzled stage -- and are the
 // epilogue afterwards, three warps per tensor-memory quarter.  The ring is as deep as the CTA's share of the
 // reduction where that fits, so that all copies are in flight at once.
+// Activations that the copy engine cannot address (a convolution whose channel count is not a multiple of 16) are
+// gathered by the same groups of warps, a thread per pixel: a k-block is then 128 codes of the packed reduction order,
+// whichever taps they belong to.  (A MobileNet-v2 block whose first layer is 24 -> 144 channels on 200,704 pixels: 16.5 ms
+// with that layer on the CUDA cores, 0.15 ms so.)
 // Every mbarrier wait is bounded; when one runs out RMSMP_ERR_TIMEOUT is recorded, the roles leave their loops, and
 // the cluster barriers are still met by every thread.  No load uses cluster multicast.
 #include <cuda.h>
@@ -44,6 +48,7 @@ struct SplitCfg {
     int tmem_cols;
     int cpo;                 // groups of eight columns per owner
     int pre;                 // 1: the A operand comes expanded from a workspace
+    int gather;              // 1: activations gathered by threads; their loads are this many bytes wide (1, 4 or 8)
     uint32_t idesc, tx_b, smem_bytes;
 };
 
@@ -72,9 +77,9 @@ __device__ __forceinline__ void split_sts128(uint32_t addr, uint32_t a, uint32_t
 }
 
 // kRQ: the epilogue writes the next layer's activation codes.  kPre: the A operand comes expanded from a workspace
-// (registers for two CTAs per SM, so that the next launch's set-up fits beside this one).
-template <int kRQ, int kPre>
-__global__ void __launch_bounds__(kSplitThreads, kPre ? 2 : 1)
+// (registers for two CTAs per SM, so that the next launch's set-up fits beside this one).  kGather: see the top.
+template <int kRQ, int kPre, int kGather>
+__global__ void __launch_bounds__(kSplitThreads, kPre || kGather ? 2 : 1)
 split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitMaps maps)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -92,7 +97,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < cfg.nst; ++s) {
-            mbar_init(smem_u32(&s_full[s]), kPre ? 2 : 5);     // activation producer, and weight producer or the four warps of a group
+            mbar_init(smem_u32(&s_full[s]), kPre ? 2 : kGather ? 4 : 5);     // activation producer, and weight producer or the four warps of a group
             mbar_init(smem_u32(&s_empty[s]), 1);
         }
         mbar_init(smem_u32(&s_tfull), 1);
@@ -118,7 +123,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     auto full = [&](int s) { return smem_u32(&s_full[s]); };
     auto empty = [&](int s) { return smem_u32(&s_empty[s]); };
 
-    if (warp == 0 || (warp == kSplitFirst && kPre)) {
+    if ((warp == 0 && !kGather) || (warp == kSplitFirst && kPre)) {
         // ---------------------------------------------------------- TMA producers
         if (lane == 0) {
             int tap = kb0 / cfg.cpt, cc = kb0 - tap * cfg.cpt;
@@ -154,7 +159,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
             for (int i = 0; i < n_kb; ++i) {
                 if (!mbar_wait(full(s), ph, abort_flag)) { ok = false; break; }
                 tc_fence_after();
-                const int ksteps = cc == cfg.cpt - 1 ? cfg.last_ksteps : cfg.bk >> 5;
+                const int ksteps = (kGather ? kb0 + i == cfg.nkb - 1 : cc == cfg.cpt - 1) ? cfg.last_ksteps : cfg.bk >> 5;
                 const uint32_t a_lo = (uint32_t)da + s * a_step, b_lo = (uint32_t)db + s * b_step;
                 for (int k = 0; k < ksteps; ++k)
                     mma_i8_halves(tmem_base, a_lo + 2 * k, b_lo + 2 * k, hi, cfg.idesc, (i | k) ? 1u : 0u);
@@ -165,7 +170,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
             if (ok) mma_commit(smem_u32(&s_tfull));
         }
         __syncwarp();
-    } else if (!kPre) {
+    } else if (!kPre && warp >= kSplitFirst) {
         // ---------------------------------------------------------- expanders
         const int grp = (warp - kSplitFirst) >> 2;
         // A thread expands one row, in original order: eight neighbouring lanes store to eight different swizzle phases.
@@ -187,12 +192,22 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         const bool eight = kind == kFixed8;
         uint4 raw[8];
         auto fetch_pos = [&](int i, int& ksteps) -> const uint4* {
-            const int kb = kb0 + i, tap = kb / cfg.cpt, cc = kb - tap * cfg.cpt;
+            const int kb = kb0 + i, tap = kGather ? 0 : kb / cfg.cpt, cc = kb - tap * cfg.cpt;
             const int koff = tap * p.Cp + cc * cfg.bk;
-            ksteps = i >= n_kb ? 0 : (cc == cfg.cpt - 1 ? cfg.last_ksteps : cfg.bk >> 5);
+            ksteps = i >= n_kb ? 0 : ((kGather ? kb == cfg.nkb - 1 : cc == cfg.cpt - 1) ? cfg.last_ksteps : cfg.bk >> 5);
             return reinterpret_cast<const uint4*>(src + (eight ? koff : koff >> 1));
         };
         auto pieces_of = [&](int ksteps) { return kind < 0 ? 0 : (eight ? 2 * ksteps : ksteps); };      // 16-byte pieces of a row
+        // this thread's pixel of the tile (kGather): its image, and the input position of its tap (0, 0)
+        int px_y = 0, px_x = 0;
+        const int8_t* px_img = p.act;
+        const bool px_ok = kGather && row < cfg.npix && (int64_t)nt * cfg.npix + row < p.N;
+        if (px_ok) {
+            const uint32_t n = (uint32_t)((int64_t)nt * cfg.npix + row), t = n / (uint32_t)p.Wo, b = t / (uint32_t)p.Ho;
+            px_x = (int)(n - t * (uint32_t)p.Wo) * p.stride - p.pad;
+            px_y = (int)(t - b * (uint32_t)p.Ho) * p.stride - p.pad;
+            px_img = p.act + (int64_t)b * p.H * p.W * p.pix_pitch;
+        }
         int ksteps;
         {
             const uint4* q = fetch_pos(grp, ksteps);
@@ -207,6 +222,42 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
             const int next_pieces = pieces_of(next_ksteps);
             if (i >= cfg.nst && !mbar_wait_warp(empty(s), ((i / cfg.nst) & 1) ^ 1, abort_flag)) break;
             const uint32_t dst = sA + s * cfg.a_bytes + row_off;
+            if (kGather) {
+                // 32 codes of one tap at a time; a Cp is a multiple of 32, so a step never spans two taps
+                const bool b_row = row < cfg.n_pad;                        // (the stage has no more rows than that)
+                const uint32_t bdst = sB + s * cfg.b_bytes + (uint32_t)row * 128u;
+#pragma unroll 1
+                for (int u = 0; u < ksteps; ++u) {
+                    const int k = (kb0 + i) * 128 + 32 * u, tap = k / p.Cp, c0 = k - tap * p.Cp;
+                    const int ti = tap / p.kw, y = px_y + ti, x = px_x + tap - ti * p.kw;
+                    const int n = px_ok && (unsigned)y < (unsigned)p.H && (unsigned)x < (unsigned)p.W ? p.Cin - c0 : 0;      // codes of this tap from c0
+                    const int8_t* a = px_img + ((int64_t)y * p.W + x) * p.pix_pitch + c0;
+                    uint32_t w[8];
+                    if (cfg.gather == 8) {
+#pragma unroll
+                        for (int q8 = 0; q8 < 4; ++q8) {
+                            const uint2 v = 8 * q8 < n ? __ldg(reinterpret_cast<const uint2*>(a) + q8) : make_uint2(0u, 0u);
+                            w[2 * q8] = v.x; w[2 * q8 + 1] = v.y;
+                        }
+                    } else if (cfg.gather == 4) {
+#pragma unroll
+                        for (int q4 = 0; q4 < 8; ++q4) w[q4] = 4 * q4 < n ? __ldg(reinterpret_cast<const uint32_t*>(a) + q4) : 0u;
+                    } else {
+#pragma unroll
+                        for (int q4 = 0; q4 < 8; ++q4) {
+                            w[q4] = 0u;
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (4 * q4 + e < n) w[q4] |= (uint32_t)(uint8_t)__ldg(a + 4 * q4 + e) << (8 * e);
+                        }
+                    }
+                    __syncwarp();
+                    if (b_row) {
+                        split_sts128(bdst + (((uint32_t)(2 * u) ^ (uint32_t)(row & 7)) << 4), w[0], w[1], w[2], w[3]);
+                        split_sts128(bdst + (((uint32_t)(2 * u + 1) ^ (uint32_t)(row & 7)) << 4), w[4], w[5], w[6], w[7]);
+                    }
+                }
+            }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (u < ksteps) {
@@ -333,6 +384,16 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
 
 bool split_tile(const Problem& p, int target, SplitCfg& c)
 {
+    if (c.gather) {                                       // any run of pixels
+        const int64_t tiles = (p.N + target - 1) / target;
+        if (tiles > (1 << 24)) return false;
+        c.tb = c.th = 0;
+        c.tiles_per_image = 0;
+        c.npix = (int)((p.N + tiles - 1) / tiles);
+        c.ntn = (int)((p.N + c.npix - 1) / c.npix);
+        c.n_pad = (c.npix + 15) / 16 * 16;
+        return true;
+    }
     const int64_t hw = (int64_t)p.Ho * p.Wo;
     if (hw <= target) {
         c.tb = (int)std::min<int64_t>(target / hw, p.B);
@@ -363,9 +424,10 @@ bool split_tile(const Problem& p, int target, SplitCfg& c)
 // the grid needs.  Against every width and cluster size measured for two dozen problems (256x512 to 4096x4096, 32 to
 // 6272 pixels) its choice is within 5 % of the best.  *us: the time that the cost stands for, as fitted to the same
 // measurements (a workspace: 2.2 us + 1400 units per us, good to 0.4 us; expansion: 1.75 of that - 2 us, good to 2 us).
-bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr)
+bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr, bool gather = false)
 {
-    if (p.pix_pitch % 16 != 0 || (reinterpret_cast<uintptr_t>(p.act) & 15) != 0) return false;
+    if (!gather && (p.pix_pitch % 16 != 0 || (reinterpret_cast<uintptr_t>(p.act) & 15) != 0)) return false;
+    if (gather && (p.wexp || p.rq_codes || p.N >= (int64_t)1 << 31)) return false;
     if (p.wexp && (reinterpret_cast<uintptr_t>(p.wexp) & 15) != 0) return false;
     const int64_t sms = sm_count();
     SplitCfg c;
@@ -377,6 +439,16 @@ bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr)
     if ((int64_t)p.kh * p.kw * c.cpt > (1 << 20)) return false;
     c.nkb = p.kh * p.kw * c.cpt;
     c.last_ksteps = (p.Cin - (c.cpt - 1) * c.bk + 31) / 32;
+    if (gather) {
+        auto fits = [&](int w) { return p.pix_pitch % w == 0 && p.Cin % w == 0 && (reinterpret_cast<uintptr_t>(p.act) & (w - 1)) == 0; };
+        c.gather = fits(8) ? 8 : fits(4) ? 4 : 1;
+        const int steps = p.kh * p.kw * p.Cp / 32;
+        c.bk = 128;
+        c.a_bytes = kBlockRows * 128;
+        c.cpt = 1;
+        c.nkb = (steps + 3) / 4;
+        c.last_ksteps = steps - 4 * (c.nkb - 1);
+    }
     double best_cost = 1e30;
     static const int targets[] = {16, 32, 48, 64, 96, 128};
     for (int target : targets) {
@@ -398,7 +470,7 @@ bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr)
             // clusters of eight do not tile the SMs of every processing cluster: count 5 % fewer for each doubling
             const double usable = (double)sms * (S == 1 ? 1.0 : S == 2 ? 0.97 : S == 4 ? 0.92 : 0.85);
             const double waves = std::max(1.0, std::ceil((double)ctas / usable));
-            const double load = (c.pre ? kBlockRows + c.npix : c.npix) * 2.56, expand = c.pre ? 0.0 : 420.0 * c.bk / 128.0;
+            const double load = (c.pre ? kBlockRows + c.npix : c.npix) * 2.56, expand = c.pre ? 0.0 : (c.gather ? 900.0 : 420.0) * c.bk / 128.0;
             const double kblock = std::max(std::max(load, expand), 90.0 * (c.bk / 32));
             const double cost = waves * (1500.0 + kpc * kblock + (S > 1 ? 900.0 + 14.0 * c.n_pad : 0.0) + 14.0 * c.n_pad / S);
             if (cost < best_cost) { best_cost = cost; best = c; }
@@ -443,15 +515,22 @@ bool split_supported(const Problem& p)
     return plan_split(p, c, &us) && us < other && tensor_map_encoder() != nullptr;
 }
 
-rmsmp_status launch_split(const Problem& p, cudaStream_t st)
+// Convolutions whose activations the copy engine cannot address.
+bool gather_supported(const Problem& p)
 {
     SplitCfg c;
-    if (!plan_split(p, c)) return RMSMP_ERR_VARIANT;
+    return plan_split(p, c, nullptr, true);
+}
+
+rmsmp_status launch_split(const Problem& p, cudaStream_t st, bool gather)
+{
+    SplitCfg c;
+    if (!plan_split(p, c, nullptr, gather)) return RMSMP_ERR_VARIANT;
     EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return RMSMP_ERR_CUDA;
     SplitMaps mp;
     memset(&mp, 0, sizeof(mp));
-    if (!encode_act_maps_4(p, c.bk, c.th, c.tb, mp.act)) return RMSMP_ERR_CUDA;
+    if (!gather && !encode_act_maps_4(p, c.bk, c.th, c.tb, mp.act)) return RMSMP_ERR_CUDA;
     if (c.pre) {
         const cuuint64_t gd[2] = {(cuuint64_t)p.Kp, (cuuint64_t)p.M};
         const cuuint64_t gs[1] = {(cuuint64_t)p.Kp};
@@ -462,10 +541,10 @@ rmsmp_status launch_split(const Problem& p, cudaStream_t st)
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return RMSMP_ERR_CUDA;
     }
-    auto fn = p.rq_codes ? split_kernel<1, 1> : c.pre ? split_kernel<0, 1> : split_kernel<0, 0>;      // (re-quantizing calls have a workspace)
+    auto fn = p.rq_codes ? split_kernel<1, 1, 0> : c.pre ? split_kernel<0, 1, 0> : gather ? split_kernel<0, 0, 1> : split_kernel<0, 0, 0>;      // (re-quantizing calls have a workspace)
     if (p.rq_codes && !c.pre) return RMSMP_ERR_VARIANT;
-    static bool attr_set[3][kMaxDevices] = {};
-    if (!ensure_smem_attr(reinterpret_cast<const void*>(fn), kSplitSmem, attr_set[p.rq_codes ? 2 : c.pre])) return RMSMP_ERR_CUDA;
+    static bool attr_set[4][kMaxDevices] = {};
+    if (!ensure_smem_attr(reinterpret_cast<const void*>(fn), kSplitSmem, attr_set[p.rq_codes ? 2 : gather ? 3 : c.pre])) return RMSMP_ERR_CUDA;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // as launch_dependent
     at[0].val.programmaticStreamSerializationAllowed = 1;

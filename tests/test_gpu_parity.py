@@ -615,6 +615,33 @@ def test_small_convolutions_share_their_reduction(M, Cin, k, stride, pad, B, H, 
             assert np.array_equal(out.cpu().numpy(), c_ref)
 
 
+@pytest.mark.parametrize("M,Cin,k,stride,pad,B,H,W", [
+    (144, 24, 1, 1, 0, 3, 17, 19),       # 8-byte loads, more pixels than a tile, the last tile ragged
+    (40, 20, 3, 1, 1, 2, 9, 7),          # 4-byte loads
+    (33, 3, 7, 2, 3, 2, 21, 15),         # single bytes; 49 taps of one step
+    (130, 5, 3, 2, 1, 1, 8, 300),        # rows wider than any copy box, two row blocks
+    (16, 72, 3, 3, 0, 2, 11, 10),        # a last step of eight codes
+    (64, 200, 5, 1, 2, 1, 6, 6),         # more k-blocks than stages
+    (8, 1, 1, 1, 0, 1, 1, 1),            # one code
+    (24, 9, 2, 1, 1, 5, 3, 3),
+])
+def test_convolutions_of_any_channel_count_under_auto(M, Cin, k, stride, pad, B, H, W):
+    """Channel counts that the copy engine cannot address, any int8 code: exact, both layouts."""
+    g = synth.rng(93, M + Cin + H)
+    Wt = synth.weights_kaiming(g, M, Cin, k, k)
+    scheme, bits = _mixed_map(M, 8, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    act = g.integers(-128, 128, size=(B, H, W, Cin)).astype(np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    _, ws, acc_ref, y_ref = O.layer_conv(Wt, scheme, bits, alpha, act, np.float32(0.25), stride, pad)
+    for layout in (R.OUT_NM, R.OUT_MN):
+        for want_acc in (True, False):
+            y, acc = Hn.conv(layer, d_packed, act, stride, pad, 0.25, R.VARIANT_AUTO, layout, want_acc)
+            if want_acc:
+                assert np.array_equal(acc, acc_ref.reshape(-1, M))
+            assert np.array_equal(np.ascontiguousarray(y).view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
+
+
 # ------------------------------------------------------------------ row assignment on the device
 
 @pytest.mark.parametrize("ratio", [(60, 35, 5), (65, 30, 5), (0, 100, 0), (50, 40, 10)], ids=lambda r: "%d-%d-%d" % r)
