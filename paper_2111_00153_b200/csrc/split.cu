@@ -306,6 +306,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         shift = (!kPre && __ldg(p.kind + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
     }
     const ActFast rq = act_fast_setup(kRQ ? p.rq_alpha : 1.0f, kRQ ? p.rq_kind : 0);
+    const bool out_mn = !kRQ && p.out_mn != 0;
     // the finished sum of this lane's row at column j of the tile
     auto put = [&](int j, int sum) {
         const int a = sum >> shift;
@@ -314,7 +315,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         if (kRQ) {
             p.rq_codes[n * p.ld_codes + m] = (int8_t)act_code_exact(y, p.rq_alpha, p.rq_kind, rq);
         } else {
-            const int64_t o = p.out_mn ? (int64_t)m * p.ld_out + n : n * p.ld_out + m;
+            const int64_t o = out_mn ? (int64_t)m * p.ld_out + n : n * p.ld_out + m;
             p.out[o] = y;
             if (p.acc) p.acc[o] = a;
         }
@@ -331,7 +332,34 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
             for (int g = rank3; g < groups; g += 3) {
                 uint32_t v[8];
                 split_ld8(taddr + 8 * g, v);
-                if (row_ok) {
+                if (out_mn) {
+                    // [row][pixel]: a store straight from the lanes' rows would touch 32 sectors for 128 bytes; the group is
+                    // turned in shared memory (the stages are free: every multiplication has finished) and leaves as
+                    // four rows of 32 bytes a store
+                    const int most = min(8, nvalid - 8 * g);
+                    for (int sub = 0; sub < (p.acc ? 2 : 1); ++sub) {
+                        const uint32_t scratch = sA + (uint32_t)(warp - kSplitFirst) * 1024u;
+                        uint32_t w[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const int a = (int)v[j] >> shift;
+                            w[j] = sub ? (uint32_t)a : __float_as_uint(__fmul_rn(__int2float_rn(a), scale));
+                        }
+                        split_sts128(scratch + lane * 32, w[0], w[1], w[2], w[3]);
+                        split_sts128(scratch + lane * 32 + 16, w[4], w[5], w[6], w[7]);
+                        __syncwarp();
+                        uint32_t* o = sub ? reinterpret_cast<uint32_t*>(p.acc) : reinterpret_cast<uint32_t*>(p.out);
+                        const int row = blk * kBlockRows + quarter * 32 + (lane >> 3);
+                        o += (int64_t)row * p.ld_out + n0 + 8 * g + (lane & 7);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            uint32_t x;
+                            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(scratch + (uint32_t)(i * 128 + lane * 4)) : "memory");
+                            if (row + 4 * i < p.M && (lane & 7) < most) o[(int64_t)(4 * i) * p.ld_out] = x;
+                        }
+                        __syncwarp();
+                    }
+                } else if (row_ok) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
                         if (8 * g + j < nvalid) put(8 * g + j, (int)v[j]);
@@ -466,7 +494,7 @@ bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr, bool gat
             // fewer than three stages are not enough for the three expander groups: a group may run ahead of the others by
             // two of its own k-blocks, and a stage's barrier tells only neighbouring phases apart
             if (c.nst < 3 && c.nst < kpc) continue;
-            c.smem_bytes = (uint32_t)(c.nst * (c.a_bytes + c.b_bytes) + red + 1024);
+            c.smem_bytes = (uint32_t)std::max(c.nst * (c.a_bytes + c.b_bytes) + red, (kSplitThreads / 32 - kSplitFirst) * 1024) + 1024;
             // clusters of eight do not tile the SMs of every processing cluster: count 5 % fewer for each doubling
             const double usable = (double)sms * (S == 1 ? 1.0 : S == 2 ? 0.97 : S == 4 ? 0.92 : 0.85);
             const double waves = std::max(1.0, std::ceil((double)ctas / usable));

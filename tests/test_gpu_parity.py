@@ -561,6 +561,43 @@ def test_small_linear_layers_share_their_reduction(M, K, N, variant):
             assert np.array_equal(y.view(np.uint32), O.epilogue(acc_ref, ws, np.float32(0.25)).view(np.uint32))
 
 
+@pytest.mark.parametrize("workspace", [False, True])
+@pytest.mark.parametrize("M,K,N", [
+    (33, 64, 1), (130, 192, 37), (1088, 64, 515),      # rows and pixels beyond the last group, rows of no multiple of 16 bytes
+    (96, 2048, 67), (257, 1008, 129),                  # a reduction shared by a cluster
+    (130, 1024, 9001), (40, 160, 38001),               # more tiles than SMs
+])
+def test_outputs_by_row_of_any_length(M, K, N, workspace):
+    """[row][pixel] outputs, turned in shared memory: exact, with and without the sums, nothing beyond the matrix."""
+    import torch
+    g = synth.rng(95, M + K + N)
+    Wt = synth.weights_normal(g, (M, K))
+    scheme, bits = _mixed_map(M, 5, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    act = g.integers(-16, 17, size=(N, K)).astype(np.int8)
+    _, ws, acc_ref, _ = O.layer_linear(Wt, scheme, bits, alpha, act, np.float32(0.25))
+    y_ref = np.ascontiguousarray(O.epilogue(acc_ref, ws, np.float32(0.25)).T)
+    ld = (K + 15) // 16 * 16
+    a = torch.zeros((N, ld), dtype=torch.int8, device="cuda")
+    a[:, :K] = torch.from_numpy(act).cuda()
+    if workspace:
+        d_ws = torch.empty(R.rmsmp_workspace_bytes(layer), dtype=torch.int8, device="cuda")
+        R.rmsmp_expand_weights(layer, d_packed, d_ws)
+    for want_acc in (True, False):
+        y = torch.full((M * N + 64,), -7.0, dtype=torch.float32, device="cuda")
+        acc = torch.full((M * N + 64,), -9, dtype=torch.int32, device="cuda") if want_acc else None
+        if workspace:
+            R.rmsmp_gemm_workspace(layer, d_packed, d_ws, a, N, ld, 0.25, y, N, R.OUT_MN, acc)
+        else:
+            R.rmsmp_gemm(layer, d_packed, a, N, ld, 0.25, y, N, R.OUT_MN, acc)
+        out = y.cpu().numpy()
+        assert np.array_equal(out[:M * N].view(np.uint32), y_ref.ravel().view(np.uint32)) and (out[M * N:] == -7.0).all()
+        if want_acc:
+            out = acc.cpu().numpy()
+            assert np.array_equal(out[:M * N], acc_ref.T.ravel()) and (out[M * N:] == -9).all()
+
+
 @pytest.mark.parametrize("N", [1, 2, 31, 33, 300])
 @pytest.mark.parametrize("M,K", [(96, 1), (130, 17), (200, 127), (64, 200), (1000, 513), (20000, 72)])
 def test_linear_layers_of_any_length_under_auto(M, K, N):
