@@ -145,6 +145,7 @@ bool stream_build_table(const Problem* probs, int count, int sms, uint8_t* h_tab
 cudaError_t launch_stream(const uint8_t* d_table, int grid, uint32_t smem_bytes, int count, uint32_t conv_grid_x, cudaStream_t st);
 // returns false if the tensor variant cannot run this problem (alignment / shape)
 bool tensor_supported(const Problem& p);
+bool tensor_resident(const Problem& p);   // the weights of a row block stay in shared memory
 rmsmp_status launch_tensor(const Problem& p, cudaStream_t st);
 // fills four CUtensorMap objects (see act_parity_split; only the first is used without the split) for
 // activation boxes of bk channels x th output rows x tb images, swizzle width = bk bytes

@@ -529,12 +529,11 @@ bool split_supported(const Problem& p)
     const double sms = sm_count(), tiles = (double)((p.N + 255) / 256 * p.nblocks);
     const bool bk64 = p.Cin % 128 != 0 && p.Cin % 128 <= 64;
     const double nkb = (double)p.kh * p.kw * ((p.Cin + 127) / 128) * (bk64 && p.Cin < 128 ? 0.5 : 1.0);
-    const bool resident = p.nblocks == 1 && nkb * kBlockRows * 128 <= 72 * 1024;
     double other;
-    if (p.wexp || resident) {
+    if (p.wexp || tensor_resident(p)) {
         if (tiles >= sms) return false;
         const double n = (double)std::min<int64_t>(p.N, 256);
-        other = 3.4 + 1.2 * n / 256 + nkb * (0.28 + 0.13 * n / 256) + (p.wexp ? 0.0 : 1.5);
+        other = 3.4 + 1.2 * n / 256 + nkb * (0.28 + 0.13 * n / 256) + (p.wexp ? 0.0 : 1.7 + 0.7 * nkb);
     } else {
         other = 2.5 + std::ceil(tiles / sms) * (1.5 + nkb * (p.Wo > 1 ? 1.15 : 1.5));
     }

@@ -46,6 +46,7 @@ constexpr int kThreads = 32 * (2 + kNumExpWarps + kNumEpiWarps);
 constexpr int kWarpStage = 32 * 32 * 4;          // 4 KB: 32 pixels x 32 rows of fp32/int32
 constexpr int kRawBoxRows = 16;                  // rows per raw weight box
 constexpr int kMaxRing = 8;
+constexpr int kResidentBlocks = 16;              // row blocks of a layer with resident weights (the grid is a multiple of them)
 constexpr int kSmemLimit = 232448 - 1024;        // 227 KB per CTA less room for the static variables
 
 struct TensorCfg {
@@ -74,8 +75,9 @@ struct TensorCfg {
     int a_bytes, b_bytes;  // one A / B stage
     int fill;              // 1 (resident weights, no workspace given): the CTA expands its row block from the packed codes
                            //    itself, once, instead of copying expanded weights in
-    int ares;              // 1 (pre mode, one row block, small K): the expanded weights of all k-blocks are loaded once
-                           //    per CTA and stay in shared memory; only activation boxes flow through a ring
+    int ares;              // 1 (pre mode, small K): the expanded weights of all k-blocks are loaded once per CTA and stay in
+                           //    shared memory; only activation boxes flow through a ring.  The grid is a multiple of the row
+                           //    blocks, so that all tiles of a CTA are of one block
     int m2;                // 1 (pre mode, even number of row blocks): a tile covers TWO row blocks.  Both use the same
                            //    activation stage, so a k-block brings 64 KB for eight MMAs instead of 48 KB for four;
                            //    the two accumulators take the two halves of tensor memory
@@ -158,60 +160,75 @@ __device__ __forceinline__ void expand_task(uint32_t meta, uint32_t raw_stage, u
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst ^ 16u), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
 }
 
-// Resident weights without a workspace: every thread of the CTA expands 16-code granules of the row block
-// from the packed codes (exact int8 values, as expand_kernel writes them) straight into the resident stages,
-// at the place the bulk copy of an expanded [rows][bk] box would have put them: stage kb = (tap, channel
-// chunk) holds codes [tap * Cp + chunk * bk, + bk) of every row, 16-byte units XOR-swizzled by the row
-// (128-byte rows: unit ^ (row & 7); 64-byte rows: unit ^ ((row >> 1) & 3)), zeros beyond M and Kp; with
-// duplicated rows (M <= 64) a second copy goes to lanes 64..127.
-__device__ __forceinline__ void fill_resident_weights(const Problem& p, const TensorCfg& cfg, uint32_t sA, int tid, int nthreads)
+// Resident weights without a workspace: the threads of the CTA expand the row block from the packed codes (exact
+// int8 values, as expand_kernel writes them) straight into the resident stages, at the place the bulk copy of an
+// expanded [rows][bk] box would have put them: stage kb = (tap, channel chunk) holds codes
+// [tap * Cp + chunk * bk, + bk) of every row, 16-byte units XOR-swizzled by the row (128-byte rows: unit ^ (row & 7);
+// 64-byte rows: unit ^ ((row >> 1) & 3)), zeros beyond M and Kp; with duplicated rows (M <= 64) a second copy goes to
+// lanes 64..127.  Nothing overlaps with it in a CTA's first tile, and it is a chain (slot, codes, expansion): a few
+// threads share a row, and a thread has the loads of four pieces of 32 codes in flight at a time (512x512 N=4096, all in one tile per
+// CTA: 14.7 us with a load at a time and half of each piece kept, 10.8 so; 128x512 N=2000 10.6).
+__device__ __forceinline__ void fill_resident_weights(const Problem& p, const TensorCfg& cfg, uint32_t sA, int row_first, int tid, int nthreads)
 {
     const int rows = cfg.dup ? kBlockRows / 2 : kBlockRows;
-    const int gpr = cfg.bk >> 4;
+    const int pshift = cfg.bk == 128 ? 2 : 1;            // 32-code pieces of a row and k-block: 4 or 2
     const int n4 = p.nP + p.nF4;
-    // a few threads per row, each with every tpr-th granule of it: kind and place of the row are read once, and a
-    // thread's loads are independent of one another
     const int tpr = nthreads / rows;
     const int r = tid / tpr, sub = tid - r * tpr;
     if (r < rows) {
-        const bool have = r < p.M;
-        const int kind = have ? (int)p.kind[r] : kFixed8;
-        const int slot = have ? p.slot[r] : 0;
+        const int m = row_first + r;
+        const bool have = m < p.M;
+        const int kind = have ? (int)p.kind[m] : kFixed8;
+        const int slot = have ? p.slot[m] : 0;
         const uint8_t* src = (kind == kFixed8) ? p.q8 + (size_t)(have ? slot - n4 : 0) * p.Kp : p.q4 + (size_t)slot * (p.Kp >> 1);
         const uint32_t phase = (cfg.bk == 128) ? (uint32_t)(r & 7) : (uint32_t)((r >> 1) & 3);
         const uint32_t row_base = sA + (uint32_t)r * (uint32_t)cfg.bk;
-        const int gtot = cfg.nkb * gpr;
-#pragma unroll 4
-        for (int g = sub; g < gtot; g += tpr) {
-            const int kb = g / gpr, q = g - kb * gpr;
-            const int tap = kb / cfg.cpt, cc = kb - tap * cfg.cpt;
-            const int k = tap * p.Cp + cc * cfg.bk + q * 16;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (have && k < p.Kp) {
-                if (kind == kFixed8) {
-                    v = __ldg(reinterpret_cast<const uint4*>(src + k));
-                } else {
-                    const uint4 raw = __ldg(reinterpret_cast<const uint4*>(src + ((k >> 5) << 4)));
-                    uint32_t w[8];
-                    if (kind == kPoT4) {
-                        expand_pot_chunk(raw, w);
-                    } else {
-                        expand_fixed4_chunk_x16(raw, w);
+        const int pieces = cfg.nkb << pshift;
+        auto code_of = [&](int i) {                      // first code of piece i in the packed row
+            const int kb = i >> pshift;
+            const int tap = cfg.cpt == 1 ? kb : kb / cfg.cpt;
+            return tap * p.Cp + (kb - tap * cfg.cpt) * cfg.bk + 32 * (i - (kb << pshift));
+        };
+        for (int base = sub; base < pieces; base += 4 * tpr) {
+            uint4 raw[4], raw2[4];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {       // 16 * value -> value: shift every byte right by four, keeping its sign
-                            const uint32_t x = w[j];
-                            w[j] = ((x >> 4) & 0x0F0F0F0Fu) | (((x >> 7) & 0x01010101u) * 0xF0u);
-                        }
+            for (int u = 0; u < 4; ++u) {
+                const int i = base + u * tpr;
+                raw[u] = raw2[u] = make_uint4(0u, 0u, 0u, 0u);
+                if (have && i < pieces) {
+                    const int k = code_of(i);
+                    if (k < p.Kp) {
+                        raw[u] = __ldg(reinterpret_cast<const uint4*>(src + (kind == kFixed8 ? k : k >> 1)));
+                        if (kind == kFixed8) raw2[u] = __ldg(reinterpret_cast<const uint4*>(src + k + 16));
                     }
-                    const int h = (k >> 4) & 1;
-                    v = h ? make_uint4(w[4], w[5], w[6], w[7]) : make_uint4(w[0], w[1], w[2], w[3]);
                 }
             }
-            const uint32_t dst = row_base + (uint32_t)kb * (uint32_t)cfg.a_bytes + (((uint32_t)q ^ phase) << 4);
-            // (no memory clobber: the loads of the next granules may move above these stores)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
-            if (cfg.dup)
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(cfg.a_bytes / 2)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = base + u * tpr;
+                if (i >= pieces) continue;
+                uint32_t w[8] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w, raw2[u].x, raw2[u].y, raw2[u].z, raw2[u].w};
+                if (kind == kPoT4) {
+                    expand_pot_chunk(raw[u], w);
+                } else if (kind == kFixed4) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {        // nibbles to bytes; a set sign bit adds the 0xF0 above it
+                        const uint32_t hi = (w[j] >> 4) & 0x0F0F0F0Fu, lo = w[j] & 0x0F0F0F0Fu;
+                        w[j] = hi + (hi & 0x08080808u) * 0x1Eu;
+                        w[j + 4] = lo + (lo & 0x08080808u) * 0x1Eu;
+                    }
+                }
+                const int kb = i >> pshift;
+                const uint32_t unit = (uint32_t)(i - (kb << pshift)) * 2u;
+                const uint32_t dst = row_base + (uint32_t)kb * (uint32_t)cfg.a_bytes;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t at = dst + (((unit + (uint32_t)h) ^ phase) << 4);
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(w[4 * h]), "r"(w[4 * h + 1]), "r"(w[4 * h + 2]), "r"(w[4 * h + 3]));
+                    if (cfg.dup)
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + (uint32_t)(cfg.a_bytes / 2)), "r"(w[4 * h]), "r"(w[4 * h + 1]), "r"(w[4 * h + 2]), "r"(w[4 * h + 3]));
+                }
+            }
         }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the MMAs read these bytes through the async proxy
@@ -310,7 +327,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     if (kAres && cfg.fill && warp != 0) {
         // every warp but the activation producer's (whose first copies go out meanwhile) expands the row block;
         // one of them then reports the resident weights to the MMA thread
-        if (my_tiles > 0) fill_resident_weights(p, cfg, sA, (int)threadIdx.x - 32, kThreads - 32);
+        if (my_tiles > 0) fill_resident_weights(p, cfg, sA, (int)(first % cfg.nbt) * kBlockRows, (int)threadIdx.x - 32, kThreads - 32);
         asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32) : "memory");
         if (threadIdx.x == 32 && my_tiles > 0) mbar_arrive(bar_fullA);
     }
@@ -328,7 +345,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 for (int kb = 0; kb < cfg.nkb; ++kb) {
                     const int koff = tap * p.Cp + cc * cfg.bk;
                     const uint32_t dst = sA + kb * cfg.a_bytes;
-                    tma_load_2d(dst, &maps.wexp, bar_fullA, koff, 0);
+                    tma_load_2d(dst, &maps.wexp, bar_fullA, koff, (int)(first % cfg.nbt) * kBlockRows);
                     if (cfg.dup) tma_load_2d(dst + cfg.a_bytes / 2, &maps.wexp, bar_fullA, koff, 0);
                     if (++cc == cfg.cpt) { cc = 0; ++tap; }
                 }
@@ -397,22 +414,6 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         {
             uint32_t sb = 0, phB = 0, sr = 0, phR = 0;
             bool ok = true;
-            if (kAres && lane == 0 && my_tiles > 0) {
-                // resident weights: every k-block's rows, once
-                mbar_arrive_expect_tx(bar_fullA, (uint32_t)(cfg.nkb * cfg.a_bytes));
-                int tap = 0, cc = 0;
-                for (int kb = 0; kb < cfg.nkb; ++kb) {
-                    const int koff = tap * p.Cp + cc * cfg.bk;
-                    const uint32_t dst = sA + kb * cfg.a_bytes;
-                    if (cfg.dup) {
-                        tma_load_2d(dst, &maps.wexp, bar_fullA, koff, 0);
-                        tma_load_2d(dst + cfg.a_bytes / 2, &maps.wexp, bar_fullA, koff, 0);
-                    } else {
-                        tma_load_2d(dst, &maps.wexp, bar_fullA, koff, 0);
-                    }
-                    if (++cc == cfg.cpt) { cc = 0; ++tap; }
-                }
-            }
             for (int64_t tile = first; tile < cfg.ntiles && ok; tile += step) {
                 const int blk = (int)(tile % p.nblocks);
                 const int64_t nt = tile / p.nblocks;
@@ -436,22 +437,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 int tap = 0, cc = 0;
                 for (int kb = 0; kb < cfg.nkb; ++kb) {
                     const int c0 = cc * cfg.bk, koff = tap * p.Cp + c0;
-                    if (kAres) {
-                        // weights are resident
-                    } else if (kPre) {
-                        // weights already expanded: one swizzled 128-row box straight into the A stage
-                        if (!mbar_wait_warp(bar_emptyA + 8 * sr, phR ^ 1, abort_flag)) { ok = false; break; }
-                        if (lane == 0) {
-                            mbar_arrive_expect_tx(bar_fullA + 8 * sr, cfg.a_bytes);
-                            if (cfg.dup) {
-                                tma_load_2d(sA + sr * cfg.a_bytes, &maps.wexp, bar_fullA + 8 * sr, koff, 0);
-                                tma_load_2d(sA + sr * cfg.a_bytes + cfg.a_bytes / 2, &maps.wexp, bar_fullA + 8 * sr, koff, 0);
-                            } else {
-                                tma_load_2d(sA + sr * cfg.a_bytes, &maps.wexp, bar_fullA + 8 * sr, koff, blk * kBlockRows);
-                            }
-                        }
-                        if (++sr == (uint32_t)cfg.nA) { sr = 0; phR ^= 1; }
-                    } else {
+                    {
                         // packed weights of this tile's rows, group by group
                         if (!mbar_wait_warp(bar_emptyR + 8 * sr, phR ^ 1, abort_flag)) { ok = false; break; }
                         const uint32_t rbar = bar_fullR + 8 * sr;
@@ -990,13 +976,10 @@ bool plan(const Problem& p, TensorCfg& c)
     c.colshift = 0;
     c.pre = p.wexp ? 1 : 0;
     c.fill = 0;
-    if (!p.wexp && p.nblocks == 1 && !p.rq_codes) {
-        // no workspace, but the whole row block's expanded weights would stay resident: the CTA expands them once
-        // itself and the layer runs in the workspace form
-        const int bk = ((p.Cin % 128 != 0) && (p.Cin % 128 <= 64)) ? 64 : 128;
-        const int64_t nkb = (int64_t)p.kh * p.kw * ((p.Cin + bk - 1) / bk);
-        if (nkb * kBlockRows * bk <= 72 * 1024) { c.pre = 1; c.fill = 1; }
-    }
+    const bool resident = tensor_resident(p);
+    // no workspace, but a whole row block's expanded weights stay resident: the CTA expands them once itself and the
+    // layer runs in the workspace form
+    if (!p.wexp && resident) { c.pre = 1; c.fill = 1; }
     // 64-byte k-blocks when a 128-byte row would be at most half used by the (last) channel chunk
     c.bk = (c.pre && (p.Cin % 128 != 0) && (p.Cin % 128 <= 64)) ? 64 : 128;
     c.a_bytes = kBlockRows * c.bk;
@@ -1017,7 +1000,7 @@ bool plan(const Problem& p, TensorCfg& c)
         c.nA = (c.bk == 64) ? 6 : 3; c.nB = (c.bk == 64) ? 8 : 4; c.nR = 0; c.raw_bytes = 0; c.out_bufs = 1;
         c.epi_warps = kNumExpWarps + kNumEpiWarps - 1;   // warp 2 fetches the weights (unless they are resident)
         c.dup = (p.M <= 64) ? 1 : 0;
-        if (p.nblocks == 1 && (int64_t)c.nkb * c.a_bytes <= 72 * 1024) {
+        if (resident) {
             c.ares = 1;
             c.epi_warps = kNumExpWarps + kNumEpiWarps;
             c.nA = c.nkb;
@@ -1097,6 +1080,21 @@ bool encode_act_maps_4(const Problem& p, int bk, int th, int tb, void* maps4)
     EncodeTiledFn enc = encode_fn();
     return enc && encode_act_maps(enc, p, bk, th, tb, bk == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                                   static_cast<CUtensorMap*>(maps4));
+}
+
+// Whether the persistent kernel keeps a row block's expanded weights in shared memory: they fit beside the activation
+// ring, and the grid can be a multiple of the row blocks (a CTA then stays with one).  Without a workspace that is always
+// the better form: the codes are expanded once per CTA, not per tile (144x160 on 740,050 pixels 355 against 131 us,
+// 2048x512 N=4096 20.9 against 13.8).  With one, the weights of several row blocks are a stream that the activations of a
+// first tile would wait behind (1024x512 N=4096, a tile per CTA: 8.1 us resident, 7.3 through the rings), and save
+// shared-memory fills from two tiles per CTA up (144x32 on 200,704 pixels 39.7 against 36.1, 3x3 256x64 on 50,176 20.7
+// against 17.7).
+bool tensor_resident(const Problem& p)
+{
+    if (p.nblocks > kResidentBlocks || (!p.wexp && p.rq_codes)) return false;
+    const int bk = ((p.Cin % 128 != 0) && (p.Cin % 128 <= 64)) ? 64 : 128;
+    if ((int64_t)p.kh * p.kw * ((p.Cin + bk - 1) / bk) * kBlockRows * bk > 72 * 1024) return false;
+    return !p.wexp || p.nblocks == 1 || (p.N + kTileN - 1) / kTileN * p.nblocks >= 2 * (int64_t)sm_count();
 }
 
 bool tensor_supported(const Problem& p)
@@ -1202,7 +1200,7 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
     if (!fn) return RMSMP_ERR_VARIANT;
     static bool attr_set[4][2][3][kMaxDevices] = {};
     if (!ensure_smem_attr(reinterpret_cast<const void*>(fn), kSmemLimit, attr_set[mode][i2][io])) return RMSMP_ERR_CUDA;
-    const int grid = (int)std::min<int64_t>(c.ntiles, sm_count());
+    const int grid = (int)std::min<int64_t>(c.ntiles, c.ares ? sm_count() / c.nbt * c.nbt : sm_count());
     if (launch_dependent(fn, (unsigned)grid, kThreads, c.smem_bytes, st, p, c, mp) != cudaSuccess) {
         cudaGetLastError();
         return RMSMP_ERR_CUDA;

@@ -948,3 +948,25 @@ def test_linear_layer_without_workspace_on_resident_weights(M, K, N, layout):
     y, acc = Hn.gemm(layer, d_packed, act, 0.125, R.VARIANT_TENSOR, out_layout=layout)
     v_ref, ws = O.quantize_rows(W, scheme, bits, alpha)
     _check_layer_outputs(y, acc, O.matmul(v_ref, act), ws, np.float32(0.125), alpha, scheme, bits)
+
+
+@pytest.mark.parametrize("variant", [R.VARIANT_AUTO, Hn.WORKSPACE], ids=["plain", "workspace"])
+@pytest.mark.parametrize("M,Cin,k,B,H,W", [
+    (130, 64, 1, 38001, 1, 1),      # two row blocks, the second of two rows; more than two tiles per SM
+    (1930, 96, 1, 5121, 1, 1),      # sixteen row blocks: a grid of 144 CTAs, a last tile of one pixel
+    (300, 160, 1, 27, 41, 37),      # 64-byte k-blocks with a half-used last chunk, tiles of whole image rows
+    (200, 64, 3, 13, 56, 56),       # three taps per stage, shifted columns
+    (140, 64, 3, 1, 9, 13),         # a tile per row block
+])
+def test_resident_weights_of_several_row_blocks(M, Cin, k, B, H, W, variant):
+    """Every CTA keeps the weights of one of the layer's row blocks: exact sums and outputs for every block."""
+    g = synth.rng(96, M + Cin + W)
+    Wt = synth.weights_kaiming(g, M, Cin, k, k)
+    scheme, bits = _mixed_map(M, M + k, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    act = g.integers(-8, 16, size=(B, H, W, Cin)).astype(np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    _, ws, acc_ref, y_ref = O.layer_conv(Wt, scheme, bits, alpha, act, np.float32(0.25), 1, k // 2)
+    y, acc = Hn.conv(layer, d_packed, act, 1, k // 2, 0.25, variant)
+    assert np.array_equal(acc, acc_ref.reshape(-1, M))
+    assert np.array_equal(y.view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
