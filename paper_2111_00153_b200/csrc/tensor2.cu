@@ -42,7 +42,7 @@ struct PairCfg {
     int tb, th;              // images / output rows per half
     int npix_h;              // pixels per half
     int nh_pad;              // npix_h rounded up to 8: accumulator columns per half
-    int halves_per_image;    // Ho/th when tb == 1 and th < Ho, else 0
+    int halves_per_image;    // ceil(Ho/th) when tb == 1 and th < Ho, else 0 (the last half of an image ends at row Ho)
     int64_t nhalves;         // halves in the problem
     int64_t ntiles_n;        // pixel tiles = ceil(nhalves / 2)
     int nbt;                 // row-block pairs
@@ -182,7 +182,7 @@ __device__ __forceinline__ HalfPos half_pos(const Problem& p, const PairCfg& cfg
     HalfPos r;
     if (cfg.halves_per_image) {
         r.b0 = (int)(hf / cfg.halves_per_image);
-        r.h0 = (int)(hf - (int64_t)r.b0 * cfg.halves_per_image) * cfg.th;
+        r.h0 = min((int)(hf - (int64_t)r.b0 * cfg.halves_per_image) * cfg.th, p.Ho - cfg.th);
         r.n0 = ((int64_t)r.b0 * p.Ho + r.h0) * p.Wo;
     } else {
         r.b0 = (int)(hf * cfg.tb);
@@ -444,11 +444,10 @@ bool plan_pair(const Problem& p, PairCfg& c)
         c.halves_per_image = 0;
         c.nhalves = (p.B + c.tb - 1) / c.tb;
     } else {
-        int th = 1;
-        for (int d = 1; d <= p.Ho; ++d)
-            if (p.Ho % d == 0 && (int64_t)d * p.Wo <= 128) th = d;
-        c.th = th; c.tb = 1;
-        c.halves_per_image = p.Ho / th;
+        const int most = std::min(128 / p.Wo, 256 / p.stride);
+        c.halves_per_image = (p.Ho + most - 1) / most;
+        c.th = (p.Ho + c.halves_per_image - 1) / c.halves_per_image;
+        c.tb = 1;
         c.nhalves = (int64_t)p.B * c.halves_per_image;
     }
     if ((int64_t)c.th * p.stride > 256) return false;

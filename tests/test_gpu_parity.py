@@ -970,3 +970,28 @@ def test_resident_weights_of_several_row_blocks(M, Cin, k, B, H, W, variant):
     y, acc = Hn.conv(layer, d_packed, act, 1, k // 2, 0.25, variant)
     assert np.array_equal(acc, acc_ref.reshape(-1, M))
     assert np.array_equal(y.view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
+
+
+@pytest.mark.parametrize("layout", [R.OUT_NM, R.OUT_MN], ids=["nm", "mn"])
+@pytest.mark.parametrize("variant", [R.VARIANT_AUTO, Hn.WORKSPACE], ids=["plain", "workspace"])
+@pytest.mark.parametrize("M,Cin,k,stride,B,H,W", [
+    (130, 64, 3, 1, 40, 29, 31),     # four tiles of eight rows: three rows twice
+    (96, 160, 3, 1, 60, 23, 32),     # tiles of 256 pixels that start at no multiple of the tile
+    (256, 128, 3, 1, 45, 17, 19),    # halves of six rows for pairs of CTAs, pixels of no multiple of 32
+    (64, 16, 5, 2, 40, 74, 41),      # a stride of two
+    (72, 32, 1, 1, 90, 29, 23),      # a 1x1 layer: tiles across images
+])
+def test_images_whose_rows_no_tile_divides(M, Cin, k, stride, B, H, W, variant, layout):
+    """The last tile of an image repeats rows of the one before it: exact everywhere, nothing beyond."""
+    g = synth.rng(97, M + Cin + W)
+    Wt = synth.weights_kaiming(g, M, Cin, k, k)
+    scheme, bits = _mixed_map(M, M + k, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    act = g.integers(-8, 16, size=(B, H, W, Cin)).astype(np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    _, ws, acc_ref, y_ref = O.layer_conv(Wt, scheme, bits, alpha, act, np.float32(0.25), stride, k // 2)
+    for want_acc in (True, False):
+        y, acc = Hn.conv(layer, d_packed, act, stride, k // 2, 0.25, variant, layout, want_acc)
+        if want_acc:
+            assert np.array_equal(acc, acc_ref.reshape(-1, M))
+        assert np.array_equal(np.ascontiguousarray(y).view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
