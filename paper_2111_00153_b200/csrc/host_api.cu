@@ -744,6 +744,9 @@ static rmsmp_status conv_impl(const rmsmp_layer* L, const void* d_packed, const 
     p.act = d_act;
     p.B = B; p.H = H; p.W = W; p.Ho = Ho; p.Wo = Wo; p.stride = stride; p.pad = pad;
     p.pix_pitch = L->Cin; p.N = N;
+    // A 1x1 convolution of step one is a linear layer over all pixels: tiles need not end with an image's rows, nor are
+    // they cut to whole ones (192x32 on 64 images of 56x56, codes out: 34.2 against 30.5 us; 512x256 of 28x28 24.7, 22.8).
+    if (L->kh == 1 && L->kw == 1 && stride == 1 && pad == 0 && N <= INT32_MAX) { p.B = (int)N; p.H = p.W = p.Ho = p.Wo = 1; }
     p.act_step = act_step; p.out = d_out; p.acc = d_acc;
     p.out_mn = (out_layout == RMSMP_OUT_MN);
     p.ld_out = p.out_mn ? N : L->M;
