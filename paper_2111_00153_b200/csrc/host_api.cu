@@ -123,7 +123,6 @@ void fill_problem(Problem& p, const rmsmp_layer* L, const void* d_packed)
     p.status = reinterpret_cast<uint32_t*>(const_cast<uint8_t*>(blob) + kStatusOffset);
     p.M = L->M; p.Cin = L->Cin; p.kh = L->kh; p.kw = L->kw; p.Cp = L->Cp; p.Kp = L->Kp;
     p.nP = L->nP; p.nF4 = L->nF4; p.n8 = L->n8; p.nblocks = L->nblocks;
-    p.raw_stage_bytes = L->raw_stage_bytes;
     p.wexp = nullptr;
     p.ragged_k = 0;
     p.rq_codes = nullptr; p.rq_alpha = 1.0f; p.rq_kind = 0; p.ld_codes = 0;

@@ -521,9 +521,10 @@ bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr, bool gat
 // Which of the two kernels takes a problem.  With a workspace the persistent kernel takes whatever fills the chip;
 // below that its time is one tile's: 3.4 us + 1.2 for the output of 256 pixels + 0.28 to 0.41 per k-block of 128 codes
 // (measured: 256x512 N=64 4.8 us against 4.1 here, 256x2304 N=196 11.7 against 5.4, 512x4608 N=49 16 against 6,
-// 768x3072 N=512 13.5 against 10.2, N=2048 13.7 against 14).  Without one it expands the codes again for every tile,
-// 1.15 us (tiles of up to 224 pixels) or 1.5 us (256 tokens) a k-block and round of tiles: 768x3072 N=512 40 us against
-// 12.4 here, 256x2304 N=6272 23.2 against 15.7, N=25088 41 against 63.
+// 768x3072 N=512 13.5 against 10.2, N=2048 13.7 against 14).  Without one it expands the weights first, 1.7 us + 0.7 a
+// k-block, if they stay resident (128x512 N=2000 10.6 against 6.5, 1024x512 N=4096 10.9 against 17.4), and otherwise
+// again for every tile, 0.59 us a k-block and round of tiles (768x3072 N=1024 21.5 against 14.7, N=4096 22.2 against 37.5;
+// 3x3 256x256 on 6272 pixels 17.8 against 15.9, on 12,544 18.2 against 31.5).
 bool split_supported(const Problem& p)
 {
     const double sms = sm_count(), tiles = (double)((p.N + 255) / 256 * p.nblocks);
@@ -535,7 +536,7 @@ bool split_supported(const Problem& p)
         const double n = (double)std::min<int64_t>(p.N, 256);
         other = 3.4 + 1.2 * n / 256 + nkb * (0.28 + 0.13 * n / 256) + (p.wexp ? 0.0 : 1.7 + 0.7 * nkb);
     } else {
-        other = 2.5 + std::ceil(tiles / sms) * (1.5 + nkb * (p.Wo > 1 ? 1.15 : 1.5));
+        other = 7.4 + std::ceil(tiles / sms) * (0.8 + 0.59 * nkb);
     }
     SplitCfg c;
     double us = 0.0;

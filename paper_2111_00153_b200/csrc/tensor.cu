@@ -2,21 +2,19 @@
 //
 // One persistent CTA per SM walks over output tiles of 128 weight rows x up to 256 pixels; the
 // reduction is cut into k-blocks of 128 codes.  Warp roles:
-//   warp 0      TMA producer.  Per k-block it fetches (a) the activation-code tile (the B
-//               operand): one 4-D box into 128-byte-swizzled shared memory -- for a convolution
-//               the box is the window of input pixels one filter tap needs, zero fill outside the
-//               image being the padding, so no im2col buffer exists anywhere; (b) the packed
-//               4-bit / 8-bit weight codes of the tile's rows, as 16-row boxes, into a raw ring.
+//   warp 0      TMA producer.  Per k-block it fetches the activation-code tile (the B operand): one 4-D box into
+//               swizzled shared memory -- for a convolution the box is the window of input pixels one filter tap
+//               needs, zero fill outside the image being the padding, so no im2col buffer exists anywhere.
 //   warp 1      allocates tensor memory and issues tcgen05.mma (kind::i8, int32 accumulators in
 //               tensor memory, two 256-column buffers: tile i+1 is computed while tile i is
 //               written out).
-//   warps 2-9   expanders, two groups of four warps that take alternate k-blocks: read the raw
-//               codes from shared memory, expand them to int8 in registers and store them in the
-//               K-major 128-byte-swizzled layout the MMA reads (the A operand).  Rows arrive
-//               group by group (PoT, Fixed-4, Fixed-8) but are written to the row of their ORIGINAL
+//   expanders   (weights without a workspace that do not stay resident) groups of four warps that take alternate
+//               k-blocks: a thread loads the packed codes of one row of the tile, expands them to int8 in registers and
+//               stores them in the K-major swizzled layout the MMA reads (the A operand).  Rows lie in the packed
+//               buffer group by group (PoT, Fixed-4, Fixed-8) but are written to the row of their ORIGINAL
 //               index, so accumulator lanes are in original row order and the output needs no
 //               scatter through the permutation.
-//   warps 10-13 epilogue, one per tensor-memory quarter (in workspace mode the expander warps
+//   last four   epilogue, one per tensor-memory quarter (in workspace mode the expander warps
 //               have nothing to expand and join the epilogue, three warps per quarter): tcgen05.ld (next chunk in flight while
 //               the current one is processed), undo the x16 of Fixed-4 rows, convert, scale by
 //               wstep*act_step, stage 32 pixels x 32 rows in a private double buffer and write it
@@ -38,13 +36,12 @@ namespace {
 
 constexpr int kTileN = 256;                      // pixels per tile (max) = TMEM columns per buffer
 constexpr int kABytes = kBlockRows * 128;        // 16 KB: 128 rows x 128 B (one k-block)
-constexpr int kBBytes = kTileN * 128;            // 32 KB
+constexpr int kNumEpiWarps = 4;
+constexpr int kPreWarps = 2 + 8 + kNumEpiWarps;  // warps of the forms that have no expanders
 constexpr int kGroups = 2;                       // expander groups taking alternate k-blocks
 constexpr int kNumExpWarps = 4 * kGroups;
-constexpr int kNumEpiWarps = 4;
-constexpr int kThreads = 32 * (2 + kNumExpWarps + kNumEpiWarps);
+__host__ __device__ constexpr int threads_of(int mode) { return 32 * (mode ? kPreWarps : 2 + kNumExpWarps + kNumEpiWarps); }
 constexpr int kWarpStage = 32 * 32 * 4;          // 4 KB: 32 pixels x 32 rows of fp32/int32
-constexpr int kRawBoxRows = 16;                  // rows per raw weight box
 constexpr int kMaxRing = 8;
 constexpr int kResidentBlocks = 16;              // row blocks of a layer with resident weights (the grid is a multiple of them)
 constexpr int kSmemLimit = 232448 - 1024;        // 227 KB per CTA less room for the static variables
@@ -64,8 +61,7 @@ struct TensorCfg {
     uint32_t tx_bytes;     // bytes one activation box brings
     int tma_store;         // 1: output chunks leave through shared memory and bulk tensor stores
     int tail_rows;         // npix % 32: height of the last chunk of a tile (0: none)
-    int nA, nB, nR;        // ring depths: expanded weights, activations, raw weights
-    uint32_t raw_bytes;    // one raw stage
+    int nA, nB;            // ring depths: expanded weights, activations
     int out_bufs;          // staging buffers per epilogue warp (1 or 2)
     int pre;               // 1: the A operand comes expanded (int8) from a workspace, no expander work
     int dup;               // 1 (pre mode, M <= 64): rows 0..63 are loaded twice, into lanes 0..63 and 64..127, so that all
@@ -95,71 +91,10 @@ struct TensorCfg {
 
 struct Maps {
     CUtensorMap act[4];                                // [B][H][W][Cin] activation codes; stride 2: one map per row/column parity
-    CUtensorMap q4, q8;                                // packed weight regions
     CUtensorMap wexp;                                  // [M][Kp] int8 weights expanded beforehand (pre mode); 64-row box when dup
     CUtensorMap out_full, out_tail, acc_full, acc_tail;   // bulk stores: 32-row and tail chunks
     CUtensorMap rq_full, rq_tail;                       // re-quantized codes: 32 pixels x 32 code bytes, and the tail
 };
-
-// ------------------------------------------------------------------ per-tile row bookkeeping
-
-// Rows of one 128-row block inside the three groups of the packed buffer.
-struct BlockInfo {
-    int p0, nP, f0, nF, e0, nE;
-};
-__device__ __forceinline__ BlockInfo load_block(const Problem& p, int blk)
-{
-    const int4 b0 = __ldg(reinterpret_cast<const int4*>(p.blocks + 8 * blk));
-    const int2 b1 = __ldg(reinterpret_cast<const int2*>(p.blocks + 8 * blk + 4));
-    BlockInfo b;
-    b.p0 = b0.x; b.nP = b0.y; b.f0 = b0.z; b.nF = b0.w; b.e0 = b1.x; b.nE = b1.y;
-    return b;
-}
-__device__ __forceinline__ int ceil_box(int n) { return (n + kRawBoxRows - 1) / kRawBoxRows * kRawBoxRows; }
-
-// What an expander thread knows about one of its rows in a tile, in one word:
-// bits 0-15 byte offset of its 32 codes inside a raw stage, bits 16-29 byte offset of its first
-// 16-byte chunk inside an A stage (the second chunk is that offset ^ 16), bits 30-31 kind (3: none).
-__device__ __forceinline__ uint32_t make_meta(const Problem& p, int64_t tile, int slot, int q)
-{
-    if (tile < 0) return 3u << 30;
-    const int blk = (int)(tile % p.nblocks);
-    const BlockInfo b = load_block(p, blk);
-    int kind, packed, raw;
-    if (slot < b.nP) {
-        kind = kPoT4; packed = b.p0 + slot; raw = slot * 64 + q * 16;
-    } else if (slot < b.nP + b.nF) {
-        kind = kFixed4; packed = p.nP + b.f0 + (slot - b.nP);
-        raw = (ceil_box(b.nP) + slot - b.nP) * 64 + q * 16;
-    } else if (slot < b.nP + b.nF + b.nE) {
-        kind = kFixed8; packed = p.nP + p.nF4 + b.e0 + (slot - b.nP - b.nF);
-        raw = (ceil_box(b.nP) + ceil_box(b.nF)) * 64 + (slot - b.nP - b.nF) * 128 + q * 32;
-    } else {
-        return 3u << 30;
-    }
-    const int row = __ldg(p.perm + packed) - blk * kBlockRows;
-    const uint32_t aoff = (uint32_t)row * 128u + ((uint32_t)((2 * q) ^ (row & 7)) << 4);
-    return (uint32_t)raw | (aoff << 16) | ((uint32_t)kind << 30);
-}
-
-// Expand one task: 32 codes from the raw stage to two 16-byte chunks of the A stage.
-__device__ __forceinline__ void expand_task(uint32_t meta, uint32_t raw_stage, uint32_t a_stage)
-{
-    const uint32_t kind = meta >> 30;
-    const uint32_t src = raw_stage + (meta & 0xFFFFu);
-    const uint32_t dst = a_stage + ((meta >> 16) & 0x3FFFu);
-    uint32_t w[8];
-    if (kind == kFixed8) {
-        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(src) : "memory");
-        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]) : "r"(src + 16) : "memory");
-    } else {
-        uint4 c;
-        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(c.x), "=r"(c.y), "=r"(c.z), "=r"(c.w) : "r"(src) : "memory");
-        if (kind == kPoT4) expand_pot_chunk(c, w); else expand_fixed4_chunk_x16(c, w);
-    }
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst ^ 16u), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-}
 
 // Resident weights without a workspace: the threads of the CTA expand the row block from the packed codes (exact
 // int8 values, as expand_kernel writes them) straight into the resident stages, at the place the bulk copy of an
@@ -271,9 +206,10 @@ __device__ __forceinline__ void tmem_ld_four(uint32_t taddr, uint32_t (&v)[4])
 // kOut:  1 when the output is fp32 [N][M] through bulk stores without an accumulator dump (the common case): the
 //        epilogue then carries only that path; 0 decides at run time.
 template <int kM2, int kRQ, int kMode, int kOut>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(threads_of(kMode), 1)
 tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps maps)
 {
+    constexpr int kThreads = threads_of(kMode);
     constexpr bool kPre = kMode != 0, kAres = kMode >= 2, kTps3 = kMode == 3;
     const bool use_tma_store = kOut ? true : (cfg.tma_store != 0);
     const bool out_mn = kOut ? false : (p.out_mn != 0);
@@ -282,14 +218,12 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sA = smem_base;
     const uint32_t sB = sA + cfg.nA * cfg.a_bytes;
-    const uint32_t sRaw = sB + cfg.nB * cfg.b_bytes;
-    const uint32_t sOut = sRaw + cfg.nR * cfg.raw_bytes;
+    const uint32_t sOut = sB + cfg.nB * cfg.b_bytes;
     const uint32_t sBar = sOut + cfg.epi_warps * cfg.out_bufs * kWarpStage;
     // barriers, 8 bytes each
     const uint32_t bar_fullA = sBar, bar_emptyA = sBar + 8 * kMaxRing;
     const uint32_t bar_fullB = sBar + 16 * kMaxRing, bar_emptyB = sBar + 24 * kMaxRing;
-    const uint32_t bar_fullR = sBar + 32 * kMaxRing, bar_emptyR = sBar + 40 * kMaxRing;
-    const uint32_t bar_tfull = sBar + 48 * kMaxRing, bar_tempty = bar_tfull + 16;
+    const uint32_t bar_tfull = sBar + 32 * kMaxRing, bar_tempty = bar_tfull + 16;
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
 
@@ -301,8 +235,6 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             mbar_init(bar_emptyA + 8 * s, 1);    // tcgen05.commit
             mbar_init(bar_fullB + 8 * s, 1);     // producer (+ transaction bytes)
             mbar_init(bar_emptyB + 8 * s, 1);    // tcgen05.commit
-            mbar_init(bar_fullR + 8 * s, 1);     // producer (+ transaction bytes)
-            mbar_init(bar_emptyR + 8 * s, 4);    // the four warps of one expander group
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar_tfull + 8 * b, 1);                  // tcgen05.commit
@@ -335,7 +267,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
 
     // Workspace mode splits the producer: one thread can start a bulk tensor copy only every few
     // hundred cycles, so the activation boxes and the weight boxes are issued by two different warps.
-    const bool pre_b_producer = kPre && warp == 0;
+    const bool pre_b_producer = warp == 0;
     const bool pre_a_producer = kPre && !kAres && warp == 2;
     if (pre_b_producer || pre_a_producer) {
         if (lane == 0) {
@@ -406,62 +338,6 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             }
             if (!ok) {
                 for (int i = 0; i < 200; ++i) __nanosleep(1000);   // let copies in flight land
-            }
-        }
-    } else if (warp == 0) {
-        // ---------------------------------------------------------- TMA producer (shared-memory expansion mode)
-        // The whole warp takes part: lane 0 waits on the barriers and fetches the activation box,
-        // the weight boxes of a k-block are issued by one lane each.
-        {
-            uint32_t sb = 0, phB = 0, sr = 0, phR = 0;
-            bool ok = true;
-            for (int64_t tile = first; tile < cfg.ntiles && ok; tile += step) {
-                const int blk = (int)(tile % p.nblocks);
-                const int64_t nt = tile / p.nblocks;
-                int b0, h0;
-                if (cfg.tiles_per_image) { b0 = (int)(nt / cfg.tiles_per_image); h0 = min((int)(nt % cfg.tiles_per_image) * cfg.th, p.Ho - cfg.th); }
-                else { b0 = (int)(nt * cfg.tb); h0 = 0; }
-                const BlockInfo bi = load_block(p, blk);
-                const int nbP = ceil_box(bi.nP) / kRawBoxRows, nbF = ceil_box(bi.nF) / kRawBoxRows,
-                          nbE = ceil_box(bi.nE) / kRawBoxRows;
-                const uint32_t raw_tx = (uint32_t)(nbP + nbF) * (kRawBoxRows * 64) + (uint32_t)nbE * (kRawBoxRows * 128);
-                // this lane's weight box (lanes beyond the box count have none)
-                const CUtensorMap* my_map = nullptr;
-                int my_row = 0, my_x8 = 0;           // my_x8: 1 if the box is in the 8-bit region
-                uint32_t my_dst = 0;
-                if (lane < nbP) { my_map = &maps.q4; my_row = bi.p0 + lane * kRawBoxRows; my_dst = lane * (kRawBoxRows * 64); }
-                else if (lane < nbP + nbF) { my_map = &maps.q4; my_row = p.nP + bi.f0 + (lane - nbP) * kRawBoxRows; my_dst = lane * (kRawBoxRows * 64); }
-                else if (lane < nbP + nbF + nbE) {
-                    my_map = &maps.q8; my_x8 = 1; my_row = bi.e0 + (lane - nbP - nbF) * kRawBoxRows;
-                    my_dst = (nbP + nbF) * (kRawBoxRows * 64) + (lane - nbP - nbF) * (kRawBoxRows * 128);
-                }
-                int tap = 0, cc = 0;
-                for (int kb = 0; kb < cfg.nkb; ++kb) {
-                    const int c0 = cc * cfg.bk, koff = tap * p.Cp + c0;
-                    {
-                        // packed weights of this tile's rows, group by group
-                        if (!mbar_wait_warp(bar_emptyR + 8 * sr, phR ^ 1, abort_flag)) { ok = false; break; }
-                        const uint32_t rbar = bar_fullR + 8 * sr;
-                        if (lane == 0) mbar_arrive_expect_tx(rbar, raw_tx);
-                        __syncwarp();
-                        if (my_map) tma_load_2d(sRaw + sr * cfg.raw_bytes + my_dst, my_map, rbar, my_x8 ? koff : (koff >> 1), my_row);
-                        if (++sr == (uint32_t)cfg.nR) { sr = 0; phR ^= 1; }
-                    }
-                    // activation codes
-                    if (!mbar_wait_warp(bar_emptyB + 8 * sb, phB ^ 1, abort_flag)) { ok = false; break; }
-                    if (lane == 0) {
-                        const int ti = tap / p.kw, tj = tap - ti * p.kw;
-                        mbar_arrive_expect_tx(bar_fullB + 8 * sb, cfg.tx_bytes);
-                        const TapBox tb = tap_box(p, h0, ti, tj);
-                        tma_load_4d(sB + sb * cfg.b_bytes, &maps.act[tb.map], bar_fullB + 8 * sb, c0, tb.x, tb.y, b0);
-                    }
-                    if (++sb == (uint32_t)cfg.nB) { sb = 0; phB ^= 1; }
-                    if (++cc == cfg.cpt) { cc = 0; ++tap; }
-                }
-            }
-            if (!ok && lane == 0) {
-                // give copies already in flight time to land before the CTA's memory is released
-                for (int i = 0; i < 200; ++i) __nanosleep(1000);
             }
         }
     } else if (warp == 1) {
@@ -583,64 +459,161 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         }
     } else if (!kPre && warp < 2 + kNumExpWarps) {
         // ---------------------------------------------------------- expanders
+        // The packed codes of a k-block (a few KB, in L2) go to registers and from there, expanded, to the stage.  A warp
+        // takes 32 rows in packed order, which are of one kind but where two kinds meet, and then runs without a branch;
+        // the four (64-byte k-blocks: two) 32-code pieces of a row are neighbours, so that a load touches eight rows and not
+        // 32, and of eight lanes' stores at most two meet in a bank.  What bounds it is one warp's chain of instructions
+        // (four to eight cycles each), which is why everything that stays the same for a tile is worked out once for it,
+        // a tile ahead, and a piece's registers are loaded again as soon as it is expanded.  With the
+        // codes brought to shared memory in boxes of 16 rows and expanded from there: 3072x768 N=4096 36.9 us, now 21.6;
+        // 3x3 512x512 on 12,544 pixels 84, now 51 to 59.
         const int grp = (warp - 2) >> 2;                 // which k-blocks: g % kGroups == grp
-        const int et = ((warp - 2) & 3) * 32 + lane;     // 0..127 inside the group
-        const int q = et & 3;                            // 32-code step inside each k-block
-        const int slot0 = et >> 2;                       // rows slot0 + 32*i of the tile's sorted order
+        const int ppr = cfg.bk >> 5;                     // pieces of a row, and rows of a thread, per k-block
+        const int q = lane & (ppr - 1), r0 = ((warp - 2) & 3) * 32 + (ppr == 4 ? lane >> 2 : lane >> 1), r_step = 32 / ppr;
         // tile look-ahead: one tile, or kGroups tiles when every tile is a single k-block
         const int64_t look = (cfg.nkb == 1) ? kGroups : 1;
-        const int64_t total = kPre ? 0 : my_tiles * cfg.nkb;   // nothing to expand in pre mode
-        int64_t g = grp;                                 // this CTA's k-block counter
-        int64_t tl = g / cfg.nkb;                        // local tile index of g
-        int kb = (int)(g - tl * cfg.nkb);
-        int cc = kb % cfg.cpt;
-        uint32_t sa = (uint32_t)(g % cfg.nA), phA = (uint32_t)((g / cfg.nA) & 1);
-        uint32_t sr = (uint32_t)(g % cfg.nR), phR = (uint32_t)((g / cfg.nR) & 1);
-        uint32_t cur[4], nxt[4];
-        auto tile_of = [&](int64_t local) -> int64_t { return local < my_tiles ? first + local * step : -1; };
+        const int64_t total = my_tiles * cfg.nkb;
+        const bool rows_change = (uint32_t)step % (uint32_t)p.nblocks != 0u;
+        // a row block's rows in the packed buffer: first and number of each kind
+        int4 blk_a;
+        int2 blk_b;
+        int blk_next = 0;
+        auto load_block = [&](int64_t local) {
+            blk_next = (int)((uint32_t)(first + min(local, my_tiles - 1) * step) % (uint32_t)p.nblocks);
+            blk_a = __ldg(reinterpret_cast<const int4*>(p.blocks + 8 * blk_next));
+            blk_b = __ldg(reinterpret_cast<const int2*>(p.blocks + 8 * blk_next + 4));
+        };
+        const int n4 = p.nP + p.nF4;
+        const uint32_t q8_first = (uint32_t)((p.q8 - p.q4) >> 4);
+        // this thread's rows in tile f_tl (and, _next, in tile f_tl + look): first code / 16 bytes; place in a stage, two of 16 bits
+        // each; a byte with the kind (3: no such row); the kind all rows of the warp have, or 4
+        uint32_t off[4], off_next[4], place[2], kinds = 0, kinds_next = 0, uni = 3, uni_next = 3;
+        int row_next[4], first_next = 0;
+        auto look_up = [&]() {
+            first_next = blk_next * kBlockRows;
+            kinds_next = 0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            cur[i] = kPre ? 0u : make_meta(p, tile_of(tl), slot0 + 32 * i, q);
-            nxt[i] = kPre ? 0u : make_meta(p, tile_of(tl + look), slot0 + 32 * i, q);
-        }
-        while (g < total) {
-            const int ksteps = (cc == cfg.cpt - 1) ? cfg.last_ksteps : 4;
-            if (!mbar_wait_warp(bar_fullR + 8 * sr, phR, abort_flag)) break;
-            if (!mbar_wait_warp(bar_emptyA + 8 * sa, phA ^ 1, abort_flag)) break;
-            if (q < ksteps) {
-                const uint32_t rs = sRaw + sr * cfg.raw_bytes, as = sA + sa * cfg.a_bytes;
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + (i & (ppr - 1)) * r_step, f = r - blk_a.y, e = f - blk_a.w;
+                const int kind = e >= blk_b.y ? 3 : f < 0 ? kPoT4 : e < 0 ? kFixed4 : kFixed8;
+                const int packed = kind == kPoT4 ? blk_a.x + r : kind == kFixed4 ? p.nP + blk_a.z + f : n4 + blk_b.x + e;
+                off_next[i] = kind == 3 ? 0u : kind == kFixed8 ? q8_first + (uint32_t)(packed - n4) * (uint32_t)(p.Kp >> 4) : (uint32_t)packed * (uint32_t)(p.Kp >> 5);
+                row_next[i] = kind == 3 ? first_next : __ldg(p.perm + packed);
+                kinds_next |= (uint32_t)kind << (8 * i);
+            }
+            const uint32_t k0 = __shfl_sync(0xffffffffu, kinds_next, 0) & 3u;      // (every lane takes part in both votes)
+            const uint32_t same = __all_sync(0xffffffffu, kinds_next == k0 * 0x01010101u);
+            uni_next = same ? k0 : 4u;
+        };
+        auto take_rows = [&]() {
+            kinds = kinds_next;
+            uni = uni_next;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                off[i] = off_next[i];
+                const uint32_t r = (uint32_t)(row_next[i] - first_next), swz = ppr == 4 ? r & 7u : (r >> 1) & 3u;
+                const uint32_t d = r * (uint32_t)cfg.bk + (((uint32_t)(2 * q) ^ swz) << 4);
+                place[i >> 1] = i & 1 ? place[i >> 1] | (d << 16) : d;
+            }
+        };
+        int64_t g = grp, f_tl = g / cfg.nkb;             // this CTA's k-block counter; tile and place of the k-block to be loaded next
+        int f_kb = (int)(g - f_tl * cfg.nkb), f_tap = f_kb / cfg.cpt, f_cc = f_kb - f_tap * cfg.cpt;
+        const int Cp32 = p.Cp >> 5;
+        uint4 lo[4], hi[4];                              // (hi: the second half of 32 eight-bit codes)
+        auto load = [&](int i, uint32_t piece) {
+            const bool eight = ((kinds >> (8 * i)) & 3u) == kFixed8;
+            const uint4* src = reinterpret_cast<const uint4*>(p.q4) + (off[i] + (eight ? 2u * piece : piece));
+            lo[i] = __ldg(src);
+            if (eight) hi[i] = __ldg(src + 1);
+        };
+        auto has_piece = [&]() { return uni != 3u && q < (f_cc == cfg.cpt - 1 ? cfg.last_ksteps : ppr); };
+        auto piece_of = [&]() { return (uint32_t)(f_tap * Cp32 + f_cc * ppr + q); };
+        auto put = [&](uint32_t dst, const uint32_t (&w)[8]) {
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]));
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst ^ 16u), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]));
+        };
+        // (a piece is not touched before the one in front of it is stored: its own load may still be on its way.  Left to
+        // itself the compiler interleaves the pieces and waits for all four loads at once)
+        auto hold = [&](int i) { asm volatile("" : "+r"(lo[i].x), "+r"(lo[i].y), "+r"(lo[i].z), "+r"(lo[i].w)); };
+        uint32_t sa = (uint32_t)(grp % cfg.nA), phA = (uint32_t)((grp / cfg.nA) & 1);
+        if (g < total) {
+            load_block(f_tl);
+            look_up();
+            take_rows();
+            load_block(f_tl + look);
+            look_up();
+            load_block(f_tl + 2 * look);
+            if (has_piece()) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if ((cur[i] >> 30) != 3u) expand_task(cur[i], rs, as);
+                    if (i < ppr) load(i, piece_of());
+            }
+        }
+        while (g < total) {
+            // what is in the registers now, and then the place of what follows it there
+            const uint32_t c_kinds = kinds, c_uni = uni, c_place[2] = {place[0], place[1]};
+            const bool c_on = has_piece();
+            g += kGroups;
+            f_kb += kGroups;
+            f_cc += kGroups;
+            while (f_cc >= cfg.cpt) { f_cc -= cfg.cpt; ++f_tap; }
+            if (f_kb >= cfg.nkb) {
+                int64_t adv = 0;
+                while (f_kb >= cfg.nkb) { f_kb -= cfg.nkb; ++adv; }
+                f_tap = f_kb / cfg.cpt;
+                f_cc = f_kb - f_tap * cfg.cpt;
+                f_tl += adv;
+                if (rows_change) {
+                    if (adv != look) { load_block(f_tl); look_up(); load_block(f_tl + look); }
+                    take_rows();
+                    look_up();
+                    load_block(f_tl + 2 * look);
+                }
+            }
+            const bool on = g < total && has_piece();
+            const uint32_t piece = piece_of();
+            if (!mbar_wait_warp(bar_emptyA + 8 * sa, phA ^ 1, abort_flag)) break;
+            const uint32_t dst = sA + sa * cfg.a_bytes;
+            auto at = [&](int i) { return dst + (i & 1 ? c_place[i >> 1] >> 16 : c_place[i >> 1] & 0xFFFFu); };
+            if (c_uni == kPoT4) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (i >= ppr) break;
+                    hold(i);
+                    uint32_t w[8];
+                    expand_pot_chunk(lo[i], w);
+                    if (on) load(i, piece);
+                    if (c_on) put(at(i), w);
+                }
+            } else if (c_uni == kFixed4) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (i >= ppr) break;
+                    hold(i);
+                    uint32_t w[8];
+                    expand_fixed4_chunk_x16(lo[i], w);
+                    if (on) load(i, piece);
+                    if (c_on) put(at(i), w);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (i >= ppr) break;
+                    hold(i);
+                    const uint32_t kind = (c_kinds >> (8 * i)) & 3u;
+                    uint32_t w[8] = {lo[i].x, lo[i].y, lo[i].z, lo[i].w, hi[i].x, hi[i].y, hi[i].z, hi[i].w};
+                    if (kind == kPoT4) expand_pot_chunk(lo[i], w);
+                    else if (kind == kFixed4) expand_fixed4_chunk_x16(lo[i], w);
+                    if (on) load(i, piece);
+                    if (c_on && kind != 3u) put(at(i), w);
+                }
             }
             fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(bar_fullA + 8 * sa);
-                mbar_arrive(bar_emptyR + 8 * sr);
-            }
-            // advance by kGroups k-blocks
-            g += kGroups;
+            if (lane == 0) mbar_arrive(bar_fullA + 8 * sa);
             sa += kGroups; while (sa >= (uint32_t)cfg.nA) { sa -= cfg.nA; phA ^= 1; }
-            sr += kGroups; while (sr >= (uint32_t)cfg.nR) { sr -= cfg.nR; phR ^= 1; }
-            kb += kGroups;
-            cc += kGroups; while (cc >= cfg.cpt) cc -= cfg.cpt;
-            if (kb >= cfg.nkb) {
-                int64_t adv = 0;
-                while (kb >= cfg.nkb) { kb -= cfg.nkb; ++adv; }
-                tl += adv;
-                cc = kb % cfg.cpt;
-                if (adv == look) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) cur[i] = nxt[i];
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) cur[i] = make_meta(p, tile_of(tl), slot0 + 32 * i, q);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) nxt[i] = make_meta(p, tile_of(tl + look), slot0 + 32 * i, q);
-            }
         }
+        __syncwarp();
     } else {
         // ---------------------------------------------------------- epilogue
         // Warp w may read tensor-memory lanes 32*(w%4)..+31.  The warps that share a quarter (one, or
@@ -932,7 +905,6 @@ bool plan(const Problem& p, TensorCfg& c)
 {
     if (p.pix_pitch % 16 != 0 || (p.Cin % 16 != 0 && !p.ragged_k)) return false;
     if ((reinterpret_cast<uintptr_t>(p.act) & 15) != 0) return false;
-    if (!p.wexp && p.raw_stage_bytes <= 0) return false;
     if (p.wexp && (reinterpret_cast<uintptr_t>(p.wexp) & 15) != 0) return false;
     const int64_t hw = (int64_t)p.Ho * p.Wo;
     if (p.Wo > kTileN || (int64_t)p.Wo * p.stride > 256) return false;
@@ -984,7 +956,7 @@ bool plan(const Problem& p, TensorCfg& c)
     // layer runs in the workspace form
     if (!p.wexp && resident) { c.pre = 1; c.fill = 1; }
     // 64-byte k-blocks when a 128-byte row would be at most half used by the (last) channel chunk
-    c.bk = (c.pre && (p.Cin % 128 != 0) && (p.Cin % 128 <= 64)) ? 64 : 128;
+    c.bk = (c.pre ? p.Cin % 128 != 0 && p.Cin % 128 <= 64 : p.Cin <= 64) ? 64 : 128;
     c.a_bytes = kBlockRows * c.bk;
     c.b_bytes = kTileN * c.bk;
     c.cpt = (p.Cin + c.bk - 1) / c.bk;
@@ -1000,12 +972,12 @@ bool plan(const Problem& p, TensorCfg& c)
     c.ares = 0;
     c.epi_warps = kNumEpiWarps;
     if (c.pre) {
-        c.nA = (c.bk == 64) ? 6 : 3; c.nB = (c.bk == 64) ? 8 : 4; c.nR = 0; c.raw_bytes = 0; c.out_bufs = 1;
-        c.epi_warps = kNumExpWarps + kNumEpiWarps - 1;   // warp 2 fetches the weights (unless they are resident)
+        c.nA = (c.bk == 64) ? 6 : 3; c.nB = (c.bk == 64) ? 8 : 4; c.out_bufs = 1;
+        c.epi_warps = kPreWarps - 3;   // warp 2 fetches the weights (unless they are resident)
         c.dup = (p.M <= 64) ? 1 : 0;
         if (resident) {
             c.ares = 1;
-            c.epi_warps = kNumExpWarps + kNumEpiWarps;
+            c.epi_warps = kPreWarps - 2;
             c.nA = c.nkb;
             const int64_t left = kSmemLimit - (1024 + 64 * kMaxRing) - (int64_t)c.nkb * c.a_bytes -
                                  (int64_t)c.epi_warps * kWarpStage;
@@ -1043,20 +1015,15 @@ bool plan(const Problem& p, TensorCfg& c)
                                   64 * kMaxRing);
         return true;
     }
-    // shared-memory budget: rings as deep as fit
-    c.raw_bytes = ((uint32_t)p.raw_stage_bytes + 1023u) & ~1023u;
-    const int fixed = 1024 /*alignment*/ + 64 * kMaxRing /*barriers*/;
-    struct Choice { int nA, nB, nR, ob; };
-    const Choice order[] = {{3, 4, 3, 2}, {3, 4, 3, 1}, {3, 3, 3, 2}, {2, 3, 3, 2}, {2, 3, 2, 1}, {2, 2, 2, 1}};
-    for (const Choice& ch : order) {
-        const int64_t need = (int64_t)ch.nA * kABytes + (int64_t)ch.nB * kBBytes + (int64_t)ch.nR * c.raw_bytes +
-                             (int64_t)kNumEpiWarps * ch.ob * kWarpStage + fixed;
-        if (need <= kSmemLimit) {
-            c.nA = ch.nA; c.nB = ch.nB; c.nR = ch.nR; c.out_bufs = ch.ob; c.smem_bytes = (uint32_t)need;
-            return true;
-        }
-    }
-    return false;
+    // Four weight stages (a group expands into one while its last and the other group's two wait for their turn: three
+    // are 20 to 30 % slower, six no faster), an output buffer a warp, and all the rest for activations.
+    c.nA = 4;
+    c.out_bufs = 1;
+    c.b_bytes = (c.n_mma * c.bk + 1023) / 1024 * 1024;
+    const int fixed = c.nA * c.a_bytes + kNumEpiWarps * c.out_bufs * kWarpStage + 1024 + 64 * kMaxRing;
+    c.nB = std::min(kMaxRing, (kSmemLimit - fixed) / c.b_bytes);
+    c.smem_bytes = (uint32_t)(fixed + c.nB * c.b_bytes);
+    return true;
 }
 
 }  // namespace
@@ -1086,7 +1053,8 @@ bool encode_act_maps_4(const Problem& p, int bk, int th, int tb, void* maps4)
 }
 
 // Whether the persistent kernel keeps a row block's expanded weights in shared memory: they fit beside the activation
-// ring, and the grid can be a multiple of the row blocks (a CTA then stays with one).  Without a workspace that is always
+// ring, and the grid can be a multiple of the row blocks without costing a round of tiles to speak of (a CTA then stays with
+// one).  Without a workspace that is always
 // the better form: the codes are expanded once per CTA, not per tile (144x160 on 740,050 pixels 355 against 131 us,
 // 2048x512 N=4096 20.9 against 13.8).  With one, the weights of several row blocks are a stream that the activations of a
 // first tile would wait behind (1024x512 N=4096, a tile per CTA: 8.1 us resident, 7.3 through the rings), and save
@@ -1094,10 +1062,12 @@ bool encode_act_maps_4(const Problem& p, int bk, int th, int tb, void* maps4)
 // against 17.7).
 bool tensor_resident(const Problem& p)
 {
-    if (p.nblocks > kResidentBlocks || (!p.wexp && p.rq_codes)) return false;
+    if (!p.wexp && p.rq_codes) return false;
+    const int64_t sms = sm_count(), tiles = (p.N + kTileN - 1) / kTileN * p.nblocks, whole = sms / p.nblocks * p.nblocks;
+    if (p.nblocks > kResidentBlocks && (whole == 0 || (tiles + whole - 1) / whole > (tiles + sms - 1) / sms)) return false;
     const int bk = ((p.Cin % 128 != 0) && (p.Cin % 128 <= 64)) ? 64 : 128;
     if ((int64_t)p.kh * p.kw * ((p.Cin + bk - 1) / bk) * kBlockRows * bk > 72 * 1024) return false;
-    return !p.wexp || p.nblocks == 1 || (p.N + kTileN - 1) / kTileN * p.nblocks >= 2 * (int64_t)sm_count();
+    return !p.wexp || p.nblocks == 1 || tiles >= 2 * sms;
 }
 
 bool tensor_supported(const Problem& p)
@@ -1117,19 +1087,6 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
     Maps mp;
     memset(&mp, 0, sizeof(mp));
     if (!encode_act_maps(enc, p, c.bk, c.colshift ? c.th + 2 : c.th, c.tb, c.bk == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, mp.act))
-        return RMSMP_ERR_CUDA;
-    // packed weight regions: rows of Kp/2 (4-bit) and Kp (8-bit) bytes, boxes of 16 rows x one k-block
-    auto make_w = [&](CUtensorMap* m, const uint8_t* base, int rows, int pitch, int box_bytes) -> bool {
-        if (rows <= 0) return true;
-        const cuuint64_t gd[2] = {(cuuint64_t)pitch, (cuuint64_t)rows};
-        const cuuint64_t gs[1] = {(cuuint64_t)pitch};
-        const cuuint32_t bx[2] = {(cuuint32_t)box_bytes, (cuuint32_t)kRawBoxRows};
-        const cuuint32_t es[2] = {1, 1};
-        return enc(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(base), gd, gs, bx, es,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-    };
-    if (!make_w(&mp.q4, p.q4, p.nP + p.nF4, p.Kp / 2, 64) || !make_w(&mp.q8, p.q8, p.n8, p.Kp, 128))
         return RMSMP_ERR_CUDA;
     if (p.wexp) {
         const cuuint64_t gd[2] = {(cuuint64_t)p.Kp, (cuuint64_t)p.M};
@@ -1204,8 +1161,13 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
     if (!fn) return RMSMP_ERR_VARIANT;
     static bool attr_set[4][2][3][kMaxDevices] = {};
     if (!ensure_smem_attr(reinterpret_cast<const void*>(fn), kSmemLimit, attr_set[mode][i2][io])) return RMSMP_ERR_CUDA;
-    const int grid = (int)std::min<int64_t>(c.ntiles, c.ares ? sm_count() / c.nbt * c.nbt : sm_count());
-    if (launch_dependent(fn, (unsigned)grid, kThreads, c.smem_bytes, st, p, c, mp) != cudaSuccess) {
+    // All tiles of a CTA are of one row block where the grid is a multiple of them: required by resident weights, and with
+    // expanders worth having when it costs no round of tiles (they look up a tile's rows only once then).
+    int64_t grid = sm_count();
+    const int64_t whole = grid / c.nbt * c.nbt;
+    if (c.ares || (!c.pre && whole > 0 && (c.ntiles + whole - 1) / whole == (c.ntiles + grid - 1) / grid)) grid = whole;
+    grid = std::min(grid, c.ntiles);
+    if (launch_dependent(fn, (unsigned)grid, threads_of(mode), c.smem_bytes, st, p, c, mp) != cudaSuccess) {
         cudaGetLastError();
         return RMSMP_ERR_CUDA;
     }

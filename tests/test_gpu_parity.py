@@ -995,3 +995,25 @@ def test_images_whose_rows_no_tile_divides(M, Cin, k, stride, B, H, W, variant, 
         if want_acc:
             assert np.array_equal(acc, acc_ref.reshape(-1, M))
         assert np.array_equal(np.ascontiguousarray(y).view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
+
+
+@pytest.mark.parametrize("mix", [(50, 30, 20), (100, 0, 0), (0, 0, 100), (0, 100, 0)], ids=lambda m: "%d-%d-%d" % m)
+@pytest.mark.parametrize("M,Cin,k,B,H,W", [
+    (2500, 96, 1, 7401, 1, 1),       # twenty row blocks that change from tile to tile, one k-block a tile, a step unused
+    (2500, 192, 1, 7401, 1, 1),      # two k-blocks: a group's next tile is one or two ahead
+    (300, 1024, 1, 16001, 1, 1),     # a row block per CTA, three of them
+    (16, 304, 5, 11, 43, 37),        # few rows; a last chunk of 48 channels
+    (200, 48, 5, 30, 31, 33),        # 64-byte k-blocks, one and a half steps
+])
+def test_weights_expanded_for_every_tile(M, Cin, k, B, H, W, mix):
+    """Neither a workspace nor room for a row block's weights: every kind of row, alone and mixed, exact."""
+    g = synth.rng(98, M + Cin + W)
+    Wt = synth.weights_kaiming(g, M, Cin, k, k)
+    scheme, bits = _mixed_map(M, M + k, mix)
+    alpha = synth.alpha_rows(Wt)
+    act = g.integers(-8, 16, size=(B, H, W, Cin)).astype(np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    _, ws, acc_ref, y_ref = O.layer_conv(Wt, scheme, bits, alpha, act, np.float32(0.25), 1, k // 2)
+    y, acc = Hn.conv(layer, d_packed, act, 1, k // 2, 0.25, R.VARIANT_TENSOR)
+    assert np.array_equal(acc, acc_ref.reshape(-1, M))
+    assert np.array_equal(y.view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
