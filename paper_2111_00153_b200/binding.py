@@ -184,7 +184,7 @@ def _check(st: int, where: str):
         raise RmsmpError(st, where)
 
 
-# The calls that a program makes per layer and pass are marshalled by the extension module (csrc/marshal.cpp); it is
+# The calls that a program makes per layer are marshalled by the extension module (csrc/marshal.cpp); it is
 # loaded with the library on the first use of one of them.
 _NATIVE = (
     "rmsmp_quantize_act",
@@ -200,12 +200,17 @@ _NATIVE = (
     "rmsmp_im2col_codes",
     "rmsmp_expand_weights",
     "rmsmp_assign_quantize_pack",
+    "rmsmp_quantize_pack",
     "rmsmp_gemm_grouped_launch",
 )
 
 
 def _raise(status: int, where: str):
     raise RmsmpError(status, where)
+
+
+def _host_array(a, fmt: str):
+    return np.ascontiguousarray(a, dtype=np.uint8 if fmt == "B" else np.float32)
 
 
 def __getattr__(name):
@@ -216,7 +221,7 @@ def __getattr__(name):
         from . import _marshal
     except ImportError as e:
         raise RuntimeError(f"the extension module _marshal is missing: build it with `python -m {__package__}.build`") from e
-    _marshal.setup({n: C.cast(getattr(L, n), C.c_void_p).value for n in _NATIVE}, _current_stream, _raise)
+    _marshal.setup({n: C.cast(getattr(L, n), C.c_void_p).value for n in _NATIVE}, _current_stream, _raise, _host_array)
     for n in _NATIVE:
         globals()[n] = getattr(_marshal, n)
     return globals()[name]
@@ -246,20 +251,6 @@ def rmsmp_layer_init(M: int, Cin: int, kh: int, kw: int, h_scheme, h_bits) -> rm
     _check(lib().rmsmp_layer_init(C.byref(layer), M, Cin, kh, kw, _hp(scheme), _hp(bits)),
            "rmsmp_layer_init")
     return layer
-
-
-def rmsmp_quantize_pack(d_W, w_layout: int, layer: rmsmp_layer, h_scheme, h_bits, h_alpha,
-                        pot_mode: int, d_packed, packed_bytes: int | None = None, stream=None):
-    scheme = np.ascontiguousarray(h_scheme, dtype=np.uint8)
-    bits = np.ascontiguousarray(h_bits, dtype=np.uint8)
-    alpha = np.ascontiguousarray(h_alpha, dtype=np.float32)
-    if not (scheme.size == bits.size == alpha.size == layer.M):
-        raise ValueError("scheme/bits/alpha need M entries")
-    if packed_bytes is None:
-        packed_bytes = d_packed.numel() * d_packed.element_size()
-    _check(lib().rmsmp_quantize_pack(_dp(d_W), w_layout, C.byref(layer), _hp(scheme), _hp(bits),
-                                     _hp(alpha), pot_mode, _dp(d_packed), packed_bytes,
-                                     _stream(stream)), "rmsmp_quantize_pack")
 
 
 def rmsmp_unpack_codes(layer: rmsmp_layer, d_packed, d_values, d_perm=None, d_wstep=None,

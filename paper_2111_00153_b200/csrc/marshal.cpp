@@ -29,11 +29,13 @@ struct Api {
     decltype(&rmsmp_im2col_codes) im2col_codes;
     decltype(&rmsmp_expand_weights) expand_weights;
     decltype(&rmsmp_assign_quantize_pack) assign_quantize_pack;
+    decltype(&rmsmp_quantize_pack) quantize_pack;
     decltype(&rmsmp_gemm_grouped_launch) gemm_grouped_launch;
 } api;
 
 PyObject* g_stream;          // callable: the current stream's handle
 PyObject* g_error;           // callable(status, where): raises RmsmpError
+PyObject* g_array;           // callable(object, format): a contiguous array of bytes ('B') or floats ('f') with its values
 PyObject *s_data_ptr, *s_numel, *s_element_size, *s_cuda_stream;
 
 // Arguments of one call, positions filled from positional and keyword arguments; conversions record the first failure.
@@ -388,6 +390,54 @@ DEF(assign_quantize_pack)
     Py_RETURN_NONE;
 }
 
+// A host array: the object's own memory where it is contiguous and of the type asked for, otherwise a converted copy.
+struct HostArray {
+    Py_buffer b{};
+    bool held = false;
+    ~HostArray() { if (held) PyBuffer_Release(&b); }
+    bool take(PyObject* o, char format)
+    {
+        if (PyObject_GetBuffer(o, &b, PyBUF_C_CONTIGUOUS | PyBUF_FORMAT) != 0) { PyErr_Clear(); return false; }
+        held = true;
+        if (b.format && b.format[0] == format && b.format[1] == 0) return true;
+        PyBuffer_Release(&b);
+        held = false;
+        return false;
+    }
+    const void* get(Call& c, int i, char format)
+    {
+        if (!c.ok) return nullptr;
+        if (take(c.a[i], format)) return b.buf;
+        PyObject* copy = PyObject_CallFunction(g_array, "OC", c.a[i], (int)format);
+        if (copy && !take(copy, format)) PyErr_SetString(PyExc_TypeError, "not an array of numbers");
+        Py_XDECREF(copy);                                       // (the buffer holds it)
+        if (!held) c.ok = false;
+        return held ? b.buf : nullptr;
+    }
+    Py_ssize_t count() const { return b.itemsize ? b.len / b.itemsize : 0; }
+};
+
+DEF(quantize_pack)
+{
+    ARGS("rmsmp_quantize_pack", 8, "d_W", "w_layout", "layer", "h_scheme", "h_bits", "h_alpha", "pot_mode", "d_packed", "packed_bytes", "stream")
+    void* W = c.ptr(0);
+    const int w_layout = c.i32(1);
+    const rmsmp_layer* L = c.structure<rmsmp_layer>(2);
+    HostArray scheme, bits, alpha;
+    const void *hs = scheme.get(c, 3, 'B'), *hb = bits.get(c, 4, 'B'), *ha = alpha.get(c, 5, 'f');
+    if (c.ok && (scheme.count() != L->M || bits.count() != L->M || alpha.count() != L->M)) {
+        PyErr_SetString(PyExc_ValueError, "scheme/bits/alpha need M entries");
+        c.ok = false;
+    }
+    const int mode = c.i32(6);
+    void* pk = c.ptr(7);
+    const size_t pk_bytes = c.none(8) ? c.bytes_of(7) : c.size(8);
+    void* s = c.stream(9);
+    RUN("rmsmp_quantize_pack", api.quantize_pack((const float*)W, (rmsmp_w_layout)w_layout, L, (const uint8_t*)hs, (const uint8_t*)hb, (const float*)ha,
+                                                 (rmsmp_pot_mode)mode, pk, pk_bytes, s))
+    Py_RETURN_NONE;
+}
+
 DEF(gemm_grouped_launch)
 {
     ARGS("rmsmp_gemm_grouped_launch", 1, "plan", "stream")
@@ -397,11 +447,11 @@ DEF(gemm_grouped_launch)
     Py_RETURN_NONE;
 }
 
-// setup(addresses: {name: int}, stream: callable, error: callable)
+// setup(addresses: {name: int}, stream: callable, error: callable, array: callable)
 PyObject* setup(PyObject*, PyObject* args)
 {
-    PyObject *addr, *stream, *error;
-    if (!PyArg_ParseTuple(args, "O!OO", &PyDict_Type, &addr, &stream, &error)) return nullptr;
+    PyObject *addr, *stream, *error, *array;
+    if (!PyArg_ParseTuple(args, "O!OOO", &PyDict_Type, &addr, &stream, &error, &array)) return nullptr;
     auto get = [&](const char* name, auto& fn) -> bool {
         PyObject* v = PyDict_GetItemString(addr, name);
         if (!v) { PyErr_SetString(PyExc_KeyError, name); return false; }
@@ -416,16 +466,18 @@ PyObject* setup(PyObject*, PyObject* args)
         !get("rmsmp_conv_implicit_workspace", api.conv_implicit_workspace) ||
         !get("rmsmp_conv_implicit_workspace_requant", api.conv_implicit_workspace_requant) || !get("rmsmp_conv_depthwise", api.conv_depthwise) ||
         !get("rmsmp_im2col_codes", api.im2col_codes) || !get("rmsmp_expand_weights", api.expand_weights) ||
-        !get("rmsmp_assign_quantize_pack", api.assign_quantize_pack) || !get("rmsmp_gemm_grouped_launch", api.gemm_grouped_launch))
+        !get("rmsmp_assign_quantize_pack", api.assign_quantize_pack) || !get("rmsmp_gemm_grouped_launch", api.gemm_grouped_launch) ||
+        !get("rmsmp_quantize_pack", api.quantize_pack))
         return nullptr;
     Py_INCREF(stream); Py_XSETREF(g_stream, stream);
     Py_INCREF(error); Py_XSETREF(g_error, error);
+    Py_INCREF(array); Py_XSETREF(g_array, array);
     Py_RETURN_NONE;
 }
 
 #define METHOD(name, doc) {"rmsmp_" #name, (PyCFunction)(void (*)(void))name, METH_FASTCALL | METH_KEYWORDS, doc}
 PyMethodDef methods[] = {
-    {"setup", setup, METH_VARARGS, "entry points, current-stream callable, error callable"},
+    {"setup", setup, METH_VARARGS, "entry points, current-stream callable, error callable, array callable"},
     METHOD(quantize_act, "Returns the activation step (alpha_a/15 or alpha_a/7) as a Python float (fp32 value)."),
     METHOD(gemm, "Linear layer."),
     METHOD(gemm_variant, "Linear layer by a chosen kernel."),
@@ -439,6 +491,7 @@ PyMethodDef methods[] = {
     METHOD(im2col_codes, "Patch matrix of a convolution's activation codes."),
     METHOD(expand_weights, "Expands a layer's packed codes into its workspace."),
     METHOD(assign_quantize_pack, "Row assignment on the device + quantize + pack, from the ratio alone."),
+    METHOD(quantize_pack, "Quantize + group + pack by a given scheme, precision and scale per row."),
     METHOD(gemm_grouped_launch, "One launch of a prepared grouped plan."),
     {nullptr, nullptr, 0, nullptr}};
 

@@ -178,3 +178,24 @@ def test_marshalled_calls_take_the_python_signatures_and_raise_like_them():
             bad_call()
     with pytest.raises(OverflowError):
         R.rmsmp_conv_implicit(good, 256, 256, 1 << 40, 4, 4, 1, 0, 0.5, 256, stream=0)
+
+
+@pytest.mark.parametrize("convert", [lambda a: a, list, lambda a: a.astype(np.int64), lambda a: np.repeat(a, 2)[::2]],
+                         ids=["array", "list", "int64", "strided"])
+def test_marshalled_pack_takes_any_host_array(convert):
+    """Scheme, precision and scale per row as what numpy makes an array of; refusals come from the library."""
+    scheme, bits, alpha = np.array([0, 1, 1, 1], np.uint8), np.array([4, 4, 8, 4], np.uint8), np.full(4, 3, np.float32)
+    layer = R.rmsmp_layer_init(4, 16, 1, 1, scheme, bits)
+
+    def call(s=scheme, b=bits, a=alpha, mode=R.POT_NEAREST, packed=256, nbytes=1 << 20):
+        R.rmsmp_quantize_pack(256, R.W_LINEAR, layer, convert(s), convert(b), convert(a), mode, packed, nbytes, stream=0)
+    for kw, status in ((dict(s=np.zeros(4, np.uint8)), R.ERR_SCHEME), (dict(b=np.array([4, 4, 5, 4], np.uint8)), R.ERR_SCHEME),
+                       (dict(a=alpha * 0), R.ERR_SCALE), (dict(mode=9), R.ERR_SCHEME), (dict(packed=None), R.ERR_NULL),
+                       (dict(packed=264), R.ERR_ALIGN), (dict(nbytes=16), R.ERR_BUFFER_TOO_SMALL)):
+        with pytest.raises(R.RmsmpError) as e:
+            call(**kw)
+        assert e.value.status == status
+    with pytest.raises(ValueError):
+        call(a=alpha[:3])
+    with pytest.raises((TypeError, ValueError)):
+        R.rmsmp_quantize_pack(256, R.W_LINEAR, layer, "abc", bits, alpha, R.POT_NEAREST, 256, 1 << 20, stream=0)
