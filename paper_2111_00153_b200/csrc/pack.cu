@@ -312,7 +312,9 @@ __global__ void __launch_bounds__(256) quantize_act_kernel(const float* __restri
     if (vec) {
         // A warp takes 1024 consecutive values per step: eight 128-bit loads per lane, each
         // instruction covering 512 contiguous bytes, then eight 32-bit stores of 128 contiguous
-        // bytes each.  The remaining 16-value groups follow one lane at a time.
+        // bytes each.  The remaining 16-value groups follow one lane at a time.  The values are read once and leave L2
+        // first; the codes are stored to stay, the layer reads them next (stored streaming: ResNet-18 at batch 256
+        // 1062 us against 1042, the MobileNet-v2 block 127.6 against 125.8).
         const size_t n16 = count / 16;
         const size_t n1024 = count / 1024;
         const int lane = threadIdx.x & 31;
@@ -325,7 +327,7 @@ __global__ void __launch_bounds__(256) quantize_act_kernel(const float* __restri
             for (int j = 0; j < 8; ++j) v[j] = __ldcs(src + j * 32);
             uint32_t* dst = reinterpret_cast<uint32_t*>(codes) + i * 256 + lane;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) __stcs(dst + j * 32, act_codes4(v[j], alpha, kind, fast));
+            for (int j = 0; j < 8; ++j) dst[j * 32] = act_codes4(v[j], alpha, kind, fast);
         }
         for (size_t i = n1024 * 64 + tid; i < n16; i += nthr) {
             const float4* src = reinterpret_cast<const float4*>(x) + i * 4;
