@@ -12,7 +12,7 @@
 // bytes, eight permutes), which makes the three taps of a kernel row one dot product; a thread owns a
 // channel quad and four neighbouring columns and walks down a strip of rows, so that every input row is
 // loaded and transposed once for the three output rows that it touches, and the next row's loads are in
-// flight meanwhile (46 us).
+// flight meanwhile (44 us; what is left is load latency at two blocks per SM).
 // Other filters: a word is split into four one-channel words, one output per work item.
 #include <algorithm>
 #include "common.cuh"
@@ -44,35 +44,41 @@ __device__ __forceinline__ void dw_transpose(uint32_t w0, uint32_t w1, uint32_t 
     t[2] = dw_prmt(c, d, 0x5410u); t[3] = dw_prmt(c, d, 0x7632u);
 }
 
-// One input row of a thread's strip, ready for the dot products: for every channel the words whose bytes 0..2
-// are the three columns under a kernel row.
-struct DwRow { uint32_t w[4][kDwCols]; };      // [channel][output column]
+// One input row of a thread's strip, ready for the dot products.  Stride 1: for every channel the words whose bytes 0..2
+// are the three columns under a kernel row.  Stride 2: the transposed columns, from which dw_word forms those words
+// where they are used -- a row serves one or two output rows there, and its sixteen words took registers that the
+// loads ahead need (56 x 56 x 192 at batch 64, launches back to back: 22.6 us with them, 19.5 so; stride 1, three output rows a row, 49.8 and 51.0).
+template <int kS> struct DwRow { uint32_t g[4], t[kS == 1 ? 12 : 5]; };
 
 template <int kS>
-__device__ __forceinline__ void dw_arrange(const uint32_t (&a)[3 * kS + 3], DwRow& r)
+__device__ __forceinline__ void dw_arrange(const uint32_t (&a)[3 * kS + 3], DwRow<kS>& r)
 {
-    uint32_t g[4];
-    dw_transpose(a[0], a[1], a[2], a[3], g);
+    dw_transpose(a[0], a[1], a[2], a[3], r.g);                                              // columns 0 1 2 (3)
     if constexpr (kS == 1) {
         const uint32_t lo = dw_prmt(a[4], a[5], 0x5140u), hi = dw_prmt(a[4], a[5], 0x7362u);      // columns 4, 5: channels 0, 1 / 2, 3
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            r.w[c][0] = g[c];                                                               // columns 0 1 2
-            r.w[c][1] = g[c] >> 8;                                                          // columns 1 2 3
-            r.w[c][2] = dw_prmt(g[c], c < 2 ? lo : hi, (c & 1) ? 0x6632u : 0x4432u);        // columns 2 3 4
-            r.w[c][3] = dw_prmt(g[c], c < 2 ? lo : hi, (c & 1) ? 0x7763u : 0x5543u);        // columns 3 4 5
+            r.t[3 * c] = r.g[c] >> 8;                                                       // columns 1 2 3
+            r.t[3 * c + 1] = dw_prmt(r.g[c], c < 2 ? lo : hi, (c & 1) ? 0x6632u : 0x4432u); // columns 2 3 4
+            r.t[3 * c + 2] = dw_prmt(r.g[c], c < 2 ? lo : hi, (c & 1) ? 0x7763u : 0x5543u); // columns 3 4 5
         }
     } else {
         uint32_t h[4];
         dw_transpose(a[4], a[5], a[6], a[7], h);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            r.w[c][0] = g[c];                                                               // columns 0 1 2
-            r.w[c][1] = dw_prmt(g[c], h[c], 0x4432u);                                       // columns 2 3 4
-            r.w[c][2] = h[c];                                                               // columns 4 5 6
-            r.w[c][3] = dw_prmt(h[c], a[8], 0x0032u | (uint32_t)(4 + c) << 8 | (uint32_t)(4 + c) << 12);      // columns 6 7 8
-        }
+        for (int c = 0; c < 4; ++c) r.t[c] = h[c];
+        r.t[4] = a[8];
     }
+}
+
+// The columns under output column j of channel c, in bytes 0..2.
+template <int kS>
+__device__ __forceinline__ uint32_t dw_word(const DwRow<kS>& r, int c, int j)
+{
+    if (j == 0) return r.g[c];
+    if constexpr (kS == 1) return r.t[3 * c + j - 1];
+    else if (j == 1) return dw_prmt(r.g[c], r.t[c], 0x4432u);                                              // columns 2 3 4
+    else return j == 2 ? r.t[c] : dw_prmt(r.t[c], r.t[4], 0x0032u | (uint32_t)(4 + c) << 8 | (uint32_t)(4 + c) << 12);      // 4 5 6, 6 7 8
 }
 
 __device__ __forceinline__ void dw_store(const Problem& p, uint32_t n, int q, const int* acc)
@@ -88,7 +94,8 @@ __device__ __forceinline__ void dw_store(const Problem& p, uint32_t n, int q, co
 }
 
 // kS = 1, 2: 3 x 3 filters of that stride, strips of `strip` output rows; kS = 0: any filter, one output per item.
-template <int kS>
+// kAcc: the sums are wanted too (their addresses take registers that the strips need: 5 % of the time).
+template <int kS, bool kAcc>
 __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const Problem p, const int strip)
 {
     extern __shared__ uint32_t s_w[];                     // [tap][quad]: channel 4q+j in byte j
@@ -139,9 +146,10 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
                 uint32_t in_x = 0;                                     // which of the columns lie inside the image
 #pragma unroll
                 for (int x = 0; x < kXW; ++x) in_x |= ((unsigned)(x0 + x) < (unsigned)p.W ? 1u : 0u) << x;
+                const int y_end = min(p.H, (ho0 + rows - 1) * kS - p.pad + 3);     // behind the last input row of the strip
                 auto load = [&](int y, uint32_t (&a)[kXW]) {           // rows and columns outside the image read as zero
                     const int8_t* r = src + (int64_t)y * row_pitch;
-                    if ((unsigned)y >= (unsigned)p.H) {
+                    if ((unsigned)y >= (unsigned)y_end) {
 #pragma unroll
                         for (int x = 0; x < kXW; ++x) a[x] = 0u;
                     } else if (in_x == (1u << kXW) - 1u) {             // the usual case, without a predicate per column
@@ -153,29 +161,29 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
                     }
                 };
                 float* out = p.out + ((size_t)b * p.Ho * p.Wo + (size_t)ho0 * p.Wo + wo0) * p.ld_out + 4 * q;
-                int32_t* acc_out = p.acc ? p.acc + (out - p.out) : nullptr;
+                int32_t* const acc_out = kAcc ? p.acc + (out - p.out) : nullptr;
                 const uint32_t ld = (uint32_t)p.ld_out;
                 const size_t row_out = (size_t)p.Wo * p.ld_out;
                 // one output row from the three arranged input rows under it
-                auto emit = [&](int h, const DwRow& r0, const DwRow& r1, const DwRow& r2) {
+                auto emit = [&](int h, const DwRow<kS>& r0, const DwRow<kS>& r1, const DwRow<kS>& r2) {
                     float* o = out + (size_t)h * row_out;
 #pragma unroll
                     for (int j = 0; j < kDwCols; ++j) {
                         int acc[4];
 #pragma unroll
                         for (int c = 0; c < 4; ++c)
-                            acc[c] = __dp4a((int)r2.w[c][j], (int)f[2][c], __dp4a((int)r1.w[c][j], (int)f[1][c], __dp4a((int)r0.w[c][j], (int)f[0][c], kDwMagicBits)));
+                            acc[c] = __dp4a((int)dw_word(r2, c, j), (int)f[2][c], __dp4a((int)dw_word(r1, c, j), (int)f[1][c], __dp4a((int)dw_word(r0, c, j), (int)f[0][c], kDwMagicBits)));
                         if (j < cols) {
                             *reinterpret_cast<float4*>(o + (uint32_t)j * ld) =
                                 make_float4(__fmul_rn(__fsub_rn(__int_as_float(acc[0]), kDwMagic), sc[0]), __fmul_rn(__fsub_rn(__int_as_float(acc[1]), kDwMagic), sc[1]),
                                             __fmul_rn(__fsub_rn(__int_as_float(acc[2]), kDwMagic), sc[2]), __fmul_rn(__fsub_rn(__int_as_float(acc[3]), kDwMagic), sc[3]));
-                            if (acc_out)
+                            if (kAcc)
                                 *reinterpret_cast<int4*>(acc_out + (size_t)h * row_out + (uint32_t)j * ld) =
                                     make_int4(acc[0] - kDwMagicBits, acc[1] - kDwMagicBits, acc[2] - kDwMagicBits, acc[3] - kDwMagicBits);
                         }
                     }
                 };
-                DwRow r[3];
+                DwRow<kS> r[3];
                 uint32_t a[kXW], nx[kXW];
                 int y = ho0 * kS - p.pad;                              // the input row to arrange next
                 if constexpr (kS == 1) {
@@ -253,11 +261,13 @@ cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
 {
     const size_t smem = (size_t)p.kh * p.kw * p.M;
     const int variant = (p.kh == 3 && p.kw == 3 && (p.stride == 1 || p.stride == 2)) ? p.stride : 0;
-    static bool attr_set[3][kMaxDevices] = {};
-    const void* fn = variant == 1 ? reinterpret_cast<const void*>(depthwise_kernel<1>)
-                   : variant == 2 ? reinterpret_cast<const void*>(depthwise_kernel<2>)
-                                  : reinterpret_cast<const void*>(depthwise_kernel<0>);
-    if (smem > 48 * 1024 && !ensure_smem_attr(fn, 200 * 1024, attr_set[variant])) return cudaErrorUnknown;
+    const bool acc = variant != 0 && p.acc;
+    static bool attr_set[3][2][kMaxDevices] = {};
+    void (*const kernel)(const Problem, const int) = variant == 1 ? (acc ? depthwise_kernel<1, true> : depthwise_kernel<1, false>)
+                                                   : variant == 2 ? (acc ? depthwise_kernel<2, true> : depthwise_kernel<2, false>)
+                                                                  : depthwise_kernel<0, false>;
+    const void* fn = reinterpret_cast<const void*>(kernel);
+    if (smem > 48 * 1024 && !ensure_smem_attr(fn, 200 * 1024, attr_set[variant][acc])) return cudaErrorUnknown;
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kDwThreads, smem);
     if (e != cudaSuccess) return e;
@@ -285,8 +295,7 @@ cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
     }
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    return launch_dependent(variant == 1 ? depthwise_kernel<1> : variant == 2 ? depthwise_kernel<2> : depthwise_kernel<0>, (unsigned)blocks,
-                            kDwThreads, smem, st, p, strip);
+    return launch_dependent(kernel, (unsigned)blocks, kDwThreads, smem, st, p, strip);
 }
 
 }  // namespace rmsmp
