@@ -64,8 +64,10 @@ struct TensorCfg {
     int nA, nB;            // ring depths: expanded weights, activations
     int out_bufs;          // staging buffers per epilogue warp (1 or 2)
     int pre;               // 1: the A operand comes expanded (int8) from a workspace, no expander work
-    int dup;               // 1 (pre mode, M <= 64): rows 0..63 are loaded twice, into lanes 0..63 and 64..127, so that all
+    int dup;               // 1 (pre mode, M <= 64, or resident weights whose last row block is at most half full): that block's
+                           //    first 64 rows are loaded twice, into lanes 0..63 and 64..127, so that all
                            //    four tensor-memory quarters hold valid rows and every epilogue warp has work
+    int cta_full;          // > 0: CTAs of every row block but the last, which gets the rest of the grid (its tiles take less)
     int epi_warps;         // epilogue warps: 4, or 12 in pre mode (the idle expander warps join)
     int bk;                // codes per k-block and bytes per operand row in shared memory: 128, or 64 (pre mode,
                            //    channel counts that would leave half of a 128-byte row empty)
@@ -91,7 +93,8 @@ struct TensorCfg {
 
 struct Maps {
     CUtensorMap act[4];                                // [B][H][W][Cin] activation codes; stride 2: one map per row/column parity
-    CUtensorMap wexp;                                  // [M][Kp] int8 weights expanded beforehand (pre mode); 64-row box when dup
+    CUtensorMap wexp;                                  // [M][Kp] int8 weights expanded beforehand (pre mode); 64-row box when all rows are dup
+    CUtensorMap wexp_dup;                              // the same in 64-row boxes, where only the last of several row blocks is dup
     CUtensorMap out_full, out_tail, acc_full, acc_tail;   // bulk stores: 32-row and tail chunks
     CUtensorMap rq_full, rq_tail;                       // re-quantized codes: 32 pixels x 32 code bytes, and the tail
 };
@@ -104,9 +107,9 @@ struct Maps {
 // lanes 64..127.  Nothing overlaps with it in a CTA's first tile, and it is a chain (slot, codes, expansion): a few
 // threads share a row, and a thread has the loads of four pieces of 32 codes in flight at a time (512x512 N=4096, all in one tile per
 // CTA: 14.7 us with a load at a time and half of each piece kept, 10.8 so; 128x512 N=2000 10.6).
-__device__ __forceinline__ void fill_resident_weights(const Problem& p, const TensorCfg& cfg, uint32_t sA, int row_first, int tid, int nthreads)
+__device__ __forceinline__ void fill_resident_weights(const Problem& p, const TensorCfg& cfg, uint32_t sA, int row_first, bool dup, int tid, int nthreads)
 {
-    const int rows = cfg.dup ? kBlockRows / 2 : kBlockRows;
+    const int rows = dup ? kBlockRows / 2 : kBlockRows;
     const int pshift = cfg.bk == 128 ? 2 : 1;            // 32-code pieces of a row and k-block: 4 or 2
     const int n4 = p.nP + p.nF4;
     const int tpr = nthreads / rows;
@@ -161,7 +164,7 @@ __device__ __forceinline__ void fill_resident_weights(const Problem& p, const Te
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t at = dst + (((unit + (uint32_t)h) ^ phase) << 4);
                     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(w[4 * h]), "r"(w[4 * h + 1]), "r"(w[4 * h + 2]), "r"(w[4 * h + 3]));
-                    if (cfg.dup)
+                    if (dup)
                         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + (uint32_t)(cfg.a_bytes / 2)), "r"(w[4 * h]), "r"(w[4 * h + 1]), "r"(w[4 * h + 2]), "r"(w[4 * h + 3]));
                 }
             }
@@ -254,13 +257,25 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
 
-    const int64_t first = blockIdx.x, step = gridDim.x;
-    const int64_t my_tiles = (cfg.ntiles > first) ? (cfg.ntiles - first + step - 1) / step : 0;
+    // (tile indices fit 32 bits with a step to spare: checked on the host)
+    const uint32_t ntiles = (uint32_t)cfg.ntiles;
+    uint32_t first = blockIdx.x, step = gridDim.x;
+    if (kAres && cfg.cta_full) {
+        // (see TensorCfg::cta_full) the CTA's row block, and its place among that block's CTAs
+        const uint32_t rest = (uint32_t)cfg.nbt - 1u, full = (uint32_t)cfg.cta_full * rest;
+        const bool last = blockIdx.x >= full;
+        const uint32_t mine = last ? rest : blockIdx.x % rest, at = last ? blockIdx.x - full : blockIdx.x / rest;
+        first = at * (uint32_t)cfg.nbt + mine;
+        step = (last ? gridDim.x - full : (uint32_t)cfg.cta_full) * (uint32_t)cfg.nbt;
+    }
+    const int my_blk = kAres ? (int)(first % (uint32_t)cfg.nbt) : 0;
+    const bool dup = cfg.dup && (!kAres || my_blk == cfg.nbt - 1);
+    const int64_t my_tiles = (ntiles > first) ? (ntiles - first + step - 1) / step : 0;
 
     if (kAres && cfg.fill && warp != 0) {
         // every warp but the activation producer's (whose first copies go out meanwhile) expands the row block;
         // one of them then reports the resident weights to the MMA thread
-        if (my_tiles > 0) fill_resident_weights(p, cfg, sA, (int)(first % cfg.nbt) * kBlockRows, (int)threadIdx.x - 32, kThreads - 32);
+        if (my_tiles > 0) fill_resident_weights(p, cfg, sA, my_blk * kBlockRows, dup, (int)threadIdx.x - 32, kThreads - 32);
         asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32) : "memory");
         if (threadIdx.x == 32 && my_tiles > 0) mbar_arrive(bar_fullA);
     }
@@ -278,8 +293,9 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 for (int kb = 0; kb < cfg.nkb; ++kb) {
                     const int koff = tap * p.Cp + cc * cfg.bk;
                     const uint32_t dst = sA + kb * cfg.a_bytes;
-                    tma_load_2d(dst, &maps.wexp, bar_fullA, koff, (int)(first % cfg.nbt) * kBlockRows);
-                    if (cfg.dup) tma_load_2d(dst + cfg.a_bytes / 2, &maps.wexp, bar_fullA, koff, 0);
+                    const CUtensorMap* map = dup && cfg.nbt > 1 ? &maps.wexp_dup : &maps.wexp;
+                    tma_load_2d(dst, map, bar_fullA, koff, my_blk * kBlockRows);
+                    if (dup) tma_load_2d(dst + cfg.a_bytes / 2, map, bar_fullA, koff, my_blk * kBlockRows);
                     if (++cc == cfg.cpt) { cc = 0; ++tap; }
                 }
             }
@@ -288,9 +304,9 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             const uint32_t bar_f = pre_b_producer ? bar_fullB : bar_fullA;
             uint32_t s = 0, ph = 0;
             bool ok = true;
-            for (int64_t tile = first; tile < cfg.ntiles && ok; tile += step) {
-                const uint32_t nt = (uint32_t)tile / (uint32_t)cfg.nbt;
-                const int blk = (int)((uint32_t)tile - nt * (uint32_t)cfg.nbt) << kM2;
+            for (uint32_t tile = first; tile < ntiles && ok; tile += step) {
+                const uint32_t nt = tile / (uint32_t)cfg.nbt;
+                const int blk = (int)(tile - nt * (uint32_t)cfg.nbt) << kM2;
                 int b0, h0;
                 if (cfg.tiles_per_image) {
                     b0 = (int)(nt / (uint32_t)cfg.tiles_per_image);
@@ -299,7 +315,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     b0 = (int)nt * cfg.tb;
                     h0 = 0;
                 }
-                const int row_a = cfg.dup ? 0 : blk * kBlockRows;
+                const int row_a = blk * kBlockRows;
                 int tap = 0, cc = 0, ti = 0, tj = 0;
                 for (int kb = 0; kb < cfg.nkb; ++kb) {
                     if (!mbar_wait(bar_e + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
@@ -330,7 +346,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                         const int koff = tap * p.Cp + cc * cfg.bk;
                         mbar_arrive_expect_tx(bar_f + 8 * s, cfg.a_bytes);
                         tma_load_2d(sA + s * cfg.a_bytes, &maps.wexp, bar_f + 8 * s, koff, row_a);
-                        if (cfg.dup) tma_load_2d(sA + s * cfg.a_bytes + cfg.a_bytes / 2, &maps.wexp, bar_f + 8 * s, koff, row_a);
+                        if (dup) tma_load_2d(sA + s * cfg.a_bytes + cfg.a_bytes / 2, &maps.wexp, bar_f + 8 * s, koff, row_a);
                     }
                     if (++s == nring) { s = 0; ph ^= 1; }
                     if (++cc == cfg.cpt) { cc = 0; ++tap; if (++tj == p.kw) { tj = 0; ++ti; } }
@@ -350,7 +366,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             const uint64_t desc_a0 = smem_desc_kmajor(sA, cfg.bk), desc_b0 = smem_desc_kmajor(sB, cfg.bk);
             const uint32_t desc_lo0_a = (uint32_t)desc_a0, desc_lo0_b = (uint32_t)desc_b0, desc_hi = (uint32_t)(desc_a0 >> 32);
             bool have_a = !kAres || my_tiles == 0 || mbar_wait(bar_fullA, 0, abort_flag);
-            for (int64_t tile = first; tile < cfg.ntiles && have_a && !*abort_flag; tile += step, ++it) {
+            for (uint32_t tile = first; tile < ntiles && have_a && !*abort_flag; tile += step, ++it) {
                 // one accumulator per tile, alternating; or (two row blocks per tile) both, every tile
                 const uint32_t ab = kM2 ? 0u : (it & 1);
                 const uint32_t tpar = kM2 ? ((it & 1) ^ 1) : (((it >> 1) & 1) ^ 1);
@@ -473,13 +489,13 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         // tile look-ahead: one tile, or kGroups tiles when every tile is a single k-block
         const int64_t look = (cfg.nkb == 1) ? kGroups : 1;
         const int64_t total = my_tiles * cfg.nkb;
-        const bool rows_change = (uint32_t)step % (uint32_t)p.nblocks != 0u;
+        const bool rows_change = step % (uint32_t)p.nblocks != 0u;
         // a row block's rows in the packed buffer: first and number of each kind
         int4 blk_a;
         int2 blk_b;
         int blk_next = 0;
         auto load_block = [&](int64_t local) {
-            blk_next = (int)((uint32_t)(first + min(local, my_tiles - 1) * step) % (uint32_t)p.nblocks);
+            blk_next = (int)((uint32_t)(first + (uint32_t)min(local, my_tiles - 1) * step) % (uint32_t)p.nblocks);
             blk_a = __ldg(reinterpret_cast<const int4*>(p.blocks + 8 * blk_next));
             blk_b = __ldg(reinterpret_cast<const int2*>(p.blocks + 8 * blk_next + 4));
         };
@@ -625,24 +641,24 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         // how many epilogue warps share a quarter, and this warp's rank among them
         auto count_q = [&](int q) { const int f = first_epi + ((q - first_epi) & 3); return (kThreads / 32 - 1 - f) / 4 + 1; };
         const int my_rank = (warp - (first_epi + ((quarter - first_epi) & 3))) >> 2;
-        const int row0 = cfg.dup ? (quarter & 1) * 32 : quarter * 32;       // first row (within the block) of this warp
-        const int cstride = cfg.dup ? count_q(quarter & 1) + count_q((quarter & 1) + 2) : count_q(quarter);
-        const int cfirst = (cfg.dup && (quarter >> 1)) ? count_q(quarter & 1) + my_rank : my_rank;
+        const int row0 = dup ? (quarter & 1) * 32 : quarter * 32;       // first row (within the block) of this warp
+        const int cstride = dup ? count_q(quarter & 1) + count_q((quarter & 1) + 2) : count_q(quarter);
+        const int cfirst = (dup && (quarter >> 1)) ? count_q(quarter & 1) + my_rank : my_rank;
         const uint32_t my_stage = sOut + (uint32_t)ew * (cfg.out_bufs * kWarpStage);
         uint32_t it = 0, stg_count = 0;
         bool alive = true;
         int scale_blk = -1, shift = 0;
         float scale = 0.f;
         const ActFast rq_fast = act_fast_setup(kRQ ? p.rq_alpha : 1.0f, kRQ ? p.rq_kind : 0);
-        for (int64_t tile = first; tile < cfg.ntiles && alive; tile += step, ++it) {
+        for (uint32_t tile = first; tile < ntiles && alive; tile += step, ++it) {
           // a tile is one row block (accumulators alternate between tiles), or two (one accumulator each)
           for (int half = 0; half <= kM2; ++half) {
             const uint32_t ab = kM2 ? (uint32_t)half : (it & 1);
             const uint32_t tpar = kM2 ? (it & 1) : ((it >> 1) & 1);
             // tile indices fit 32 bits (checked on the host): 32-bit divisions, a fraction of the 64-bit ones' cost,
             // which every epilogue warp would otherwise pay in front of each tile
-            const uint32_t nt = (uint32_t)tile / (uint32_t)cfg.nbt;
-            const int blk = ((int)((uint32_t)tile - nt * (uint32_t)cfg.nbt) << kM2) + half;
+            const uint32_t nt = tile / (uint32_t)cfg.nbt;
+            const int blk = ((int)(tile - nt * (uint32_t)cfg.nbt) << kM2) + half;
             int64_t n0;
             if (cfg.tiles_per_image) {
                 const uint32_t img = nt / (uint32_t)cfg.tiles_per_image, tin = nt - img * (uint32_t)cfg.tiles_per_image;
@@ -943,7 +959,7 @@ bool plan(const Problem& p, TensorCfg& c)
     c.npix = c.tb * c.th * p.Wo;
     c.n_mma = (c.npix + 15) / 16 * 16;
     c.ntiles = c.ntiles_n * p.nblocks;
-    if (c.ntiles >= (1ll << 31)) return false;
+    if (c.ntiles >= (1ll << 31)) return false;       // (the kernel counts in 32 bits, a step beyond the last)
     c.m2 = 0;
     c.nbt = p.nblocks;
     c.tps = 1;
@@ -970,6 +986,7 @@ bool plan(const Problem& p, TensorCfg& c)
     c.tma_store = 0;
     c.dup = 0;
     c.ares = 0;
+    c.cta_full = 0;
     c.epi_warps = kNumEpiWarps;
     if (c.pre) {
         c.nA = (c.bk == 64) ? 6 : 3; c.nB = (c.bk == 64) ? 8 : 4; c.out_bufs = 1;
@@ -1082,6 +1099,27 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
     if (pair_supported(p)) return launch_pair(p, st);
     TensorCfg c;
     if (!plan(p, c)) return RMSMP_ERR_VARIANT;
+    // All tiles of a CTA are of one row block where the grid is a multiple of them: required by resident weights, and with
+    // expanders worth having when it costs no round of tiles (they look up a tile's rows only once then).
+    int64_t grid = sm_count();
+    const int64_t whole = grid / c.nbt * c.nbt;
+    if (c.ares || (!c.pre && whole > 0 && (c.ntiles + whole - 1) / whole == (c.ntiles + grid - 1) / grid)) grid = whole;
+    grid = std::min(grid, c.ntiles);
+    if (c.ares && c.nbt > 1 && p.M % kBlockRows >= 1 && p.M % kBlockRows <= kBlockRows / 2) {
+        // Shares of the grid by what a tile takes: the last block's output, done by all warps for half of the rows or less,
+        // takes 0.5 to 0.7 of a full one's (256 pixels: 2.8 us; the products 0.17 to 0.41 a k-block).  Equal shares and a
+        // half of the warps idle: 192x32 on 200,704 pixels 33.3 us against 31.7, codes out 30.5 and 27.8, 160x64 on 50,176
+        // 10.5 and 8.9, 144x160 on 740,050 134 and 108.
+        const double n = c.npix / 256.0, mma = c.nkb * (0.28 + 0.13 * n) * (c.bk == 64 ? 0.6 : 1.0), out = 2.8 * n;
+        const double full_us = std::max(mma, out), last_us = std::max(mma, (p.rq_codes ? 0.72 : 0.45 + 0.15 * (p.M % kBlockRows) / 64.0) * out);
+        const int64_t sms = sm_count(), even = whole / c.nbt;
+        double best = 0.95 * std::ceil((double)c.ntiles_n / even) * full_us;
+        for (int64_t last = 1; last < even; ++last) {
+            const int64_t full = (sms - last) / (c.nbt - 1);
+            const double us = std::max(std::ceil((double)c.ntiles_n / full) * full_us, std::ceil((double)c.ntiles_n / last) * last_us);
+            if (c.ntiles_n >= full && us < best) { best = us; c.cta_full = (int)full; c.dup = 1; grid = full * (c.nbt - 1) + last; }
+        }
+    }
     EncodeTiledFn enc = encode_fn();
     if (!enc) return RMSMP_ERR_CUDA;
     Maps mp;
@@ -1091,12 +1129,14 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
     if (p.wexp) {
         const cuuint64_t gd[2] = {(cuuint64_t)p.Kp, (cuuint64_t)p.M};
         const cuuint64_t gs[1] = {(cuuint64_t)p.Kp};
-        const cuuint32_t bx[2] = {(cuuint32_t)c.bk, (cuuint32_t)(c.dup ? kBlockRows / 2 : (c.m2 ? 2 * kBlockRows : kBlockRows))};
         const cuuint32_t es[2] = {1, 1};
-        if (enc(&mp.wexp, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t*>(p.wexp), gd, gs, bx, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, c.bk == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        auto make = [&](CUtensorMap* m, int rows) -> bool {
+            const cuuint32_t bx[2] = {(cuuint32_t)c.bk, (cuuint32_t)rows};
+            return enc(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t*>(p.wexp), gd, gs, bx, es,
+                       CU_TENSOR_MAP_INTERLEAVE_NONE, c.bk == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+        };
+        if (!make(&mp.wexp, c.m2 ? 2 * kBlockRows : (c.dup && c.nbt == 1 ? kBlockRows / 2 : kBlockRows)) || (c.dup && c.nbt > 1 && !make(&mp.wexp_dup, kBlockRows / 2)))
             return RMSMP_ERR_CUDA;
     }
 
@@ -1161,12 +1201,6 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
     if (!fn) return RMSMP_ERR_VARIANT;
     static bool attr_set[4][2][3][kMaxDevices] = {};
     if (!ensure_smem_attr(reinterpret_cast<const void*>(fn), kSmemLimit, attr_set[mode][i2][io])) return RMSMP_ERR_CUDA;
-    // All tiles of a CTA are of one row block where the grid is a multiple of them: required by resident weights, and with
-    // expanders worth having when it costs no round of tiles (they look up a tile's rows only once then).
-    int64_t grid = sm_count();
-    const int64_t whole = grid / c.nbt * c.nbt;
-    if (c.ares || (!c.pre && whole > 0 && (c.ntiles + whole - 1) / whole == (c.ntiles + grid - 1) / grid)) grid = whole;
-    grid = std::min(grid, c.ntiles);
     if (launch_dependent(fn, (unsigned)grid, threads_of(mode), c.smem_bytes, st, p, c, mp) != cudaSuccess) {
         cudaGetLastError();
         return RMSMP_ERR_CUDA;

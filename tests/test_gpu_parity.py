@@ -1017,3 +1017,29 @@ def test_weights_expanded_for_every_tile(M, Cin, k, B, H, W, mix):
     y, acc = Hn.conv(layer, d_packed, act, 1, k // 2, 0.25, R.VARIANT_TENSOR)
     assert np.array_equal(acc, acc_ref.reshape(-1, M))
     assert np.array_equal(y.view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
+
+
+@pytest.mark.parametrize("M", [129, 144, 192, 193, 336])
+@pytest.mark.parametrize("variant", [R.VARIANT_AUTO, Hn.WORKSPACE], ids=["plain", "workspace"])
+def test_resident_weights_whose_last_row_block_is_short(M, variant):
+    """The last block's rows lie twice in tensor memory and its tiles go to fewer CTAs: exact, and the codes of the
+    re-quantizing call are the quantizer's."""
+    import torch
+    Cin, B, H, W = 64, 61, 31, 29
+    g = synth.rng(99, M)
+    Wt = synth.weights_kaiming(g, M, Cin, 1, 1)
+    scheme, bits = _mixed_map(M, M, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    act = g.integers(0, 16, size=(B, H, W, Cin)).astype(np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    _, ws, acc_ref, y_ref = O.layer_conv(Wt, scheme, bits, alpha, act, np.float32(0.25), 1, 0)
+    y, acc = Hn.conv(layer, d_packed, act, 1, 0, 0.25, variant)
+    assert np.array_equal(acc, acc_ref.reshape(-1, M))
+    assert np.array_equal(y.view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
+    if variant == Hn.WORKSPACE:
+        want, _ = O.quantize_act(y_ref.reshape(-1, M), 4.0, R.ACT_U4)
+        codes = torch.full((B * H * W, M), 99, dtype=torch.int8, device="cuda")
+        d_ws = torch.empty(R.rmsmp_workspace_bytes(layer), dtype=torch.int8, device="cuda")
+        R.rmsmp_expand_weights(layer, d_packed, d_ws)
+        R.rmsmp_conv_implicit_workspace_requant(layer, d_packed, d_ws, torch.from_numpy(act).cuda(), B, H, W, 1, 0, 0.25, 4.0, R.ACT_U4, codes)
+        assert np.array_equal(codes.cpu().numpy(), want)
