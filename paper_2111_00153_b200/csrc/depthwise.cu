@@ -146,7 +146,9 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
                 uint32_t in_x = 0;                                     // which of the columns lie inside the image
 #pragma unroll
                 for (int x = 0; x < kXW; ++x) in_x |= ((unsigned)(x0 + x) < (unsigned)p.W ? 1u : 0u) << x;
-                const int y_end = min(p.H, (ho0 + rows - 1) * kS - p.pad + 3);     // behind the last input row of the strip
+                // behind the last input row of the strip; 0 where the whole strip lies in the padding above the image, so
+                // that the one unsigned comparison in load() rules out rows in front of the image too
+                const int y_end = max(0, min(p.H, (ho0 + rows - 1) * kS - p.pad + 3));
                 auto load = [&](int y, uint32_t (&a)[kXW]) {           // rows and columns outside the image read as zero
                     const int8_t* r = src + (int64_t)y * row_pitch;
                     if ((unsigned)y >= (unsigned)y_end) {

@@ -828,6 +828,39 @@ def test_depthwise_strips_on_the_whole_code_range(C, pad, B, H, W, stride):
         assert np.array_equal(y.cpu().numpy().view(np.uint32), O.epilogue(acc_ref, wstep, np.float32(0.5)).view(np.uint32))
 
 
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("C,pad,B,H,W", [
+    (32, 4, 1, 8, 8), (32, 4, 2, 8, 8),        # strips of one output row, the first of them above every input row
+    (32, 5, 1, 14, 14), (64, 8, 2, 14, 14),
+    (192, 6, 4, 28, 28),                       # strips of two rows
+    (8, 16, 3, 1, 5), (4, 16, 2, 6, 1),        # the widest padding
+])
+def test_depthwise_strips_that_lie_in_the_padding(C, pad, B, H, W, stride):
+    """Outputs without an input row under them are zero.  The activations are the middle of a buffer of non-zero codes,
+    so that a row read from outside the image stays inside the buffer and shows in the sums."""
+    import torch
+    g = synth.rng(89, C + H + W + pad)
+    Wt = synth.weights_kaiming(g, C, 1, 3, 3)
+    scheme, bits = O.assign_rows(Wt, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    codes = g.integers(0, 16, size=(B, H, W, C), dtype=np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    v_ref, wstep = O.quantize_rows(Wt.reshape(C, -1), scheme, bits, alpha)
+    acc_ref = O.conv_depthwise(v_ref.reshape(C, 3, 3), codes, stride, pad)
+    margin = (pad + 4) * (W + 2 * pad) * C // 16 * 16
+    buf = torch.full((margin + codes.size + margin,), 15, dtype=torch.int8, device="cuda")
+    act = buf[margin:margin + codes.size]
+    act.copy_(torch.from_numpy(codes).cuda().view(-1))
+    for with_acc in (True, False):
+        y = torch.full(acc_ref.shape, float("nan"), dtype=torch.float32, device="cuda")
+        acc = torch.full(acc_ref.shape, -5, dtype=torch.int32, device="cuda")
+        R.rmsmp_conv_depthwise(layer, d_packed, act, B, H, W, stride, pad, 0.5, y, acc if with_acc else None)
+        torch.cuda.synchronize()
+        if with_acc:
+            assert np.array_equal(acc.cpu().numpy(), acc_ref)
+        assert np.array_equal(y.cpu().numpy().view(np.uint32), O.epilogue(acc_ref, wstep, np.float32(0.5)).view(np.uint32))
+
+
 def test_depthwise_conv_rejects_what_it_cannot_run():
     import torch
     g = synth.rng(86, 1)
