@@ -36,10 +36,41 @@ struct RowStats {             // scratch, 16 bytes per row
     float* amax;              // max |w|, 1 for an all-zero row
 };
 
+// The definition's variance: two plain passes in reduction order, every operation rounded on its own.
+__device__ __noinline__ double exact_variance(const float* __restrict__ w, int K)
+{
+    double mean = 0.0, acc = 0.0;
+    for (int pass = 0; pass < 2; ++pass) {
+        acc = 0.0;
+        auto add = [&](float v) {
+            if (pass == 0) {
+                acc = __dadd_rn(acc, (double)v);
+            } else {
+                const double d = __dsub_rn((double)v, mean);
+                acc = __dadd_rn(acc, __dmul_rn(d, d));
+            }
+        };
+        if ((K & 3) == 0) {
+            const float4* w4 = reinterpret_cast<const float4*>(w);
+            float4 v = __ldg(w4);
+            for (int i = 0; i < (K >> 2); ++i) {
+                const float4 nx = __ldg(w4 + min(i + 1, (K >> 2) - 1));
+                add(v.x); add(v.y); add(v.z); add(v.w);
+                v = nx;
+            }
+        } else {
+            for (int i = 0; i < K; ++i) add(__ldg(w + i));
+        }
+        if (pass == 0) mean = acc / (double)K;
+    }
+    return acc / (double)K;
+}
+
 // One pass with the row's first weight as the origin: x = w - c, s1 = sum x, s2 = sum x^2, variance
 // (s2 - s1^2 / K) / K.  With u = 2^-53 and q = s2 / K, any order of additions leaves |error| <= 4 (K + 8) u q
 // (|s1| sum|x| <= K s2), and the definition's own two passes are off by at most (K + 4) u var + 2 ((K + 1) u A)^2
 // with A = mean |w|, A^2 <= 2 (c^2 + q); G = 2 (K + 16) u below leaves a factor of more than two.
+// A row whose bound leaves the range of fp32 (weights of 1e25 and more) gets the definition's chain here.
 __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(const float* __restrict__ W, int K, RowStats out)
 {
     pdl_wait();
@@ -86,41 +117,12 @@ __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(const float* __
         double v = fabs(fmax((s2 - s1 * s1 / (double)K) / (double)K, 0.0));
         float e = __double2float_ru(6.0 * G * q + 4.0 * G * G * (c * c + q));
         if (mx == 0.0f) { v = 0.0; e = 0.0f; }                     // an all-zero row's variance is exactly zero
-        if (!(v <= 1e300) || !(e <= 3e38f)) { v = __longlong_as_double(0x7FF0000000000000ll); e = 0.0f; }     // not finite: last, by row index
+        if (!(e <= 3e38f)) { v = exact_variance(w, K); e = 0.0f; }
+        if (!(v <= 1e300)) { v = __longlong_as_double(0x7FF0000000000000ll); e = 0.0f; }     // not finite: last, by row index
         out.var[row] = v;
         out.err[row] = e;
         out.amax[row] = (mx == 0.0f) ? 1.0f : mx;
     }
-}
-
-// The definition's variance: two plain passes in reduction order, every operation rounded on its own.
-__device__ double exact_variance(const float* __restrict__ w, int K)
-{
-    double mean = 0.0, acc = 0.0;
-    for (int pass = 0; pass < 2; ++pass) {
-        acc = 0.0;
-        auto add = [&](float v) {
-            if (pass == 0) {
-                acc = __dadd_rn(acc, (double)v);
-            } else {
-                const double d = __dsub_rn((double)v, mean);
-                acc = __dadd_rn(acc, __dmul_rn(d, d));
-            }
-        };
-        if ((K & 3) == 0) {
-            const float4* w4 = reinterpret_cast<const float4*>(w);
-            float4 v = __ldg(w4);
-            for (int i = 0; i < (K >> 2); ++i) {
-                const float4 nx = __ldg(w4 + min(i + 1, (K >> 2) - 1));
-                add(v.x); add(v.y); add(v.z); add(v.w);
-                v = nx;
-            }
-        } else {
-            for (int i = 0; i < K; ++i) add(__ldg(w + i));
-        }
-        if (pass == 0) mean = acc / (double)K;
-    }
-    return acc / (double)K;
 }
 
 struct MetaArgs {

@@ -737,10 +737,14 @@ def _rows_at_the_cuts(name, g, M, K):
     elif name == "permuted":                            # the same weights in another order: sums differ in the last bits only
         for r in range(1, M):
             W[r] = W[0][g.permutation(K)]
+    elif name == "huge":                                # squares far beyond fp32, rows of several magnitudes
+        W *= np.exp2(g.integers(80, 120, size=(M, 1))).astype(np.float32)
+    elif name == "tiny":                                # squares below fp32's smallest number
+        W *= np.exp2(-g.integers(80, 110, size=(M, 1))).astype(np.float32)
     return np.ascontiguousarray(W)
 
 
-@pytest.mark.parametrize("name", ["normal", "copies", "all_equal", "constant", "zero_rows", "offset", "permuted"])
+@pytest.mark.parametrize("name", ["normal", "copies", "all_equal", "constant", "zero_rows", "offset", "permuted", "huge", "tiny"])
 @pytest.mark.parametrize("M,K,ratio", [(1, 5, (60, 35, 5)), (33, 31, (60, 35, 5)), (257, 100, (50, 40, 10)),
                                        (1024, 36, (60, 35, 5)), (1100, 36, (60, 35, 5)), (2500, 64, (65, 30, 5)),
                                        (4100, 20, (60, 35, 5)), (300, 64, (95, 0, 5)), (128, 16, (0, 100, 0))])
