@@ -8,16 +8,19 @@
 // ranking.  So:
 //   row_stats_kernel   one block per row, one pass over the weights: the variance summed in parallel, a bound
 //                      on how far it can be from the definition's value, and max |w|.
-//   assign_kernel      one block: finds the two cuts by a radix selection over the parallel variances; a row
-//                      whose interval reaches across a cut (in practice: rows that are copies of one another)
-//                      is undecided, gets the definition's chain of additions, and the undecided rows are
-//                      ordered by the exact key.  Then the kind of every row, the stable grouping by prefix
-//                      sums in original order, and every metadata section of the packed buffer.
+//   assign_kernel      one block (and some that help): finds the two cuts by a radix selection over the parallel
+//                      variances; a row whose interval reaches across a cut (in practice: rows that are copies
+//                      of one another) is undecided and gets the definition's chain of additions; a second
+//                      selection finds the cuts among the undecided rows, and of those at a cut's very key the
+//                      first by row index lie in front (all-zero rows: 70 % of 65,536 1.0 ms; every undecided
+//                      row compared with every other was 268 ms).  Then the kind of every row, the stable
+//                      grouping by prefix sums in original order, and every metadata section of the packed buffer.
 //   assign_small_kernel  the same for up to 4096 rows that the parallel variances decide, up to eight rows a thread: each cut
 //                      is a threshold found by bisection, one counting barrier a step, and nothing goes through
 //                      memory between the statistics and the metadata (64 to 512 rows 9 us -> 4).  Otherwise it leaves the
 //                      layer to assign_kernel's code.
 // The result is the definition's in every case.
+#include <type_traits>
 #include "common.cuh"
 
 namespace rmsmp {
@@ -70,7 +73,9 @@ __device__ __noinline__ double exact_variance(const float* __restrict__ w, int K
 // (s2 - s1^2 / K) / K.  With u = 2^-53 and q = s2 / K, any order of additions leaves |error| <= 4 (K + 8) u q
 // (|s1| sum|x| <= K s2), and the definition's own two passes are off by at most (K + 4) u var + 2 ((K + 1) u A)^2
 // with A = mean |w|, A^2 <= 2 (c^2 + q); G = 2 (K + 16) u below leaves a factor of more than two.
-// A row whose bound leaves the range of fp32 (weights of 1e25 and more) gets the definition's chain here.
+// A row whose bound says nothing -- it leaves the range of fp32 (weights of 1e25 and more), or is as large as the variance
+// (weights all the same: the definition's variance is rounding noise) -- gets the definition's chain here, where every SM
+// has rows to work on.
 __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(const float* __restrict__ W, int K, RowStats out)
 {
     pdl_wait();
@@ -117,7 +122,7 @@ __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(const float* __
         double v = fabs(fmax((s2 - s1 * s1 / (double)K) / (double)K, 0.0));
         float e = __double2float_ru(6.0 * G * q + 4.0 * G * G * (c * c + q));
         if (mx == 0.0f) { v = 0.0; e = 0.0f; }                     // an all-zero row's variance is exactly zero
-        if (!(e <= 3e38f)) { v = exact_variance(w, K); e = 0.0f; }
+        if (!(e <= 3e38f) || (e > 0.0f && (double)e >= v)) { v = exact_variance(w, K); e = 0.0f; }
         if (!(v <= 1e300)) { v = __longlong_as_double(0x7FF0000000000000ll); e = 0.0f; }     // not finite: last, by row index
         out.var[row] = v;
         out.err[row] = e;
@@ -167,17 +172,69 @@ __device__ __forceinline__ void block_reduce(T (&v)[N], Op op, T* s, T id)
     }
 }
 
+// Share `rank` of `ranks` of the listed rows' variances by the definition; neighbouring rows go to different blocks and warps.
+__device__ __forceinline__ void exact_variances(const MetaArgs& a, const int32_t* list, int n, int rank, int ranks)
+{
+    const int nt = blockDim.x, u = (threadIdx.x & 31) * (nt >> 5) + (threadIdx.x >> 5);
+    for (int i = u * ranks + rank; i < n; i += nt * ranks) {
+        const int r = list[i];
+        if (a.st.err[r] != 0.0f) a.st.var[r] = exact_variance(a.W + (size_t)r * a.K, a.K);
+    }
+}
+
+// assign_kernel is a cluster of kHelpers blocks, of which the first assigns.  The others sleep at the cluster's barrier until it
+// knows how many undecided rows need the definition's chain of additions, take their share and leave: copies of four rows,
+// 65,536 of 1024 weights 9.6 ms on one SM, 2.1 ms so; random weights no slower.  For up to 4096 rows there are no helpers:
+// the cluster costs random weights 1 us of 26 to 32, and copies of four rows take 118 to 745 us without them (226 with three).
+constexpr int kHelpers = 8;
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// What a block other than the first does.  s_rows: its own word, which the first block fills.
+__device__ __forceinline__ void help(const MetaArgs& a, int* s_rows)
+{
+    if (threadIdx.x == 0) *s_rows = 0;
+    cluster_arrive();                                     // (1) this block runs and its word is clear
+    cluster_wait();
+    cluster_arrive();                                     // (2) the first block knows the number of rows
+    cluster_wait();
+    const int n = *reinterpret_cast<volatile int*>(s_rows);
+    if (n > 0) {
+        exact_variances(a, reinterpret_cast<const int32_t*>(a.blob + a.off_slot), n, (int)blockIdx.x, kHelpers);
+        cluster_arrive();                                 // (3) this share is done
+    }
+}
+
+// The first block's side: n listed rows' variances.
+__device__ __forceinline__ void exact_variances_with_helpers(const MetaArgs& a, int* s_rows, const int32_t* list, int n)
+{
+    cluster_wait();                                       // (1)
+    if (n > 0 && threadIdx.x > 0 && threadIdx.x < kHelpers) {
+        uint32_t at;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(s_rows)), "r"(threadIdx.x));
+        asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(at), "r"(n) : "memory");
+    }
+    cluster_arrive();                                     // (2)
+    if (n == 0) return;
+    cluster_wait();
+    exact_variances(a, list, n, 0, kHelpers);
+    cluster_arrive();                                     // (3)
+    cluster_wait();
+}
+
 // One block: everything here is latency (a few barriers per step), so the statistics are copied to shared memory
 // first and the selection starts at the first bit in which the variances differ at all (their exponents mostly
 // agree): two or three digits for random weights instead of eight.
-__device__ __forceinline__ void assign_rows_block(const MetaArgs& a)
+// kBlocks: the blocks that share the chains of additions, s_rows the helpers' word (see help()).
+template <int kBlocks>
+__device__ __forceinline__ void assign_rows_block(const MetaArgs& a, int* s_rows)
 {
     __shared__ int s_hist[2][256];
     __shared__ unsigned long long s_prefix[2];
     __shared__ int s_left[2], s_same[2];
     __shared__ double s_dbl[4 * 32];
-    __shared__ unsigned long long s_u64[32];
-    __shared__ int s_int[2 * 32];
+    __shared__ unsigned long long s_u64[4 * 32];
+    __shared__ int s_int[4 * 32];
     __shared__ int s_undecided;
     __shared__ int s_warp[3][32];
     __shared__ int s_start[3][kAssignMaxBlocks + 1];      // rows of each kind in front of every 128-row block
@@ -195,71 +252,117 @@ __device__ __forceinline__ void assign_rows_block(const MetaArgs& a)
     bool need[2];
     for (int c = 0; c < 2; ++c) need[c] = cut[c] > 0 && cut[c] < M && (c == 0 || cut[1] != cut[0]);
 
-    // ---- the statistics, and the bits in which the keys differ (a non-negative double orders like its bits)
-    const unsigned long long key0 = (unsigned long long)__double_as_longlong(a.st.var[0]);
-    unsigned long long diff[1] = {0ull};
-    for (int r = t; r < M; r += nt) {
-        const double v = a.st.var[r];
-        if (local) { s_var[r] = v; s_err[r] = a.st.err[r]; }
-        diff[0] |= (unsigned long long)__double_as_longlong(v) ^ key0;
+    // ---- the statistics in shared memory
+    if (local) {
+        for (int r = t; r < M; r += nt) { s_var[r] = a.st.var[r]; s_err[r] = a.st.err[r]; }
     }
-    for (int i = t; i < 256; i += nt) { s_hist[0][i] = 0; s_hist[1][i] = 0; }
     if (t == 0) s_undecided = 0;
-    block_reduce<1>(diff, [](unsigned long long x, unsigned long long y) { return x | y; }, s_u64, 0ull);
-    int top = 64 - __clzll((long long)diff[0]);           // bits from `top` up are common to all keys
-    if (t < 2) { s_prefix[t] = top < 64 ? key0 & (~0ull << top) : 0ull; s_left[t] = cut[t]; s_same[t] = M; }
     __syncthreads();
 
-    // ---- the largest key in front of each cut, up to eight bits at a time
-    while (top > 0) {
-        const int shift = max(top - 8, 0);
-        const unsigned long long above = top < 64 ? ~0ull << top : 0ull;
-        const unsigned long long pre0 = s_prefix[0], pre1 = s_prefix[1];
-        const bool one = pre0 == pre1 && need[0] && need[1];       // both cuts still in the same bin: one histogram
+    // For each cut c with open[c]: the key of the want[c]-th of the rows that in(c, r) names (s_prefix), how many of the rows
+    // with that key are among those want[c] (s_left), and how many there are (s_same).  Radix selection, up to eight bits
+    // at a time, from the first bit in which the keys differ at all: two or three digits for random weights (their
+    // exponents mostly agree), none where all keys are the same.  (A non-negative double orders like its bits.)
+    // all_rows: in() is true everywhere; one histogram does for both cuts while they are in the same bin then.  Otherwise the rows
+    // are those at a cut, many of which tie: a warp counts the digit of the first of its rows in one addition (20,000 rows
+    // of random weights 7 % slower so, copies of four rows twice as fast).
+    auto select = [&](auto all_rows, auto in, const bool (&open)[2], const int (&want)[2]) {
+        constexpr bool kAll = decltype(all_rows)::value;
+        unsigned long long bits[4] = {0ull, 0ull, 0ull, 0ull};         // per cut: bits set in a key, bits clear in a key
         for (int r = t; r < M; r += nt) {
             const unsigned long long key = (unsigned long long)__double_as_longlong(var[r]);
-            const int d = (int)((key & ~above) >> shift);
-            if (need[0] && (key & above) == pre0) atomicAdd(&s_hist[0][d], 1);
-            if (need[1] && !one && (key & above) == pre1) atomicAdd(&s_hist[1][d], 1);
-        }
-        __syncthreads();
-        if (warp < 2 && need[warp]) {
-            // the digit in which the cut's last row lies: a warp scans the 256 counters, eight to a lane
-            const int* h = s_hist[one ? 0 : warp];
-            int n[8], sum = 0;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { n[j] = h[8 * lane + j]; sum += n[j]; }
-            int incl = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
-            int before = incl - sum;
-            const int left = s_left[warp];
-            __syncwarp();
-            if (before < left && left <= incl) {
-                int j = 0;
-                while (before + n[j] < left) before += n[j++];
-                s_left[warp] = left - before;
-                s_same[warp] = n[j];
-                s_prefix[warp] |= (unsigned long long)(8 * lane + j) << shift;
-            }
-        }
-        __syncthreads();
-        top = shift;
-        if (top > 0 && (!need[0] || s_same[0] == 1) && (!need[1] || s_same[1] == 1)) {
-            // one row left at each cut: its key is the rest of the digits
-            const unsigned long long known = ~0ull << shift, k0 = s_prefix[0], k1 = s_prefix[1];
-            __syncthreads();
-            for (int r = t; r < M; r += nt) {
-                const unsigned long long key = (unsigned long long)__double_as_longlong(var[r]);
-                if (need[0] && (key & known) == k0) s_prefix[0] = key;
-                if (need[1] && (key & known) == k1) s_prefix[1] = key;
-            }
-            __syncthreads();
-            break;
+            for (int c = 0; c < 2; ++c)
+                if (open[c] && in(c, r)) { bits[2 * c] |= key; bits[2 * c + 1] |= ~key; }
         }
         for (int i = t; i < 256; i += nt) { s_hist[0][i] = 0; s_hist[1][i] = 0; }
+        block_reduce<4>(bits, [](unsigned long long x, unsigned long long y) { return x | y; }, s_u64, 0ull);
+        int top = 64 - __clzll((long long)((bits[0] & bits[1]) | (bits[2] & bits[3])));      // bits from `top` up are common to a cut's keys
+        if (t < 2) {
+            s_prefix[t] = top < 64 ? (t == 0 ? bits[0] : bits[2]) & (~0ull << top) : 0ull;
+            s_left[t] = t == 0 ? want[0] : want[1];
+            s_same[t] = M;                                // (counted below)
+        }
         __syncthreads();
-    }
+        if (top == 0) {                                   // one key a cut
+            int n[2] = {0, 0};
+            for (int r = t; r < M; r += nt) { n[0] += open[0] && in(0, r); n[1] += open[1] && in(1, r); }
+            block_reduce<2>(n, [](int x, int y) { return x + y; }, s_int, 0);
+            if (t < 2) s_same[t] = t == 0 ? n[0] : n[1];
+            __syncthreads();
+        }
+        while (top > 0) {
+            const int shift = max(top - 8, 0);
+            const unsigned long long above = top < 64 ? ~0ull << top : 0ull;
+            const unsigned long long pre[2] = {s_prefix[0], s_prefix[1]};
+            const bool one = kAll && pre[0] == pre[1] && open[0] && open[1];
+            if (kAll) {
+                for (int r = t; r < M; r += nt) {
+                    const unsigned long long key = (unsigned long long)__double_as_longlong(var[r]);
+                    const int d = (int)((key & ~above) >> shift);
+                    if (open[0] && (key & above) == pre[0]) atomicAdd(&s_hist[0][d], 1);
+                    if (open[1] && !one && (key & above) == pre[1]) atomicAdd(&s_hist[1][d], 1);
+                }
+            }
+            for (int r0 = kAll ? M : t - lane; r0 < M; r0 += nt) {
+                const int r = r0 + lane;
+                const unsigned long long key = r < M ? (unsigned long long)__double_as_longlong(var[r]) : 0ull;
+                const int d = (int)((key & ~above) >> shift);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    if (!open[c]) continue;
+                    // (rows that tie share their digits: the first row's digit is counted once for the warp)
+                    const bool on = r < M && (key & above) == pre[c] && in(c, r);
+                    const unsigned m = __ballot_sync(0xffffffffu, on);
+                    if (m == 0u) continue;
+                    const int lead = __ffs((int)m) - 1, d0 = __shfl_sync(0xffffffffu, d, lead);
+                    const unsigned same = __ballot_sync(0xffffffffu, on && d == d0);
+                    if (lane == lead) atomicAdd(&s_hist[c][d0], __popc(same));
+                    else if (on && d != d0) atomicAdd(&s_hist[c][d], 1);
+                }
+            }
+            __syncthreads();
+            if (warp < 2 && (warp == 0 ? open[0] : open[1])) {
+                // the digit in which the cut's last row lies: a warp scans the 256 counters, eight to a lane
+                const int* h = s_hist[one ? 0 : warp];
+                int n[8], sum = 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) { n[j] = h[8 * lane + j]; sum += n[j]; }
+                int incl = sum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+                int before = incl - sum;
+                const int left = s_left[warp];
+                __syncwarp();
+                if (before < left && left <= incl) {
+                    int j = 0;
+                    while (before + n[j] < left) before += n[j++];
+                    s_left[warp] = left - before;
+                    s_same[warp] = n[j];
+                    s_prefix[warp] |= (unsigned long long)(8 * lane + j) << shift;
+                }
+            }
+            __syncthreads();
+            top = shift;
+            if (top > 0 && (!open[0] || s_same[0] == 1) && (!open[1] || s_same[1] == 1)) {
+                // one row left at each cut: its key is the rest of the digits
+                const unsigned long long known = ~0ull << shift, k0 = s_prefix[0], k1 = s_prefix[1];
+                __syncthreads();
+                for (int r = t; r < M; r += nt) {
+                    const unsigned long long key = (unsigned long long)__double_as_longlong(var[r]);
+                    if (open[0] && (key & known) == k0 && in(0, r)) s_prefix[0] = key;
+                    if (open[1] && (key & known) == k1 && in(1, r)) s_prefix[1] = key;
+                }
+                __syncthreads();
+                break;
+            }
+            for (int i = t; i < 256; i += nt) { s_hist[0][i] = 0; s_hist[1][i] = 0; }
+            __syncthreads();
+        }
+    };
+
+    // ---- the largest key in front of each cut
+    select(std::true_type{}, [](int, int) { return true; }, need, cut);
     if (cut[1] == cut[0] && t == 0) { s_prefix[1] = s_prefix[0]; s_left[1] = s_left[0]; s_same[1] = s_same[0]; }
     __syncthreads();
 
@@ -299,41 +402,68 @@ __device__ __forceinline__ void assign_rows_block(const MetaArgs& a)
     }
     __syncthreads();
     const int nu = s_undecided;
+    // Undecided rows by the exact key: in front of a cut are those below und_key and the first und_left (by row index) of
+    // those at it.
+    unsigned long long und_key[2] = {0ull, 0ull};
+    int und_left[2] = {0, 0}, und_n[2] = {0, 0};
+    if (kBlocks > 1) exact_variances_with_helpers(a, s_rows, slot, nu);
     if (nu > 0) {
-        block_reduce<2>(in_front, [](int x, int y) { return x + y; }, s_int, 0);
-        const int want0 = cut[0] - in_front[0], want1 = cut[1] - in_front[1];
-        for (int i = t; i < nu; i += nt) {
-            const int r = slot[i];
-            if (err[r] != 0.0f) { var[r] = exact_variance(a.W + (size_t)r * a.K, a.K); err[r] = 0.0f; }
+        if (kBlocks == 1) {
+            exact_variances(a, slot, nu, 0, 1);
+            __syncthreads();
         }
-        __syncthreads();
-        for (int i = t; i < nu; i += nt) {
-            const int r = slot[i];
-            const double v = var[r];
-            const int sides = kind[r];
-            int before0 = 0, before1 = 0;                 // undecided rows of the same cut that come first
-            for (int j = 0; j < nu; ++j) {
-                const int r2 = slot[j];
-                const double v2 = var[r2];
-                if (!(v2 < v || (v2 == v && r2 < r))) continue;
-                // (bits 4-7 keep a row's result apart from its sides, which other threads still read)
-                before0 += (kind[r2] & 3) == 2; before1 += ((kind[r2] >> 2) & 3) == 2;
-            }
-            int res = sides;
-            if ((sides & 3) == 2) res |= (before0 < want0 ? 0 : 1) << 4;
-            if (((sides >> 2) & 3) == 2) res |= (before1 < want1 ? 0 : 1) << 5;
-            kind[r] = (uint8_t)res;
+        if (local) {
+            for (int i = t; i < nu; i += nt) s_var[slot[i]] = __ldcg(a.st.var + slot[i]);
         }
-        __syncthreads();
+        auto undecided = [&](int c, int r) { return ((kind[r] >> (2 * c)) & 3) == 2; };
+        int n[4] = {in_front[0], in_front[1], 0, 0};
+        for (int i = t; i < nu; i += nt) { n[2] += undecided(0, slot[i]); n[3] += undecided(1, slot[i]); }
+        block_reduce<4>(n, [](int x, int y) { return x + y; }, s_int, 0);      // (and the exact variances are there)
+        const int want[2] = {cut[0] - n[0], cut[1] - n[1]};
+        const bool open[2] = {want[0] > 0 && want[0] < n[2], want[1] > 0 && want[1] < n[3]};
+        select(std::false_type{}, undecided, open, want);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            und_n[c] = n[2 + c];
+            und_key[c] = open[c] ? s_prefix[c] : (want[c] > 0 ? ~0ull : 0ull);
+            und_left[c] = open[c] ? s_left[c] : 0;
+        }
     }
+    // the side of an undecided row; `at` counts the rows at a cut's key as they come
+    auto decide = [&](int c, int s, int r, int (&at)[2]) -> int {
+        if (s != 2) return s;
+        const unsigned long long key = (unsigned long long)__double_as_longlong(var[r]);
+        if (key != und_key[c]) return key < und_key[c] ? 0 : 1;
+        return at[c]++ < und_left[c] ? 0 : 1;
+    };
 
     // ---- stable grouping: consecutive rows per thread, prefix sums over the threads
     const int per = (M + nt - 1) / nt;
     const int r0 = min(M, t * per), r1 = min(M, r0 + per);
+    int at[2] = {0, 0};                                   // undecided rows at each cut's key in front of this thread's
+    if (nu > 0) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            if (und_n[c] == 0) continue;                  // (the same for every thread)
+            int n = 0;
+            for (int r = r0; r < r1; ++r)
+                n += ((kind[r] >> (2 * c)) & 3) == 2 && (unsigned long long)__double_as_longlong(var[r]) == und_key[c];
+            int incl = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+            if (lane == 31) s_warp[c][warp] = incl;
+            __syncthreads();
+            int before = lane < warp ? s_warp[c][lane] : 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+            at[c] = before + incl - n;
+        }
+        __syncthreads();
+    }
     int cnt[3] = {0, 0, 0};
     for (int r = r0; r < r1; ++r) {
         const int s = kind[r];
-        const int s0 = (s & 3) == 2 ? (s >> 4) & 1 : s & 3, s1 = ((s >> 2) & 3) == 2 ? (s >> 5) & 1 : (s >> 2) & 3;
+        const int s0 = decide(0, s & 3, r, at), s1 = decide(1, (s >> 2) & 3, r, at);
         const int k = s0 == 0 ? kPoT4 : (s1 == 0 ? kFixed4 : kFixed8);
         kind[r] = (uint8_t)k;
         cnt[0] += k == 0; cnt[1] += k == 1; cnt[2] += k == 2;
@@ -393,9 +523,12 @@ __device__ __forceinline__ void assign_rows_block(const MetaArgs& a)
 
 __global__ void __launch_bounds__(kAssignThreads, 1) assign_kernel(MetaArgs a)
 {
+    __shared__ int s_rows;
     pdl_wait();
     pdl_trigger();
-    assign_rows_block(a);
+    if (blockIdx.x > 0) { help(a, &s_rows); return; }
+    cluster_arrive();                                     // (1)
+    assign_rows_block<kHelpers>(a, &s_rows);
 }
 
 // Up to kSmallThreads * R rows, R of them per thread (row i * threads + t); 128 threads or more, so that the other form can take over.
@@ -498,7 +631,7 @@ __global__ void __launch_bounds__(kSmallThreads) assign_small_kernel(MetaArgs a)
     const bool clear0 = cut[0] <= 0 || cut[0] >= M || (found[0] && edge[0] < ~edge[1]);
     const bool clear1 = cut[1] <= 0 || cut[1] >= M || (found[1] && edge[2] < ~edge[3]);
     if (!clear0 || !clear1) {
-        assign_rows_block(a);
+        assign_rows_block<1>(a, nullptr);
         return;
     }
 
@@ -588,7 +721,7 @@ cudaError_t launch_assign_meta(const float* dW, const rmsmp_layer& L, const floa
     a.M = M; a.Cin = L.Cin; a.kh = L.kh; a.kw = L.kw; a.Cp = L.Cp; a.Kp = L.Kp;
     a.nP = L.nP; a.nF4 = L.nF4; a.n8 = L.n8; a.nblocks = L.nblocks; a.pot_mode = pot_mode;
     // few warps: cheap barriers, and a block that finds room on an SM while the statistics still run
-    if (M > 8 * kSmallThreads) return launch_dependent(assign_kernel, 1, kAssignThreads, 0, st, a);
+    if (M > 8 * kSmallThreads) return launch_dependent_cluster(assign_kernel, kHelpers, kHelpers, kAssignThreads, 0, st, a);
     if (M > 2 * kSmallThreads) return launch_dependent(assign_small_kernel<8>, 1, kSmallThreads, 0, st, a);
     if (M > kSmallThreads) return launch_dependent(assign_small_kernel<2>, 1, kSmallThreads, 0, st, a);
     return launch_dependent(assign_small_kernel<1>, 1, (unsigned)(M <= 128 ? 128 : (M + 31) / 32 * 32), 0, st, a);

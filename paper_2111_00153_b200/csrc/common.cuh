@@ -93,6 +93,21 @@ inline cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigne
     return cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
 }
 
+// The same in clusters of `cluster` blocks.
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent_cluster(void (*kernel)(P...), unsigned cluster, unsigned grid, unsigned block, size_t smem, cudaStream_t st, const A&... args)
+{
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(grid); lc.blockDim = dim3(block); lc.dynamicSmemBytes = smem; lc.stream = st;
+    lc.attrs = at; lc.numAttrs = 2;
+    return cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
+}
+
 // Re-quantizing epilogue request (rmsmp_*_workspace_requant): the next layer's clip value, kind and code buffer.
 struct Requant {
     float alpha;

@@ -747,7 +747,8 @@ def _rows_at_the_cuts(name, g, M, K):
 @pytest.mark.parametrize("name", ["normal", "copies", "all_equal", "constant", "zero_rows", "offset", "permuted", "huge", "tiny"])
 @pytest.mark.parametrize("M,K,ratio", [(1, 5, (60, 35, 5)), (33, 31, (60, 35, 5)), (257, 100, (50, 40, 10)),
                                        (1024, 36, (60, 35, 5)), (1100, 36, (60, 35, 5)), (2500, 64, (65, 30, 5)),
-                                       (4100, 20, (60, 35, 5)), (300, 64, (95, 0, 5)), (128, 16, (0, 100, 0))])
+                                       (4100, 20, (60, 35, 5)), (300, 64, (95, 0, 5)), (128, 16, (0, 100, 0)),
+                                       (2500, 27, (0, 40, 60)), (20000, 12, (60, 35, 5))])
 def test_assignment_at_the_cuts_of_the_ranking(M, K, ratio, name):
     """Whole-number result (which row gets which scheme), so no tolerance: it is the oracle's for rows whose
     variances tie, or differ by less than the summation error, at a cut; fewer and more rows than threads, and more
@@ -769,6 +770,30 @@ def test_assignment_at_the_cuts_of_the_ranking(M, K, ratio, name):
     for off, n in ((0, 68), (layer.off_perm, 4 * M), (layer.off_slot, 4 * M), (layer.off_wstep, 4 * M), (layer.off_alpha, 4 * M),
                    (layer.off_kind, M), (layer.off_blocks, 32 * layer.nblocks)):
         assert torch.equal(d_packed[off:off + n], ref[off:off + n])
+
+
+@pytest.mark.parametrize("name", ["copies", "constant", "zero_rows"])
+def test_assignment_of_many_tied_rows_takes_no_quadratic_time(name):
+    """20,000 rows of which most tie at a cut: within fifteen times what rows take that do not (100 us against 15 to
+    32 ms when every tied row was compared with every other)."""
+    import torch
+    M, K, ratio = 20000, 64, (60, 35, 5)
+    layer = R.rmsmp_layer_init_ratio(M, K, 1, 1, ratio)
+    d_packed = torch.empty(layer.packed_bytes, dtype=torch.uint8, device="cuda")
+    scratch = torch.empty(R.rmsmp_assign_scratch_bytes(M), dtype=torch.uint8, device="cuda")
+    times = {}
+    for which in ("normal", name):
+        d_W = torch.from_numpy(_rows_at_the_cuts(which, synth.rng(90, M), M, K)).cuda()
+        runs = []
+        for _ in range(4):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            R.rmsmp_assign_quantize_pack(d_W, R.W_LINEAR, layer, ratio, None, R.POT_NEAREST, d_packed, scratch)
+            end.record()
+            torch.cuda.synchronize()
+            runs.append(start.elapsed_time(end))
+        times[which] = min(runs)
+    assert times[name] <= 15.0 * times["normal"], times
 
 
 # ------------------------------------------------------------------ depthwise convolution
