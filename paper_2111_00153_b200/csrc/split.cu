@@ -495,8 +495,9 @@ bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr, bool gat
             // two of its own k-blocks, and a stage's barrier tells only neighbouring phases apart
             if (c.nst < 3 && c.nst < kpc) continue;
             c.smem_bytes = (uint32_t)std::max(c.nst * (c.a_bytes + c.b_bytes) + red, (kSplitThreads / 32 - kSplitFirst) * 1024) + 1024;
-            // clusters of eight do not tile the SMs of every processing cluster: count 5 % fewer for each doubling
-            const double usable = (double)sms * (S == 1 ? 1.0 : S == 2 ? 0.97 : S == 4 ? 0.92 : 0.85);
+            // clusters do not tile the SMs of every processing cluster (of 148, 128 CTAs in clusters of four are placed at once but
+            // not 136 -- 3x3 48x368 on 17 images of 15x11 17.6 us so, 11.0 in pairs --, 112 in clusters of eight but not 128)
+            const double usable = (double)sms * (S == 1 ? 1.0 : S == 2 ? 0.97 : S == 4 ? 0.9 : 0.85);
             const double waves = std::max(1.0, std::ceil((double)ctas / usable));
             const double load = (c.pre ? kBlockRows + c.npix : c.npix) * 2.56, expand = c.pre ? 0.0 : (c.gather ? 900.0 : 420.0) * c.bk / 128.0;
             const double kblock = std::max(std::max(load, expand), 90.0 * (c.bk / 32));
@@ -533,8 +534,10 @@ bool split_supported(const Problem& p)
     double other;
     if (p.wexp || tensor_resident(p)) {
         if (tiles >= sms) return false;
-        const double n = (double)std::min<int64_t>(p.N, 256);
+        const int64_t hw = (int64_t)p.Ho * p.Wo;          // (its tiles are whole images: 3x3 256x256 on 32 of 14x14 11.7 us there, 12.5 here)
+        const double n = (double)std::min<int64_t>(p.N, hw <= 256 && !bk64 ? 256 / hw * hw : 256);
         other = 3.4 + 1.2 * n / 256 + nkb * (0.28 + 0.13 * n / 256) + (p.wexp ? 0.0 : 1.7 + 0.7 * nkb);
+        if (p.out_mn && p.N < 32) other += 1.4;           // (no bulk stores: 64x64 N=8 5.2 us there, 3.3 here)
     } else {
         other = 7.4 + std::ceil(tiles / sms) * (0.8 + 0.59 * nkb);
     }

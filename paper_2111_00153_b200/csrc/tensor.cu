@@ -930,7 +930,8 @@ bool plan(const Problem& p, TensorCfg& c)
         // Narrower tiles where the widest ones leave SMs idle in the last round: a k-block takes 0.28 us + 0.13 per 256
         // pixels, the output of 256 pixels 0.8 beside the next tile's k-blocks and 1.2 at the end (768x768 N=4096: 96 tiles
         // of 256 tokens, or 144 of 176: 7.7 against 7.2 us); not for gains
-        // below a tenth, which measure as losses as often.
+        // below a tenth, which measure as losses as often.  [row][pixel] outputs keep to whole chunks of 32 pixels, without
+        // which they leave through direct stores (256x64 N=20000 16.5 us with tiles of 144 pixels).
         if (p.wexp) {
             const int64_t sms = sm_count();
             const double nkb = (double)p.kh * p.kw * ((p.Cin + 127) / 128);
@@ -940,8 +941,9 @@ bool plan(const Problem& p, TensorCfg& c)
             };
             double best = 0.9 * cost(c.tb);
             const int most = c.tb, step = hw == 1 ? 16 : 1;
+            const bool whole = p.out_mn && p.ld_out % 4 == 0 && p.N % 4 == 0 && most * hw % 32 == 0;
             for (int tb = (most - 1) / step * step; tb >= 1 && 2 * tb >= most; tb -= step)
-                if (cost(tb) < best) { best = cost(tb); c.tb = tb; }
+                if (!(whole && tb * hw % 32 != 0) && cost(tb) < best) { best = cost(tb); c.tb = tb; }
         }
         c.tiles_per_image = 0;
         c.ntiles_n = (p.B + c.tb - 1) / c.tb;

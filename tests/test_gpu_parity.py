@@ -679,6 +679,64 @@ def test_convolutions_of_any_channel_count_under_auto(M, Cin, k, stride, pad, B,
             assert np.array_equal(np.ascontiguousarray(y).view(np.uint32), y_ref.reshape(-1, M).view(np.uint32))
 
 
+# ------------------------------------------------------------------ choice of tiles and kernels: neighbours cost about the same
+
+def _call_us(M, Cin, k, pad, B, H, W, layout):
+    """GPU time of one call on a workspace (a linear layer where k is 0: B tokens), and its exact sums' check."""
+    import torch
+    g = synth.rng(91, M + Cin + B)
+    kk = max(k, 1)
+    Wt = synth.weights_kaiming(g, M, Cin, kk, kk)
+    scheme, bits = _mixed_map(M, 9)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, synth.alpha_rows(Wt))
+    ws = Hn._workspace(layer, d_packed)
+    N = B if k == 0 else B * (H + 2 * pad - k + 1) * (W + 2 * pad - k + 1)
+    act = torch.randint(0, 16, (B, H, W, Cin) if k else (N, Cin), dtype=torch.int8, device="cuda")
+    y = torch.empty((N, M) if layout == R.OUT_NM else (M, N), dtype=torch.float32, device="cuda")
+
+    def call():
+        if k:
+            R.rmsmp_conv_implicit_workspace(layer, d_packed, ws, act, B, H, W, 1, pad, 0.5, y, layout)
+        else:
+            R.rmsmp_gemm_workspace(layer, d_packed, ws, act, N, Cin, 0.5, y, y.shape[1], layout)
+
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        call()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            for _ in range(10):
+                call()
+        runs = []
+        for _ in range(8):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record(stream)
+            graph.replay()
+            end.record(stream)
+            torch.cuda.synchronize()
+            runs.append(100.0 * start.elapsed_time(end))
+    assert R.rmsmp_last_device_status(d_packed) == R.OK
+    # the call against the kernel that shares no code with it
+    ref = torch.empty_like(y)
+    if k:
+        R.rmsmp_conv_implicit_variant(layer, d_packed, act, B, H, W, 1, pad, 0.5, ref, layout, None, R.VARIANT_SIMPLE)
+    else:
+        R.rmsmp_gemm_variant(layer, d_packed, act, N, Cin, 0.5, ref, ref.shape[1], layout, None, R.VARIANT_SIMPLE)
+    assert torch.equal(y.view(torch.int32), ref.view(torch.int32))
+    return min(runs)
+
+
+@pytest.mark.parametrize("call,other,bound", [
+    # 256 rows, 20,000 tokens as [M][N] against [N][M]: 7.6 us and 6.8; tiles no multiple of 32 tokens 16.5
+    ((256, 64, 0, 0, 20000, 1, 1, R.OUT_MN), (256, 64, 0, 0, 20000, 1, 1, R.OUT_NM), 1.7),
+])
+def test_neighbouring_problems_cost_about_the_same(call, other, bound):
+    """(M, Cin, k, pad, B, H, W, layout): a rule that picks tiles or a kernel badly for one of two like problems shows in their
+    times.  Each bound lies halfway between what the rule gives and what it gave when it was wrong (in the comments)."""
+    assert _call_us(*call) <= bound * _call_us(*other)
+
+
 # ------------------------------------------------------------------ row assignment on the device
 
 @pytest.mark.parametrize("ratio", [(60, 35, 5), (65, 30, 5), (0, 100, 0), (50, 40, 10)], ids=lambda r: "%d-%d-%d" % r)
