@@ -930,14 +930,16 @@ bool plan(const Problem& p, TensorCfg& c)
         // Narrower tiles where the widest ones leave SMs idle in the last round: a k-block takes 0.28 us + 0.13 per 256
         // pixels, the output of 256 pixels 0.8 beside the next tile's k-blocks and 1.2 at the end (768x768 N=4096: 96 tiles
         // of 256 tokens, or 144 of 176: 7.7 against 7.2 us); not for gains
-        // below a tenth, which measure as losses as often.  [row][pixel] outputs keep to whole chunks of 32 pixels, without
+        // below a tenth, which measure as losses as often, nor where reading the activations takes as long (10x4096 N=20000:
+        // 24.1 us with 256 tokens a tile, 28.3 with 144).  [row][pixel] outputs keep to whole chunks of 32 pixels, without
         // which they leave through direct stores (256x64 N=20000 16.5 us with tiles of 144 pixels).
         if (p.wexp) {
             const int64_t sms = sm_count();
             const double nkb = (double)p.kh * p.kw * ((p.Cin + 127) / 128);
+            const double read = (double)p.N * p.Cin / 6.3e6;
             auto cost = [&](int tb) {
                 const double n = (double)tb * hw / 256.0, waves = (double)((((int64_t)p.B + tb - 1) / tb * p.nblocks + sms - 1) / sms);
-                return waves * std::max(nkb * (0.28 + 0.13 * n), 0.4 + 0.8 * n) + 1.2 * n;
+                return std::max(waves * std::max(nkb * (0.28 + 0.13 * n), 0.4 + 0.8 * n) + 1.2 * n, read);
             };
             double best = 0.9 * cost(c.tb);
             const int most = c.tb, step = hw == 1 ? 16 : 1;

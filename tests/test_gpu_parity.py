@@ -730,6 +730,8 @@ def _call_us(M, Cin, k, pad, B, H, W, layout):
 @pytest.mark.parametrize("call,other,bound", [
     # 256 rows, 20,000 tokens as [M][N] against [N][M]: 7.6 us and 6.8; tiles no multiple of 32 tokens 16.5
     ((256, 64, 0, 0, 20000, 1, 1, R.OUT_MN), (256, 64, 0, 0, 20000, 1, 1, R.OUT_NM), 1.7),
+    # ten rows against 64: 24 us and 17; 28 with narrow tiles
+    ((10, 4096, 0, 0, 20000, 1, 1, R.OUT_NM), (64, 4096, 0, 0, 20000, 1, 1, R.OUT_NM), 1.56),
 ])
 def test_neighbouring_problems_cost_about_the_same(call, other, bound):
     """(M, Cin, k, pad, B, H, W, layout): a rule that picks tiles or a kernel badly for one of two like problems shows in their
