@@ -955,7 +955,23 @@ bool plan(const Problem& p, TensorCfg& c)
         // 29x29 454 against 81.)
         const int most = std::min(kTileN / p.Wo, 256 / p.stride);
         c.tiles_per_image = (p.Ho + most - 1) / most;
+        // Lower tiles where the tallest leave SMs idle (few images): a k-block takes 0.25 us (128-byte rows 0.33) + 0.04 per 256
+        // pixels + 0.1 with every SM busy, the output of 256 pixels 1.7.  3x3 64x32 on 2 of 49x49, tiles of five rows 8.3 us,
+        // of one 6.0.  Not for a few rows, whose boxes of weights lie mostly outside the matrix and then take longer than the
+        // activations' (3x3 16x16 on 12 of 62x8 6.6 and 9.9).
+        if (p.wexp && p.M > 32) {
+            const double sms = sm_count(), bk = p.Cin % 128 != 0 && p.Cin % 128 <= 64 ? 64 : 128;
+            const double nkb = p.kh * p.kw * std::ceil(p.Cin / bk);
+            auto cost = [&](int per_image) {
+                const double n = (double)((p.Ho + per_image - 1) / per_image * p.Wo) / 256.0;
+                return 3.8 + 1.7 * n + nkb * ((bk == 64 ? 0.25 : 0.33) + 0.04 * n + 0.1 * ((double)p.B * per_image * p.nblocks / sms));
+            };
+            double best = 0.9 * cost(c.tiles_per_image);
+            for (int per_image = c.tiles_per_image + 1; per_image <= p.Ho && (double)p.B * per_image * p.nblocks <= sms; ++per_image)
+                if (cost(per_image) < best) { best = cost(per_image); c.tiles_per_image = per_image; }
+        }
         c.th = (p.Ho + c.tiles_per_image - 1) / c.tiles_per_image;
+        c.tiles_per_image = (p.Ho + c.th - 1) / c.th;
         c.tb = 1;
         c.ntiles_n = (int64_t)p.B * c.tiles_per_image;
     }

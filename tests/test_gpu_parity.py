@@ -732,6 +732,8 @@ def _call_us(M, Cin, k, pad, B, H, W, layout):
     ((256, 64, 0, 0, 20000, 1, 1, R.OUT_MN), (256, 64, 0, 0, 20000, 1, 1, R.OUT_NM), 1.7),
     # ten rows against 64: 24 us and 17; 28 with narrow tiles
     ((10, 4096, 0, 0, 20000, 1, 1, R.OUT_NM), (64, 4096, 0, 0, 20000, 1, 1, R.OUT_NM), 1.56),
+    # two images of 49 x 49 against eight: 6.0 us and 8.3; 8.3 with tiles of five rows
+    ((64, 32, 3, 1, 2, 49, 49, R.OUT_NM), (64, 32, 3, 1, 8, 49, 49, R.OUT_NM), 0.87),
 ])
 def test_neighbouring_problems_cost_about_the_same(call, other, bound):
     """(M, Cin, k, pad, B, H, W, layout): a rule that picks tiles or a kernel badly for one of two like problems shows in their
