@@ -1096,15 +1096,24 @@ bool encode_act_maps_4(const Problem& p, int bk, int th, int tb, void* maps4)
 // 2048x512 N=4096 20.9 against 13.8).  With one, the weights of several row blocks are a stream that the activations of a
 // first tile would wait behind (1024x512 N=4096, a tile per CTA: 8.1 us resident, 7.3 through the rings), and save
 // shared-memory fills from two tiles per CTA up (144x32 on 200,704 pixels 39.7 against 36.1, 3x3 256x64 on 50,176 20.7
-// against 17.7).
+// against 17.7).  Beside 64 KB of them fewer than four activation stages of 128-byte rows are left, too few for a linear layer
+// with fp32 outputs (192x512 on 200,000 tokens 56.3 us against 46.1, 512x512 on 50,176 28.6 against 26.3, 1024x512 on 20,000
+// 23.2 against 21.5; codes out 37.0 against 38.1, 21.0 against 21.9, 19.1 against 19.6).
 bool tensor_resident(const Problem& p)
 {
     if (!p.wexp && p.rq_codes) return false;
     const int64_t sms = sm_count(), tiles = (p.N + kTileN - 1) / kTileN * p.nblocks, whole = sms / p.nblocks * p.nblocks;
-    if (p.nblocks > kResidentBlocks && (whole == 0 || (tiles + whole - 1) / whole > (tiles + sms - 1) / sms)) return false;
+    if (whole == 0 || (p.nblocks > kResidentBlocks && (tiles + whole - 1) / whole > (tiles + sms - 1) / sms)) return false;
     const int bk = ((p.Cin % 128 != 0) && (p.Cin % 128 <= 64)) ? 64 : 128;
-    if ((int64_t)p.kh * p.kw * ((p.Cin + bk - 1) / bk) * kBlockRows * bk > 72 * 1024) return false;
-    return !p.wexp || p.nblocks == 1 || tiles >= 2 * sms;
+    const int64_t bytes = (int64_t)p.kh * p.kw * ((p.Cin + bk - 1) / bk) * kBlockRows * bk;
+    if (bytes > 72 * 1024) return false;
+    if (!p.wexp || p.nblocks == 1) return true;
+    if (tiles < 2 * sms) return false;
+    if (p.rq_codes) return true;
+    // (two rounds of full tiles against three: 1872x160 on 4880 tokens, 20 tiles for the nine CTAs of a block, 14.4 us
+    // resident, 11.7 through the rings)
+    if ((p.N / kTileN * p.nblocks + sms - 1) / sms <= 2 && (tiles + whole - 1) / whole > 2) return false;
+    return p.kh * p.kw > 1 || bk == 64 || bytes < 64 * 1024;
 }
 
 bool tensor_supported(const Problem& p)

@@ -734,6 +734,10 @@ def _call_us(M, Cin, k, pad, B, H, W, layout):
     ((10, 4096, 0, 0, 20000, 1, 1, R.OUT_NM), (64, 4096, 0, 0, 20000, 1, 1, R.OUT_NM), 1.56),
     # two images of 49 x 49 against eight: 6.0 us and 8.3; 8.3 with tiles of five rows
     ((64, 32, 3, 1, 2, 49, 49, R.OUT_NM), (64, 32, 3, 1, 8, 49, 49, R.OUT_NM), 0.87),
+    # 192 rows against 256: 46 us and 53; 56 with resident weights
+    ((192, 512, 0, 0, 200000, 1, 1, R.OUT_NM), (256, 512, 0, 0, 200000, 1, 1, R.OUT_NM), 0.97),
+    # 4880 tokens against 4864 and 1872 rows against 1920: 11.7 us and 10.2; 14.4 with three rounds of tiles
+    ((1872, 160, 0, 0, 4880, 1, 1, R.OUT_MN), (1920, 160, 0, 0, 4864, 1, 1, R.OUT_MN), 1.28),
 ])
 def test_neighbouring_problems_cost_about_the_same(call, other, bound):
     """(M, Cin, k, pad, B, H, W, layout): a rule that picks tiles or a kernel badly for one of two like problems shows in their
