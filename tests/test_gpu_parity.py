@@ -738,6 +738,10 @@ def _call_us(M, Cin, k, pad, B, H, W, layout):
     ((192, 512, 0, 0, 200000, 1, 1, R.OUT_NM), (256, 512, 0, 0, 200000, 1, 1, R.OUT_NM), 0.97),
     # 4880 tokens against 4864 and 1872 rows against 1920: 11.7 us and 10.2; 14.4 with three rounds of tiles
     ((1872, 160, 0, 0, 4880, 1, 1, R.OUT_MN), (1920, 160, 0, 0, 4864, 1, 1, R.OUT_MN), 1.28),
+    # 17 images against 16: 10.9 us and 10; 17.6 with more clusters than the chip places at once
+    ((48, 368, 3, 1, 17, 15, 11, R.OUT_NM), (48, 368, 3, 1, 16, 15, 11, R.OUT_NM), 1.35),
+    # eight tokens as [M][N] against [N][M]: 3.3 us and 3.9; 5.5 on the persistent kernel
+    ((64, 64, 0, 0, 8, 1, 1, R.OUT_MN), (64, 64, 0, 0, 8, 1, 1, R.OUT_NM), 1.15),
 ])
 def test_neighbouring_problems_cost_about_the_same(call, other, bound):
     """(M, Cin, k, pad, B, H, W, layout): a rule that picks tiles or a kernel badly for one of two like problems shows in their
