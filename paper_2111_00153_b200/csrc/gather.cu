@@ -14,6 +14,7 @@ namespace rmsmp {
 namespace {
 
 constexpr int kGatherThreads = 256;
+constexpr size_t kRowsSmem = 100 * 1024;                  // im2col_rows_kernel's most
 
 struct GatherArgs {
     const int8_t* act;
@@ -77,11 +78,14 @@ __global__ void __launch_bounds__(kGatherThreads) im2col_kernel(const GatherArgs
 struct RowsArgs {
     int zero_left, rowb;      // bytes of zeros in front of a staged row (a multiple of 16, at least 16 + pad * C), bytes per staged row
     int tile;                 // pixels assembled at a time
+    int wide;                 // padded pixels: bytes per copy into shared memory (16, 4 or 1), 0: a word a pixel
 };
 // One run's share of a unit (sixteen columns): which input row, the byte that would be the unit's column 0 relative to
 // the pixel's first byte in that row, and the columns that are this run's.
 struct alignas(32) Piece { uint32_t keep[4]; int row, off, last, pad; };      // last: 1 on a unit's last piece
 
+// kDense: pixels follow one another without padding bytes.
+template <bool kDense>
 __global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(const GatherArgs a, const RowsArgs ra)
 {
     extern __shared__ __align__(32) uint8_t s_mem[];
@@ -94,7 +98,6 @@ __global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(const Gathe
     const int run = a.kw * a.C;
     const int row_bytes = a.W * a.C;                                       // a staged row's own bytes
     const int chunks = ra.rowb >> 4;
-    const bool dense = a.pix_pitch == a.C;
     const int rows_total = a.B * a.Ho;
     if (tid < a.units) {
         // a unit's pieces; in front of it lie as many pieces as whole units, and one more for every run that ended inside one
@@ -113,13 +116,18 @@ __global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(const Gathe
             s_piece[n].last = (e == 16 || i + 1 == a.kh) ? 1 : 0;
         }
     }
+    if (!kDense) {
+        // padded pixels are copied one by one to the same place of every row: the zeros around them are written once
+        for (int q = tid; q < a.kh * chunks; q += kGatherThreads) *reinterpret_cast<uint4*>(s_rows + 16 * q) = make_uint4(0u, 0u, 0u, 0u);
+        if (tid < a.kh) s_base[tid] = tid * ra.rowb + ra.zero_left - a.pad * a.C;
+    }
     pdl_wait();
     pdl_trigger();
     for (int r = blockIdx.x; r < rows_total; r += gridDim.x) {
         const int b = r / a.Ho, ho = r - b * a.Ho;
         const int y0 = ho * a.stride - a.pad;
         __syncthreads();                                                   // the previous row's readers are done
-        if (dense) {
+        if constexpr (kDense) {
             // rows of packed pixels: 16-byte granules of global memory to the same place inside a granule of shared memory
             for (int q = tid; q < a.kh * chunks; q += kGatherThreads) {
                 const int i = q / chunks, j = q - i * chunks;
@@ -143,16 +151,49 @@ __global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(const Gathe
                 if (j == 0) s_base[i] = i * ra.rowb + ra.zero_left + lead - a.pad * a.C;
             }
         } else {
-            for (int q = tid; q < a.kh * ra.rowb; q += kGatherThreads) {
-                const int i = q / ra.rowb, at = q - i * ra.rowb - ra.zero_left;
+            const int pixels = a.kh * a.W;
+            auto source = [&](int q, int& i, int& x) -> const int8_t* {        // pixel q of the kh rows; null outside the image
+                i = q / a.W; x = q - i * a.W;
                 const int y = y0 + i;
-                uint8_t v = 0;
-                if ((unsigned)y < (unsigned)a.H && (unsigned)at < (unsigned)row_bytes) {
-                    const int x = at / a.C;
-                    v = (uint8_t)__ldg(a.act + ((int64_t)(b * a.H + y) * a.W + x) * a.pix_pitch + (at - x * a.C));
+                return (unsigned)y < (unsigned)a.H ? a.act + ((int64_t)(b * a.H + y) * a.W + x) * a.pix_pitch : nullptr;
+            };
+            if (ra.wide == 0) {
+                // up to four channels in pixels of whole words: eight words on their way at a time.  (The tensor's last
+                // pixel byte by byte: what lies behind its channels need not be there.)
+                const int8_t* last = a.act + ((int64_t)a.B * a.H * a.W - 1) * a.pix_pitch;
+                for (int q0 = tid; q0 < pixels; q0 += 8 * kGatherThreads) {
+                    uint32_t w[8];
+                    uint8_t* dst[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int q = q0 + u * kGatherThreads;
+                        int i = 0, x = 0;
+                        const int8_t* src = q < pixels ? source(q, i, x) : nullptr;
+                        dst[u] = s_rows + i * ra.rowb + ra.zero_left + x * a.C;
+                        w[u] = 0u;
+                        if (src != nullptr && src != last) w[u] = __ldg(reinterpret_cast<const uint32_t*>(src));
+                        else if (src != nullptr) for (int c = 0; c < a.C; ++c) w[u] |= (uint32_t)(uint8_t)__ldg(src + c) << (8 * c);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (q0 + u * kGatherThreads < pixels)
+                            for (int c = 0; c < a.C; ++c) dst[u][c] = (uint8_t)(w[u] >> (8 * c));
                 }
-                s_rows[q] = v;
-                if (at == -ra.zero_left) s_base[i] = i * ra.rowb + ra.zero_left - a.pad * a.C;
+            } else {
+                for (int q = tid; q < pixels; q += kGatherThreads) {
+                    int i, x;
+                    const int8_t* src = source(q, i, x);
+                    uint8_t* dst = s_rows + i * ra.rowb + ra.zero_left + x * a.C;
+                    if (ra.wide == 16) {
+                        for (int c = 0; c < a.C; c += 16)
+                            *reinterpret_cast<uint4*>(dst + c) = src ? __ldg(reinterpret_cast<const uint4*>(src + c)) : make_uint4(0u, 0u, 0u, 0u);
+                    } else if (ra.wide == 4) {
+                        for (int c = 0; c < a.C; c += 4)
+                            *reinterpret_cast<uint32_t*>(dst + c) = src ? __ldg(reinterpret_cast<const uint32_t*>(src + c)) : 0u;
+                    } else {
+                        for (int c = 0; c < a.C; ++c) dst[c] = src ? (uint8_t)__ldg(src + c) : (uint8_t)0;
+                    }
+                }
             }
         }
         for (int p0 = 0; p0 < a.Wo; p0 += ra.tile) {
@@ -208,7 +249,7 @@ cudaError_t launch_im2col(const int8_t* act, int B, int H, int W, int C, int64_t
     a.units = (int)(ld_cols >> 4);
     if (a.N == 0) return cudaSuccess;
     if (a.units > kGatherThreads) return cudaErrorInvalidValue;
-    // input rows in shared memory when they fit without opting in to more, beside the tile that is assembled
+    // input rows in shared memory when they fit, beside the tile that is assembled
     RowsArgs ra;
     auto up16 = [](int n) { return (n + 15) & ~15; };
     ra.zero_left = up16(pad * C) + 16;
@@ -216,10 +257,21 @@ cudaError_t launch_im2col(const int8_t* act, int B, int H, int W, int C, int64_t
     ra.tile = (int)std::min<int64_t>(Wo, std::max<int64_t>(1, 20 * 1024 / ld_cols));
     if (ra.tile < Wo && ra.tile >= 32) ra.tile &= ~31;
     const size_t smem = ((size_t)ra.tile * ld_cols + (size_t)kh * ra.rowb + 31) / 32 * 32 + 32 + sizeof(Piece) * (size_t)(a.units + kh);
-    if (smem <= 46 * 1024) {
+    auto whole = [&](int w) { return pix_pitch % w == 0 && (reinterpret_cast<uintptr_t>(act) & (w - 1)) == 0; };
+    ra.wide = C <= 4 && whole(4) ? 0 : C % 16 == 0 && whole(16) ? 16 : C % 4 == 0 && whole(4) ? 4 : 1;
+    // Rows too wide for the shared memory that needs no opting in (7 x 7 x 3 from about 1000 pixels): fewer blocks share an SM, which
+    // is worth it for few channels and rows enough (7 x 7, two images of 1080 x 1920 x 3 237 us by the other kernel, 74 so, and 130
+    // with a fourth byte a pixel; 3 x 3, two of 224 x 224 x 64 47 and 71; 32 rows of 2000 x 3 10.7 and 18.8).
+    static bool attr_set[2][kMaxDevices] = {};
+    const bool dense = pix_pitch == C;
+    void (*const rows_kernel)(const GatherArgs, const RowsArgs) = dense ? im2col_rows_kernel<true> : im2col_rows_kernel<false>;
+    const bool small = smem <= 46 * 1024, large = smem <= kRowsSmem && C <= 16 && (int64_t)B * Ho >= sm_count();
+    if (small || (large && ensure_smem_attr(reinterpret_cast<const void*>(rows_kernel), (int)kRowsSmem, attr_set[dense]))) {
         const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, 200 * 1024 / smem));
         const int64_t blocks = std::min<int64_t>((int64_t)B * Ho, (int64_t)sm_count() * per_sm);
-        return launch_dependent(im2col_rows_kernel, (unsigned)blocks, kGatherThreads, smem, st, a, ra);
+        // Rows that are not small take at least 40 KB, five blocks an SM: a launch is placed while the one in front drains, and more of them crowd together where
+        // that leaves first (8 x 56 x 56 x 64 20.4 us against 22.6 with as many as fit; 2 x 640 x 640 x 3 10.3, 12.9).
+        return launch_dependent(rows_kernel, (unsigned)blocks, kGatherThreads, dense && smem > 16 * 1024 ? std::max<size_t>(smem, 40 * 1024) : smem, st, a, ra);
     }
     const int ppg = kGatherThreads / a.units;
     const int64_t blocks = std::min<int64_t>((a.N + ppg - 1) / ppg, (int64_t)sm_count() * 16);

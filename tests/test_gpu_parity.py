@@ -727,6 +727,30 @@ def _call_us(M, Cin, k, pad, B, H, W, layout):
     return min(runs)
 
 
+def test_patch_matrix_of_wide_rows_in_proportion():
+    """720 rows of 1280 pixels against 448 of 640 (three and a fifth times the work): 34 us and 11 for two images and
+    one; 105 when rows that wide went to the other kernel."""
+    import torch
+
+    def us(H, W):
+        Ho, Wo = (H - 1) // 2 + 1, (W - 1) // 2 + 1
+        act = torch.randint(0, 16, (2, H, W, 3), dtype=torch.int8, device="cuda")
+        cols = torch.empty((2 * Ho * Wo, 160), dtype=torch.int8, device="cuda")
+        runs = []
+        for _ in range(8):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            start.record()
+            for _ in range(10):
+                R.rmsmp_im2col_codes(act, 2, H, W, 3, 3, 7, 7, 2, 3, cols, 160)
+            end.record()
+            torch.cuda.synchronize()
+            runs.append(100.0 * start.elapsed_time(end))
+        return min(runs)
+
+    assert us(720, 1280) <= 6.0 * us(448, 640)
+
+
 @pytest.mark.parametrize("call,other,bound", [
     # 256 rows, 20,000 tokens as [M][N] against [N][M]: 7.6 us and 6.8; tiles no multiple of 32 tokens 16.5
     ((256, 64, 0, 0, 20000, 1, 1, R.OUT_MN), (256, 64, 0, 0, 20000, 1, 1, R.OUT_NM), 1.7),
@@ -1044,6 +1068,37 @@ def test_patch_matrix_pieces(C, kh, kw, stride, pad, B, H, W, ld, offset):
     got = out.cpu().numpy()
     assert np.array_equal(got[128:-128].reshape(ref.shape), ref)
     assert (got[:128] == 99).all() and (got[-128:] == 99).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("C,pitch,k,stride,pad,B,H,W,offset", [
+    (3, 4, 7, 2, 3, 2, 9, 77, 0), (4, 16, 3, 1, 1, 2, 6, 40, 0), (1, 4, 5, 1, 2, 1, 5, 9, 4),      # a word a pixel
+    (3, 4, 3, 1, 1, 1, 5, 6, 1), (24, 25, 3, 1, 1, 2, 5, 8, 0), (5, 7, 5, 3, 4, 2, 6, 11, 3),      # byte by byte
+    (24, 32, 3, 1, 1, 2, 6, 9, 0), (12, 20, 3, 2, 0, 1, 7, 9, 8),                                   # four bytes at a time
+    (32, 48, 3, 1, 1, 2, 5, 9, 0), (16, 64, 5, 1, 2, 1, 6, 7, 16),                                  # sixteen
+    (3, 3, 7, 2, 3, 1, 320, 1100, 0), (3, 4, 7, 2, 3, 1, 320, 1100, 0),                             # rows that need more shared memory
+    (16, 16, 5, 1, 2, 1, 160, 300, 0), (8, 12, 5, 1, 2, 1, 160, 500, 4),
+    (3, 4, 7, 2, 3, 1, 20, 1100, 0),                                                                # ... and too few of them for that
+])
+def test_patch_matrix_of_padded_and_wide_pixels(C, pitch, k, stride, pad, B, H, W, offset):
+    """The bytes between pixels are not zero and must not show; the tensor ends with the last pixel's channels."""
+    import torch
+    g = synth.rng(94, C + pitch + W)
+    act = g.integers(-128, 128, size=(B, H, W, C), dtype=np.int8)
+    pixels = np.full((B * H * W, pitch), 55, np.int8)
+    pixels[:, :C] = act.reshape(-1, C)
+    flat = pixels.reshape(-1)[:(B * H * W - 1) * pitch + C]
+    a = torch.full((offset + flat.size,), 55, dtype=torch.int8, device="cuda")
+    a[offset:] = torch.from_numpy(flat).cuda()
+    Ho, Wo = O.conv_out_hw(H, W, k, k, stride, pad)
+    ld = (k * k * C + 15) // 16 * 16
+    N = B * Ho * Wo
+    buf = torch.full((N * ld + 256,), 99, dtype=torch.int8, device="cuda")
+    R.rmsmp_im2col_codes(a[offset:], B, H, W, C, pitch, k, k, stride, pad, buf[128:128 + N * ld], ld)
+    torch.cuda.synchronize()
+    assert np.array_equal(buf[128:128 + N * ld].cpu().numpy().reshape(N, ld), O.im2col(act, k, k, stride, pad, ld))
+    assert (buf[:128] == 99).all() and (buf[128 + N * ld:] == 99).all()
+
 
 
 @pytest.mark.gpu
