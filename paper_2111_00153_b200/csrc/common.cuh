@@ -90,7 +90,9 @@ inline cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigne
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(grid); lc.blockDim = dim3(block); lc.dynamicSmemBytes = smem; lc.stream = st;
     lc.attrs = at; lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();            // (a refused launch is this call's error, not the next one's)
+    return e;
 }
 
 // The same in clusters of `cluster` blocks.
@@ -105,7 +107,9 @@ inline cudaError_t launch_dependent_cluster(void (*kernel)(P...), unsigned clust
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(grid); lc.blockDim = dim3(block); lc.dynamicSmemBytes = smem; lc.stream = st;
     lc.attrs = at; lc.numAttrs = 2;
-    return cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 // Re-quantizing epilogue request (rmsmp_*_workspace_requant): the next layer's clip value, kind and code buffer.

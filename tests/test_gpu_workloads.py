@@ -527,3 +527,32 @@ def test_calls_in_a_row_on_the_same_buffers_are_ordered(M, K, N):
     torch.cuda.synchronize()
     for i, out in got:
         assert all(torch.equal(a, b) for a, b in zip(out, want[i]))
+
+
+def test_a_refused_launch_leaves_no_error_for_the_next_call():
+    """While a blocking stream is captured the driver refuses launches on the legacy default stream: that call reports
+    it, and what comes after runs as if nothing had been."""
+    import ctypes
+    import torch
+    g = synth.rng(95, 1)
+    M, K, N = 40, 64, 3
+    Wt = synth.weights_normal(g, (M, K))
+    scheme, bits = O.assign_rows(Wt, (60, 35, 5))
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, synth.alpha_rows(Wt))
+    act = torch.zeros((N, K), dtype=torch.int8, device="cuda")
+    y = torch.empty((N, M), dtype=torch.float32, device="cuda")
+    values = torch.empty((M, K), dtype=torch.int8, device="cuda")
+    rt = ctypes.CDLL("libcudart.so.%s" % torch.version.cuda.split(".")[0])
+    stream, graph = ctypes.c_void_p(), ctypes.c_void_p()
+    torch.cuda.synchronize()
+    assert rt.cudaStreamCreate(ctypes.byref(stream)) == 0
+    assert rt.cudaStreamBeginCapture(stream, 0) == 0
+    with pytest.raises(R.RmsmpError) as e:
+        R.rmsmp_gemm_variant(layer, d_packed, act, N, K, 0.5, y, M, R.OUT_NM, None, R.VARIANT_SIMT, stream=0)
+    rt.cudaStreamEndCapture(stream, ctypes.byref(graph))       # (the refused launch has invalidated the capture)
+    assert rt.cudaStreamDestroy(stream) == 0
+    rt.cudaGetLastError()
+    assert e.value.status == R.ERR_CUDA
+    R.rmsmp_unpack_codes(layer, d_packed, values)
+    torch.cuda.synchronize()
+    assert np.array_equal(values.cpu().numpy(), O.quantize_rows(Wt, scheme, bits, synth.alpha_rows(Wt))[0])
