@@ -23,6 +23,7 @@
 #include <cstring>
 #include <algorithm>
 #include "common.cuh"
+#include "tmap.cuh"
 
 namespace rmsmp {
 
@@ -391,28 +392,6 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
 
 // ------------------------------------------------------------------ host side
 
-typedef CUresult (*EncodeTiledFn2)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
-                                   CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                   CUtensorMapFloatOOBfill);
-
-EncodeTiledFn2 encode_fn2()
-{
-    static EncodeTiledFn2 fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void* ptr = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn2>(ptr);
-        else
-            cudaGetLastError();
-    }
-    return fn;
-}
-
 // The pair kernel takes: expanded weights, an even number of row blocks, full 128-channel chunks,
 // fp32 [N][M] output through bulk stores, no accumulator dump, no re-quantizing epilogue.
 bool plan_pair(const Problem& p, PairCfg& c)
@@ -473,7 +452,7 @@ bool plan_pair(const Problem& p, PairCfg& c)
 bool pair_supported(const Problem& p)
 {
     PairCfg c;
-    if (!plan_pair(p, c) || !encode_fn2()) return false;
+    if (!plan_pair(p, c) || !tensor_map_encoder()) return false;
     return c.nkb >= 16 && c.npix_h >= 64;
 }
 
@@ -481,7 +460,7 @@ rmsmp_status launch_pair(const Problem& p, cudaStream_t st)
 {
     PairCfg c;
     if (!plan_pair(p, c)) return RMSMP_ERR_VARIANT;
-    EncodeTiledFn2 enc = encode_fn2();
+    EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return RMSMP_ERR_CUDA;
     PairMaps mp;
     memset(&mp, 0, sizeof(mp));

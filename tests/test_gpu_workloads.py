@@ -5,6 +5,10 @@ The ResNet-18 stack is compared in full at the benchmark's batch; of the BERT-ba
 largest ones are compared on randomly sampled outputs the oracle computes one by one plus every
 row (the integer sums are exact, so each sampled element is as strict as in a full comparison).
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -14,6 +18,8 @@ from paper_2111_00153_b200 import synth
 from tests import harness as Hn
 
 pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _expected(acc, ws, act_step):
@@ -556,3 +562,38 @@ def test_a_refused_launch_leaves_no_error_for_the_next_call():
     R.rmsmp_unpack_codes(layer, d_packed, values)
     torch.cuda.synchronize()
     assert np.array_equal(values.cpu().numpy(), O.quantize_rows(Wt, scheme, bits, synth.alpha_rows(Wt))[0])
+
+
+def test_first_calls_of_several_threads_at_once():
+    """A process whose first tensor-core calls come from eight threads together: none is refused while another looks
+    the tensor-map encoder up."""
+    code = """
+import threading, numpy as np, torch
+from paper_2111_00153_b200 import binding as R
+M, K, N, T = 256, 512, 64, 8
+scheme, bits = np.ones(M, np.uint8), np.full(M, 4, np.uint8)
+layer = R.rmsmp_layer_init(M, K, 1, 1, scheme, bits)
+packed = torch.empty(layer.packed_bytes, dtype=torch.uint8, device="cuda")
+R.rmsmp_quantize_pack(torch.randn(M, K, device="cuda"), R.W_LINEAR, layer, scheme, bits, np.ones(M, np.float32), 0, packed)
+ws = torch.empty(R.rmsmp_workspace_bytes(layer), dtype=torch.int8, device="cuda")
+R.rmsmp_expand_weights(layer, packed, ws)
+act = torch.ones((N, K), dtype=torch.int8, device="cuda")
+out = [torch.empty((N, M), device="cuda") for _ in range(T)]
+torch.cuda.synchronize()
+gate, errors = threading.Barrier(T), []
+def work(i):
+    gate.wait()
+    try:
+        R.rmsmp_gemm_workspace(layer, packed, ws, act, N, K, 0.5, out[i], M, stream=0)
+    except Exception as e:
+        errors.append(str(e))
+threads = [threading.Thread(target=work, args=(i,)) for i in range(T)]
+for t in threads: t.start()
+for t in threads: t.join()
+torch.cuda.synchronize()
+assert not errors, errors
+assert all(torch.equal(o, out[0]) for o in out)
+"""
+    for _ in range(2):
+        r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300, cwd=ROOT)
+        assert r.returncode == 0, r.stderr[-2000:]
