@@ -213,9 +213,7 @@ def _host_array(a, fmt: str):
     return np.ascontiguousarray(a, dtype=np.uint8 if fmt == "B" else np.float32)
 
 
-def __getattr__(name):
-    if name not in _NATIVE:
-        raise AttributeError(f"module {__name__!r} has no attribute {name!r}")
+def _load_native():
     L = lib()
     try:
         from . import _marshal
@@ -224,6 +222,20 @@ def __getattr__(name):
     _marshal.setup({n: C.cast(getattr(L, n), C.c_void_p).value for n in _NATIVE}, _current_stream, _raise, _host_array)
     for n in _NATIVE:
         globals()[n] = getattr(_marshal, n)
+
+
+def __getattr__(name):
+    if name not in _NATIVE:
+        raise AttributeError(f"module {__name__!r} has no attribute {name!r}")
+    try:
+        _load_native()
+    except (RuntimeError, OSError):
+        # not built: the name is there all the same, as for the other calls, and the call says what is missing
+        def call(*args, **kwargs):
+            _load_native()
+            return globals()[name](*args, **kwargs)
+        call.__name__ = name
+        return call
     return globals()[name]
 
 

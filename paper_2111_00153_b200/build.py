@@ -11,7 +11,8 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "librmsmp.so")
 MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
-MARSHAL = os.path.join(_HERE, "_marshal.so")
+# named for the interpreter it was built for, so that another one does not load it
+MARSHAL = os.path.join(_HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ("host_api.cu", "pack.cu", "simt.cu", "tensor.cu", "tensor2.cu", "split.cu", "peak.cu", "builtin_scratch.cu", "stream.cu", "assign.cu", "depthwise.cu", "gather.cu")
 HEADERS = tuple(sorted(f for f in os.listdir(CSRC) if f.endswith((".cuh", ".h")))) + \
           (os.path.join("..", "..", "include", "rmsmp.h"),)
@@ -48,6 +49,9 @@ def build_marshal(force: bool = False) -> str:
     header = os.path.join(CSRC, "..", "..", "include", "rmsmp.h")
     if not force and not _older(MARSHAL, [MARSHAL_SOURCE, header, os.path.abspath(__file__)]):
         return MARSHAL
+    untagged = os.path.join(_HERE, "_marshal.so")         # the name of earlier builds, which any interpreter would load
+    if os.path.exists(untagged):
+        os.remove(untagged)
     tmp = MARSHAL + ".%d.tmp" % os.getpid()
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], MARSHAL_SOURCE, "-o", tmp])
     os.replace(tmp, MARSHAL)

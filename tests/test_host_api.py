@@ -199,3 +199,29 @@ def test_marshalled_pack_takes_any_host_array(convert):
         call(a=alpha[:3])
     with pytest.raises((TypeError, ValueError)):
         R.rmsmp_quantize_pack(256, R.W_LINEAR, layer, "abc", bits, alpha, R.POT_NEAREST, 256, 1 << 20, stream=0)
+
+
+def test_marshalling_module_is_named_for_its_interpreter():
+    import sysconfig
+    assert os.path.basename(B.MARSHAL) == "_marshal" + sysconfig.get_config_var("EXT_SUFFIX")
+    assert os.path.exists(B.MARSHAL) and not os.path.exists(os.path.join(os.path.dirname(B.MARSHAL), "_marshal.so"))
+
+
+def test_names_are_there_without_the_library_and_calls_say_what_is_missing():
+    import subprocess
+    import sys
+    code = """
+from paper_2111_00153_b200 import binding as R
+R.LIB_PATH = "/nonexistent/librmsmp.so"
+from paper_2111_00153_b200.binding import rmsmp_gemm, rmsmp_workspace_bytes
+assert hasattr(R, "rmsmp_quantize_act") and not hasattr(R, "rmsmp_no_such_call")
+for call in (rmsmp_gemm, R.rmsmp_quantize_act):
+    try:
+        call()
+    except RuntimeError as e:
+        assert "is missing" in str(e)
+    else:
+        raise SystemExit("no error")
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300, cwd=ROOT)
+    assert r.returncode == 0, r.stdout + r.stderr
