@@ -580,8 +580,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 f_cc = f_kb - f_tap * cfg.cpt;
                 f_tl += adv;
                 if (rows_change) {
-                    if (adv != look) { load_block(f_tl); look_up(); load_block(f_tl + look); }
-                    take_rows();
+                    take_rows();                          // (the look-ahead's tile: with two groups adv is look, 2 for nkb == 1 and else 1)
                     look_up();
                     load_block(f_tl + 2 * look);
                 }
