@@ -1064,7 +1064,7 @@ bool plan(const Problem& p, TensorCfg& c)
 
 }  // namespace
 
-EncodeTiledFn tensor_map_encoder()
+static EncodeTiledFn driver_encoder()
 {
     // (threads that come while another looks it up wait for it)
     static const EncodeTiledFn fn = []() -> EncodeTiledFn {
@@ -1078,6 +1078,24 @@ EncodeTiledFn tensor_map_encoder()
     }();
     return fn;
 }
+
+// The driver's call needs a current context, which a thread has only after a runtime call that makes one: a thread whose first
+// call comes here gets its device's.
+static CUresult encode_tiled(CUtensorMap* map, CUtensorMapDataType type, cuuint32_t rank, void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                             const cuuint32_t* box, const cuuint32_t* steps, CUtensorMapInterleave interleave, CUtensorMapSwizzle swizzle,
+                             CUtensorMapL2promotion promotion, CUtensorMapFloatOOBfill fill)
+{
+    const EncodeTiledFn fn = driver_encoder();
+    CUresult r = fn(map, type, rank, base, dims, strides, box, steps, interleave, swizzle, promotion, fill);
+    if (r == CUDA_ERROR_INVALID_CONTEXT || r == CUDA_ERROR_NOT_INITIALIZED) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) { cudaGetLastError(); return r; }
+        r = fn(map, type, rank, base, dims, strides, box, steps, interleave, swizzle, promotion, fill);
+    }
+    return r;
+}
+
+EncodeTiledFn tensor_map_encoder() { return driver_encoder() ? encode_tiled : nullptr; }
 
 bool encode_act_maps_4(const Problem& p, int bk, int th, int tb, void* maps4)
 {

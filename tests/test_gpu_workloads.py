@@ -565,8 +565,8 @@ def test_a_refused_launch_leaves_no_error_for_the_next_call():
 
 
 def test_first_calls_of_several_threads_at_once():
-    """A process whose first tensor-core calls come from eight threads together: none is refused while another looks
-    the tensor-map encoder up."""
+    """A process whose first tensor-core calls come from eight threads together, for which they are the first CUDA calls
+    too: none is refused while another looks the tensor-map encoder up, or for want of a current context."""
     code = """
 import threading, numpy as np, torch
 from paper_2111_00153_b200 import binding as R
