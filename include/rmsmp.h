@@ -96,7 +96,8 @@ typedef struct rmsmp_layer {
     int32_t Cp, Kp;             /* padded channel count per tap, padded packed row length */
     int32_t nP, nF4, n8;        /* rows per group */
     int32_t nblocks;            /* ceil(M/128) */
-    int32_t raw_stage_bytes;    /* most bytes of packed codes that a 128-row block has per 128 of a row (rows of a kind in 16s) */
+    int32_t raw_stage_bytes;    /* most bytes of packed codes that a 128-row block has per 128 of a row (rows of a kind in 16s);
+                                   kept for the structure's layout, no kernel reads it */
     uint64_t off_perm, off_slot, off_wstep, off_alpha, off_kind, off_blocks, off_q4, off_q8;
     uint64_t packed_bytes;      /* size the packed buffer must have */
 } rmsmp_layer;

@@ -74,13 +74,19 @@ bool ensure_smem_attr(const void* fn, int bytes, bool* done);
 // Every kernel that a layer call queues is launched as a programmatic dependent of whatever is in front of it on the
 // stream: its CTAs are placed, and its set-up runs, while the kernel in front drains, which takes the launch gap from
 // 1.9 to about 1 us, and such a launch also costs the host less (2.3 against 3 us).  The order of memory accesses is
-// kept by two rules.  (1) pdl_wait() comes before a kernel's first access to global memory; it returns when the kernels
+// kept by these rules.  (1) pdl_wait() comes before a kernel's first access to global memory; it returns when the kernels
 // in front have finished and their writes are visible.  (2) pdl_trigger() (the next kernel may be placed) comes after
-// it, so that a kernel whose successor runs has no unfinished predecessor itself; kernels that write what the grouped
-// stream kernel reads ahead of its own wait (packed codes and the packed buffer's metadata) end in pack_kernel, which
-// never triggers.  The tensor-core kernels do not trigger either: a small kernel whose blocks are placed beside their
-// CTAs has to live with what 200 KB of shared memory leaves of the L1 (the activation quantizer behind a convolution:
-// ResNet-18 at batch 256 1168 us with the trigger, 1146 with it just before the end, 1075 without, 1138 with plain launches).
+// it, so that a kernel whose successor runs has no unfinished predecessor itself.  Two kernels are exempt, those of the
+// grouped tensor-core launch (stream.cu): act_e4m3_kernel and stream_kernel trigger at once and read ahead of their wait
+// the launch's table (both) and, of every layer, packed codes, perm and wstep (stream_kernel).  Activations, the copies of
+// them, outputs and status words stay behind it, and each of the two waits before it ends, so that neither ends before what
+// is in front of it.  (3) So whatever writes a table, packed codes or a packed buffer's metadata must be complete before
+// any kernel behind it can be placed: the last kernel of such a call never triggers (pack_kernel; everything else that
+// writes them is a copy or a kernel in front of pack_kernel).  A new writer that triggered would be a race.
+// Without a trigger for another reason: tensor_kernel and pair_kernel, because a small kernel whose blocks are placed
+// beside their CTAs has to live with what 200 KB of shared memory leaves of the L1 (the activation quantizer behind a
+// convolution: ResNet-18 at batch 256 1168 us with the trigger, 1146 with it just before the end, 1075 without, 1138 with
+// plain launches; split_kernel, for problems that leave SMs free, triggers), and the general depthwise form (depthwise.cu).
 template <typename... P, typename... A>
 inline cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, const A&... args)
 {
@@ -211,11 +217,13 @@ __host__ __device__ inline TapBox tap_box(const Problem& p, int h0, int ti, int 
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// A pointer that cannot be known before this point, so that no read-only load through it moves in front of pdl_wait().
+// A pointer that cannot be known before this point, so that no read-only load (__ldg: to the compiler a function of the
+// address alone) through it moves in front of pdl_wait().  Every kernel launched as a dependent takes the pointers of such
+// loads through this, or reads them from memory behind the wait.
 template <typename T>
 __device__ __forceinline__ T* pdl_ordered(T* p)
 {
-    asm volatile("" : "+l"(p) :: "memory");
+    asm volatile("" : "+l"(p));
     return p;
 }
 

@@ -96,11 +96,13 @@ __device__ __forceinline__ void dw_store(const Problem& p, uint32_t n, int q, co
 // kS = 1, 2: 3 x 3 filters of that stride, strips of `strip` output rows; kS = 0: any filter, one output per item.
 // kAcc: the sums are wanted too (their addresses take registers that the strips need: 5 % of the time).
 template <int kS, bool kAcc>
-__global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const Problem p, const int strip)
+__global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const Problem given, const int strip)
 {
     extern __shared__ uint32_t s_w[];                     // [tap][quad]: channel 4q+j in byte j
-    const int taps = p.kh * p.kw, C = p.M;
     pdl_wait();
+    Problem p = given;
+    p.act = pdl_ordered(p.act); p.wstep = pdl_ordered(p.wstep);
+    const int taps = p.kh * p.kw, C = p.M;
     // (the other form's blocks stay for its whole time: placed early, the next launch's crowd together where these leave
     // first; 960 channels, 64 images of 28 x 28, stride 3 56.4 us with the trigger, 49.7 without)
     if (kS != 0) pdl_trigger();

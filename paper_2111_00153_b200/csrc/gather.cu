@@ -23,12 +23,13 @@ struct GatherArgs {
     int B, H, W, C, kh, kw, stride, pad, Ho, Wo, K, units;      // units: 16-byte pieces per output row
 };
 
-__global__ void __launch_bounds__(kGatherThreads) im2col_kernel(const GatherArgs a)
+__global__ void __launch_bounds__(kGatherThreads) im2col_kernel(GatherArgs a)
 {
     // thread <-> (pixel of the block's current group, 16-byte piece of its row): fixed per thread; the pixel index
     // advances by whole groups; 32-bit index arithmetic (the host checks the counts)
     pdl_wait();
     pdl_trigger();
+    a.act = pdl_ordered(a.act);
     const int upr = a.units;
     const int ppg = kGatherThreads / upr;                 // pixels per group (units <= kGatherThreads is checked by the host)
     const int my_p = threadIdx.x / upr, k0 = (threadIdx.x - my_p * upr) << 4;
@@ -86,7 +87,7 @@ struct alignas(32) Piece { uint32_t keep[4]; int row, off, last, pad; };      //
 
 // kDense: pixels follow one another without padding bytes.
 template <bool kDense>
-__global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(const GatherArgs a, const RowsArgs ra)
+__global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(GatherArgs a, const RowsArgs ra)
 {
     extern __shared__ __align__(32) uint8_t s_mem[];
     uint8_t* const s_out = s_mem;                                          // [tile][ld_cols]
@@ -123,6 +124,7 @@ __global__ void __launch_bounds__(kGatherThreads) im2col_rows_kernel(const Gathe
     }
     pdl_wait();
     pdl_trigger();
+    a.act = pdl_ordered(a.act);
     for (int r = blockIdx.x; r < rows_total; r += gridDim.x) {
         const int b = r / a.Ho, ho = r - b * a.Ho;
         const int y0 = ho * a.stride - a.pad;
@@ -264,7 +266,7 @@ cudaError_t launch_im2col(const int8_t* act, int B, int H, int W, int C, int64_t
     // with a fourth byte a pixel; 3 x 3, two of 224 x 224 x 64 47 and 71; 32 rows of 2000 x 3 10.7 and 18.8).
     static bool attr_set[2][kMaxDevices] = {};
     const bool dense = pix_pitch == C;
-    void (*const rows_kernel)(const GatherArgs, const RowsArgs) = dense ? im2col_rows_kernel<true> : im2col_rows_kernel<false>;
+    void (*const rows_kernel)(GatherArgs, const RowsArgs) = dense ? im2col_rows_kernel<true> : im2col_rows_kernel<false>;
     const bool small = smem <= 46 * 1024, large = smem <= kRowsSmem && C <= 16 && (int64_t)B * Ho >= sm_count();
     if (small || (large && ensure_smem_attr(reinterpret_cast<const void*>(rows_kernel), (int)kRowsSmem, attr_set[dense]))) {
         const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, 200 * 1024 / smem));

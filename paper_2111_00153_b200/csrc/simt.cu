@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(256) rowwarp_kernel(Problem p)
 {
     pdl_wait();
     pdl_trigger();
+    p.act = pdl_ordered(p.act); p.q4 = pdl_ordered(p.q4); p.q8 = pdl_ordered(p.q8); p.wstep = pdl_ordered(p.wstep);
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;

@@ -182,9 +182,10 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         const uint8_t* src = p.q4;
         if (m_row < p.M) {
             kind = p.kind[m_row];
-            const int packed = __ldg(p.slot + m_row);
+            const int packed = __ldg(pdl_ordered(p.slot) + m_row);
             src = kind == kFixed8 ? p.q8 + (size_t)(packed - p.nP - p.nF4) * p.Kp : p.q4 + (size_t)packed * (p.Kp >> 1);
         }
+        src = pdl_ordered(src);
         const uint32_t swz = cfg.bk == 128 ? (uint32_t)(row & 7) : (uint32_t)((row >> 1) & 3);
         const uint32_t row_off = (uint32_t)row * (uint32_t)cfg.bk;
         // The codes of a k-block are in registers before its turn comes: the next one's are loaded as soon as this one's
@@ -200,13 +201,13 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         auto pieces_of = [&](int ksteps) { return kind < 0 ? 0 : (eight ? 2 * ksteps : ksteps); };      // 16-byte pieces of a row
         // this thread's pixel of the tile (kGather): its image, and the input position of its tap (0, 0)
         int px_y = 0, px_x = 0;
-        const int8_t* px_img = p.act;
+        const int8_t* px_img = pdl_ordered(p.act);
         const bool px_ok = kGather && row < cfg.npix && (int64_t)nt * cfg.npix + row < p.N;
         if (px_ok) {
             const uint32_t n = (uint32_t)((int64_t)nt * cfg.npix + row), t = n / (uint32_t)p.Wo, b = t / (uint32_t)p.Ho;
             px_x = (int)(n - t * (uint32_t)p.Wo) * p.stride - p.pad;
             px_y = (int)(t - b * (uint32_t)p.Ho) * p.stride - p.pad;
-            px_img = p.act + (int64_t)b * p.H * p.W * p.pix_pitch;
+            px_img += (int64_t)b * p.H * p.W * p.pix_pitch;
         }
         int ksteps;
         {
@@ -302,8 +303,8 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     float scale = 0.0f;
     int shift = 0;
     if (row_ok) {
-        scale = __fmul_rn(__ldg(p.wstep + m), p.act_step);
-        shift = (!kPre && __ldg(p.kind + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
+        scale = __fmul_rn(__ldg(pdl_ordered(p.wstep) + m), p.act_step);
+        shift = (!kPre && __ldg(pdl_ordered(p.kind) + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
     }
     const ActFast rq = act_fast_setup(kRQ ? p.rq_alpha : 1.0f, kRQ ? p.rq_kind : 0);
     const bool out_mn = !kRQ && p.out_mn != 0;

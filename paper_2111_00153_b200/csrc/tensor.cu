@@ -120,6 +120,7 @@ __device__ __forceinline__ void fill_resident_weights(const Problem& p, const Te
         const int kind = have ? (int)p.kind[m] : kFixed8;
         const int slot = have ? p.slot[m] : 0;
         const uint8_t* src = (kind == kFixed8) ? p.q8 + (size_t)(have ? slot - n4 : 0) * p.Kp : p.q4 + (size_t)slot * (p.Kp >> 1);
+        src = pdl_ordered(src);
         const uint32_t phase = (cfg.bk == 128) ? (uint32_t)(r & 7) : (uint32_t)((r >> 1) & 3);
         const uint32_t row_base = sA + (uint32_t)r * (uint32_t)cfg.bk;
         const int pieces = cfg.nkb << pshift;
@@ -491,13 +492,15 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         const int64_t total = my_tiles * cfg.nkb;
         const bool rows_change = step % (uint32_t)p.nblocks != 0u;
         // a row block's rows in the packed buffer: first and number of each kind
+        const int32_t* const blocks = pdl_ordered(p.blocks), *const perm = pdl_ordered(p.perm);
+        const uint4* const codes = reinterpret_cast<const uint4*>(pdl_ordered(p.q4));
         int4 blk_a;
         int2 blk_b;
         int blk_next = 0;
         auto load_block = [&](int64_t local) {
             blk_next = (int)((uint32_t)(first + (uint32_t)min(local, my_tiles - 1) * step) % (uint32_t)p.nblocks);
-            blk_a = __ldg(reinterpret_cast<const int4*>(p.blocks + 8 * blk_next));
-            blk_b = __ldg(reinterpret_cast<const int2*>(p.blocks + 8 * blk_next + 4));
+            blk_a = __ldg(reinterpret_cast<const int4*>(blocks + 8 * blk_next));
+            blk_b = __ldg(reinterpret_cast<const int2*>(blocks + 8 * blk_next + 4));
         };
         const int n4 = p.nP + p.nF4;
         const uint32_t q8_first = (uint32_t)((p.q8 - p.q4) >> 4);
@@ -514,7 +517,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 const int kind = e >= blk_b.y ? 3 : f < 0 ? kPoT4 : e < 0 ? kFixed4 : kFixed8;
                 const int packed = kind == kPoT4 ? blk_a.x + r : kind == kFixed4 ? p.nP + blk_a.z + f : n4 + blk_b.x + e;
                 off_next[i] = kind == 3 ? 0u : kind == kFixed8 ? q8_first + (uint32_t)(packed - n4) * (uint32_t)(p.Kp >> 4) : (uint32_t)packed * (uint32_t)(p.Kp >> 5);
-                row_next[i] = kind == 3 ? first_next : __ldg(p.perm + packed);
+                row_next[i] = kind == 3 ? first_next : __ldg(perm + packed);
                 kinds_next |= (uint32_t)kind << (8 * i);
             }
             const uint32_t k0 = __shfl_sync(0xffffffffu, kinds_next, 0) & 3u;      // (every lane takes part in both votes)
@@ -538,7 +541,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         uint4 lo[4], hi[4];                              // (hi: the second half of 32 eight-bit codes)
         auto load = [&](int i, uint32_t piece) {
             const bool eight = ((kinds >> (8 * i)) & 3u) == kFixed8;
-            const uint4* src = reinterpret_cast<const uint4*>(p.q4) + (off[i] + (eight ? 2u * piece : piece));
+            const uint4* src = codes + (off[i] + (eight ? 2u * piece : piece));
             lo[i] = __ldg(src);
             if (eight) hi[i] = __ldg(src + 1);
         };
@@ -674,8 +677,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 scale = 0.f;
                 shift = 0;
                 if (row_ok) {
-                    scale = __fmul_rn(__ldg(p.wstep + m), p.act_step);
-                    shift = (!kPre && __ldg(p.kind + m) == kFixed4) ? 4 : 0;   // expanders store Fixed-4 codes as 16 * value
+                    scale = __fmul_rn(__ldg(pdl_ordered(p.wstep) + m), p.act_step);
+                    shift = (!kPre && __ldg(pdl_ordered(p.kind) + m) == kFixed4) ? 4 : 0;   // expanders store Fixed-4 codes as 16 * value
                 }
             }
             if (!mbar_wait_warp(bar_tfull + 8 * ab, tpar, abort_flag)) { alive = false; break; }

@@ -336,7 +336,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
             const int64_t nt = tile / cfg.nbt;
             const int blk = (int)(tile - nt * cfg.nbt) * 2 + (int)rank;
             const int m = blk * kBlockRows + quarter * 32 + lane;
-            const float scale = (m < p.M) ? __fmul_rn(__ldg(p.wstep + m), p.act_step) : 0.f;
+            const float scale = (m < p.M) ? __fmul_rn(__ldg(pdl_ordered(p.wstep) + m), p.act_step) : 0.f;
             int64_t n0h[2];
             int nvalid[2];
 #pragma unroll

@@ -225,3 +225,20 @@ for call in (rmsmp_gemm, R.rmsmp_quantize_act):
 """
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300, cwd=ROOT)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_read_only_loads_go_through_pointers_ordered_behind_the_wait():
+    """To the compiler a read-only load is a function of its address: in a kernel that waits for the one in front, its
+    pointer must not exist before the wait.  Kernels take their problem by value, so a load straight through a member of
+    it is what must not be there (a local copy whose pointers were ordered may)."""
+    direct = re.compile(r"__ldg\((?:reinterpret_cast<[^>]*>\()?\s*([pa])\.(\w+)")
+    for name in sorted(os.listdir(B.CSRC)):
+        if not name.endswith(".cu") or name in ("stream.cu",):          # (its table's and packed codes' early reads are the rule's exemption)
+            continue
+        text = open(os.path.join(B.CSRC, name)).read()
+        if "pdl_wait()" not in text:
+            continue
+        for obj, member in direct.findall(text):
+            ordered = re.search(r"%s\.%s = pdl_ordered\(%s\.%s\)" % (obj, member, obj, member), text)
+            from_table = name == "simt.cu" and (obj, member) == ("p", "perm")      # (a problem read from the launch's table)
+            assert ordered or from_table, (name, obj, member)
