@@ -535,6 +535,64 @@ def test_calls_in_a_row_on_the_same_buffers_are_ordered(M, K, N):
         assert all(torch.equal(a, b) for a, b in zip(out, want[i]))
 
 
+@pytest.mark.parametrize("B,H,Cin", [(1, 9, 24), (2, 14, 32), (16, 28, 24)])
+def test_a_network_of_calls_without_anything_between_them_is_ordered(B, H, Cin):
+    """The other calls that are launched as dependents -- plain convolutions (gathered and not), depthwise layers of both
+    forms, the patch matrix, an expansion into a workspace that the last round's convolution read -- each feeding the next
+    with no other kernel in between: equal to the same calls with a synchronisation after each."""
+    import torch
+    g = synth.rng(96, B + H + Cin)
+    C = 96
+
+    def pack(shape):
+        W = synth.weights_kaiming(g, *shape)
+        scheme, bits = O.assign_rows(W.reshape(shape[0], -1), (60, 35, 5))
+        return Hn.pack_layer(W, scheme, bits, synth.alpha_rows(W.reshape(shape[0], -1)))
+
+    up, dw3, dw5, down = pack((C, Cin, 1, 1)), pack((C, 1, 3, 3)), pack((C, 1, 5, 5)), [pack((Cin, C, 3, 3)) for _ in range(2)]
+    ld = (9 * Cin + 15) // 16 * 16
+    last_W = synth.weights_normal(g, (40, ld))
+    last_scheme, last_bits = O.assign_rows(last_W, (60, 35, 5))
+    last = Hn.pack_layer(last_W, last_scheme, last_bits, synth.alpha_rows(last_W))
+    N = B * H * H
+    xs = [torch.from_numpy(synth.act_halfnormal(g, (N, Cin))).cuda() for _ in range(2)]
+    ws = torch.zeros(R.rmsmp_workspace_bytes(down[0][0]), dtype=torch.int8, device="cuda")
+    c_in, c_up, c_dw, c_out = (torch.zeros((N, n), dtype=torch.int8, device="cuda") for n in (Cin, C, C, Cin))
+    y_up, y_dw, y_out, y_last = (torch.zeros((N, n), dtype=torch.float32, device="cuda") for n in (C, C, Cin, 40))
+    cols = torch.zeros((N, ld), dtype=torch.int8, device="cuda")
+
+    def chain(i, wait):
+        x, (dl, dp) = xs[i & 1], down[(i >> 1) & 1]
+        step = R.rmsmp_quantize_act(x, N * Cin, 3.0, R.ACT_U4, c_in); wait()
+        R.rmsmp_conv_implicit(up[0], up[1], c_in, B, H, H, 1, 0, step, y_up); wait()
+        step = R.rmsmp_quantize_act(y_up, N * C, 2.0, R.ACT_U4, c_up); wait()
+        R.rmsmp_conv_depthwise(dw3[0], dw3[1], c_up, B, H, H, 1, 1, step, y_dw); wait()
+        step = R.rmsmp_quantize_act(y_dw, N * C, 2.0, R.ACT_U4, c_dw); wait()
+        R.rmsmp_conv_depthwise(dw5[0], dw5[1], c_dw, B, H, H, 1, 2, step, y_up); wait()
+        step = R.rmsmp_quantize_act(y_up, N * C, 2.0, R.ACT_U4, c_up); wait()
+        R.rmsmp_expand_weights(dl, dp, ws); wait()
+        R.rmsmp_conv_implicit_workspace(dl, dp, ws, c_up, B, H, H, 1, 1, step, y_out); wait()
+        step = R.rmsmp_quantize_act(y_out, N * Cin, 2.0, R.ACT_U4, c_out); wait()
+        R.rmsmp_im2col_codes(c_out, B, H, H, Cin, Cin, 3, 3, 1, 1, cols, ld); wait()
+        R.rmsmp_gemm(last[0], last[1], cols, N, ld, step, y_last, 40); wait()
+
+    def outputs():
+        return [t.clone() for t in (y_up, y_dw, y_out, y_last, cols)]
+
+    want = []
+    for i in range(4):
+        chain(i, torch.cuda.synchronize)
+        want.append(outputs())
+    assert all(float(w[3].abs().max()) > 0 for w in want) and not torch.equal(want[0][3], want[2][3])
+    torch.cuda.synchronize()
+    for first in range(4):
+        for i in range(first, first + 12):                # rounds right behind one another
+            chain(i, lambda: None)
+        got = outputs()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, want[(first + 11) & 3]))
+
+
 def test_a_refused_launch_leaves_no_error_for_the_next_call():
     """While a blocking stream is captured the driver refuses launches on the legacy default stream: that call reports
     it, and what comes after runs as if nothing had been."""
