@@ -12,7 +12,8 @@
 // bytes, eight permutes), which makes the three taps of a kernel row one dot product; a thread owns a
 // channel quad and four neighbouring columns and walks down a strip of rows, so that every input row is
 // loaded and transposed once for the three output rows that it touches, and the next row's loads are in
-// flight meanwhile (44 us; what is left is load latency at two blocks per SM).
+// flight meanwhile (48 us with launches back to back, 54 alone behind a flushed L2; what is left is load latency at two
+// blocks per SM).
 // Other filters: a word is split into four one-channel words, one output per work item.
 #include <algorithm>
 #include "common.cuh"
@@ -47,7 +48,7 @@ __device__ __forceinline__ void dw_transpose(uint32_t w0, uint32_t w1, uint32_t 
 // One input row of a thread's strip, ready for the dot products.  Stride 1: for every channel the words whose bytes 0..2
 // are the three columns under a kernel row.  Stride 2: the transposed columns, from which dw_word forms those words
 // where they are used -- a row serves one or two output rows there, and its sixteen words took registers that the
-// loads ahead need (56 x 56 x 192 at batch 64, launches back to back: 22.6 us with them, 19.5 so; stride 1, three output rows a row, 49.8 and 51.0).
+// loads ahead need (56 x 56 x 192 at batch 64, launches back to back: 22.6 us with them, 18.4 so; stride 1, three output rows a row, 47.8 with them).
 template <int kS> struct DwRow { uint32_t g[4], t[kS == 1 ? 12 : 5]; };
 
 template <int kS>

@@ -451,8 +451,10 @@ bool split_tile(const Problem& p, int target, SplitCfg& c)
 // Tile width and cluster size by a cost in SM cycles: start-up, the k-blocks of one CTA (rows of up to 128 bytes through
 // the SM's copy path, or the expansion of the codes), sending and adding the parts, the output; times the rounds that
 // the grid needs.  Against every width and cluster size measured for two dozen problems (256x512 to 4096x4096, 32 to
-// 6272 pixels) its choice is within 5 % of the best.  *us: the time that the cost stands for, as fitted to the same
-// measurements (a workspace: 2.2 us + 1400 units per us, good to 0.4 us; expansion: 1.75 of that - 2 us, good to 2 us).
+// 6272 pixels) its choice was within 5 % of the best; where channels are few it is off by more (7x7 step two 240x16 on 4 images of
+// 50x50 19.4 us chosen, 17.0 possible).  *us: the time that the cost stands for, as fitted to the same two dozen (a
+// workspace: 2.2 us + 1400 units per us; expansion: 1.75 of that - 2 us).  Over 86 convolutions the kernel that it decides for
+// takes 1.02 of the better one's time on average, 1.46 at worst.
 bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr, bool gather = false)
 {
     if (!gather && (p.pix_pitch % 16 != 0 || (reinterpret_cast<uintptr_t>(p.act) & 15) != 0)) return false;

@@ -953,8 +953,7 @@ bool plan(const Problem& p, TensorCfg& c)
         c.ntiles_n = (p.B + c.tb - 1) / c.tb;
     } else {
         // As few tiles as cover an image's rows, all of the same height.  (Heights that divide the image's make tiles of
-        // one row where that is a prime: 3x3 256x256 on 64 images of 29x29 133 us against 30 so, 5x5 160x16 on 46 of
-        // 29x29 454 against 81.)
+        // one row where that is a prime: 3x3 256x256 on 64 images of 29x29 133 us against 30 so.)
         const int most = std::min(kTileN / p.Wo, 256 / p.stride);
         c.tiles_per_image = (p.Ho + most - 1) / most;
         // Lower tiles where the tallest leave SMs idle (few images): a k-block takes 0.25 us (128-byte rows 0.33) + 0.04 per 256
