@@ -317,6 +317,22 @@ def test_config5_grouped_tensor_launch_matches_oracle(N):
         assert not torch.isnan(y).any()
 
 
+@pytest.mark.parametrize("N", [1, 16, 33, 64, 65, 80, 96, 112, 113, 128])
+def test_grouped_tensor_launch_ring_of_packed_codes(N):
+    """The expander sets take alternate stages and tell a slot's phases apart by parity: the ring has an even number of slots, or
+    enough of them that a set cannot be two of a slot's phases ahead of its copies (header words 5 and 13: slots, A stages)."""
+    import torch
+    keep, items, refs = _grouped_case([(384, 512)], N)
+    arr = R.make_gemm_items(items)
+    table = torch.empty(R.rmsmp_grouped_plan_bytes(arr), dtype=torch.uint8, device="cuda")
+    R.rmsmp_gemm_grouped_prepare(arr, R.OUT_NM, table)
+    torch.cuda.synchronize()
+    header = table[:128].cpu().numpy().view(np.int32)
+    slots, a_stages = int(header[5]), int(header[13])
+    assert a_stages % 2 == 0 and slots >= 2
+    assert slots % 2 == 0 or slots >= a_stages + 2
+
+
 def test_grouped_tensor_launch_mn_layout_and_single_layer():
     import torch
     keep, items, refs = _grouped_case([(384, 512), (200, 256)], 33, R.OUT_MN)
