@@ -1230,3 +1230,31 @@ def test_resident_weights_whose_last_row_block_is_short(M, variant):
         R.rmsmp_expand_weights(layer, d_packed, d_ws)
         R.rmsmp_conv_implicit_workspace_requant(layer, d_packed, d_ws, torch.from_numpy(act).cuda(), B, H, W, 1, 0, 0.25, 4.0, R.ACT_U4, codes)
         assert np.array_equal(codes.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("k,stride,pad,B,H,W,offset", [
+    (7, 2, 3, 3, 37, 64, 0),       # eight output rows a pass, the last one of an image has three
+    (7, 2, 3, 1, 9, 223, 1),       # two rows a pass; rows that start at any byte
+    (7, 3, 0, 2, 40, 65, 3),
+    (3, 2, 1, 2, 31, 31, 0),       # more rows a pass than pixels would need
+    (3, 1, 4, 1, 5, 6, 2),         # padding wider than the filter
+    (3, 2, 1, 1, 200, 500, 0),
+    (5, 2, 2, 2, 33, 47, 7),       # rows of five units
+    (5, 4, 2, 1, 17, 300, 0),
+    (7, 2, 3, 1, 3, 1, 5),         # a row of one pixel
+])
+def test_patch_matrix_of_three_channels(k, stride, pad, B, H, W, offset):
+    """Bytes are copied: the oracle's, and nothing around them."""
+    import torch
+    g = synth.rng(143, k + H + W)
+    act = g.integers(-128, 128, size=(B, H, W, 3), dtype=np.int8)
+    raw = torch.full((offset + act.size,), 77, dtype=torch.int8, device="cuda")
+    raw[offset:] = torch.from_numpy(act.reshape(-1)).cuda()
+    ld = (3 * k * k + 15) // 16 * 16
+    ref = O.im2col(act, k, k, stride, pad, ld)
+    out = torch.full((ref.size + 256,), 99, dtype=torch.int8, device="cuda")
+    R.rmsmp_im2col_codes(raw[offset:], B, H, W, 3, 3, k, k, stride, pad, out[128:], ld)
+    torch.cuda.synchronize()
+    got = out.cpu().numpy()
+    assert np.array_equal(got[128:-128].reshape(ref.shape), ref)
+    assert (got[:128] == 99).all() and (got[-128:] == 99).all()
