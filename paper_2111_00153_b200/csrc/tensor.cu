@@ -42,6 +42,7 @@ constexpr int kGroups = 2;                       // expander groups taking alter
 constexpr int kNumExpWarps = 4 * kGroups;
 __host__ __device__ constexpr int threads_of(int mode) { return 32 * (mode ? kPreWarps : 2 + kNumExpWarps + kNumEpiWarps); }
 constexpr int kWarpStage = 32 * 32 * 4;          // 4 KB: 32 pixels x 32 rows of fp32/int32
+constexpr int kWideEpi = 8;                      // epilogue warps of the form with 144 KB of resident weights
 constexpr int kMaxRing = 8;
 constexpr int kResidentBlocks = 16;              // row blocks of a layer with resident weights (the grid is a multiple of them)
 constexpr int kSmemLimit = 232448 - 1024;        // 227 KB per CTA less room for the static variables
@@ -84,9 +85,10 @@ struct TensorCfg {
     int tps;               // k-blocks per activation stage: 1, or 3 (resident weights, 64-byte k-blocks, 3-wide kernels):
                            //    one barrier round trip then covers a whole kernel row instead of a single tap
     int b_sub;             // bytes of one k-block inside an activation stage
-    int colshift;          // 1 (with tps == 3; 3x3, stride 1, tiles of whole output rows of one image, W % 8 == 0): an activation
+    int colshift;          // 1 (with tps == 3; 3x3, stride 1, tiles of whole output rows of one image): an activation
                            //    stage holds the th + 2 input rows the tile needs at ONE column shift j, fetched once; the
-                           //    taps (0..2, j) read it at row offsets of W pixels (whole swizzle atoms).  The copy engine
+                           //    taps (0..2, j) read it at row offsets of W pixels (the swizzle goes by the address: rows may start
+                           //    anywhere in its pattern; 3x3 64x48 on 60 images of 51x51 29.0 us without, 19.4 so).  The copy engine
                            //    then moves 3 (th + 2) rows per tile instead of 9 th
     uint32_t smem_bytes;
 };
@@ -325,7 +327,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                             // one stage = one column shift: the th + kh - 1 input rows the tile needs, fetched once
                             // and read by the kh taps of that column at row offsets (see TensorCfg::colshift)
                             mbar_arrive_expect_tx(bar_f + 8 * s, cfg.tx_bytes);
-                            tma_load_4d(sB + s * cfg.b_bytes, &maps.act[0], bar_f + 8 * s, 0, ti - p.pad, h0 - p.pad, b0);
+                            tma_load_4d(sB + s * cfg.b_bytes, &maps.act[0], bar_f + 8 * s, cc * cfg.bk, ti - p.pad, h0 - p.pad, b0);
+                            if (++cc == cfg.cpt) { cc = 0; ++ti; }
                         } else {
                             // one stage = the taps of one kernel row (one channel chunk per tap in this mode)
                             mbar_arrive_expect_tx(bar_f + 8 * s, cfg.tps * cfg.tx_bytes);
@@ -333,8 +336,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                                 const TapBox tb = tap_box(p, h0, ti, tj + t);
                                 tma_load_4d(sB + s * cfg.b_bytes + t * cfg.b_sub, &maps.act[tb.map], bar_f + 8 * s, 0, tb.x, tb.y, b0);
                             }
+                            ++ti;
                         }
-                        ++ti;
                         kb += cfg.tps - 1;
                         if (++s == nring) { s = 0; ph ^= 1; }
                         continue;
@@ -382,10 +385,11 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     // reading one buffer at three row offsets
                     const uint32_t a_step = (uint32_t)cfg.a_bytes >> 4, b_step = (uint32_t)cfg.b_bytes >> 4;
                     const uint32_t t_step = cfg.colshift ? ((uint32_t)(p.W * cfg.bk) >> 4) : ((uint32_t)cfg.b_sub >> 4);
-                    const uint32_t a_t = cfg.colshift ? 3 * a_step : a_step;       // between the three MMAs of a stage
+                    const uint32_t a_t = cfg.colshift ? 3 * a_step * (uint32_t)cfg.cpt : a_step;       // between the three taps of a stage
                     const uint32_t a_adv = cfg.colshift ? a_step : 3 * a_step;     // from stage to stage
                     uint32_t a_lo = desc_lo0_a, b_lo = desc_lo0_b + sb * b_step;
-                    const bool two = (cfg.last_ksteps == 2);
+                    const bool two_last = (cfg.last_ksteps == 2);
+                    bool two = two_last || cfg.cpt > 1;                            // (of two chunks the first is whole)
                     for (int kb = 0; kb < cfg.nkb; kb += 3) {
                         if (!mbar_wait(bar_fullB + 8 * sb, phB, abort_flag)) { ok = false; break; }
                         tc_fence_after();
@@ -400,6 +404,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                         }
                         a_lo += a_adv;
                         b_lo += b_step;
+                        if (cfg.cpt > 1) two = !two || two_last;
                         if (++sb == (uint32_t)cfg.nB) { sb = 0; phB ^= 1; b_lo = desc_lo0_b; }
                     }
                 } else if (!kAres && cfg.bk == 128 && cfg.last_ksteps == 4) {
@@ -632,7 +637,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             sa += kGroups; while (sa >= (uint32_t)cfg.nA) { sa -= cfg.nA; phA ^= 1; }
         }
         __syncwarp();
-    } else {
+    } else if (warp >= kThreads / 32 - cfg.epi_warps) {
         // ---------------------------------------------------------- epilogue
         // Warp w may read tensor-memory lanes 32*(w%4)..+31.  The warps that share a quarter (one, or
         // three in pre mode) take alternate 32-pixel chunks; with duplicated rows the two quarters
@@ -919,6 +924,20 @@ bool encode_act_maps(EncodeTiledFn enc, const Problem& p, int bk, int th, int tb
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// One row block of a 3x3 convolution of step one with 65 to 128 channels, on expanded weights: they stay resident (144 KB, as two
+// 64-channel k-blocks a tap) beside a ring of column-shift stages, from two tiles per CTA up.  Through the rings a tile brings 373 KB
+// into the SM, so 97: 128x128 on 256 images of 28x28 36.0 against 34.8 us, codes out 35.0 and 29.4 (three stages, and
+// eight epilogue warps, are what fits).
+bool wide_shift(const Problem& p)
+{
+    const int most = p.Wo <= kTileN ? kTileN / p.Wo : 0;
+    if (!p.wexp || p.nblocks != 1 || p.Cin <= 64 || p.Cin > 128 || p.kh != 3 || p.kw != 3 || p.stride != 1 || p.pad != 1 || most < 1) return false;
+    if ((int64_t)p.Ho * p.Wo <= kTileN && 2 * (int64_t)p.Ho * p.Wo <= kTileN) return false;      // (several images a tile)
+    const int per_image = (p.Ho + most - 1) / most, th = (p.Ho + per_image - 1) / per_image;
+    return 3 * (((th + 2) * p.W * 64 + 1023) / 1024 * 1024) <= kSmemLimit - (1024 + 64 * kMaxRing) - 18 * kBlockRows * 64 - kWideEpi * kWarpStage &&
+           (int64_t)p.B * per_image >= 2 * sm_count();
+}
+
 bool plan(const Problem& p, TensorCfg& c)
 {
     if (p.pix_pitch % 16 != 0 || (p.Cin % 16 != 0 && !p.ragged_k)) return false;
@@ -993,7 +1012,8 @@ bool plan(const Problem& p, TensorCfg& c)
     // layer runs in the workspace form
     if (!p.wexp && resident) { c.pre = 1; c.fill = 1; }
     // 64-byte k-blocks when a 128-byte row would be at most half used by the (last) channel chunk
-    c.bk = (c.pre ? p.Cin % 128 != 0 && p.Cin % 128 <= 64 : p.Cin <= 64) ? 64 : 128;
+    const bool wide = wide_shift(p);
+    c.bk = wide || (c.pre ? p.Cin % 128 != 0 && p.Cin % 128 <= 64 : p.Cin <= 64) ? 64 : 128;
     c.a_bytes = kBlockRows * c.bk;
     c.b_bytes = kTileN * c.bk;
     c.cpt = (p.Cin + c.bk - 1) / c.bk;
@@ -1015,7 +1035,7 @@ bool plan(const Problem& p, TensorCfg& c)
         c.dup = (p.M <= 64) ? 1 : 0;
         if (resident) {
             c.ares = 1;
-            c.epi_warps = kPreWarps - 2;
+            c.epi_warps = wide ? kWideEpi : kPreWarps - 2;
             c.nA = c.nkb;
             const int64_t left = kSmemLimit - (1024 + 64 * kMaxRing) - (int64_t)c.nkb * c.a_bytes -
                                  (int64_t)c.epi_warps * kWarpStage;
@@ -1023,11 +1043,11 @@ bool plan(const Problem& p, TensorCfg& c)
         }
         c.tps = 1;
         c.b_sub = c.b_bytes;
-        if (c.ares && c.bk == 64 && c.cpt == 1 && p.kw == 3 && c.last_ksteps <= 2) {
+        if (c.ares && c.bk == 64 && (c.cpt == 1 || wide) && p.kw == 3 && c.last_ksteps <= 2) {
             c.tps = 3;
             c.b_sub = (c.n_mma * c.bk + 1023) / 1024 * 1024;
             c.b_bytes = c.tps * c.b_sub;
-            if (p.kh == 3 && p.stride == 1 && p.Wo == p.W && c.tb == 1 && p.W % 8 == 0 && c.npix == c.th * p.W) {
+            if (p.kh == 3 && p.stride == 1 && p.Wo == p.W && c.tb == 1 && c.npix == c.th * p.W) {
                 c.colshift = 1;
                 c.tx_bytes = (uint32_t)((c.th + 2) * p.W * c.bk);
                 c.b_bytes = ((c.th + 2) * p.W * c.bk + 1023) / 1024 * 1024;
@@ -1121,6 +1141,7 @@ bool tensor_resident(const Problem& p)
     if (!p.wexp && p.rq_codes) return false;
     const int64_t sms = sm_count(), tiles = (p.N + kTileN - 1) / kTileN * p.nblocks, whole = sms / p.nblocks * p.nblocks;
     if (whole == 0 || (p.nblocks > kResidentBlocks && (tiles + whole - 1) / whole > (tiles + sms - 1) / sms)) return false;
+    if (wide_shift(p)) return true;
     const int bk = ((p.Cin % 128 != 0) && (p.Cin % 128 <= 64)) ? 64 : 128;
     const int64_t bytes = (int64_t)p.kh * p.kw * ((p.Cin + bk - 1) / bk) * kBlockRows * bk;
     if (bytes > 72 * 1024) return false;

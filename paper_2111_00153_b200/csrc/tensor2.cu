@@ -37,6 +37,8 @@ constexpr int kEpiWarps2 = 8;
 constexpr int kFirstEpi2 = 6;                   // warps 6-13, two per tensor-memory quarter
 constexpr int kRing2 = 3;                       // stages; a stage holds TWO k-blocks of each operand (64 KB per CTA)
 constexpr int kSub2 = 2;
+constexpr int kPairSmem = 232448 - 1024;         // 227 KB per CTA less room for the static variables
+constexpr int kPairRest = kEpiWarps2 * kWarpStage2 + 1024 + 64 * 2 * kRing2;      // all but the stages
 constexpr long long kWaitCycles2 = 2000000000LL;
 
 struct PairCfg {
@@ -50,9 +52,14 @@ struct PairCfg {
     int64_t ntiles;          // ntiles_n * nbt
     int cpt;                 // 128-channel chunks per tap
     int nkb;                 // k-blocks per tile
+    int shift;               // 1: column-shift stages (see plan_pair)
+    int ring, b_stage;       // stages; bytes of a stage's activation operand
+    int img_pix, img_cols;   // pixels stored as one run and the accumulator columns from one run to the next: all of a half,
+                             // or (column shift) an image's
+    int runs;                // of them in a half
     uint32_t idesc;
     uint32_t tx_b;           // bytes one activation box brings
-    int tail_rows;           // npix_h % 32
+    int tail_rows;           // img_pix % 32
     uint32_t smem_bytes;
 };
 
@@ -193,14 +200,18 @@ __device__ __forceinline__ HalfPos half_pos(const Problem& p, const PairCfg& cfg
     return r;
 }
 
+// kShift: column-shift stages (PairCfg::shift).
+template <bool kShift>
 __global__ void __launch_bounds__(kThreads2, 1)
 pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps maps)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (s32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sA = smem_base;
-    const uint32_t sB = sA + kRing2 * kSub2 * kStageA;
-    const uint32_t sOut = sB + kRing2 * kSub2 * kStageB;
+    const int ring = kShift ? cfg.ring : kRing2;
+    const uint32_t a_stage = kShift ? 3 * kStageA : kSub2 * kStageA, b_stage = kShift ? (uint32_t)cfg.b_stage : kSub2 * kStageB;
+    const uint32_t sB = sA + ring * a_stage;
+    const uint32_t sOut = sB + ring * b_stage;
     const uint32_t sBar = sOut + kEpiWarps2 * kWarpStage2;
     const uint32_t bar_full = sBar, bar_empty = sBar + 8 * kRing2;
     const uint32_t bar_tfull = sBar + 16 * kRing2, bar_tempty = bar_tfull + 16;
@@ -211,7 +222,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     const uint32_t rank = cluster_rank();                 // 0 = leader: owns the "full" and "accumulator free" barriers
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kRing2; ++s) {
+        for (int s = 0; s < kRing2; ++s) {               // (a ring has no more stages than that)
             bar_init(bar_full + 8 * s, 1);       // the leader's activation producer announces all four copies' bytes; leader only
             bar_init(bar_empty + 8 * s, 1);      // the leader's commit, delivered to both CTAs
         }
@@ -238,7 +249,39 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     const int64_t first = blockIdx.x >> 1, step = gridDim.x >> 1;      // cluster index, clusters in the grid
     const uint32_t lead_full = map_to_rank(bar_full, 0), lead_tempty = map_to_rank(bar_tempty, 0);
 
-    if (warp == 0 || warp == 2 || warp == 3 || warp == 4) {
+    if (kShift && (warp == 0 || (warp >= 2 && warp <= 4))) {
+        // ---------------------------------------------------------- producers, column-shift stages
+        // A stage is one kernel column j of one channel chunk: warp 0 fetches the th + 2 input rows at that shift, warps 2 to 4
+        // the weights of the taps (0, j), (1, j), (2, j).
+        if (lane == 0) {
+            const int ti = warp - 2;
+            uint32_t s = 0, ph = 0;
+            bool ok = true;
+            for (int64_t tile = first; tile < cfg.ntiles && ok; tile += step) {
+                const int64_t nt = tile / cfg.nbt;
+                const int blk = (int)(tile - nt * cfg.nbt) * 2 + (int)rank;
+                const HalfPos hp = half_pos(p, cfg, 2 * nt + rank);
+                int cc = 0, tj = 0;
+                for (int st = 0; st < 3 * cfg.cpt; ++st) {
+                    if (!bar_wait(bar_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
+                    const uint32_t fb = lead_full + 8 * s;
+                    if (warp == 0) {
+                        if (rank == 0)
+                            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                                         ::"r"(bar_full + 8 * s), "r"(2u * (cfg.tx_b + 3u * (uint32_t)kStageA)) : "memory");
+                        pair_load_4d(sB + s * b_stage, &maps.act[0], fb, cc * 128, tj - 1, hp.h0 - 1, hp.b0);
+                    } else {
+                        pair_load_2d(sA + s * a_stage + ti * kStageA, &maps.wexp, fb, (3 * ti + tj) * p.Cp + cc * 128, blk * kBlockRows);
+                    }
+                    if (++s == (uint32_t)ring) { s = 0; ph ^= 1; }
+                    if (++tj == 3) { tj = 0; ++cc; }
+                }
+            }
+            if (!ok) {
+                for (int i = 0; i < 200; ++i) __nanosleep(1000);   // let copies in flight land
+            }
+        }
+    } else if (!kShift && (warp == 0 || warp == 2 || warp == 3 || warp == 4)) {
       if (lane == 0) {
         // ---------------------------------------------------------- producers (both CTAs)
         // One thread can start a bulk tensor copy only every ~300 ns, about the time four MMAs take,
@@ -287,7 +330,8 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
             uint32_t s = 0, ph = 0, it = 0;
             const uint32_t hi = (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);     // SBO 1024 B, version 1, 128-byte swizzle
             const uint32_t a_lo0 = ((sA >> 4) & 0x3FFFu) | (1u << 16), b_lo0 = ((sB >> 4) & 0x3FFFu) | (1u << 16);
-            const uint32_t a_step = (kSub2 * kStageA) >> 4, b_step = (kSub2 * kStageB) >> 4;
+            const uint32_t a_step = a_stage >> 4, b_step = b_stage >> 4;
+            const uint32_t row_step = (uint32_t)(p.W * 128) >> 4;                      // (column shift) a tap's rows lie W pixels further on
             uint32_t a_lo = a_lo0, b_lo = b_lo0;
             for (int64_t tile = first; tile < cfg.ntiles && !*abort_flag; tile += step, ++it) {
                 const uint32_t ab = it & 1;
@@ -295,10 +339,22 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d_tmem = tmem_base + ab * 256;
                 bool ok = true;
-                for (int kb = 0; kb < cfg.nkb; kb += kSub2) {
+                for (int kb = 0; kb < cfg.nkb; kb += kShift ? 3 : kSub2) {
                     if (!bar_wait(bar_full + 8 * s, ph, abort_flag)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    if (issuer) {
+                    if (kShift) {
+                        if (issuer) {
+#pragma unroll
+                            for (int i = 0; i < 3; ++i) {
+                                const uint32_t a1 = a_lo + i * (kStageA >> 4), b1 = b_lo + i * row_step;
+                                pair_mma(d_tmem, a1, b1, hi, cfg.idesc, (kb | i) ? 1u : 0u);
+                                pair_mma(d_tmem, a1 + 2, b1 + 2, hi, cfg.idesc, 1u);
+                                pair_mma(d_tmem, a1 + 4, b1 + 4, hi, cfg.idesc, 1u);
+                                pair_mma(d_tmem, a1 + 6, b1 + 6, hi, cfg.idesc, 1u);
+                            }
+                            pair_commit(bar_empty + 8 * s);
+                        }
+                    } else if (issuer) {
                         pair_mma(d_tmem, a_lo, b_lo, hi, cfg.idesc, kb ? 1u : 0u);
                         pair_mma(d_tmem, a_lo + 2, b_lo + 2, hi, cfg.idesc, 1u);
                         pair_mma(d_tmem, a_lo + 4, b_lo + 4, hi, cfg.idesc, 1u);
@@ -314,7 +370,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                     }
                     a_lo += a_step;
                     b_lo += b_step;
-                    if (++s == kRing2) { s = 0; ph ^= 1; a_lo = a_lo0; b_lo = b_lo0; }
+                    if (++s == (uint32_t)ring) { s = 0; ph ^= 1; a_lo = a_lo0; b_lo = b_lo0; }
                 }
                 if (!ok) break;
                 if (issuer) pair_commit(bar_tfull + 8 * ab);
@@ -328,7 +384,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
         const int my_rank = (warp - (first_epi + ((quarter - first_epi) & 3))) >> 2;
         const int cstride = count_q(quarter);
         const uint32_t my_stage = sOut + (uint32_t)(warp - first_epi) * kWarpStage2;
-        const int nch = (cfg.npix_h + 31) >> 5;              // 32-pixel chunks per half
+        const int nch = (cfg.img_pix + 31) >> 5;             // 32-pixel chunks per run of pixels
         uint32_t it = 0;
         bool alive = true;
         for (int64_t tile = first; tile < cfg.ntiles && alive; tile += step, ++it) {
@@ -349,12 +405,14 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + ab * 256;
             const bool rows_ok = blk * kBlockRows + quarter * 32 < p.M;
-            // chunk index i = h * nch + c; this warp takes i = my_rank, my_rank + cstride, ...
+            // chunk index i = (h * runs + e) * nch + c; this warp takes i = my_rank, my_rank + cstride, ...
             uint32_t v[32];
-            for (int i = my_rank; i < 2 * nch; i += cstride) {
-                const int h = i >= nch, c = i - h * nch;
-                if (!rows_ok || c * 32 >= nvalid[h]) continue;
-                ld_issue(taddr + h * cfg.nh_pad + c * 32, v);
+            const int per_half = kShift ? cfg.runs * nch : nch;
+            for (int i = my_rank; i < 2 * per_half; i += cstride) {
+                const int h = i >= per_half, u = i - h * per_half, e = kShift ? u / nch : 0, c = u - e * nch;
+                const int at = e * cfg.img_pix + c * 32;                 // the chunk's first pixel in its half
+                if (!rows_ok || at >= nvalid[h]) continue;
+                ld_issue(taddr + h * cfg.nh_pad + e * cfg.img_cols + c * 32, v);
                 ld_wait(v);
                 if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 __syncwarp();
@@ -367,8 +425,8 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) {
-                    const bool tail = cfg.tail_rows && (c == (cfg.npix_h >> 5));
-                    store_2d(tail ? &maps.out_tail : &maps.out_full, my_stage, blk * kBlockRows + quarter * 32, (int)(n0h[h] + c * 32));
+                    const bool tail = cfg.tail_rows && (c == (cfg.img_pix >> 5));
+                    store_2d(tail ? &maps.out_tail : &maps.out_full, my_stage, blk * kBlockRows + quarter * 32, (int)(n0h[h] + at));
                 }
             }
             // accumulators of this tile are out of tensor memory: tell the leader
@@ -431,17 +489,45 @@ bool plan_pair(const Problem& p, PairCfg& c)
     }
     if ((int64_t)c.th * p.stride > 256) return false;
     c.npix_h = c.tb * c.th * p.Wo;
-    c.nh_pad = (c.npix_h + 7) / 8 * 8;
-    c.ntiles_n = (c.nhalves + 1) / 2;
-    c.nbt = p.nblocks / 2;
-    c.ntiles = c.ntiles_n * c.nbt;
     c.cpt = p.Cin / 128;
     c.nkb = p.kh * p.kw * c.cpt;
     c.tx_b = (uint32_t)c.npix_h * 128u;
-    c.tail_rows = c.npix_h & 31;
+    c.shift = 0;
+    c.ring = kRing2;
+    c.b_stage = kSub2 * kStageB;
+    c.runs = 1;
+    c.img_pix = c.img_cols = c.npix_h;
+    // Column-shift stages (3x3, step one): a stage holds, for one kernel column and channel chunk, the th + 2 input rows of the half
+    // once and the weights of the three taps of that column, which read it at row offsets of W pixels (of several images, with the
+    // staged rows between them as accumulator columns that nobody stores).  Where a pixel then costs fewer rows of copies
+    // (weights: 128 rows of nine taps to a half) and two stages fit: 256x256 on 256 images of 14x14 30.6 us without, 29.0 so, 512x512
+    // of 7x7 26.9 and 26.0, 256x256 on 64 of 29x29 32.0 and 31.7.
+    if (p.kh == 3 && p.kw == 3 && p.stride == 1 && p.pad == 1) {
+        const int hw1 = p.Ho * p.Wo, pitch = (c.th + 2) * p.W;           // staged pixels from one image to the next
+        const int tb = c.halves_per_image || hw1 > 128 ? 1 : std::min(c.tb, (128 - hw1) / pitch + 1);
+        const int rows = tb * pitch, pix = tb * c.th * p.Wo;
+        const int64_t stage = 3 * kStageA + ((int64_t)rows * 128 + 1023) / 1024 * 1024;
+        const int ring = (int)std::min<int64_t>(kRing2, (kPairSmem - kPairRest) / stage);
+        if (ring >= 2 && c.th + 2 <= 256 && (1152.0 + 3 * rows) / pix < (1152.0 + 9 * c.npix_h) / c.npix_h) {
+            c.shift = 1;
+            c.ring = ring;
+            c.b_stage = (int)stage - 3 * kStageA;
+            if (tb != c.tb) { c.tb = tb; c.nhalves = (p.B + tb - 1) / tb; }
+            c.npix_h = pix;
+            c.tx_b = (uint32_t)rows * 128u;
+            c.runs = tb;
+            c.img_pix = c.th * p.Wo;
+            c.img_cols = pitch;
+        }
+    }
+    c.nh_pad = (c.shift ? (c.runs - 1) * c.img_cols + c.img_pix + 7 : c.npix_h + 7) / 8 * 8;
+    c.ntiles_n = (c.nhalves + 1) / 2;
+    c.nbt = p.nblocks / 2;
+    c.ntiles = c.ntiles_n * c.nbt;
+    c.tail_rows = c.img_pix & 31;
     // kind::i8, int32 accumulate, signed 8-bit A and B, K-major; N = both halves, M = 256 over the pair
     c.idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * c.nh_pad) >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
-    c.smem_bytes = (uint32_t)(kRing2 * kSub2 * (kStageA + kStageB) + kEpiWarps2 * kWarpStage2 + 1024 + 64 * 2 * kRing2);
+    c.smem_bytes = (uint32_t)(c.ring * ((c.shift ? 3 * kStageA : kSub2 * kStageA) + c.b_stage) + kPairRest);
     return true;
 }
 
@@ -464,7 +550,7 @@ rmsmp_status launch_pair(const Problem& p, cudaStream_t st)
     if (!enc) return RMSMP_ERR_CUDA;
     PairMaps mp;
     memset(&mp, 0, sizeof(mp));
-    if (!encode_act_maps_4(p, 128, c.th, c.tb, mp.act)) return RMSMP_ERR_CUDA;
+    if (!encode_act_maps_4(p, 128, c.shift ? c.th + 2 : c.th, c.tb, mp.act)) return RMSMP_ERR_CUDA;
     {
         const cuuint64_t gd[2] = {(cuuint64_t)p.Kp, (cuuint64_t)p.M};
         const cuuint64_t gs[1] = {(cuuint64_t)p.Kp};
@@ -486,8 +572,9 @@ rmsmp_status launch_pair(const Problem& p, cudaStream_t st)
     if (!make_out(&mp.out_full, 32)) return RMSMP_ERR_CUDA;
     if (c.tail_rows && !make_out(&mp.out_tail, c.tail_rows)) return RMSMP_ERR_CUDA;
 
-    static bool attr_set[kMaxDevices] = {};
-    if (!ensure_smem_attr(reinterpret_cast<const void*>(pair_kernel), (int)c.smem_bytes, attr_set)) return RMSMP_ERR_CUDA;
+    void (*const kernel)(const Problem, const PairCfg, const PairMaps) = c.shift ? pair_kernel<true> : pair_kernel<false>;
+    static bool attr_set[2][kMaxDevices] = {};
+    if (!ensure_smem_attr(reinterpret_cast<const void*>(kernel), kPairSmem, attr_set[c.shift])) return RMSMP_ERR_CUDA;
     const int clusters = (int)std::min<int64_t>(c.ntiles, sm_count() / 2);
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof(lc));
@@ -502,7 +589,7 @@ rmsmp_status launch_pair(const Problem& p, cudaStream_t st)
     at[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = 2;
-    if (cudaLaunchKernelEx(&lc, pair_kernel, p, c, mp) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&lc, kernel, p, c, mp) != cudaSuccess) {
         cudaGetLastError();
         return RMSMP_ERR_CUDA;
     }

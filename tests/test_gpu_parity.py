@@ -1232,6 +1232,58 @@ def test_resident_weights_whose_last_row_block_is_short(M, variant):
         assert np.array_equal(codes.cpu().numpy(), want)
 
 
+# ------------------------------------------------------------------ column-shift stages
+
+def _check_some_images(Wt, scheme, bits, alpha, act, stride, pad, y, acc, images):
+    """Sums and outputs of those images against the oracle's convolution of them alone."""
+    M, B = Wt.shape[0], act.shape[0]
+    _, _, acc_ref, y_ref = O.layer_conv(Wt, scheme, bits, alpha, np.ascontiguousarray(act[images]), np.float32(0.25), stride, pad)
+    assert np.array_equal(y.reshape(B, -1, M)[images].view(np.uint32), y_ref.reshape(len(images), -1, M).view(np.uint32))
+    if acc is not None:
+        assert np.array_equal(acc.reshape(B, -1, M)[images], acc_ref.reshape(len(images), -1, M))
+
+
+@pytest.mark.parametrize("M,Cin,B,H,W", [
+    (48, 64, 300, 13, 11),         # rows of 11 pixels: a tap's rows start anywhere in the swizzle pattern
+    (100, 32, 35, 37, 35),        # tiles of seven rows, the last one repeats rows; one 32-code step a tap
+    (64, 48, 16, 51, 51),
+    (128, 80, 150, 29, 9),        # two chunks a tap (the second of one step), weights of 144 KB resident
+    (20, 128, 150, 29, 9),        # the same with duplicated rows
+    (72, 96, 300, 15, 17),        # one image of 255 pixels a tile
+])
+def test_column_shift_stages_of_any_width(M, Cin, B, H, W):
+    g = synth.rng(140, M + Cin + W)
+    Wt = synth.weights_kaiming(g, M, Cin, 3, 3)
+    scheme, bits = _mixed_map(M, 11, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    act = g.integers(-16, 17, size=(B, H, W, Cin)).astype(np.int8)
+    images = sorted({0, 1, B // 2, B - 1})
+    for want_acc in (True, False):
+        y, acc = Hn.conv(layer, d_packed, act, 1, 1, 0.25, Hn.WORKSPACE, want_acc=want_acc)
+        _check_some_images(Wt, scheme, bits, alpha, act, 1, 1, y, acc, images)
+
+
+@pytest.mark.parametrize("Cin,B,H,W", [
+    (256, 387, 7, 7),             # two images a half with staged rows between them, the last half has one
+    (256, 200, 11, 13),           # halves of six rows, the last of an image repeats one
+    (256, 100, 14, 14),
+    (384, 230, 9, 9),             # three channel chunks, an image a half
+    (256, 40, 5, 100),            # halves of a row: no column shift
+    (256, 35, 20, 28),            # stages so large that two of them make the ring
+])
+def test_column_shift_stages_of_cta_pairs(Cin, B, H, W):
+    M = 256
+    g = synth.rng(141, Cin + W)
+    Wt = synth.weights_kaiming(g, M, Cin, 3, 3)
+    scheme, bits = _mixed_map(M, 12, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    act = g.integers(-16, 17, size=(B, H, W, Cin)).astype(np.int8)
+    y, _ = Hn.conv(layer, d_packed, act, 1, 1, 0.25, Hn.WORKSPACE, want_acc=False)
+    _check_some_images(Wt, scheme, bits, alpha, act, 1, 1, y, None, sorted({0, 1, B // 2, B - 2, B - 1}))
+
+
 @pytest.mark.parametrize("k,stride,pad,B,H,W,offset", [
     (7, 2, 3, 3, 37, 64, 0),       # eight output rows a pass, the last one of an image has three
     (7, 2, 3, 1, 9, 223, 1),       # two rows a pass; rows that start at any byte
