@@ -1284,6 +1284,40 @@ def test_column_shift_stages_of_cta_pairs(Cin, B, H, W):
     _check_some_images(Wt, scheme, bits, alpha, act, 1, 1, y, None, sorted({0, 1, B // 2, B - 2, B - 1}))
 
 
+@pytest.mark.parametrize("kind", [R.ACT_U4, R.ACT_S4])
+@pytest.mark.parametrize("M,Cin,k,B,H,W,ld_extra", [
+    (144, 32, 1, 40, 31, 33, 16),       # a second row block of one 16-byte piece, ragged tiles, padding columns
+    (48, 64, 3, 100, 21, 19, 0),        # duplicated rows, 48 of 64; column shift
+    (128, 128, 3, 150, 29, 9, 0),       # resident weights of two chunks a tap
+])
+def test_requantized_codes_leave_in_sixteen_byte_pieces(M, Cin, k, B, H, W, ld_extra, kind):
+    import torch
+    g = synth.rng(142, M + Cin)
+    Wt = synth.weights_kaiming(g, M, Cin, k, k)
+    scheme, bits = O.assign_rows(Wt, (60, 35, 5))
+    alpha = synth.alpha_rows(Wt)
+    act = synth.act_codes_uniform(g, (B, H, W, Cin))
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    ws = torch.empty(R.rmsmp_workspace_bytes(layer), dtype=torch.int8, device="cuda")
+    R.rmsmp_expand_weights(layer, d_packed, ws)
+    N, pad = B * H * W, k // 2
+    images = [0, B // 2, B - 1]
+    _, _, _, y_ref = O.layer_conv(Wt, scheme, bits, alpha, np.ascontiguousarray(act[images]), np.float32(0.125), 1, pad)
+    na = _next_alpha(y_ref)
+    want, _ = O.quantize_act(y_ref.reshape(len(images), H * W, M), na, kind)
+    a = torch.from_numpy(act).cuda()
+    out = torch.full((N, M + ld_extra), 99, dtype=torch.int8, device="cuda")
+    if ld_extra:
+        R.rmsmp_gemm_workspace_requant(layer, d_packed, ws, a, N, Cin, 0.125, na, kind, out, M + ld_extra)
+    else:
+        R.rmsmp_conv_implicit_workspace_requant(layer, d_packed, ws, a, B, H, W, 1, pad, 0.125, na, kind, out)
+    torch.cuda.synchronize()
+    assert R.rmsmp_last_device_status(d_packed) == R.OK
+    got = out.cpu().numpy()
+    assert np.array_equal(got[:, :M].reshape(B, H * W, M)[images], want)
+    assert (got[:, M:] == 99).all()
+
+
 @pytest.mark.parametrize("k,stride,pad,B,H,W,offset", [
     (7, 2, 3, 3, 37, 64, 0),       # eight output rows a pass, the last one of an image has three
     (7, 2, 3, 1, 9, 223, 1),       # two rows a pass; rows that start at any byte
