@@ -140,6 +140,12 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t sr
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
+// Fetches a descriptor, so that the first copy through it does not wait for that.
+__device__ __forceinline__ void tensormap_prefetch(const CUtensorMap* m)
+{
+    asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major rows of `row_bytes` (128 or 64) with the swizzle of that
 // width; groups of 8 rows are 8*row_bytes apart.
 __device__ __forceinline__ uint64_t smem_desc_kmajor(uint32_t addr, int row_bytes)

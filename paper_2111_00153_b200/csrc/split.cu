@@ -112,8 +112,8 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     __syncthreads();
     tc_fence_after();
     if (cfg.S > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");      // this CTA runs: its shared memory may be written
-    pdl_wait();
-    pdl_trigger();
+    // From here on the weights: packed codes, their rows' places and scales, or the expanded copy.  What the kernel in front
+    // writes or reads -- activations, outputs, the status word -- stays behind the waits further down (see launch_dependent).
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
 
@@ -126,6 +126,12 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     if ((warp == 0 && !kGather) || (warp == kSplitFirst && kPre)) {
         // ---------------------------------------------------------- TMA producers
         if (lane == 0) {
+            if (warp == 0) {
+                tensormap_prefetch(&maps.act[0]);
+                if (act_parity_split(p)) { tensormap_prefetch(&maps.act[1]); tensormap_prefetch(&maps.act[2]); tensormap_prefetch(&maps.act[3]); }
+                pdl_wait();
+                pdl_trigger();
+            }
             int tap = kb0 / cfg.cpt, cc = kb0 - tap * cfg.cpt;
             int ti = tap / p.kw, tj = tap - ti * p.kw;
             int s = 0;
@@ -182,10 +188,9 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         const uint8_t* src = p.q4;
         if (m_row < p.M) {
             kind = p.kind[m_row];
-            const int packed = __ldg(pdl_ordered(p.slot) + m_row);
+            const int packed = __ldg(p.slot + m_row);
             src = kind == kFixed8 ? p.q8 + (size_t)(packed - p.nP - p.nF4) * p.Kp : p.q4 + (size_t)packed * (p.Kp >> 1);
         }
-        src = pdl_ordered(src);
         const uint32_t swz = cfg.bk == 128 ? (uint32_t)(row & 7) : (uint32_t)((row >> 1) & 3);
         const uint32_t row_off = (uint32_t)row * (uint32_t)cfg.bk;
         // The codes of a k-block are in registers before its turn comes: the next one's are loaded as soon as this one's
@@ -201,7 +206,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         auto pieces_of = [&](int ksteps) { return kind < 0 ? 0 : (eight ? 2 * ksteps : ksteps); };      // 16-byte pieces of a row
         // this thread's pixel of the tile (kGather): its image, and the input position of its tap (0, 0)
         int px_y = 0, px_x = 0;
-        const int8_t* px_img = pdl_ordered(p.act);
+        const int8_t* px_img = p.act;
         const bool px_ok = kGather && row < cfg.npix && (int64_t)nt * cfg.npix + row < p.N;
         if (px_ok) {
             const uint32_t n = (uint32_t)((int64_t)nt * cfg.npix + row), t = n / (uint32_t)p.Wo, b = t / (uint32_t)p.Ho;
@@ -215,6 +220,11 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
             const int pieces = pieces_of(ksteps);
 #pragma unroll
             for (int u = 0; u < 8; ++u) raw[u] = u < pieces ? __ldg(q + u) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        if (kGather) {
+            pdl_wait();
+            pdl_trigger();
+            px_img = pdl_ordered(px_img);
         }
         for (int i = grp; i < n_kb; i += 3) {
             const int s = i % cfg.nst;
@@ -303,9 +313,10 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     float scale = 0.0f;
     int shift = 0;
     if (row_ok) {
-        scale = __fmul_rn(__ldg(pdl_ordered(p.wstep) + m), p.act_step);
-        shift = (!kPre && __ldg(pdl_ordered(p.kind) + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
+        scale = __fmul_rn(__ldg(p.wstep + m), p.act_step);
+        shift = (!kPre && __ldg(p.kind + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
     }
+    pdl_wait();                                           // the outputs
     const ActFast rq = act_fast_setup(kRQ ? p.rq_alpha : 1.0f, kRQ ? p.rq_kind : 0);
     const bool out_mn = !kRQ && p.out_mn != 0;
     // the finished sum of this lane's row at column j of the tile

@@ -232,12 +232,6 @@ __device__ __forceinline__ void mma_f8f6f4_tmem_a(uint32_t d_tmem, uint32_t a_tm
         : "memory");
 }
 
-// The tensor maps live in the table in global memory (written by a copy before the launch); fetching a
-// tile's descriptor one tile ahead keeps its first copy from waiting for it.
-__device__ __forceinline__ void tensormap_prefetch(const CUtensorMap* m)
-{
-    asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
-}
 // E4M3 copies of the activation codes of every layer with PoT rows: [N][Kp], zeros beyond the layer's
 // reduction length.  blockIdx.y = layer; layers whose bytes can be read as they are have no copy.  The launch behind
 // waits for this kernel, so it is all latency: the table is read ahead of the wait for the launch in front, a thread
@@ -419,7 +413,8 @@ stream_kernel(const uint8_t* __restrict__ table)
                 const int bi = box_index(v.rows);
                 const CUtensorMap* map = (v.kind == kFixed8) ? &v.P->q8[bi] : &v.P->q4[bi];
                 if (it + 1 < it1) {
-                    // fetch the next tile's descriptor now, so that its first copy does not wait for it
+                    // (the tensor maps live in the table, in global memory: the next tile's descriptor is fetched now, so that
+                    // its first copy does not wait for it)
                     const ItemView nv = view(it + 1);
                     const int nb = box_index(nv.rows);
                     tensormap_prefetch((nv.kind == kFixed8) ? &nv.P->q8[nb] : &nv.P->q4[nb]);

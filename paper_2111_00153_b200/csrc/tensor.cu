@@ -121,7 +121,6 @@ __device__ __forceinline__ void fill_resident_weights(const Problem& p, const Te
         const int kind = have ? (int)p.kind[m] : kFixed8;
         const int slot = have ? p.slot[m] : 0;
         const uint8_t* src = (kind == kFixed8) ? p.q8 + (size_t)(have ? slot - n4 : 0) * p.Kp : p.q4 + (size_t)slot * (p.Kp >> 1);
-        src = pdl_ordered(src);
         const uint32_t phase = (cfg.bk == 128) ? (uint32_t)(r & 7) : (uint32_t)((r >> 1) & 3);
         const uint32_t row_base = sA + (uint32_t)r * (uint32_t)cfg.bk;
         const int pieces = cfg.nkb << pshift;
@@ -255,7 +254,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();                                           // and no trigger: see launch_dependent
+    // (the weights are read ahead of the wait for the kernel in front, activations and outputs behind it; no trigger: see
+    // launch_dependent)
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
 
@@ -300,6 +300,10 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     if (dup) tma_load_2d(dst + cfg.a_bytes / 2, map, bar_fullA, koff, my_blk * kBlockRows);
                     if (++cc == cfg.cpt) { cc = 0; ++tap; }
                 }
+            }
+            if (pre_b_producer) {
+                tensormap_prefetch(&maps.act[0]);
+                pdl_wait();
             }
             const uint32_t nring = pre_b_producer ? (uint32_t)cfg.nB : (uint32_t)cfg.nA;
             const uint32_t bar_e = pre_b_producer ? bar_emptyB : bar_emptyA;
@@ -496,8 +500,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         const int64_t total = my_tiles * cfg.nkb;
         const bool rows_change = step % (uint32_t)p.nblocks != 0u;
         // a row block's rows in the packed buffer: first and number of each kind
-        const int32_t* const blocks = pdl_ordered(p.blocks), *const perm = pdl_ordered(p.perm);
-        const uint4* const codes = reinterpret_cast<const uint4*>(pdl_ordered(p.q4));
+        const int32_t* const blocks = p.blocks, *const perm = p.perm;
+        const uint4* const codes = reinterpret_cast<const uint4*>(p.q4);
         int4 blk_a;
         int2 blk_b;
         int blk_next = 0;
@@ -656,6 +660,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         int scale_blk = -1, shift = 0;
         float scale = 0.f;
         const ActFast rq_fast = act_fast_setup(kRQ ? p.rq_alpha : 1.0f, kRQ ? p.rq_kind : 0);
+        pdl_wait();                                                        // the outputs
         for (uint32_t tile = first; tile < ntiles && alive; tile += step, ++it) {
           // a tile is one row block (accumulators alternate between tiles), or two (one accumulator each)
           for (int half = 0; half <= kM2; ++half) {
@@ -681,8 +686,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 scale = 0.f;
                 shift = 0;
                 if (row_ok) {
-                    scale = __fmul_rn(__ldg(pdl_ordered(p.wstep) + m), p.act_step);
-                    shift = (!kPre && __ldg(pdl_ordered(p.kind) + m) == kFixed4) ? 4 : 0;   // expanders store Fixed-4 codes as 16 * value
+                    scale = __fmul_rn(__ldg(p.wstep + m), p.act_step);
+                    shift = (!kPre && __ldg(p.kind + m) == kFixed4) ? 4 : 0;   // expanders store Fixed-4 codes as 16 * value
                 }
             }
             if (!mbar_wait_warp(bar_tfull + 8 * ab, tpar, abort_flag)) { alive = false; break; }

@@ -242,7 +242,8 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     __syncthreads();
     cluster_sync_all();                                   // both CTAs' barriers exist before anyone signals the peer
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    pdl_wait();                                           // and no trigger: see launch_dependent
+    // (the weights are read ahead of the wait for the kernel in front, activations and outputs behind it; no trigger: see
+    // launch_dependent)
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
 
@@ -255,6 +256,10 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
         // the weights of the taps (0, j), (1, j), (2, j).
         if (lane == 0) {
             const int ti = warp - 2;
+            if (warp == 0) {
+                asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.act[0]) : "memory");
+                pdl_wait();
+            }
             uint32_t s = 0, ph = 0;
             bool ok = true;
             for (int64_t tile = first; tile < cfg.ntiles && ok; tile += step) {
@@ -288,6 +293,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
         // so each operand has two producer threads taking alternate stages.
         const bool is_b = (warp == 0 || warp == 3);
         const uint32_t mine = (warp >= 3) ? 1u : 0u;
+        if (is_b) pdl_wait();
         uint32_t s = 0, ph = 0, g = 0;
         bool ok = true;
         for (int64_t tile = first; tile < cfg.ntiles && ok; tile += step) {
@@ -387,12 +393,13 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
         const int nch = (cfg.img_pix + 31) >> 5;             // 32-pixel chunks per run of pixels
         uint32_t it = 0;
         bool alive = true;
+        pdl_wait();                                          // the outputs
         for (int64_t tile = first; tile < cfg.ntiles && alive; tile += step, ++it) {
             const uint32_t ab = it & 1;
             const int64_t nt = tile / cfg.nbt;
             const int blk = (int)(tile - nt * cfg.nbt) * 2 + (int)rank;
             const int m = blk * kBlockRows + quarter * 32 + lane;
-            const float scale = (m < p.M) ? __fmul_rn(__ldg(pdl_ordered(p.wstep) + m), p.act_step) : 0.f;
+            const float scale = (m < p.M) ? __fmul_rn(__ldg(p.wstep + m), p.act_step) : 0.f;
             int64_t n0h[2];
             int nvalid[2];
 #pragma unroll
