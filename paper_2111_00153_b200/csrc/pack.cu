@@ -50,7 +50,7 @@ __device__ __forceinline__ int pot_nibble(float w, float alpha, int mode)   // E
 }
 
 // ------------------------------------------------------------------ pack kernel
-// One block per packed row.  Phase 1: coalesced (128-bit where aligned) reads of the fp32 row,
+// One block per row, in original order.  Phase 1: coalesced (128-bit where aligned) reads of the fp32 row,
 // quantize, scatter the codes as bytes into shared memory at their packed position k'.
 // Phase 2: every thread turns 32 code bytes into one 16-byte (4-bit rows) or two 16-byte
 // (8-bit rows) chunks and stores them with 128-bit stores, consecutive threads to consecutive
@@ -59,7 +59,7 @@ __device__ __forceinline__ int pot_nibble(float w, float alpha, int mode)   // E
 struct PackArgs {
     const float* W;
     uint8_t* blob;
-    uint64_t off_perm, off_alpha, off_kind, off_q4, off_q8;
+    uint64_t off_slot, off_alpha, off_kind, off_q4, off_q8;
     int M, K, taps, Cin, Cp, Kp, n4, seg;   // seg: codes per shared-memory segment
     int conv, pot_mode;
 };
@@ -67,16 +67,28 @@ struct PackArgs {
 __global__ void __launch_bounds__(256) pack_kernel(PackArgs a)
 {
     extern __shared__ __align__(16) uint8_t s_code[];
+    const int r = blockIdx.x;
+    const float* wrow = a.W + (size_t)r * a.K;
+    const bool vec4 = ((a.K & 3) == 0);   // row starts stay 16-byte aligned
+    const int stride = blockDim.x * 4;
+    // Four 128-bit loads in flight per thread before any code is formed: a block walks one row, so its time is the number
+    // of dependent load rounds.  The first four go out ahead of the wait for the metadata: the kernel in front (the
+    // metadata's writer) triggered behind its own wait, so whatever was in front of that, and the weights with it, is complete.
+    float4 w[4];
+    auto load = [&](int idx0, int k_hi) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (idx0 + u * stride < k_hi) w[u] = __ldg(reinterpret_cast<const float4*>(wrow + idx0 + u * stride));
+    };
+    const int k_first = a.conv ? a.K : min(a.K, a.seg);       // where the first segment's weights end
+    if (vec4) load(threadIdx.x * 4, k_first);
     pdl_wait();                                              // and no trigger: see launch_dependent
-    const int p = blockIdx.x;
-    const int r = reinterpret_cast<const int32_t*>(a.blob + a.off_perm)[p];
+    const int p = reinterpret_cast<const int32_t*>(a.blob + a.off_slot)[r];
     const float alpha = reinterpret_cast<const float*>(a.blob + a.off_alpha)[r];
     const int kind = (a.blob + a.off_kind)[r];
-    const float* wrow = a.W + (size_t)r * a.K;
     const float Q = (kind == kFixed8) ? 127.0f : 7.0f;
     uint8_t* dst = (kind == kFixed8) ? a.blob + a.off_q8 + (size_t)(p - a.n4) * a.Kp
                                      : a.blob + a.off_q4 + (size_t)p * (a.Kp / 2);
-    const bool vec4 = ((a.K & 3) == 0);   // row starts stay 16-byte aligned
 
     for (int seg0 = 0; seg0 < a.Kp; seg0 += a.seg) {
         const int seg_len = min(a.seg, a.Kp - seg0);
@@ -86,28 +98,26 @@ __global__ void __launch_bounds__(256) pack_kernel(PackArgs a)
         // original indices covered by this segment (linear: k' = k; conv: whole row in one segment)
         const int k_lo = a.conv ? 0 : seg0;
         const int k_hi = a.conv ? a.K : min(a.K, seg0 + seg_len);
-        auto put = [&](int idx, float w) {
-            int code = (kind == kPoT4) ? pot_nibble(w, alpha, a.pot_mode) : fixed_q(w, alpha, Q);
-            int kp = a.conv ? ((idx % a.taps) * a.Cp + idx / a.taps) : idx;
-            s_code[kp - seg0] = (uint8_t)code;
-        };
+        auto code_of = [&](float v) { return (uint8_t)((kind == kPoT4) ? pot_nibble(v, alpha, a.pot_mode) : fixed_q(v, alpha, Q)); };
         if (vec4) {
-            // four 128-bit loads in flight per thread before any code is formed: a block walks one
-            // row, so its time is the number of dependent load rounds
-            const int stride = blockDim.x * 4;
             for (int idx0 = k_lo + threadIdx.x * 4; idx0 < k_hi; idx0 += 4 * stride) {
-                float4 w[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (idx0 + u * stride < k_hi) w[u] = __ldg(reinterpret_cast<const float4*>(wrow + idx0 + u * stride));
+                if (idx0 >= 4 * stride) load(idx0, k_hi);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int idx = idx0 + u * stride;
-                    if (idx < k_hi) { put(idx, w[u].x); put(idx + 1, w[u].y); put(idx + 2, w[u].z); put(idx + 3, w[u].w); }
+                    if (idx >= k_hi) break;
+                    const float v[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+                    int c = a.conv ? idx / a.taps : 0, tap = idx - c * a.taps;      // (one division for four codes)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        s_code[a.conv ? tap * a.Cp + c : idx + e - seg0] = code_of(v[e]);
+                        if (++tap == a.taps) { tap = 0; ++c; }
+                    }
                 }
             }
         } else {
-            for (int idx = k_lo + threadIdx.x; idx < k_hi; idx += blockDim.x) put(idx, wrow[idx]);
+            for (int idx = k_lo + threadIdx.x; idx < k_hi; idx += blockDim.x)
+                s_code[(a.conv ? (idx % a.taps) * a.Cp + idx / a.taps : idx) - seg0] = code_of(wrow[idx]);
         }
         __syncthreads();
         for (int c = threadIdx.x; c < seg_len / 32; c += blockDim.x) {
@@ -148,7 +158,7 @@ cudaError_t launch_pack(const float* dW, int conv_oihw, const rmsmp_layer& L, in
 {
     PackArgs a;
     a.W = dW; a.blob = blob;
-    a.off_perm = L.off_perm; a.off_alpha = L.off_alpha; a.off_kind = L.off_kind;
+    a.off_slot = L.off_slot; a.off_alpha = L.off_alpha; a.off_kind = L.off_kind;
     a.off_q4 = L.off_q4; a.off_q8 = L.off_q8;
     a.M = L.M; a.K = L.Cin * L.kh * L.kw; a.taps = L.kh * L.kw; a.Cin = L.Cin; a.Cp = L.Cp;
     a.Kp = L.Kp; a.n4 = L.nP + L.nF4;
