@@ -119,6 +119,9 @@ struct StreamHeader {               // first 128 bytes of the table
     uint32_t pad[9];
 };
 static_assert(sizeof(StreamHeader) == 128, "header is 128 bytes");
+// Behind it: the first item of every CTA's list (and the end of the last one's), then the lists.
+constexpr uint32_t kOffFirst = sizeof(StreamHeader);
+__host__ __device__ constexpr uint32_t off_items(uint32_t grid) { return (kOffFirst + 4u * (grid + 1u) + 15u) & ~15u; }
 
 __host__ __device__ inline int box_index(int rows) { return rows > 64 ? 0 : (rows > 32 ? 1 : 2); }   // 128, 64 or 32 rows high
 
@@ -301,8 +304,10 @@ stream_kernel(const uint8_t* __restrict__ table)
     // hence no launch, ends before the launch in front of it has.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const StreamHeader* H = reinterpret_cast<const StreamHeader*>(table);
-    const int32_t* cta_first = reinterpret_cast<const int32_t*>(table + H->off_first);
-    const StreamItem* items = reinterpret_cast<const StreamItem*>(table + H->off_items);
+    // (where the lists lie follows from the grid, so that the first of them and the header are fetched side by side)
+    const int32_t* cta_first = reinterpret_cast<const int32_t*>(table + kOffFirst);
+    const StreamItem* items = reinterpret_cast<const StreamItem*>(table + off_items(gridDim.x));
+    const int it0 = __ldg(cta_first + blockIdx.x), it1 = __ldg(cta_first + blockIdx.x + 1);
     const StreamProblem* probs = reinterpret_cast<const StreamProblem*>(table + H->off_probs);
     const int n_pad = H->n_pad, nS = H->nS, nch = H->nch, nB = H->nB, nAst = H->nAst;
     const uint32_t stage_bytes = H->stage_bytes, b_bytes = H->b_bytes, idesc = H->idesc, idesc_fp = H->idesc_fp;
@@ -324,7 +329,6 @@ stream_kernel(const uint8_t* __restrict__ table)
     __shared__ int4 s_items[kLocalItems];                 // the head of this CTA's list of items (prob, kind / k-blocks / rows, row0, packed0)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int it0 = __ldg(cta_first + blockIdx.x), it1 = __ldg(cta_first + blockIdx.x + 1);
     for (int i = threadIdx.x; i < min(it1 - it0, kLocalItems); i += kStreamThreads) {
         s_items[i] = __ldg(reinterpret_cast<const int4*>(items + it0 + i));
     }
@@ -443,6 +447,7 @@ stream_kernel(const uint8_t* __restrict__ table)
         // ---------------------------------------------------------- producer of the activation tiles (lanes 0 / 1: first / second k-block)
         uint32_t sb = 0, phB = 0;
         bool ok = true;
+        if (lane == 0) { const int4 a = s_items[0]; tensormap_prefetch(item_kind(a.y) == kPoT4 ? &probs[a.x].act_fp : &probs[a.x].act); }
         // the E4M3 copies come from the kernel in front of this one
         asm volatile("griddepcontrol.wait;" ::: "memory");
         for (int it = it0; it < it1 && ok; ++it) {
@@ -736,9 +741,9 @@ Layout table_layout(int count, int nitems, int grid)
 {
     Layout L;
     L.grid = grid; L.nitems = nitems;
-    size_t off = sizeof(StreamHeader);
-    L.off_first = off; off = up(off + sizeof(int32_t) * (size_t)(grid + 1), 16);
-    L.off_items = off; off = up(off + sizeof(StreamItem) * (size_t)nitems, 128);
+    size_t off;
+    L.off_first = kOffFirst;
+    off = L.off_items = off_items((uint32_t)grid); off = up(off + sizeof(StreamItem) * (size_t)nitems, 128);
     L.off_probs = off; off += sizeof(StreamProblem) * (size_t)count;
     L.bytes = up(off, 256);
     L.off_act = L.bytes;
