@@ -91,6 +91,30 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
     if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort_flag);
     return __all_sync(0xffffffffu, ok);
 }
+__device__ __forceinline__ bool mbar_wait_parked_step(uint32_t bar, uint32_t parity, volatile int* abort_flag)      // (see mbar_wait_step)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 16; ++i)
+            if (__all_sync(0xffffffffu, mbar_try_wait_parked(bar, parity, 20000u))) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0 || clock64() - t0 > kWaitCycles)) { *abort_flag = 1; return false; }
+    }
+}
+// The form of a warp that walks its loop in step: every lane polls, and the verdict is a vote, so that what follows is the
+// same for the whole warp to the compiler too.
+__device__ __forceinline__ bool mbar_wait_step(uint32_t bar, uint32_t parity, volatile int* abort_flag)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 64; ++i)
+            if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0 || clock64() - t0 > kWaitCycles)) { *abort_flag = 1; return false; }
+    }
+}
 __device__ __forceinline__ void fence_proxy_async_smem()
 {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -172,6 +196,68 @@ __device__ __forceinline__ void mma_i8_halves(uint32_t d_tmem, uint32_t a_lo, ui
         "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %4, p;\n\t}"
         ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
         : "memory");
+}
+// The MMAs of a warp in step: all lanes take part, the elected one issues.  What a warp can issue is what bounds tiles of fewer
+// than 256 columns: measured with one wait and one commit to every four MMAs, lane 0 in a branch of its own takes 124 cycles an
+// MMA whatever its size; each MMA behind an election of its own 101; four behind one election 63 to 69 up to 128 columns
+// and, from 160, the N / 2 that the tensor pipe takes.  (The branch, and a flag in a register as the predicate, leave the compiler in
+// doubt about how many lanes issue, and operands in uniform registers out of reach.)
+// One 32-code step; two (a 64-byte k-block); four (a 128-byte k-block): 32 bytes further on in both operands' rows each.
+#define RMSMP_MMA_HEAD "{\n\t.reg .pred p, e;\n\t.reg .b64 da, db;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+#define RMSMP_MMA_NEXT "add.s64 da, da, 2;\n\tadd.s64 db, db, 2;\n\t"
+#define RMSMP_MMA_I8(group) "@e tcgen05.mma.cta_group::" group ".kind::i8 [%0], da, db, %4, p;\n\t"
+#define RMSMP_MMA_ADD "setp.eq.u32 p, 0, 0;\n\t"
+template <int kSteps>
+__device__ __forceinline__ void mma_i8_step(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate)
+{
+    static_assert(kSteps == 1 || kSteps == 2 || kSteps == 4, "");
+    if (kSteps == 1)
+        asm volatile(RMSMP_MMA_HEAD RMSMP_MMA_I8("1") "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
+    else if (kSteps == 2)
+        asm volatile(RMSMP_MMA_HEAD RMSMP_MMA_I8("1") RMSMP_MMA_ADD RMSMP_MMA_NEXT RMSMP_MMA_I8("1") "}"
+                     ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
+    else
+        asm volatile(RMSMP_MMA_HEAD RMSMP_MMA_I8("1") RMSMP_MMA_ADD RMSMP_MMA_NEXT RMSMP_MMA_I8("1") RMSMP_MMA_NEXT RMSMP_MMA_I8("1") RMSMP_MMA_NEXT RMSMP_MMA_I8("1") "}"
+                     ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+// One to four steps.
+__device__ __forceinline__ void mma_i8_steps(int steps, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate)
+{
+    if (steps == 4) {
+        mma_i8_step<4>(d_tmem, a_lo, b_lo, hi, idesc, accumulate);
+    } else {
+        if (steps & 2) mma_i8_step<2>(d_tmem, a_lo, b_lo, hi, idesc, accumulate);
+        if (steps & 1) mma_i8_step<1>(d_tmem, a_lo + 2 * (steps & 2), b_lo + 2 * (steps & 2), hi, idesc, accumulate | (uint32_t)(steps & 2));
+    }
+}
+// Four steps of a CTA pair (256 rows, 128 in each CTA).
+__device__ __forceinline__ void mma_i8_pair_step(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(RMSMP_MMA_HEAD RMSMP_MMA_I8("2") RMSMP_MMA_ADD RMSMP_MMA_NEXT RMSMP_MMA_I8("2") RMSMP_MMA_NEXT RMSMP_MMA_I8("2") RMSMP_MMA_NEXT RMSMP_MMA_I8("2") "}"
+                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+// Four steps with the A operand in tensor memory (8 columns a step); kFp: E3M2 x E4M3 operands and fp32 accumulators.
+template <bool kFp>
+__device__ __forceinline__ void mma_tmem_a_step(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate)
+{
+#define RMSMP_MMA_TMEM(kind, at) "@e tcgen05.mma.cta_group::1.kind::" kind " [%0], [" at "], db, %4, p;\n\tadd.s64 db, db, 2;\n\t"
+#define RMSMP_MMA_TMEM4(kind) \
+    asm volatile("{\n\t.reg .pred p, e;\n\t.reg .b64 db;\n\t.reg .b32 a1, a2, a3;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 db, {%2, %3};\n\t" \
+                 "add.u32 a1, %1, 8;\n\tadd.u32 a2, %1, 16;\n\tadd.u32 a3, %1, 24;\n\t" \
+                 RMSMP_MMA_TMEM(kind, "%1") RMSMP_MMA_ADD RMSMP_MMA_TMEM(kind, "a1") RMSMP_MMA_TMEM(kind, "a2") RMSMP_MMA_TMEM(kind, "a3") "}" \
+                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory")
+    if (kFp) RMSMP_MMA_TMEM4("f8f6f4"); else RMSMP_MMA_TMEM4("i8");
+#undef RMSMP_MMA_TMEM4
+#undef RMSMP_MMA_TMEM
+}
+#undef RMSMP_MMA_HEAD
+#undef RMSMP_MMA_NEXT
+#undef RMSMP_MMA_I8
+#undef RMSMP_MMA_ADD
+__device__ __forceinline__ void mma_commit_step(uint32_t bar)
+{
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar)
 {

@@ -89,7 +89,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     __shared__ __align__(8) uint64_t s_full[kSplitRing], s_empty[kSplitRing], s_tfull;
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;      // (a shuffle: the same for the warp to the compiler too)
     const uint32_t rank = cfg.S > 1 ? split_rank() : 0u;
     const uint32_t tile = blockIdx.x / (uint32_t)cfg.S;
     const int nt = (int)(tile / (uint32_t)p.nblocks), blk = (int)(tile - (uint32_t)nt * (uint32_t)p.nblocks);
@@ -114,7 +114,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     if (cfg.S > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");      // this CTA runs: its shared memory may be written
     // From here on the weights: packed codes, their rows' places and scales, or the expanded copy.  What the kernel in front
     // writes or reads -- activations, outputs, the status word -- stays behind the waits further down (see launch_dependent).
-    const uint32_t tmem_base = s_tmem_base;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
 
     int b0, h0;
@@ -155,27 +155,23 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ---------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            const uint64_t da = smem_desc_kmajor(sA, cfg.bk), db = smem_desc_kmajor(sB, cfg.bk);
-            const uint32_t hi = (uint32_t)(da >> 32), a_step = (uint32_t)cfg.a_bytes >> 4, b_step = (uint32_t)cfg.b_bytes >> 4;
-            int s = 0, cc = kb0 % cfg.cpt;
-            uint32_t ph = 0;
-            bool ok = true;
-            for (int i = 0; i < n_kb; ++i) {
-                if (!mbar_wait(full(s), ph, abort_flag)) { ok = false; break; }
-                tc_fence_after();
-                const int ksteps = (kGather ? kb0 + i == cfg.nkb - 1 : cc == cfg.cpt - 1) ? cfg.last_ksteps : cfg.bk >> 5;
-                const uint32_t a_lo = (uint32_t)da + s * a_step, b_lo = (uint32_t)db + s * b_step;
-                for (int k = 0; k < ksteps; ++k)
-                    mma_i8_halves(tmem_base, a_lo + 2 * k, b_lo + 2 * k, hi, cfg.idesc, (i | k) ? 1u : 0u);
-                mma_commit(empty(s));
-                if (++s == cfg.nst) { s = 0; ph ^= 1; }
-                if (++cc == cfg.cpt) cc = 0;
-            }
-            if (ok) mma_commit(smem_u32(&s_tfull));
+        // ---------------------------------------------------------- MMA issuer (the warp walks in step, the elected lane issues)
+        const uint64_t da = smem_desc_kmajor(sA, cfg.bk), db = smem_desc_kmajor(sB, cfg.bk);
+        const uint32_t hi = (uint32_t)(da >> 32), a_step = (uint32_t)cfg.a_bytes >> 4, b_step = (uint32_t)cfg.b_bytes >> 4;
+        int s = 0, cc = kb0 % cfg.cpt;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int i = 0; i < n_kb; ++i) {
+            if (!mbar_wait_step(full(s), ph, abort_flag)) { ok = false; break; }
+            tc_fence_after();
+            const int ksteps = (kGather ? kb0 + i == cfg.nkb - 1 : cc == cfg.cpt - 1) ? cfg.last_ksteps : cfg.bk >> 5;
+            const uint32_t a_lo = (uint32_t)da + s * a_step, b_lo = (uint32_t)db + s * b_step;
+            mma_i8_steps(ksteps, tmem_base, a_lo, b_lo, hi, cfg.idesc, i ? 1u : 0u);
+            mma_commit_step(empty(s));
+            if (++s == cfg.nst) { s = 0; ph ^= 1; }
+            if (++cc == cfg.cpt) cc = 0;
         }
-        __syncwarp();
+        if (ok) mma_commit_step(smem_u32(&s_tfull));
     } else if (!kPre && warp >= kSplitFirst) {
         // ---------------------------------------------------------- expanders
         const int grp = (warp - kSplitFirst) >> 2;

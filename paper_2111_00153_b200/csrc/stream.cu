@@ -28,9 +28,9 @@
 //                within 0..15 are read as they are (as an E4M3 number such a byte is the code times
 //                2^-9, subnormals included); otherwise the E4M3 copy of a layer's codes is written
 //                once per launch by a small kernel in front of this one (act_e4m3_kernel, into
-//                scratch behind the table).  One thread gets an
-//                MMA out only every ~150 cycles whatever its size (measured; two issuing threads
-//                give twice the rate), so with few tokens the steps of a stage are dealt to up to
+//                scratch behind the table).  One warp gets an
+//                MMA out every 63 cycles at best (ptx.cuh; 150 when a lane issued them one by one),
+//                so with few tokens the stages are dealt to up to
 //                four issuers, each with an accumulator chain of its own (the chains are added up
 //                in the epilogue).  Warp 4 allocates tensor memory.  Accumulator buffers take turns
 //                between items so that an item's output overlaps the next items' stream.
@@ -72,8 +72,8 @@ constexpr int kAStageCols = 64;                                       // 256 cod
 constexpr int kMaxTokens = 128;                                       // accumulator columns of one chain at most
 constexpr int kRingMax = 12;
 constexpr int kStreamMaxK = 16384;                                    // reduction length up to which the fp32 sums of PoT tiles are exact
-constexpr int kLocalItems = 96;                                        // items of a CTA's list kept in shared memory
-constexpr int kStreamSmem = 232448 - 1024 - kLocalItems * 16;
+constexpr int kLocalItems = 64;                                        // items of a CTA's list kept in shared memory
+constexpr int kStreamSmem = 232448 - 64 - kLocalItems * 16;            // (for 128 tokens just enough for six slots of packed codes)
 constexpr uint32_t kPlanMagic = 0x53545247u;                          // "STRG"
 
 // One layer of the launch as the kernel sees it (device table, 128-byte aligned: it starts with
@@ -208,33 +208,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])
         : "r"(taddr) : "memory");
 }
 
-// One MMA with the A operand in tensor memory (128 lanes x 8 columns = 128 rows x 32 codes) and the
-// B operand in shared memory (descriptor given as 32-bit halves).
-__device__ __forceinline__ void mma_i8_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi,
-                                              uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], db, %4, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// The same with E3M2 x E4M3 operands and fp32 accumulators.
-__device__ __forceinline__ void mma_f8f6f4_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi,
-                                                  uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], db, %4, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 // E4M3 copies of the activation codes of every layer with PoT rows: [N][Kp], zeros beyond the layer's
 // reduction length.  blockIdx.y = layer; layers whose bytes can be read as they are have no copy.  The launch behind
 // waits for this kernel, so it is all latency: the table is read ahead of the wait for the launch in front, a thread
@@ -328,7 +301,7 @@ stream_kernel(const uint8_t* __restrict__ table)
     __shared__ int s_abort;
     __shared__ int4 s_items[kLocalItems];                 // the head of this CTA's list of items (prob, kind / k-blocks / rows, row0, packed0)
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;      // (a shuffle: the same for the warp to the compiler too)
     for (int i = threadIdx.x; i < min(it1 - it0, kLocalItems); i += kStreamThreads) {
         s_items[i] = __ldg(reinterpret_cast<const int4*>(items + it0 + i));
     }
@@ -472,63 +445,66 @@ stream_kernel(const uint8_t* __restrict__ table)
     } else if (warp < kFirstMma) {
         // warps 2-3 have no role
     } else if (warp < kFirstExp) {
-        // ---------------------------------------------------------- MMA issuers (lane 0 issues; the warp walks in step)
-        // Every tcgen05 instruction holds its thread for ~150 cycles, the commit included, so a stage is one
+        // ---------------------------------------------------------- MMA issuers (the warp walks in step, the elected lane issues)
+        // A tcgen05 instruction holds its warp for 60 cycles and more, the commit included, so a stage is one
         // issuer's: its four or eight MMAs and ONE commit, which frees the stage's A columns and activation slot.
         // The issuers take the CTA's stages in turn; stage st of an item adds to accumulator chain st % nch.
         const int me = warp - kFirstMma;
         if (me < nch) {
-            const bool issuer = (lane == 0);
+            // (what comes from memory is shuffled, so that the compiler knows it to be the same for the warp too)
+            auto same = [](uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); };
+            const uint32_t tmem = same(tmem_base), acc_base = tmem + same(a_base_col), buffer_cols = same(acc_cols), buffers = same(nAcc);
+            const uint32_t chains = same((uint32_t)nch), stages = same((uint32_t)nAst), chain_cols = same((uint32_t)n_pad);
+            const uint32_t b_step = same(b_bytes) >> 4, b_half = same(b_sub) >> 4, desc_i8 = same(idesc), desc_fp = same(idesc_fp);
+            const int first_it = (int)same((uint32_t)it0), end_it = (int)same((uint32_t)it1);
             uint32_t sa = (uint32_t)me, phA = 0, n = 0, t = 0;        // t: stages of the items before this one
             const uint64_t desc_b0 = smem_desc_kmajor(sB, 128);
             const uint32_t b_lo0 = (uint32_t)desc_b0, desc_hi = (uint32_t)(desc_b0 >> 32);
             bool ok = true;
-            for (int it = it0; it < it1 && ok && !*abort_flag; ++it, ++n) {
+            for (int it = first_it; it < end_it && ok; ++it, ++n) {
                 const ItemView v = view(it);
                 last_status = v.P->status;
-                const uint32_t ab = n & (nAcc - 1u), lap = n >> acc_shift;      // nAcc is 2 or 4
+                const int nst = (int)same((uint32_t)v.nst), nkb = (int)same((uint32_t)v.nkb), kind = (int)same((uint32_t)v.kind);
+                const uint32_t ab = n & (buffers - 1u), lap = n >> (buffers == 4u ? 2 : 1);      // nAcc is 2 or 4
                 bool have_acc = false;                    // this issuer has made sure the item's accumulator buffer is free
                 // its own stages only: those whose index over the whole list is me modulo nch (1, 2 or 4); the A stage
                 // advances by nch with them (nch <= nAst)
-                for (int st = (int)(((uint32_t)me - t) & (uint32_t)(nch - 1)); st < v.nst; st += nch) {
+                for (int st = (int)(((uint32_t)me - t) & (chains - 1u)); st < nst; st += (int)chains) {
                     {
                         if (!have_acc) {
-                            if (!mbar_wait_parked(bar_tempty + 8 * ab, (lap & 1) ^ 1, abort_flag)) { ok = false; break; }
+                            if (!mbar_wait_parked_step(bar_tempty + 8 * ab, (lap & 1) ^ 1, abort_flag)) { ok = false; break; }
                             have_acc = true;
                         }
-                        if (!mbar_wait_parked(bar_fullB + 8 * sa, phA, abort_flag) || !mbar_wait_parked(bar_fullA + 8 * sa, phA, abort_flag)) { ok = false; break; }
+                        if (!mbar_wait_parked_step(bar_fullB + 8 * sa, phA, abort_flag) || !mbar_wait_parked_step(bar_fullA + 8 * sa, phA, abort_flag)) { ok = false; break; }
                         tc_fence_after();
-                        if (issuer) {
-                            const uint32_t chain = (uint32_t)st & (uint32_t)(nch - 1);
-                            const uint32_t d_tmem = tmem_base + ab * acc_cols + chain * (uint32_t)n_pad;
-                            const uint32_t a_t = tmem_base + a_base_col + sa * kAStageCols, b_lo = b_lo0 + sa * (b_bytes >> 4);
+                        {
+                            const uint32_t chain = (uint32_t)st & (chains - 1u);
+                            const uint32_t d_tmem = tmem + ab * buffer_cols + chain * chain_cols;
+                            const uint32_t a_t = acc_base + sa * kAStageCols, b_lo = b_lo0 + sa * b_step;
                             // a 32-code step is 8 columns of A and 32 bytes (two 16-byte units) of a B row; the first
                             // instruction into a chain in this item overwrites it
-                            const int nsteps = 4 * min(v.kbps, v.nkb - st * v.kbps);
-                            if (v.kind == kPoT4) {
-                                for (int j = 0; j < nsteps; ++j) {
-                                    const uint32_t b_j = b_lo + (uint32_t)(j >> 2) * (b_sub >> 4) + 2u * (uint32_t)(j & 3);
-                                    mma_f8f6f4_tmem_a(d_tmem, a_t + 8 * j, b_j, desc_hi, idesc_fp, (st < nch && j == 0) ? 0u : 1u);
-                                }
+                            const bool both = 2 * st + 1 < nkb;             // (an odd number of k-blocks: the last stage has one)
+                            const uint32_t first = st < (int)chains ? 0u : 1u, b_lo2 = b_lo + b_half;
+                            if (kind == kPoT4) {
+                                mma_tmem_a_step<true>(d_tmem, a_t, b_lo, desc_hi, desc_fp, first);
+                                if (both) mma_tmem_a_step<true>(d_tmem, a_t + 32, b_lo2, desc_hi, desc_fp, 1u);
                             } else {
-                                for (int j = 0; j < nsteps; ++j) {
-                                    const uint32_t b_j = b_lo + (uint32_t)(j >> 2) * (b_sub >> 4) + 2u * (uint32_t)(j & 3);
-                                    mma_i8_tmem_a(d_tmem, a_t + 8 * j, b_j, desc_hi, idesc, (st < nch && j == 0) ? 0u : 1u);
-                                }
+                                mma_tmem_a_step<false>(d_tmem, a_t, b_lo, desc_hi, desc_i8, first);
+                                if (both) mma_tmem_a_step<false>(d_tmem, a_t + 32, b_lo2, desc_hi, desc_i8, 1u);
                             }
-                            mma_commit(bar_emptyA + 8 * sa);
+                            mma_commit_step(bar_emptyA + 8 * sa);
                         }
                     }
-                    sa += (uint32_t)nch;
-                    if (sa >= (uint32_t)nAst) { sa -= (uint32_t)nAst; phA ^= 1; }
+                    sa += chains;
+                    if (sa >= stages) { sa -= stages; phA ^= 1; }
                 }
-                t += (uint32_t)v.nst;
+                t += (uint32_t)nst;
                 if (!ok) break;
                 // Every issuer reports once per item, whether or not a stage of it was its own.  An issuer without
                 // stages in short items can be items ahead of the others: before it reports on this buffer again
                 // it makes sure that the buffer's previous item has everybody's report (one arrival per phase).
-                if (lap >= 1 && !mbar_wait_parked(bar_tfull + 8 * ab, (lap - 1) & 1, abort_flag)) break;
-                if (issuer) mma_commit(bar_tfull + 8 * ab);
+                if (lap >= 1 && !mbar_wait_parked_step(bar_tfull + 8 * ab, (lap - 1) & 1, abort_flag)) break;
+                mma_commit_step(bar_tfull + 8 * ab);
             }
         }
     } else if (warp < kFirstEpi) {
@@ -812,7 +788,7 @@ bool stream_build_table(const Problem* probs, int count, int sms, uint8_t* h_tab
     StreamHeader* H = reinterpret_cast<StreamHeader*>(h_table);
     H->magic = kPlanMagic; H->nprob = count; H->nitems = (int32_t)nitems; H->grid = grid;
     H->n_pad = std::max(16, (int)((maxN + 15) / 16 * 16));
-    // consecutive MMAs of one thread are ~150 cycles apart; with few tokens the accumulator buffer has room
+    // consecutive MMAs of one warp are 60 cycles and more apart; with few tokens the accumulator buffer has room
     // for several chains, one per issuing thread (summed in the epilogue)
     H->nch = H->n_pad <= 32 ? 4 : (H->n_pad <= 64 ? 2 : 1);
     H->acc_cols = H->nch * H->n_pad;                              // <= 128

@@ -231,7 +231,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;      // (a shuffle: the same for the warp to the compiler too)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxRing; ++s) {
@@ -256,7 +256,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     tc_fence_after();
     // (the weights are read ahead of the wait for the kernel in front, activations and outputs behind it; no trigger: see
     // launch_dependent)
-    const uint32_t tmem_base = s_tmem_base;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
 
     // (tile indices fit 32 bits with a step to spare: checked on the host)
@@ -365,19 +365,18 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA issuer
-        // The whole warp walks the loops in step (so that ring positions and descriptors are
-        // warp-uniform values); lane 0 alone issues the MMAs and commits.
-        const bool issuer = (lane == 0);
+        // The whole warp walks the loops in step, so that ring positions and descriptors are the same for all lanes and known to
+        // be; the elected lane issues the MMAs and commits.
         {
             uint32_t sa = 0, phA = 0, sb = 0, phB = 0, it = 0;
             const uint64_t desc_a0 = smem_desc_kmajor(sA, cfg.bk), desc_b0 = smem_desc_kmajor(sB, cfg.bk);
             const uint32_t desc_lo0_a = (uint32_t)desc_a0, desc_lo0_b = (uint32_t)desc_b0, desc_hi = (uint32_t)(desc_a0 >> 32);
-            bool have_a = !kAres || my_tiles == 0 || mbar_wait(bar_fullA, 0, abort_flag);
-            for (uint32_t tile = first; tile < ntiles && have_a && !*abort_flag; tile += step, ++it) {
+            bool have_a = !kAres || my_tiles == 0 || mbar_wait_step(bar_fullA, 0, abort_flag);
+            for (uint32_t tile = first; tile < ntiles && have_a; tile += step, ++it) {
                 // one accumulator per tile, alternating; or (two row blocks per tile) both, every tile
                 const uint32_t ab = kM2 ? 0u : (it & 1);
                 const uint32_t tpar = kM2 ? ((it & 1) ^ 1) : (((it >> 1) & 1) ^ 1);
-                if (!mbar_wait(bar_tempty + 8 * ab, tpar, abort_flag)) break;
+                if (!mbar_wait_step(bar_tempty + 8 * ab, tpar, abort_flag)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + ab * kTileN;
                 bool ok = true;
@@ -394,16 +393,19 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     const bool two_last = (cfg.last_ksteps == 2);
                     bool two = two_last || cfg.cpt > 1;                            // (of two chunks the first is whole)
                     for (int kb = 0; kb < cfg.nkb; kb += 3) {
-                        if (!mbar_wait(bar_fullB + 8 * sb, phB, abort_flag)) { ok = false; break; }
+                        if (!mbar_wait_step(bar_fullB + 8 * sb, phB, abort_flag)) { ok = false; break; }
                         tc_fence_after();
-                        if (issuer) {
-                            mma_i8_halves(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
-                            if (two) mma_i8_halves(d_tmem, a_lo + 2, b_lo + 2, desc_hi, cfg.idesc, 1u);
-                            mma_i8_halves(d_tmem, a_lo + a_t, b_lo + t_step, desc_hi, cfg.idesc, 1u);
-                            if (two) mma_i8_halves(d_tmem, a_lo + a_t + 2, b_lo + t_step + 2, desc_hi, cfg.idesc, 1u);
-                            mma_i8_halves(d_tmem, a_lo + 2 * a_t, b_lo + 2 * t_step, desc_hi, cfg.idesc, 1u);
-                            if (two) mma_i8_halves(d_tmem, a_lo + 2 * a_t + 2, b_lo + 2 * t_step + 2, desc_hi, cfg.idesc, 1u);
-                            mma_commit(bar_emptyB + 8 * sb);
+                        {
+                            if (two) {
+                                mma_i8_step<2>(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
+                                mma_i8_step<2>(d_tmem, a_lo + a_t, b_lo + t_step, desc_hi, cfg.idesc, 1u);
+                                mma_i8_step<2>(d_tmem, a_lo + 2 * a_t, b_lo + 2 * t_step, desc_hi, cfg.idesc, 1u);
+                            } else {
+                                mma_i8_step<1>(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
+                                mma_i8_step<1>(d_tmem, a_lo + a_t, b_lo + t_step, desc_hi, cfg.idesc, 1u);
+                                mma_i8_step<1>(d_tmem, a_lo + 2 * a_t, b_lo + 2 * t_step, desc_hi, cfg.idesc, 1u);
+                            }
+                            mma_commit_step(bar_emptyB + 8 * sb);
                         }
                         a_lo += a_adv;
                         b_lo += b_step;
@@ -416,29 +418,20 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     const uint32_t a_step = (uint32_t)cfg.a_bytes >> 4, b_step = (uint32_t)cfg.b_bytes >> 4;
                     uint32_t a_lo = desc_lo0_a + sa * a_step, b_lo = desc_lo0_b + sb * b_step;
                     if (kM2) {
-                        if (!mbar_wait(bar_tempty + 8, tpar, abort_flag)) break;
+                        if (!mbar_wait_step(bar_tempty + 8, tpar, abort_flag)) break;
                         tc_fence_after();
                     }
                     for (int kb = 0; kb < cfg.nkb; ++kb) {
-                        if (!mbar_wait(bar_fullB + 8 * sb, phB, abort_flag) || !mbar_wait(bar_fullA + 8 * sa, phA, abort_flag)) {
+                        if (!mbar_wait_step(bar_fullB + 8 * sb, phB, abort_flag) || !mbar_wait_step(bar_fullA + 8 * sa, phA, abort_flag)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
                         const uint32_t acc = kb ? 1u : 0u;
-                        if (issuer) mma_i8_halves(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, acc);
-                        if (issuer) mma_i8_halves(d_tmem, a_lo + 2, b_lo + 2, desc_hi, cfg.idesc, 1u);
-                        if (issuer) mma_i8_halves(d_tmem, a_lo + 4, b_lo + 4, desc_hi, cfg.idesc, 1u);
-                        if (issuer) mma_i8_halves(d_tmem, a_lo + 6, b_lo + 6, desc_hi, cfg.idesc, 1u);
-                        if (kM2) {
-                            const uint32_t a1 = a_lo + (kABytes >> 4);
-                            if (issuer) mma_i8_halves(d_tmem + kTileN, a1, b_lo, desc_hi, cfg.idesc, acc);
-                            if (issuer) mma_i8_halves(d_tmem + kTileN, a1 + 2, b_lo + 2, desc_hi, cfg.idesc, 1u);
-                            if (issuer) mma_i8_halves(d_tmem + kTileN, a1 + 4, b_lo + 4, desc_hi, cfg.idesc, 1u);
-                            if (issuer) mma_i8_halves(d_tmem + kTileN, a1 + 6, b_lo + 6, desc_hi, cfg.idesc, 1u);
-                        }
-                        if (issuer) mma_commit(bar_emptyA + 8 * sa);
-                        if (issuer) mma_commit(bar_emptyB + 8 * sb);
+                        mma_i8_step<4>(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, acc);
+                        if (kM2) mma_i8_step<4>(d_tmem + kTileN, a_lo + (kABytes >> 4), b_lo, desc_hi, cfg.idesc, acc);
+                        mma_commit_step(bar_emptyA + 8 * sa);
+                        mma_commit_step(bar_emptyB + 8 * sb);
                         a_lo += a_step;
                         b_lo += b_step;
                         if (++sa == (uint32_t)cfg.nA) { sa = 0; phA ^= 1; a_lo = desc_lo0_a; }
@@ -450,26 +443,22 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     uint32_t a_lo = kAres ? desc_lo0_a : desc_lo0_a + sa * a_step;
                     uint32_t b_lo = desc_lo0_b + sb * b_step;
                     for (int kb = 0; kb < cfg.nkb; ++kb) {
-                        if (!mbar_wait(bar_fullB + 8 * sb, phB, abort_flag) ||
-                            (!kAres && !mbar_wait(bar_fullA + 8 * sa, phA, abort_flag))) { ok = false; break; }
+                        if (!mbar_wait_step(bar_fullB + 8 * sb, phB, abort_flag) ||
+                            (!kAres && !mbar_wait_step(bar_fullA + 8 * sa, phA, abort_flag))) { ok = false; break; }
                         tc_fence_after();
                         const int ksteps = (uniform || cc != cfg.cpt - 1) ? (cfg.bk >> 5) : cfg.last_ksteps;
-                        if (issuer) mma_i8_halves(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
-                        for (int ks = 1; ks < ksteps; ++ks)
-                            if (issuer) mma_i8_halves(d_tmem, a_lo + 2 * ks, b_lo + 2 * ks, desc_hi, cfg.idesc, 1u);
+                        mma_i8_steps(ksteps, d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
                         if (kM2) {
                             // second row block: rows 128..255 of the weight stage, second accumulator
                             if (kb == 0) {
-                                if (!mbar_wait(bar_tempty + 8, tpar, abort_flag)) { ok = false; break; }
+                                if (!mbar_wait_step(bar_tempty + 8, tpar, abort_flag)) { ok = false; break; }
                                 tc_fence_after();
                             }
                             const uint32_t a1 = a_lo + (kABytes >> 4);
-                            if (issuer) mma_i8_halves(d_tmem + kTileN, a1, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
-                            for (int ks = 1; ks < ksteps; ++ks)
-                                if (issuer) mma_i8_halves(d_tmem + kTileN, a1 + 2 * ks, b_lo + 2 * ks, desc_hi, cfg.idesc, 1u);
+                            mma_i8_steps(ksteps, d_tmem + kTileN, a1, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
                         }
-                        if (!kAres && issuer) mma_commit(bar_emptyA + 8 * sa);
-                        if (issuer) mma_commit(bar_emptyB + 8 * sb);
+                        if (!kAres) mma_commit_step(bar_emptyA + 8 * sa);
+                        mma_commit_step(bar_emptyB + 8 * sb);
                         a_lo += a_step;
                         b_lo += b_step;
                         if (++sa == (uint32_t)cfg.nA) { sa = 0; phA ^= 1; if (!kAres) a_lo = desc_lo0_a; }
@@ -478,8 +467,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     }
                 }
                 if (!ok) break;
-                if (issuer) mma_commit(bar_tfull + 8 * ab);
-                if (kM2 && issuer) mma_commit(bar_tfull + 8);
+                mma_commit_step(bar_tfull + 8 * ab);
+                if (kM2) mma_commit_step(bar_tfull + 8);
             }
         }
     } else if (!kPre && warp < 2 + kNumExpWarps) {

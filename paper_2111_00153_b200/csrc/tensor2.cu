@@ -23,6 +23,7 @@
 #include <cstring>
 #include <algorithm>
 #include "common.cuh"
+#include "ptx.cuh"
 #include "tmap.cuh"
 
 namespace rmsmp {
@@ -117,6 +118,18 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile
         if (clock64() - t0 > kWaitCycles2) { *abort_flag = 1; return false; }
     }
 }
+// (a warp that walks its loop in step: the verdict is a vote)
+__device__ __forceinline__ bool bar_wait_step(uint32_t bar, uint32_t parity, volatile int* abort_flag)
+{
+    if (__all_sync(0xffffffffu, bar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 64; ++i)
+            if (__all_sync(0xffffffffu, bar_try_wait(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0 || clock64() - t0 > kWaitCycles2)) { *abort_flag = 1; return false; }
+    }
+}
 __device__ __forceinline__ bool bar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
 {
     bool ok = true;
@@ -143,21 +156,11 @@ __device__ __forceinline__ void store_2d(const CUtensorMap* map, uint32_t src, i
                  ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
-// One MMA of the pair: 256 rows (128 per CTA) x N columns x 32 codes; descriptors as 32-bit halves.
-__device__ __forceinline__ void pair_mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "mov.b64 da, {%1, %3};\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::2.kind::i8 [%0], da, db, %4, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
-}
 // Arrive (once all MMAs issued so far have finished) on the barrier at this shared-memory offset in BOTH CTAs.
 __device__ __forceinline__ void pair_commit(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+                 "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
                  ::"r"(bar), "h"((uint16_t)3) : "memory");
 }
 __device__ __forceinline__ void ld_issue(uint32_t taddr, uint32_t (&v)[32])
@@ -218,7 +221,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();                 // 0 = leader: owns the "full" and "accumulator free" barriers
 
     if (threadIdx.x == 0) {
@@ -244,7 +247,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // (the weights are read ahead of the wait for the kernel in front, activations and outputs behind it; no trigger: see
     // launch_dependent)
-    const uint32_t tmem_base = s_tmem_base;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
 
     const int64_t first = blockIdx.x >> 1, step = gridDim.x >> 1;      // cluster index, clusters in the grid
@@ -332,46 +335,33 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA issuer (leader CTA only)
         if (rank == 0) {
-            const bool issuer = (lane == 0);
             uint32_t s = 0, ph = 0, it = 0;
             const uint32_t hi = (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);     // SBO 1024 B, version 1, 128-byte swizzle
             const uint32_t a_lo0 = ((sA >> 4) & 0x3FFFu) | (1u << 16), b_lo0 = ((sB >> 4) & 0x3FFFu) | (1u << 16);
             const uint32_t a_step = a_stage >> 4, b_step = b_stage >> 4;
             const uint32_t row_step = (uint32_t)(p.W * 128) >> 4;                      // (column shift) a tap's rows lie W pixels further on
             uint32_t a_lo = a_lo0, b_lo = b_lo0;
-            for (int64_t tile = first; tile < cfg.ntiles && !*abort_flag; tile += step, ++it) {
+            for (int64_t tile = first; tile < cfg.ntiles; tile += step, ++it) {
                 const uint32_t ab = it & 1;
-                if (!bar_wait(bar_tempty + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag)) break;
+                if (!bar_wait_step(bar_tempty + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d_tmem = tmem_base + ab * 256;
                 bool ok = true;
                 for (int kb = 0; kb < cfg.nkb; kb += kShift ? 3 : kSub2) {
-                    if (!bar_wait(bar_full + 8 * s, ph, abort_flag)) { ok = false; break; }
+                    if (!bar_wait_step(bar_full + 8 * s, ph, abort_flag)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     if (kShift) {
-                        if (issuer) {
+                        {
 #pragma unroll
                             for (int i = 0; i < 3; ++i) {
                                 const uint32_t a1 = a_lo + i * (kStageA >> 4), b1 = b_lo + i * row_step;
-                                pair_mma(d_tmem, a1, b1, hi, cfg.idesc, (kb | i) ? 1u : 0u);
-                                pair_mma(d_tmem, a1 + 2, b1 + 2, hi, cfg.idesc, 1u);
-                                pair_mma(d_tmem, a1 + 4, b1 + 4, hi, cfg.idesc, 1u);
-                                pair_mma(d_tmem, a1 + 6, b1 + 6, hi, cfg.idesc, 1u);
+                                mma_i8_pair_step(d_tmem, a1, b1, hi, cfg.idesc, (kb | i) ? 1u : 0u);
                             }
                             pair_commit(bar_empty + 8 * s);
                         }
-                    } else if (issuer) {
-                        pair_mma(d_tmem, a_lo, b_lo, hi, cfg.idesc, kb ? 1u : 0u);
-                        pair_mma(d_tmem, a_lo + 2, b_lo + 2, hi, cfg.idesc, 1u);
-                        pair_mma(d_tmem, a_lo + 4, b_lo + 4, hi, cfg.idesc, 1u);
-                        pair_mma(d_tmem, a_lo + 6, b_lo + 6, hi, cfg.idesc, 1u);
-                        if (kb + 1 < cfg.nkb) {
-                            const uint32_t a1 = a_lo + (kStageA >> 4), b1 = b_lo + (kStageB >> 4);
-                            pair_mma(d_tmem, a1, b1, hi, cfg.idesc, 1u);
-                            pair_mma(d_tmem, a1 + 2, b1 + 2, hi, cfg.idesc, 1u);
-                            pair_mma(d_tmem, a1 + 4, b1 + 4, hi, cfg.idesc, 1u);
-                            pair_mma(d_tmem, a1 + 6, b1 + 6, hi, cfg.idesc, 1u);
-                        }
+                    } else {
+                        mma_i8_pair_step(d_tmem, a_lo, b_lo, hi, cfg.idesc, kb ? 1u : 0u);
+                        if (kb + 1 < cfg.nkb) mma_i8_pair_step(d_tmem, a_lo + (kStageA >> 4), b_lo + (kStageB >> 4), hi, cfg.idesc, 1u);
                         pair_commit(bar_empty + 8 * s);
                     }
                     a_lo += a_step;
@@ -379,7 +369,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                     if (++s == (uint32_t)ring) { s = 0; ph ^= 1; a_lo = a_lo0; b_lo = b_lo0; }
                 }
                 if (!ok) break;
-                if (issuer) pair_commit(bar_tfull + 8 * ab);
+                pair_commit(bar_tfull + 8 * ab);
             }
         }
     } else if (warp >= kFirstEpi2) {
