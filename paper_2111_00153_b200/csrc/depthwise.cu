@@ -11,9 +11,9 @@
 // 74 us for 56 x 56 x 192 at batch 64).  So the words of four neighbouring columns are transposed (4 x 4
 // bytes, eight permutes), which makes the three taps of a kernel row one dot product; a thread owns a
 // channel quad and four neighbouring columns and walks down a strip of rows, so that every input row is
-// loaded and transposed once for the three output rows that it touches, and the next row's loads are in
-// flight meanwhile (48 us with launches back to back, 54 alone behind a flushed L2; what is left is load latency at two
-// blocks per SM).
+// loaded and transposed once for the three output rows that it touches.  Its next four input rows are on their way
+// meanwhile, into words of shared memory of its own (nobody waits for anybody): in registers one row was what there was room for
+// (56 x 56 x 192 at batch 64, launches back to back: 44.2 us so, 41.9 with the ring; two blocks of 128-register threads per SM).
 // Other filters: a word is split into four one-channel words, one output per work item.
 #include <algorithm>
 #include "common.cuh"
@@ -24,6 +24,10 @@ namespace {
 
 constexpr int kDwThreads = 256;
 constexpr int kDwCols = 4;                                 // output columns per thread (3 x 3 path)
+constexpr size_t kDwSmem = 226 * 1024;
+constexpr int kDwAhead = 4;                                // input rows on their way per thread (3 x 3 path)
+constexpr uint32_t kDwRingColumn = kDwThreads * 4;         // a column of a ring row: a word per thread
+__host__ __device__ constexpr int dw_ring_bytes(int s) { return (kDwAhead + 1) * (3 * s + 3) * (int)kDwRingColumn; }
 // Sums start from the bits of 1.5 * 2^23: a nine-tap sum of int8 products is below 2^18, so the finished word IS the
 // float 1.5 * 2^23 + sum and one subtraction gives float(sum) exactly.
 constexpr int kDwMagicBits = 0x4B400000;
@@ -82,6 +86,12 @@ __device__ __forceinline__ uint32_t dw_word(const DwRow<kS>& r, int c, int j)
     else return j == 2 ? r.t[c] : dw_prmt(r.t[c], r.t[4], 0x0032u | (uint32_t)(4 + c) << 8 | (uint32_t)(4 + c) << 12);      // 4 5 6, 6 7 8
 }
 
+// A word from global to shared memory without passing through a register; `bytes` 0: zeros, nothing is read.
+__device__ __forceinline__ void dw_copy(uint32_t dst, const int8_t* src, uint32_t bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ void dw_store(const Problem& p, uint32_t n, int q, const int* acc)
 {
     const float4 ws = __ldg(reinterpret_cast<const float4*>(p.wstep) + q);
@@ -130,6 +140,7 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
         const uint32_t ncol = (uint32_t)(p.Wo + kDwCols - 1) / kDwCols, nstrip = (uint32_t)(p.Ho + strip - 1) / (uint32_t)strip;
         const uint32_t n_items = (uint32_t)p.B * nstrip * ncol;
         constexpr int kXW = 3 * kS + 3;                                // input columns under four outputs
+        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_w) + (uint32_t)((taps * C + 15) & ~15) + 4u * threadIdx.x;
         for (int qi = 0; qi < qpt; ++qi) {
             const int q = my_q0 + qi * lanes_q;
             if (q >= quads) break;
@@ -154,18 +165,32 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
                 // behind the last input row of the strip; 0 where the whole strip lies in the padding above the image, so
                 // that the one unsigned comparison in load() rules out rows in front of the image too
                 const int y_end = max(0, min(p.H, (ho0 + rows - 1) * kS - p.pad + 3));
-                auto load = [&](int y, uint32_t (&a)[kXW]) {           // rows and columns outside the image read as zero
+                // The thread's next input row on its way to its own words of the ring; rows and columns outside the image become zeros.
+                int y = ho0 * kS - p.pad;                              // the input row to fetch next
+                uint32_t put = ring, got = ring;                       // where it goes, and where the next one to be used lies
+                auto fetch = [&]() {
                     const int8_t* r = src + (int64_t)y * row_pitch;
                     if ((unsigned)y >= (unsigned)y_end) {
 #pragma unroll
-                        for (int x = 0; x < kXW; ++x) a[x] = 0u;
-                    } else if (in_x == (1u << kXW) - 1u) {             // the usual case, without a predicate per column
+                        for (int x = 0; x < kXW; ++x) dw_copy(put + x * kDwRingColumn, p.act, 0u);
+                    } else if (in_x == (1u << kXW) - 1u) {             // the usual case, without a choice per column
 #pragma unroll
-                        for (int x = 0; x < kXW; ++x) a[x] = __ldg(reinterpret_cast<const uint32_t*>(r + (uint32_t)x * pitch));
+                        for (int x = 0; x < kXW; ++x) dw_copy(put + x * kDwRingColumn, r + (uint32_t)x * pitch, 4u);
                     } else {
 #pragma unroll
-                        for (int x = 0; x < kXW; ++x) a[x] = ((in_x >> x) & 1u) ? __ldg(reinterpret_cast<const uint32_t*>(r + (uint32_t)x * pitch)) : 0u;
+                        for (int x = 0; x < kXW; ++x) dw_copy(put + x * kDwRingColumn, (in_x >> x) & 1u ? r + (uint32_t)x * pitch : p.act, (in_x >> x) & 1u ? 4u : 0u);
                     }
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                    ++y;
+                    put = put == ring + (kDwAhead * kXW) * kDwRingColumn ? ring : put + kXW * kDwRingColumn;
+                };
+                // The row fetched kDwAhead rows ago; the place of the one used before it is free for the next.
+                auto take = [&](uint32_t (&a)[kXW]) {
+                    asm volatile("cp.async.wait_group %0;" ::"n"(kDwAhead - 1) : "memory");
+#pragma unroll
+                    for (int x = 0; x < kXW; ++x) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(a[x]) : "r"(got + x * kDwRingColumn) : "memory");
+                    got = got == ring + (kDwAhead * kXW) * kDwRingColumn ? ring : got + kXW * kDwRingColumn;
+                    fetch();
                 };
                 float* out = p.out + ((size_t)b * p.Ho * p.Wo + (size_t)ho0 * p.Wo + wo0) * p.ld_out + 4 * q;
                 int32_t* const acc_out = kAcc ? p.acc + (out - p.out) : nullptr;
@@ -191,35 +216,24 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
                     }
                 };
                 DwRow<kS> r[3];
-                uint32_t a[kXW], nx[kXW];
-                int y = ho0 * kS - p.pad;                              // the input row to arrange next
-                if constexpr (kS == 1) {
-                    load(y, a);
-                    load(y + 1, nx);
-                    dw_arrange<1>(a, r[0]);
-                    load(y + 2, a);
-                    dw_arrange<1>(nx, r[1]);
-                    y += 3;
-                    for (int h = 0; h < rows; h += 3) {
-                        // three output rows a turn, so that the rows' places in r[] are fixed; a row's words are
-                        // loaded while the row in front of it is worked on
-                        load(y, nx); dw_arrange<1>(a, r[2]); emit(h, r[0], r[1], r[2]);
-                        if (h + 1 < rows) { load(y + 1, a); dw_arrange<1>(nx, r[0]); emit(h + 1, r[1], r[2], r[0]); }
-                        if (h + 2 < rows) { load(y + 2, nx); dw_arrange<1>(a, r[1]); emit(h + 2, r[2], r[0], r[1]); }
+                uint32_t a[kXW];
+                asm volatile("cp.async.wait_group 0;" ::: "memory");   // (what the last item fetched behind its end: zeros)
 #pragma unroll
-                        for (int x = 0; x < kXW; ++x) a[x] = nx[x];
-                        y += 3;
+                for (int i = 0; i < kDwAhead; ++i) fetch();
+                if constexpr (kS == 1) {
+                    take(a); dw_arrange<1>(a, r[0]);
+                    take(a); dw_arrange<1>(a, r[1]);
+                    for (int h = 0; h < rows; h += 3) {
+                        // three output rows a turn, so that the rows' places in r[] are fixed
+                        take(a); dw_arrange<1>(a, r[2]); emit(h, r[0], r[1], r[2]);
+                        if (h + 1 < rows) { take(a); dw_arrange<1>(a, r[0]); emit(h + 1, r[1], r[2], r[0]); }
+                        if (h + 2 < rows) { take(a); dw_arrange<1>(a, r[1]); emit(h + 2, r[2], r[0], r[1]); }
                     }
                 } else {
-                    load(y, a);
-                    load(y + 1, nx);
-                    dw_arrange<2>(a, r[0]);
-                    load(y + 2, a);
-                    y += 3;
+                    take(a); dw_arrange<2>(a, r[0]);
                     for (int h = 0; h < rows; h += 2) {                // r[0] and r[2] take turns as the shared row
-                        dw_arrange<2>(nx, r[1]); load(y, nx); dw_arrange<2>(a, r[2]); load(y + 1, a); emit(h, r[0], r[1], r[2]);
-                        if (h + 1 < rows) { dw_arrange<2>(nx, r[1]); load(y + 2, nx); dw_arrange<2>(a, r[0]); load(y + 3, a); emit(h + 1, r[2], r[1], r[0]); }
-                        y += 4;
+                        take(a); dw_arrange<2>(a, r[1]); take(a); dw_arrange<2>(a, r[2]); emit(h, r[0], r[1], r[2]);
+                        if (h + 1 < rows) { take(a); dw_arrange<2>(a, r[1]); take(a); dw_arrange<2>(a, r[0]); emit(h + 1, r[2], r[1], r[0]); }
                     }
                 }
             }
@@ -266,15 +280,16 @@ bool depthwise_supported(const Problem& p)
 
 cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
 {
-    const size_t smem = (size_t)p.kh * p.kw * p.M;
-    const int variant = (p.kh == 3 && p.kw == 3 && (p.stride == 1 || p.stride == 2)) ? p.stride : 0;
+    const size_t table = (size_t)p.kh * p.kw * p.M, with_ring = ((table + 15) & ~(size_t)15) + dw_ring_bytes(p.stride);
+    const int variant = (p.kh == 3 && p.kw == 3 && (p.stride == 1 || p.stride == 2) && with_ring <= kDwSmem) ? p.stride : 0;
+    const size_t smem = variant ? with_ring : table;
     const bool acc = variant != 0 && p.acc;
     static bool attr_set[3][2][kMaxDevices] = {};
     void (*const kernel)(const Problem, const int) = variant == 1 ? (acc ? depthwise_kernel<1, true> : depthwise_kernel<1, false>)
                                                    : variant == 2 ? (acc ? depthwise_kernel<2, true> : depthwise_kernel<2, false>)
                                                                   : depthwise_kernel<0, false>;
     const void* fn = reinterpret_cast<const void*>(kernel);
-    if (smem > 48 * 1024 && !ensure_smem_attr(fn, 200 * 1024, attr_set[variant][acc])) return cudaErrorUnknown;
+    if (smem > 48 * 1024 && !ensure_smem_attr(fn, (int)kDwSmem, attr_set[variant][acc])) return cudaErrorUnknown;
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kDwThreads, smem);
     if (e != cudaSuccess) return e;
