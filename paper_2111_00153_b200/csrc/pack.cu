@@ -323,13 +323,15 @@ __global__ void __launch_bounds__(256) quantize_act_kernel(const float* __restri
         // instruction covering 512 contiguous bytes, then eight 32-bit stores of 128 contiguous
         // bytes each.  The remaining 16-value groups follow one lane at a time.  The values are read once and leave L2
         // first; the codes are stored to stay, the layer reads them next (stored streaming: ResNet-18 at batch 256
-        // 1062 us against 1042, the MobileNet-v2 block 127.6 against 125.8).
+        // 1062 us against 1042, the MobileNet-v2 block 127.6 against 125.8).  The last values come first: what was written last
+        // is what L2 still holds of a larger tensor (the depthwise layer's 154 MB behind it 26.9 -> 25.4 us).
         const size_t n16 = count / 16;
         const size_t n1024 = count / 1024;
         const int lane = threadIdx.x & 31;
         const size_t warp = tid >> 5, nwarp = nthr >> 5;
         const ActFast fast = act_fast_setup(alpha, kind);
-        for (size_t i = warp; i < n1024; i += nwarp) {
+        for (size_t k = warp; k < n1024; k += nwarp) {
+            const size_t i = n1024 - 1 - k;
             const float4* src = reinterpret_cast<const float4*>(x) + i * 256 + lane;
             float4 v[8];
 #pragma unroll
