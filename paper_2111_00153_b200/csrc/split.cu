@@ -116,6 +116,9 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     // writes or reads -- activations, outputs, the status word -- stays behind the waits further down (see launch_dependent).
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
+    const int32_t* const slot_of = p.slot;
+    const float* const wstep = p.wstep;
+    const uint8_t* const kind_of = p.kind;
 
     int b0, h0;
     if (cfg.tiles_per_image) { b0 = nt / cfg.tiles_per_image; h0 = (nt - b0 * cfg.tiles_per_image) * cfg.th; }
@@ -184,7 +187,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         const uint8_t* src = p.q4;
         if (m_row < p.M) {
             kind = p.kind[m_row];
-            const int packed = __ldg(p.slot + m_row);
+            const int packed = __ldg(slot_of + m_row);
             src = kind == kFixed8 ? p.q8 + (size_t)(packed - p.nP - p.nF4) * p.Kp : p.q4 + (size_t)packed * (p.Kp >> 1);
         }
         const uint32_t swz = cfg.bk == 128 ? (uint32_t)(row & 7) : (uint32_t)((row >> 1) & 3);
@@ -309,8 +312,8 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     float scale = 0.0f;
     int shift = 0;
     if (row_ok) {
-        scale = __fmul_rn(__ldg(p.wstep + m), p.act_step);
-        shift = (!kPre && __ldg(p.kind + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
+        scale = __fmul_rn(__ldg(wstep + m), p.act_step);
+        shift = (!kPre && __ldg(kind_of + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
     }
     pdl_wait();                                           // the outputs
     const ActFast rq = act_fast_setup(kRQ ? p.rq_alpha : 1.0f, kRQ ? p.rq_kind : 0);

@@ -258,6 +258,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     // launch_dependent)
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
+    const float* const wstep = p.wstep;                   // (weights: read ahead of the wait)
+    const uint8_t* const kind_of = p.kind;
 
     // (tile indices fit 32 bits with a step to spare: checked on the host)
     const uint32_t ntiles = (uint32_t)cfg.ntiles;
@@ -675,8 +677,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 scale = 0.f;
                 shift = 0;
                 if (row_ok) {
-                    scale = __fmul_rn(__ldg(p.wstep + m), p.act_step);
-                    shift = (!kPre && __ldg(p.kind + m) == kFixed4) ? 4 : 0;   // expanders store Fixed-4 codes as 16 * value
+                    scale = __fmul_rn(__ldg(wstep + m), p.act_step);
+                    shift = (!kPre && __ldg(kind_of + m) == kFixed4) ? 4 : 0;   // expanders store Fixed-4 codes as 16 * value
                 }
             }
             if (!mbar_wait_warp(bar_tfull + 8 * ab, tpar, abort_flag)) { alive = false; break; }

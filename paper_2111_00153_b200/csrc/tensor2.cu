@@ -249,6 +249,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     // launch_dependent)
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
+    const float* const wstep = p.wstep;                   // (weights: read ahead of the wait)
 
     const int64_t first = blockIdx.x >> 1, step = gridDim.x >> 1;      // cluster index, clusters in the grid
     const uint32_t lead_full = map_to_rank(bar_full, 0), lead_tempty = map_to_rank(bar_tempty, 0);
@@ -389,7 +390,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
             const int64_t nt = tile / cfg.nbt;
             const int blk = (int)(tile - nt * cfg.nbt) * 2 + (int)rank;
             const int m = blk * kBlockRows + quarter * 32 + lane;
-            const float scale = (m < p.M) ? __fmul_rn(__ldg(p.wstep + m), p.act_step) : 0.f;
+            const float scale = (m < p.M) ? __fmul_rn(__ldg(wstep + m), p.act_step) : 0.f;
             int64_t n0h[2];
             int nvalid[2];
 #pragma unroll
