@@ -40,9 +40,14 @@ constexpr int kNumEpiWarps = 4;
 constexpr int kPreWarps = 2 + 8 + kNumEpiWarps;  // warps of the forms that have no expanders
 constexpr int kGroups = 2;                       // expander groups taking alternate k-blocks
 constexpr int kNumExpWarps = 4 * kGroups;
-__host__ __device__ constexpr int threads_of(int mode) { return 32 * (mode ? kPreWarps : 2 + kNumExpWarps + kNumEpiWarps); }
+// Codes out: a chunk is some 250 instructions, most of them waiting for the one in front, and its bytes are few: more warps with
+// one set of registers each, not twelve with two (192x32 on 200,704 pixels 25.5 us with twelve, 23.9 so; 256x256 3x3 on 256 images
+// of 14x14 30.9 and 30.4).
+constexpr int kRqWarps = 22;
+__host__ __device__ constexpr int warps_of(int mode, int rq) { return mode ? (rq ? kRqWarps : kPreWarps) : 2 + kNumExpWarps + kNumEpiWarps; }
 constexpr int kWarpStage = 32 * 32 * 4;          // 4 KB: 32 pixels x 32 rows of fp32/int32
-constexpr int kWideEpi = 8;                      // epilogue warps of the form with 144 KB of resident weights
+constexpr int kRqStage = 2 * 32 * 32;            // two buffers of 32 pixels x 32 codes
+constexpr int kWideEpi = 8;                      // epilogue warps of the form with 144 KB of resident weights (codes out: twice as many)
 constexpr int kMaxRing = 8;
 constexpr int kResidentBlocks = 16;              // row blocks of a layer with resident weights (the grid is a multiple of them)
 constexpr int kSmemLimit = 232448 - 1024;        // 227 KB per CTA less room for the static variables
@@ -213,10 +218,10 @@ __device__ __forceinline__ void tmem_ld_four(uint32_t taddr, uint32_t (&v)[4])
 // kOut:  1 when the output is fp32 [N][M] through bulk stores without an accumulator dump (the common case): the
 //        epilogue then carries only that path; 0 decides at run time.
 template <int kM2, int kRQ, int kMode, int kOut>
-__global__ void __launch_bounds__(threads_of(kMode), 1)
+__global__ void __launch_bounds__(32 * warps_of(kMode, kRQ), 1)
 tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps maps)
 {
-    constexpr int kThreads = threads_of(kMode);
+    constexpr int kThreads = 32 * warps_of(kMode, kRQ);
     constexpr bool kPre = kMode != 0, kAres = kMode >= 2, kTps3 = kMode == 3;
     const bool use_tma_store = kOut ? true : (cfg.tma_store != 0);
     const bool out_mn = kOut ? false : (p.out_mn != 0);
@@ -226,7 +231,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     const uint32_t sA = smem_base;
     const uint32_t sB = sA + cfg.nA * cfg.a_bytes;
     const uint32_t sOut = sB + cfg.nB * cfg.b_bytes;
-    const uint32_t sBar = sOut + cfg.epi_warps * cfg.out_bufs * kWarpStage;
+    const uint32_t sBar = sOut + cfg.epi_warps * cfg.out_bufs * (kRQ ? kRqStage : kWarpStage);
     // barriers, 8 bytes each
     const uint32_t bar_fullA = sBar, bar_emptyA = sBar + 8 * kMaxRing;
     const uint32_t bar_fullB = sBar + 16 * kMaxRing, bar_emptyB = sBar + 24 * kMaxRing;
@@ -648,7 +653,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         const int row0 = dup ? (quarter & 1) * 32 : quarter * 32;       // first row (within the block) of this warp
         const int cstride = dup ? count_q(quarter & 1) + count_q((quarter & 1) + 2) : count_q(quarter);
         const int cfirst = (dup && (quarter >> 1)) ? count_q(quarter & 1) + my_rank : my_rank;
-        const uint32_t my_stage = sOut + (uint32_t)ew * (cfg.out_bufs * kWarpStage);
+        const uint32_t my_stage = sOut + (uint32_t)ew * (cfg.out_bufs * (kRQ ? kRqStage : kWarpStage));
         uint32_t it = 0, stg_count = 0;
         bool alive = true;
         int scale_blk = -1, shift = 0;
@@ -859,6 +864,19 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     }
                 }
             };
+            if (kRQ) {
+                // (a re-quantizing chunk may read its accumulators again: the buffer is handed back after the last one)
+                uint32_t v[32];
+#pragma unroll 1
+                for (int c = cfirst; c < nchunks; c += cstride) {
+                    tmem_ld_issue(taddr + c * 32, v);
+                    tmem_ld_wait(v);
+                    emit(v, c);
+                    __syncwarp();
+                }
+                release_tmem();
+                continue;
+            }
             // two register sets: the load of this warp's next chunk is in flight while the current one is emitted
             // (tensor-memory loads and their waits are warp-wide: every chunk ends with the warp together again)
             uint32_t va[32], vb[32];
@@ -867,18 +885,15 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             for (int c = cfirst; c < nchunks; c += 2 * cstride) {
                 const int c1 = c + cstride, c2 = c + 2 * cstride;
                 const bool more1 = c1 < nchunks;
-                // (a re-quantizing chunk may read its accumulators again: the buffer is handed back after it)
-                if (more1) tmem_ld_issue(taddr + c1 * 32, vb); else if (!kRQ) release_tmem();
+                if (more1) tmem_ld_issue(taddr + c1 * 32, vb); else release_tmem();
                 emit(va, c);
                 __syncwarp();
-                if (!more1 && kRQ) release_tmem();
                 if (more1) {
                     tmem_ld_wait(vb);
                     const bool more2 = c2 < nchunks;
-                    if (more2) tmem_ld_issue(taddr + c2 * 32, va); else if (!kRQ) release_tmem();
+                    if (more2) tmem_ld_issue(taddr + c2 * 32, va); else release_tmem();
                     emit(vb, c1);
                     __syncwarp();
-                    if (!more2 && kRQ) release_tmem();
                     if (more2) tmem_ld_wait(va);
                 }
             }
@@ -1035,16 +1050,17 @@ bool plan(const Problem& p, TensorCfg& c)
     c.ares = 0;
     c.cta_full = 0;
     c.epi_warps = kNumEpiWarps;
+    const int stage = p.rq_codes ? kRqStage : kWarpStage;
     if (c.pre) {
         c.nA = (c.bk == 64) ? 6 : 3; c.nB = (c.bk == 64) ? 8 : 4; c.out_bufs = 1;
-        c.epi_warps = kPreWarps - 3;   // warp 2 fetches the weights (unless they are resident)
+        c.epi_warps = warps_of(1, p.rq_codes != nullptr) - 3;   // warp 2 fetches the weights (unless they are resident)
         c.dup = (p.M <= 64) ? 1 : 0;
         if (resident) {
             c.ares = 1;
-            c.epi_warps = wide ? kWideEpi : kPreWarps - 2;
+            c.epi_warps = wide ? (p.rq_codes ? 2 * kWideEpi : kWideEpi) : warps_of(1, p.rq_codes != nullptr) - 2;
             c.nA = c.nkb;
             const int64_t left = kSmemLimit - (1024 + 64 * kMaxRing) - (int64_t)c.nkb * c.a_bytes -
-                                 (int64_t)c.epi_warps * kWarpStage;
+                                 (int64_t)c.epi_warps * stage;
             c.nB = (int)std::min<int64_t>(kMaxRing, left / c.b_bytes);
         }
         c.tps = 1;
@@ -1059,7 +1075,7 @@ bool plan(const Problem& p, TensorCfg& c)
                 c.b_bytes = ((c.th + 2) * p.W * c.bk + 1023) / 1024 * 1024;
             }
             const int64_t left = kSmemLimit - (1024 + 64 * kMaxRing) - (int64_t)c.nkb * c.a_bytes -
-                                 (int64_t)c.epi_warps * kWarpStage;
+                                 (int64_t)c.epi_warps * stage;
             c.nB = (int)std::min<int64_t>(kMaxRing, left / c.b_bytes);
             if (c.nB < 2) { c.tps = 1; c.colshift = 0; c.tx_bytes = (uint32_t)c.npix * (uint32_t)c.bk; c.b_bytes = kTileN * c.bk; c.b_sub = c.b_bytes; c.nB = (int)std::min<int64_t>(kMaxRing, left / c.b_bytes); }
         }
@@ -1077,7 +1093,7 @@ bool plan(const Problem& p, TensorCfg& c)
         }
         c.a_rows = c.m2 ? 2 * kBlockRows : c.nbt > 1 ? kBlockRows : (std::min(p.M, c.dup ? kBlockRows / 2 : kBlockRows) + 7) / 8 * 8;
         c.a_tx = (uint32_t)(c.a_rows * c.bk * (c.dup && c.nbt == 1 ? 2 : 1));
-        c.smem_bytes = (uint32_t)(c.nA * c.a_bytes + c.nB * c.b_bytes + c.epi_warps * c.out_bufs * kWarpStage + 1024 +
+        c.smem_bytes = (uint32_t)(c.nA * c.a_bytes + c.nB * c.b_bytes + c.epi_warps * c.out_bufs * stage + 1024 +
                                   64 * kMaxRing);
         return true;
     }
@@ -1262,7 +1278,7 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
     if (!fn) return RMSMP_ERR_VARIANT;
     static bool attr_set[4][2][3][kMaxDevices] = {};
     if (!ensure_smem_attr(reinterpret_cast<const void*>(fn), kSmemLimit, attr_set[mode][i2][io])) return RMSMP_ERR_CUDA;
-    if (launch_dependent(fn, (unsigned)grid, threads_of(mode), c.smem_bytes, st, p, c, mp) != cudaSuccess) {
+    if (launch_dependent(fn, (unsigned)grid, 32 * warps_of(mode, io == 1), c.smem_bytes, st, p, c, mp) != cudaSuccess) {
         cudaGetLastError();
         return RMSMP_ERR_CUDA;
     }
