@@ -1344,3 +1344,22 @@ def test_patch_matrix_of_three_channels(k, stride, pad, B, H, W, offset):
     got = out.cpu().numpy()
     assert np.array_equal(got[128:-128].reshape(ref.shape), ref)
     assert (got[:128] == 99).all() and (got[-128:] == 99).all()
+
+
+@pytest.mark.parametrize("stride,B", [(1, 2048), (2, 4096)])
+def test_depthwise_threads_that_take_several_strips(stride, B):
+    """A thread's copies for one strip are over before those for the next begin."""
+    import torch
+    C, H = 96, 7
+    g = synth.rng(144, B)
+    Wt = synth.weights_kaiming(g, C, 1, 3, 3)
+    scheme, bits = O.assign_rows(Wt, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    codes = g.integers(-128, 128, size=(B, H, H, C), dtype=np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    v_ref, wstep = O.quantize_rows(Wt.reshape(C, -1), scheme, bits, alpha)
+    acc_ref = O.conv_depthwise(v_ref.reshape(C, 3, 3), codes, stride, 1)
+    y = torch.full(acc_ref.shape, float("nan"), dtype=torch.float32, device="cuda")
+    R.rmsmp_conv_depthwise(layer, d_packed, torch.from_numpy(codes).cuda(), B, H, H, stride, 1, 0.5, y)
+    torch.cuda.synchronize()
+    assert np.array_equal(y.cpu().numpy().view(np.uint32), O.epilogue(acc_ref, wstep, np.float32(0.5)).view(np.uint32))
