@@ -162,18 +162,23 @@ def _stream(stream):
 
 
 _raw_stream = None
+_raw_pair = None         # torch's accessors of the current stream's handle and the current device
+_accessors = None        # the extension module's call that takes them, once it is loaded
 
 
 def _first_stream():
     """The current stream through torch's public call, which also starts CUDA up.  From then on its handle is read
     directly where this torch has the accessor: the public call builds a Stream object (3.4 us, a third of a small
     layer's call; the accessor 0.2 us)."""
-    global _raw_stream
+    global _raw_stream, _raw_pair
     import torch
     handle = torch.cuda.current_stream().cuda_stream
     raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
     if raw is not None and device is not None:
         _raw_stream = lambda: raw(device())
+        _raw_pair = (raw, device)
+        if _accessors is not None:
+            _accessors(*_raw_pair)
     else:
         _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
     return handle
@@ -214,12 +219,16 @@ def _host_array(a, fmt: str):
 
 
 def _load_native():
+    global _accessors
     L = lib()
     try:
         from . import _marshal
     except ImportError as e:
         raise RuntimeError(f"the extension module _marshal is missing: build it with `python -m {__package__}.build`") from e
     _marshal.setup({n: C.cast(getattr(L, n), C.c_void_p).value for n in _NATIVE}, _current_stream, _raise, _host_array)
+    _accessors = _marshal.stream_accessors
+    if _raw_pair is not None:
+        _accessors(*_raw_pair)
     for n in _NATIVE:
         globals()[n] = getattr(_marshal, n)
 

@@ -43,6 +43,7 @@ struct Problem {
     int B, H, W, Ho, Wo, stride, pad;
     int64_t pix_pitch;
     int64_t N;                // B*Ho*Wo
+    int sms;                  // SMs of the device (looked up once a call: the plans ask for it a dozen times)
     int ragged_k;             // linear layer under AUTO: a K that is not a multiple of 16 may take the tensor path (rows are
                               // 16-byte aligned all the same; the copy engine fills up with zeros)
     int act_nonneg;           // grouped tensor-core launch: every activation code is within 0..15
@@ -173,18 +174,18 @@ cudaError_t launch_stream(const uint8_t* d_table, int grid, uint32_t smem_bytes,
 // returns false if the tensor variant cannot run this problem (alignment / shape)
 bool tensor_supported(const Problem& p);
 bool tensor_resident(const Problem& p);   // the weights of a row block stay in shared memory
+// The contraction on the tensor cores by whichever kernel takes the problem; RMSMP_ERR_VARIANT, with nothing queued, if none can.
+// The launch_*_if_better() plan once: they return false if theirs is not the kernel to take, and otherwise launch it (*s).
 rmsmp_status launch_tensor(const Problem& p, cudaStream_t st);
 // fills four CUtensorMap objects (see act_parity_split; only the first is used without the split) for
 // activation boxes of bk channels x th output rows x tb images, swizzle width = bk bytes
 bool encode_act_maps_4(const Problem& p, int bk, int th, int tb, void* maps4);
-// two-CTA form of the workspace mode (tensor2.cu): false if it cannot, or should not, run this problem
-bool pair_supported(const Problem& p);
-rmsmp_status launch_pair(const Problem& p, cudaStream_t st);
+// two-CTA form of the workspace mode (tensor2.cu)
+bool launch_pair_if_better(const Problem& p, cudaStream_t st, rmsmp_status* s);
 // problems that do not fill the chip: narrow tiles, the reduction shared by a cluster (split.cu)
-bool split_supported(const Problem& p);
-rmsmp_status launch_split(const Problem& p, cudaStream_t st, bool gather = false);
-// the same kernel with activations gathered by threads, for what the copy engine cannot address
-bool gather_supported(const Problem& p);
+bool launch_split_if_better(const Problem& p, cudaStream_t st, rmsmp_status* s);
+// the same kernel with activations gathered by threads, for what the copy engine cannot address (RMSMP_ERR_VARIANT: not this one either)
+rmsmp_status launch_gather(const Problem& p, cudaStream_t st);
 
 // ---- activation boxes of the tensor-core kernels ----
 // A stride-2 convolution reads, for one filter tap, every second pixel of every second input row.

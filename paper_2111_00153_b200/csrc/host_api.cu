@@ -124,6 +124,7 @@ void fill_problem(Problem& p, const rmsmp_layer* L, const void* d_packed)
     p.M = L->M; p.Cin = L->Cin; p.kh = L->kh; p.kw = L->kw; p.Cp = L->Cp; p.Kp = L->Kp;
     p.nP = L->nP; p.nF4 = L->nF4; p.n8 = L->n8; p.nblocks = L->nblocks;
     p.wexp = nullptr;
+    p.sms = sm_count();
     p.ragged_k = 0;
     p.rq_codes = nullptr; p.rq_alpha = 1.0f; p.rq_kind = 0; p.ld_codes = 0;
 }
@@ -135,15 +136,14 @@ rmsmp_status dispatch(Problem& p, rmsmp_variant variant, cudaStream_t st)
         // 16384x1024 16 92 / 8.8, 30000x1024 8 85 / 17.2, 109x1333 3076 272 / 9.9); what the copy engine
         // cannot address goes to the tensor cores through gathered tiles.
         p.ragged_k = p.kh == 1 && p.kw == 1 && p.H == 1 && p.W == 1;
-        if (tensor_supported(p)) variant = RMSMP_VARIANT_TENSOR;
-        else if (gather_supported(p)) return launch_split(p, st, true);
-        else variant = RMSMP_VARIANT_SIMT;
+        rmsmp_status s = launch_tensor(p, st);
+        if (s == RMSMP_ERR_VARIANT) s = launch_gather(p, st);
+        if (s != RMSMP_ERR_VARIANT) return s;
+        variant = RMSMP_VARIANT_SIMT;
     }
     cudaError_t e = cudaSuccess;
     switch (variant) {
-        case RMSMP_VARIANT_TENSOR:
-            if (!tensor_supported(p)) return RMSMP_ERR_VARIANT;
-            return launch_tensor(p, st);
+        case RMSMP_VARIANT_TENSOR: return launch_tensor(p, st);
         case RMSMP_VARIANT_SIMT: e = launch_simt(p, false, st); break;
         case RMSMP_VARIANT_SHIFTADD: e = launch_simt(p, true, st); break;
         case RMSMP_VARIANT_SIMPLE: e = launch_simple(p, st); break;

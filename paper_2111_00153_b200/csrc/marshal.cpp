@@ -34,6 +34,7 @@ struct Api {
 } api;
 
 PyObject* g_stream;          // callable: the current stream's handle
+PyObject *g_raw, *g_device;  // torch's accessors, once CUDA has been started up: g_raw(g_device()) is that handle
 PyObject* g_error;           // callable(status, where): raises RmsmpError
 PyObject* g_array;           // callable(object, format): a contiguous array of bytes ('B') or floats ('f') with its values
 PyObject *s_data_ptr, *s_numel, *s_element_size, *s_cuda_stream;
@@ -150,7 +151,16 @@ struct Call {
     {
         if (!ok) return nullptr;
         if (!none(i) && PyLong_Check(a[i])) return address(a[i]);
-        PyObject* r = none(i) ? PyObject_CallNoArgs(g_stream) : PyObject_GetAttr(a[i], s_cuda_stream);
+        PyObject* r;
+        if (!none(i)) {
+            r = PyObject_GetAttr(a[i], s_cuda_stream);
+        } else if (g_raw) {
+            PyObject* device = PyObject_CallNoArgs(g_device);
+            r = device ? PyObject_CallOneArg(g_raw, device) : nullptr;
+            Py_XDECREF(device);
+        } else {
+            r = PyObject_CallNoArgs(g_stream);
+        }
         if (!r) { ok = false; return nullptr; }
         void* p = address(r);
         Py_DECREF(r);
@@ -475,9 +485,19 @@ PyObject* setup(PyObject*, PyObject* args)
     Py_RETURN_NONE;
 }
 
+PyObject* stream_accessors(PyObject*, PyObject* args)
+{
+    PyObject *raw, *device;
+    if (!PyArg_ParseTuple(args, "OO", &raw, &device)) return nullptr;
+    Py_INCREF(device); Py_XSETREF(g_device, device);
+    Py_INCREF(raw); Py_XSETREF(g_raw, raw);
+    Py_RETURN_NONE;
+}
+
 #define METHOD(name, doc) {"rmsmp_" #name, (PyCFunction)(void (*)(void))name, METH_FASTCALL | METH_KEYWORDS, doc}
 PyMethodDef methods[] = {
     {"setup", setup, METH_VARARGS, "entry points, current-stream callable, error callable, array callable"},
+    {"stream_accessors", stream_accessors, METH_VARARGS, "callable(device) and callable(): the current stream's handle without a Python frame"},
     METHOD(quantize_act, "Returns the activation step (alpha_a/15 or alpha_a/7) as a Python float (fp32 value)."),
     METHOD(gemm, "Linear layer."),
     METHOD(gemm_variant, "Linear layer by a chosen kernel."),

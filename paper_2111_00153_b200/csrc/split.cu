@@ -470,7 +470,7 @@ bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr, bool gat
     if (!gather && (p.pix_pitch % 16 != 0 || (reinterpret_cast<uintptr_t>(p.act) & 15) != 0)) return false;
     if (gather && (p.wexp || p.rq_codes || p.N >= (int64_t)1 << 31)) return false;
     if (p.wexp && (reinterpret_cast<uintptr_t>(p.wexp) & 15) != 0) return false;
-    const int64_t sms = sm_count();
+    const int64_t sms = p.sms;
     SplitCfg c;
     memset(&c, 0, sizeof(c));
     c.pre = p.wexp ? 1 : 0;
@@ -530,46 +530,8 @@ bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr, bool gat
     return true;
 }
 
-}  // namespace
-
-// Which of the two kernels takes a problem.  With a workspace the persistent kernel takes whatever fills the chip;
-// below that its time is one tile's: 3.4 us + 1.2 for the output of 256 pixels + 0.28 to 0.41 per k-block of 128 codes
-// (measured: 256x512 N=64 4.8 us against 4.1 here, 256x2304 N=196 11.7 against 5.4, 512x4608 N=49 16 against 6,
-// 768x3072 N=512 13.5 against 10.2, N=2048 13.7 against 14).  Without one it expands the weights first, 1.7 us + 0.7 a
-// k-block, if they stay resident (128x512 N=2000 10.6 against 6.5, 1024x512 N=4096 10.9 against 17.4), and otherwise
-// again for every tile, 0.59 us a k-block and round of tiles (768x3072 N=1024 21.5 against 14.7, N=4096 22.2 against 37.5;
-// 3x3 256x256 on 6272 pixels 17.8 against 15.9, on 12,544 18.2 against 31.5).
-bool split_supported(const Problem& p)
+rmsmp_status launch_planned(const Problem& p, const SplitCfg& c, cudaStream_t st, bool gather)
 {
-    const double sms = sm_count(), tiles = (double)((p.N + 255) / 256 * p.nblocks);
-    const bool bk64 = p.Cin % 128 != 0 && p.Cin % 128 <= 64;
-    const double nkb = (double)p.kh * p.kw * ((p.Cin + 127) / 128) * (bk64 && p.Cin < 128 ? 0.5 : 1.0);
-    double other;
-    if (p.wexp || tensor_resident(p)) {
-        if (tiles >= sms) return false;
-        const int64_t hw = (int64_t)p.Ho * p.Wo;          // (its tiles are whole images: 3x3 256x256 on 32 of 14x14 11.7 us there, 12.5 here)
-        const double n = (double)std::min<int64_t>(p.N, hw <= 256 && !bk64 ? 256 / hw * hw : 256);
-        other = 3.4 + 1.2 * n / 256 + nkb * (0.28 + 0.13 * n / 256) + (p.wexp ? 0.0 : 1.7 + 0.7 * nkb);
-        if (p.out_mn && p.N < 32) other += 1.4;           // (no bulk stores: 64x64 N=8 5.2 us there, 3.3 here)
-    } else {
-        other = 7.4 + std::ceil(tiles / sms) * (0.8 + 0.59 * nkb);
-    }
-    SplitCfg c;
-    double us = 0.0;
-    return plan_split(p, c, &us) && us < other && tensor_map_encoder() != nullptr;
-}
-
-// Convolutions whose activations the copy engine cannot address.
-bool gather_supported(const Problem& p)
-{
-    SplitCfg c;
-    return plan_split(p, c, nullptr, true);
-}
-
-rmsmp_status launch_split(const Problem& p, cudaStream_t st, bool gather)
-{
-    SplitCfg c;
-    if (!plan_split(p, c, nullptr, gather)) return RMSMP_ERR_VARIANT;
     EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return RMSMP_ERR_CUDA;
     SplitMaps mp;
@@ -602,6 +564,44 @@ rmsmp_status launch_split(const Problem& p, cudaStream_t st, bool gather)
         return RMSMP_ERR_CUDA;
     }
     return RMSMP_OK;
+}
+
+}  // namespace
+
+// Which of the two kernels takes a problem.  With a workspace the persistent kernel takes whatever fills the chip;
+// below that its time is one tile's: 3.4 us + 1.2 for the output of 256 pixels + 0.28 to 0.41 per k-block of 128 codes
+// (measured: 256x512 N=64 4.8 us against 4.1 here, 256x2304 N=196 11.7 against 5.4, 512x4608 N=49 16 against 6,
+// 768x3072 N=512 13.5 against 10.2, N=2048 13.7 against 14).  Without one it expands the weights first, 1.7 us + 0.7 a
+// k-block, if they stay resident (128x512 N=2000 10.6 against 6.5, 1024x512 N=4096 10.9 against 17.4), and otherwise
+// again for every tile, 0.59 us a k-block and round of tiles (768x3072 N=1024 21.5 against 14.7, N=4096 22.2 against 37.5;
+// 3x3 256x256 on 6272 pixels 17.8 against 15.9, on 12,544 18.2 against 31.5).
+bool launch_split_if_better(const Problem& p, cudaStream_t st, rmsmp_status* s)
+{
+    const double sms = p.sms, tiles = (double)((p.N + 255) / 256 * p.nblocks);
+    const bool bk64 = p.Cin % 128 != 0 && p.Cin % 128 <= 64;
+    const double nkb = (double)p.kh * p.kw * ((p.Cin + 127) / 128) * (bk64 && p.Cin < 128 ? 0.5 : 1.0);
+    double other;
+    if (p.wexp || tensor_resident(p)) {
+        if (tiles >= sms) return false;
+        const int64_t hw = (int64_t)p.Ho * p.Wo;          // (its tiles are whole images: 3x3 256x256 on 32 of 14x14 11.7 us there, 12.5 here)
+        const double n = (double)std::min<int64_t>(p.N, hw <= 256 && !bk64 ? 256 / hw * hw : 256);
+        other = 3.4 + 1.2 * n / 256 + nkb * (0.28 + 0.13 * n / 256) + (p.wexp ? 0.0 : 1.7 + 0.7 * nkb);
+        if (p.out_mn && p.N < 32) other += 1.4;           // (no bulk stores: 64x64 N=8 5.2 us there, 3.3 here)
+    } else {
+        other = 7.4 + std::ceil(tiles / sms) * (0.8 + 0.59 * nkb);
+    }
+    SplitCfg c;
+    double us = 0.0;
+    if (!plan_split(p, c, &us) || us >= other || tensor_map_encoder() == nullptr) return false;
+    *s = launch_planned(p, c, st, false);
+    return true;
+}
+
+// Convolutions whose activations the copy engine cannot address.
+rmsmp_status launch_gather(const Problem& p, cudaStream_t st)
+{
+    SplitCfg c;
+    return plan_split(p, c, nullptr, true) ? launch_planned(p, c, st, true) : RMSMP_ERR_VARIANT;
 }
 
 }  // namespace rmsmp

@@ -956,16 +956,23 @@ bool wide_shift(const Problem& p)
     if ((int64_t)p.Ho * p.Wo <= kTileN && 2 * (int64_t)p.Ho * p.Wo <= kTileN) return false;      // (several images a tile)
     const int per_image = (p.Ho + most - 1) / most, th = (p.Ho + per_image - 1) / per_image;
     return 3 * (((th + 2) * p.W * 64 + 1023) / 1024 * 1024) <= kSmemLimit - (1024 + 64 * kMaxRing) - 18 * kBlockRows * 64 - kWideEpi * kWarpStage &&
-           (int64_t)p.B * per_image >= 2 * sm_count();
+           (int64_t)p.B * per_image >= 2 * p.sms;
 }
 
-bool plan(const Problem& p, TensorCfg& c)
+// Whether the copy engine can fetch the activations, one box a tap.
+bool addressable(const Problem& p)
 {
     if (p.pix_pitch % 16 != 0 || (p.Cin % 16 != 0 && !p.ragged_k)) return false;
     if ((reinterpret_cast<uintptr_t>(p.act) & 15) != 0) return false;
     if (p.wexp && (reinterpret_cast<uintptr_t>(p.wexp) & 15) != 0) return false;
-    const int64_t hw = (int64_t)p.Ho * p.Wo;
     if (p.Wo > kTileN || (int64_t)p.Wo * p.stride > 256) return false;
+    return (int64_t)p.Ho * p.Wo > kTileN || (int64_t)p.Ho * p.stride <= 256;      // (tiles of whole images, or of as many rows as a box has)
+}
+
+bool plan(const Problem& p, TensorCfg& c)
+{
+    if (!addressable(p)) return false;
+    const int64_t hw = (int64_t)p.Ho * p.Wo;
     if (hw <= kTileN) {
         c.th = p.Ho;
         c.tb = (int)std::min<int64_t>(kTileN / hw, p.B);
@@ -976,7 +983,7 @@ bool plan(const Problem& p, TensorCfg& c)
         // 24.1 us with 256 tokens a tile, 28.3 with 144).  [row][pixel] outputs keep to whole chunks of 32 pixels, without
         // which they leave through direct stores (256x64 N=20000 16.5 us with tiles of 144 pixels).
         if (p.wexp) {
-            const int64_t sms = sm_count();
+            const int64_t sms = p.sms;
             const double nkb = (double)p.kh * p.kw * ((p.Cin + 127) / 128);
             const double read = (double)p.N * p.Cin / 6.3e6;
             auto cost = [&](int tb) {
@@ -1001,7 +1008,7 @@ bool plan(const Problem& p, TensorCfg& c)
         // of one 6.0.  Not for a few rows, whose boxes of weights lie mostly outside the matrix and then take longer than the
         // activations' (3x3 16x16 on 12 of 62x8 6.6 and 9.9).
         if (p.wexp && p.M > 32) {
-            const double sms = sm_count(), bk = p.Cin % 128 != 0 && p.Cin % 128 <= 64 ? 64 : 128;
+            const double sms = p.sms, bk = p.Cin % 128 != 0 && p.Cin % 128 <= 64 ? 64 : 128;
             const double nkb = p.kh * p.kw * std::ceil(p.Cin / bk);
             auto cost = [&](int per_image) {
                 const double n = (double)((p.Ho + per_image - 1) / per_image * p.Wo) / 256.0;
@@ -1016,7 +1023,6 @@ bool plan(const Problem& p, TensorCfg& c)
         c.tb = 1;
         c.ntiles_n = (int64_t)p.B * c.tiles_per_image;
     }
-    if ((int64_t)c.th * p.stride > 256) return false;
     c.npix = c.tb * c.th * p.Wo;
     c.n_mma = (c.npix + 15) / 16 * 16;
     c.ntiles = c.ntiles_n * p.nblocks;
@@ -1082,7 +1088,7 @@ bool plan(const Problem& p, TensorCfg& c)
         // Two row blocks per tile pay when K is long (the two accumulators' epilogue is only half
         // hidden behind the next tile's MMAs) and when the halved tile count does not cost more in
         // idle SMs of the last wave than the ~20 % a double tile saves.
-        const int64_t sms = sm_count();
+        const int64_t sms = p.sms;
         const int64_t waves1 = (c.ntiles + sms - 1) / sms, waves2 = (c.ntiles / 2 + sms - 1) / sms;
         if (!c.ares && !c.dup && c.bk == 128 && p.nblocks % 2 == 0 && c.nkb >= 16 && 16 * waves2 < 10 * waves1) {
             c.m2 = 1;
@@ -1163,7 +1169,7 @@ bool encode_act_maps_4(const Problem& p, int bk, int th, int tb, void* maps4)
 bool tensor_resident(const Problem& p)
 {
     if (!p.wexp && p.rq_codes) return false;
-    const int64_t sms = sm_count(), tiles = (p.N + kTileN - 1) / kTileN * p.nblocks, whole = sms / p.nblocks * p.nblocks;
+    const int64_t sms = p.sms, tiles = (p.N + kTileN - 1) / kTileN * p.nblocks, whole = sms / p.nblocks * p.nblocks;
     if (whole == 0 || (p.nblocks > kResidentBlocks && (tiles + whole - 1) / whole > (tiles + sms - 1) / sms)) return false;
     if (wide_shift(p)) return true;
     const int bk = ((p.Cin % 128 != 0) && (p.Cin % 128 <= 64)) ? 64 : 128;
@@ -1186,13 +1192,14 @@ bool tensor_supported(const Problem& p)
 
 rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
 {
-    if (split_supported(p)) return launch_split(p, st);
-    if (pair_supported(p)) return launch_pair(p, st);
+    rmsmp_status s;
+    if (!addressable(p) || !encode_fn()) return RMSMP_ERR_VARIANT;
+    if (launch_split_if_better(p, st, &s) || launch_pair_if_better(p, st, &s)) return s;
     TensorCfg c;
     if (!plan(p, c)) return RMSMP_ERR_VARIANT;
     // All tiles of a CTA are of one row block where the grid is a multiple of them: required by resident weights, and with
     // expanders worth having when it costs no round of tiles (they look up a tile's rows only once then).
-    int64_t grid = sm_count();
+    int64_t grid = p.sms;
     const int64_t whole = grid / c.nbt * c.nbt;
     if (c.ares || (!c.pre && whole > 0 && (c.ntiles + whole - 1) / whole == (c.ntiles + grid - 1) / grid)) grid = whole;
     grid = std::min(grid, c.ntiles);
@@ -1203,7 +1210,7 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
         // 10.5 and 8.9, 144x160 on 740,050 134 and 108.
         const double n = c.npix / 256.0, mma = c.nkb * (0.28 + 0.13 * n) * (c.bk == 64 ? 0.6 : 1.0), out = 2.8 * n;
         const double full_us = std::max(mma, out), last_us = std::max(mma, (p.rq_codes ? 0.72 : 0.45 + 0.15 * (p.M % kBlockRows) / 64.0) * out);
-        const int64_t sms = sm_count(), even = whole / c.nbt;
+        const int64_t sms = p.sms, even = whole / c.nbt;
         double best = 0.95 * std::ceil((double)c.ntiles_n / even) * full_us;
         for (int64_t last = 1; last < even; ++last) {
             const int64_t full = (sms - last) / (c.nbt - 1);
@@ -1212,7 +1219,6 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
         }
     }
     EncodeTiledFn enc = encode_fn();
-    if (!enc) return RMSMP_ERR_CUDA;
     Maps mp;
     memset(&mp, 0, sizeof(mp));
     if (!encode_act_maps(enc, p, c.bk, c.colshift ? c.th + 2 : c.th, c.tb, c.bk == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, mp.act))

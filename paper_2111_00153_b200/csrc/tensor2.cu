@@ -466,7 +466,7 @@ bool plan_pair(const Problem& p, PairCfg& c)
         // for the weights and the rest in proportion to its pixels (768x3072 N=4096: 48 tiles for 74 pairs of SMs, or 72
         // with halves of 88 tokens: 14.1 against 12.6 us)
         {
-            const int64_t pairs = sm_count() / 2;
+            const int64_t pairs = p.sms / 2;
             auto cost = [&](int tb) {
                 const int64_t tiles = (((int64_t)p.B + tb - 1) / tb + 1) / 2 * (p.nblocks / 2);
                 return (double)((tiles + pairs - 1) / pairs) * (0.35 + 0.65 * (double)tb * (double)hw / 128.0);
@@ -529,21 +529,8 @@ bool plan_pair(const Problem& p, PairCfg& c)
     return true;
 }
 
-}  // namespace
-
-// Worth it when K is long (short reductions are dominated by the pair's start-up and by the
-// epilogue: BERT-base FFN1 with 6 k-blocks is 40 % slower this way) and both halves are well filled.
-bool pair_supported(const Problem& p)
+rmsmp_status launch_planned(const Problem& p, const PairCfg& c, cudaStream_t st)
 {
-    PairCfg c;
-    if (!plan_pair(p, c) || !tensor_map_encoder()) return false;
-    return c.nkb >= 16 && c.npix_h >= 64;
-}
-
-rmsmp_status launch_pair(const Problem& p, cudaStream_t st)
-{
-    PairCfg c;
-    if (!plan_pair(p, c)) return RMSMP_ERR_VARIANT;
     EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return RMSMP_ERR_CUDA;
     PairMaps mp;
@@ -573,7 +560,7 @@ rmsmp_status launch_pair(const Problem& p, cudaStream_t st)
     void (*const kernel)(const Problem, const PairCfg, const PairMaps) = c.shift ? pair_kernel<true> : pair_kernel<false>;
     static bool attr_set[2][kMaxDevices] = {};
     if (!ensure_smem_attr(reinterpret_cast<const void*>(kernel), kPairSmem, attr_set[c.shift])) return RMSMP_ERR_CUDA;
-    const int clusters = (int)std::min<int64_t>(c.ntiles, sm_count() / 2);
+    const int clusters = (int)std::min<int64_t>(c.ntiles, p.sms / 2);
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof(lc));
     lc.gridDim = dim3((unsigned)(2 * clusters), 1, 1);
@@ -592,6 +579,18 @@ rmsmp_status launch_pair(const Problem& p, cudaStream_t st)
         return RMSMP_ERR_CUDA;
     }
     return RMSMP_OK;
+}
+
+}  // namespace
+
+// Worth it when K is long (short reductions are dominated by the pair's start-up and by the
+// epilogue: BERT-base FFN1 with 6 k-blocks is 40 % slower this way) and both halves are well filled.
+bool launch_pair_if_better(const Problem& p, cudaStream_t st, rmsmp_status* s)
+{
+    PairCfg c;
+    if (!plan_pair(p, c) || c.nkb < 16 || c.npix_h < 64 || !tensor_map_encoder()) return false;
+    *s = launch_planned(p, c, st);
+    return true;
 }
 
 }  // namespace rmsmp
