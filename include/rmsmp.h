@@ -14,7 +14,10 @@
  *     The only memory it obtains by itself is 2 MiB of pinned HOST memory per device, on the first
  *     rmsmp_quantize_pack, used to upload the layer metadata without stalling the stream.
  *   - `stream` is a cudaStream_t passed as void* (0 = default stream).  All device work is
- *     asynchronous on it.
+ *     asynchronous on it.  A layer's weights (packed buffer, expanded copy) are read as soon as the
+ *     kernel in front on the stream lets its programmatic dependents start: ordinary kernels and copies
+ *     that write them are ordered as always; a kernel of the caller's own that writes them must not
+ *     trigger its dependents early.
  *   - Every function returns an rmsmp_status and never throws, aborts or prints.  Everything
  *     that can be validated on the host is validated before anything is launched.
  *   - Device pointers must be 16-byte aligned unless stated otherwise.
