@@ -77,6 +77,7 @@ struct TensorCfg {
                            //    rows lie twice in tensor memory, in lanes 0..63 and 64..127; 2 (at most 32 rows): four times.  All four
                            //    tensor-memory quarters then hold valid rows and every epilogue warp has work
     int cta_full;          // > 0: CTAs of every row block but the last, which gets the rest of the grid (its tiles take less)
+    int trigger;           // 1: the grid leaves half of the SMs free, where the next launch's set-up and weights may go ahead (see launch_dependent)
     int epi_warps;         // epilogue warps: 4, or 12 in pre mode (the idle expander warps join)
     int bk;                // codes per k-block and bytes per operand row in shared memory: 128, or 64 (pre mode,
                            //    channel counts that would leave half of a 128-byte row empty)
@@ -262,8 +263,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // (the weights are read ahead of the wait for the kernel in front, activations and outputs behind it; no trigger: see
-    // launch_dependent)
+    // (the weights are read ahead of the wait for the kernel in front, activations and outputs behind it: see launch_dependent)
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
     const float* const wstep = p.wstep;                   // (weights: read ahead of the wait)
@@ -313,6 +313,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             if (pre_b_producer) {
                 tensormap_prefetch(&maps.act[0]);
                 pdl_wait();
+                if (cfg.trigger) pdl_trigger();
             }
             const uint32_t nring = pre_b_producer ? (uint32_t)cfg.nB : (uint32_t)cfg.nA;
             const uint32_t bar_e = pre_b_producer ? bar_emptyB : bar_emptyA;
@@ -1275,6 +1276,8 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
         if (ok && p.acc && c.tail_rows) ok = make(&mp.acc_tail, p.acc, CU_TENSOR_MAP_DATA_TYPE_INT32, c.tail_rows);
         c.tma_store = ok ? 1 : 0;
     }
+
+    c.trigger = 2 * grid <= p.sms;
 
     // the kernel's form (see tensor_kernel): [mode][two row blocks][1: re-quantizing epilogue, 2: plain fp32 [N][M] bulk-store output]
     typedef void (*KernelFn)(const Problem, const TensorCfg, const Maps);
