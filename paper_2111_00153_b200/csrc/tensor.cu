@@ -73,9 +73,9 @@ struct TensorCfg {
     int nA, nB;            // ring depths: expanded weights, activations
     int out_bufs;          // staging buffers per epilogue warp (1 or 2)
     int pre;               // 1: the A operand comes expanded (int8) from a workspace, no expander work
-    int dup;               // pre mode, M <= 64, or resident weights whose last row block is at most half full: 1, that block's first 64
-                           //    rows lie twice in tensor memory, in lanes 0..63 and 64..127; 2 (at most 32 rows): four times.  All four
-                           //    tensor-memory quarters then hold valid rows and every epilogue warp has work
+    int dup;               // 1 (pre mode, M <= 64, or resident weights whose last row block is at most half full): that block's
+                           //    first 64 rows are loaded twice, into lanes 0..63 and 64..127, so that all
+                           //    four tensor-memory quarters hold valid rows and every epilogue warp has work
     int cta_full;          // > 0: CTAs of every row block but the last, which gets the rest of the grid (its tiles take less)
     int trigger;           // 1: the grid leaves half of the SMs free, where the next launch's set-up and weights may go ahead (see launch_dependent)
     int epi_warps;         // epilogue warps: 4, or 12 in pre mode (the idle expander warps join)
@@ -104,8 +104,8 @@ struct TensorCfg {
 
 struct Maps {
     CUtensorMap act[4];                                // [B][H][W][Cin] activation codes; stride 2: one map per row/column parity
-    CUtensorMap wexp;                                  // [M][Kp] int8 weights expanded beforehand (pre mode)
-    CUtensorMap wexp_dup;                              // the same in lower boxes, where only the last of several row blocks is dup
+    CUtensorMap wexp;                                  // [M][Kp] int8 weights expanded beforehand (pre mode); 64-row box when all rows are dup
+    CUtensorMap wexp_dup;                              // the same in 64-row boxes, where only the last of several row blocks is dup
     CUtensorMap out_full, out_tail, acc_full, acc_tail;   // bulk stores: 32-row and tail chunks
 };
 
@@ -113,13 +113,13 @@ struct Maps {
 // int8 values, as expand_kernel writes them) straight into the resident stages, at the place the bulk copy of an
 // expanded [rows][bk] box would have put them: stage kb = (tap, channel chunk) holds codes
 // [tap * Cp + chunk * bk, + bk) of every row, 16-byte units XOR-swizzled by the row (128-byte rows: unit ^ (row & 7);
-// 64-byte rows: unit ^ ((row >> 1) & 3)), zeros beyond M and Kp; with duplicated rows a second copy goes to
+// 64-byte rows: unit ^ ((row >> 1) & 3)), zeros beyond M and Kp; with duplicated rows (M <= 64) a second copy goes to
 // lanes 64..127.  Nothing overlaps with it in a CTA's first tile, and it is a chain (slot, codes, expansion): a few
 // threads share a row, and a thread has the loads of four pieces of 32 codes in flight at a time (512x512 N=4096, all in one tile per
 // CTA: 14.7 us with a load at a time and half of each piece kept, 10.8 so; 128x512 N=2000 10.6).
-__device__ __forceinline__ void fill_resident_weights(const Problem& p, const TensorCfg& cfg, uint32_t sA, int row_first, int dup, int tid, int nthreads)
+__device__ __forceinline__ void fill_resident_weights(const Problem& p, const TensorCfg& cfg, uint32_t sA, int row_first, bool dup, int tid, int nthreads)
 {
-    const int rows = kBlockRows >> dup;
+    const int rows = dup ? kBlockRows / 2 : kBlockRows;
     const int pshift = cfg.bk == 128 ? 2 : 1;            // 32-code pieces of a row and k-block: 4 or 2
     const int n4 = p.nP + p.nF4;
     const int tpr = nthreads / rows;
@@ -174,8 +174,8 @@ __device__ __forceinline__ void fill_resident_weights(const Problem& p, const Te
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t at = dst + (((unit + (uint32_t)h) ^ phase) << 4);
                     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(w[4 * h]), "r"(w[4 * h + 1]), "r"(w[4 * h + 2]), "r"(w[4 * h + 3]));
-                    for (int c = 1; c < 1 << dup; ++c)
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + (uint32_t)(c * (cfg.a_bytes >> dup))), "r"(w[4 * h]), "r"(w[4 * h + 1]), "r"(w[4 * h + 2]), "r"(w[4 * h + 3]));
+                    if (dup)
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + (uint32_t)(cfg.a_bytes / 2)), "r"(w[4 * h]), "r"(w[4 * h + 1]), "r"(w[4 * h + 2]), "r"(w[4 * h + 3]));
                 }
             }
         }
@@ -281,7 +281,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         step = (last ? gridDim.x - full : (uint32_t)cfg.cta_full) * (uint32_t)cfg.nbt;
     }
     const int my_blk = kAres ? (int)(first % (uint32_t)cfg.nbt) : 0;
-    const int dup = !kAres || my_blk == cfg.nbt - 1 ? cfg.dup : 0;
+    const bool dup = cfg.dup && (!kAres || my_blk == cfg.nbt - 1);
     const int64_t my_tiles = (ntiles > first) ? (ntiles - first + step - 1) / step : 0;
 
     if (kAres && cfg.fill && warp != 0) {
@@ -306,7 +306,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     const int koff = tap * p.Cp + cc * cfg.bk;
                     const uint32_t dst = sA + kb * cfg.a_bytes;
                     const CUtensorMap* map = dup && cfg.nbt > 1 ? &maps.wexp_dup : &maps.wexp;
-                    for (int r = 0; r < 1 << dup; ++r) tma_load_2d(dst + r * (cfg.a_bytes >> dup), map, bar_fullA, koff, my_blk * kBlockRows);
+                    tma_load_2d(dst, map, bar_fullA, koff, my_blk * kBlockRows);
+                    if (dup) tma_load_2d(dst + cfg.a_bytes / 2, map, bar_fullA, koff, my_blk * kBlockRows);
                     if (++cc == cfg.cpt) { cc = 0; ++tap; }
                 }
             }
@@ -362,7 +363,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     } else {
                         const int koff = tap * p.Cp + cc * cfg.bk;
                         mbar_arrive_expect_tx(bar_f + 8 * s, cfg.a_tx);
-                        for (int r = 0; r < 1 << dup; ++r) tma_load_2d(sA + s * cfg.a_bytes + r * (cfg.a_bytes >> dup), &maps.wexp, bar_f + 8 * s, koff, row_a);
+                        tma_load_2d(sA + s * cfg.a_bytes, &maps.wexp, bar_f + 8 * s, koff, row_a);
+                        if (dup) tma_load_2d(sA + s * cfg.a_bytes + cfg.a_bytes / 2, &maps.wexp, bar_f + 8 * s, koff, row_a);
                     }
                     if (++s == nring) { s = 0; ph ^= 1; }
                     if (++cc == cfg.cpt) { cc = 0; ++tap; if (++tj == p.kw) { tj = 0; ++ti; } }
@@ -641,7 +643,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     } else if (warp >= kThreads / 32 - cfg.epi_warps) {
         // ---------------------------------------------------------- epilogue
         // Warp w may read tensor-memory lanes 32*(w%4)..+31.  The warps that share a quarter (one, or
-        // more in pre mode) take alternate 32-pixel chunks; with duplicated rows the quarters
+        // three in pre mode) take alternate 32-pixel chunks; with duplicated rows the two quarters
         // holding the same rows share the chunks as well.
         const int quarter = warp & 3;
         const int first_epi = kThreads / 32 - cfg.epi_warps;               // epilogue warps are the last epi_warps warps
@@ -649,16 +651,9 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         // how many epilogue warps share a quarter, and this warp's rank among them
         auto count_q = [&](int q) { const int f = first_epi + ((q - first_epi) & 3); return (kThreads / 32 - 1 - f) / 4 + 1; };
         const int my_rank = (warp - (first_epi + ((quarter - first_epi) & 3))) >> 2;
-        const int apart = 4 >> dup;                                     // from a quarter to the next one with the same rows
-        const int row0 = (quarter & (apart - 1)) * 32;                  // first row (within the block) of this warp
-        int cstride = 0, cbefore = 0;                                   // warps with those rows, and those of them in front of this quarter's
-        for (int q = quarter & (apart - 1); q < 4; q += apart) {
-            if (q < quarter) cbefore += count_q(q);
-            cstride += count_q(q);
-        }
-        // Chunks are dealt on from tile to tile: where they are no multiple of the warps, the one that had a chunk more has one
-        // less next time (64x160 on 802,816 pixels, eight chunks for six warps, 65.1 us always dealt from the first, 63.7 so).
-        int cfirst = cbefore + my_rank;
+        const int row0 = dup ? (quarter & 1) * 32 : quarter * 32;       // first row (within the block) of this warp
+        const int cstride = dup ? count_q(quarter & 1) + count_q((quarter & 1) + 2) : count_q(quarter);
+        const int cfirst = (dup && (quarter >> 1)) ? count_q(quarter & 1) + my_rank : my_rank;
         const uint32_t my_stage = sOut + (uint32_t)ew * (cfg.out_bufs * (kRQ ? kRqStage : kWarpStage));
         uint32_t it = 0, stg_count = 0;
         bool alive = true;
@@ -698,15 +693,14 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             if (!mbar_wait_warp(bar_tfull + 8 * ab, tpar, abort_flag)) { alive = false; break; }
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + ab * kTileN;
-            const int nchunks = (nvalid + 31) >> 5, cstart = cfirst;
-            cfirst = (cfirst + cstride * 16 - nchunks) % cstride;          // (at most eight chunks)
+            const int nchunks = (nvalid + 31) >> 5;
             auto release_tmem = [&]() {
                 // all accumulators of this tile are in registers: hand the buffer back
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_tempty + 8 * ab);
             };
-            if (blk * kBlockRows + row0 >= p.M || cstart >= nchunks) {      // no valid row, or no chunk, for this warp
+            if (blk * kBlockRows + row0 >= p.M || cfirst >= nchunks) {      // no valid row, or no chunk, for this warp
                 release_tmem();
                 continue;
             }
@@ -875,7 +869,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 // (a re-quantizing chunk may read its accumulators again: the buffer is handed back after the last one)
                 uint32_t v[32];
 #pragma unroll 1
-                for (int c = cstart; c < nchunks; c += cstride) {
+                for (int c = cfirst; c < nchunks; c += cstride) {
                     tmem_ld_issue(taddr + c * 32, v);
                     tmem_ld_wait(v);
                     emit(v, c);
@@ -887,9 +881,9 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             // two register sets: the load of this warp's next chunk is in flight while the current one is emitted
             // (tensor-memory loads and their waits are warp-wide: every chunk ends with the warp together again)
             uint32_t va[32], vb[32];
-            tmem_ld_issue(taddr + cstart * 32, va);
+            tmem_ld_issue(taddr + cfirst * 32, va);
             tmem_ld_wait(va);
-            for (int c = cstart; c < nchunks; c += 2 * cstride) {
+            for (int c = cfirst; c < nchunks; c += 2 * cstride) {
                 const int c1 = c + cstride, c2 = c + 2 * cstride;
                 const bool more1 = c1 < nchunks;
                 if (more1) tmem_ld_issue(taddr + c1 * 32, vb); else release_tmem();
@@ -1067,12 +1061,10 @@ bool plan(const Problem& p, TensorCfg& c)
     if (c.pre) {
         c.nA = (c.bk == 64) ? 6 : 3; c.nB = (c.bk == 64) ? 8 : 4; c.out_bufs = 1;
         c.epi_warps = warps_of(1, p.rq_codes != nullptr) - 3;   // warp 2 fetches the weights (unless they are resident)
-        // (four copies of 32 rows where there are rounds enough, or k-blocks few enough, for them: 32x192 on 200,704 pixels 14.8 us with two
-        // of 64, 14.3 so; 24x144 on 50,176 6.2 and 6.6)
-        c.dup = p.M <= 32 && (c.nkb <= 2 || c.ntiles >= 4 * p.sms) ? 2 : p.M <= 64 ? 1 : 0;
+        c.dup = (p.M <= 64) ? 1 : 0;
         if (resident) {
             c.ares = 1;
-            c.epi_warps = wide ? (p.rq_codes ? 2 * kWideEpi : kWideEpi) : warps_of(2, p.rq_codes != nullptr) - 2;
+            c.epi_warps = wide ? (p.rq_codes ? 2 * kWideEpi : kWideEpi) : warps_of(1, p.rq_codes != nullptr) - 2;
             c.nA = c.nkb;
             const int64_t left = kSmemLimit - (1024 + 64 * kMaxRing) - (int64_t)c.nkb * c.a_bytes -
                                  (int64_t)c.epi_warps * stage;
@@ -1106,8 +1098,8 @@ bool plan(const Problem& p, TensorCfg& c)
             c.a_bytes = 2 * kABytes;
             c.nA = 2; c.nB = 3;
         }
-        c.a_rows = c.m2 ? 2 * kBlockRows : c.nbt > 1 ? kBlockRows : (std::min(p.M, kBlockRows >> c.dup) + 7) / 8 * 8;
-        c.a_tx = (uint32_t)(c.a_rows * c.bk) << (c.nbt == 1 ? c.dup : 0);
+        c.a_rows = c.m2 ? 2 * kBlockRows : c.nbt > 1 ? kBlockRows : (std::min(p.M, c.dup ? kBlockRows / 2 : kBlockRows) + 7) / 8 * 8;
+        c.a_tx = (uint32_t)(c.a_rows * c.bk * (c.dup && c.nbt == 1 ? 2 : 1));
         c.smem_bytes = (uint32_t)(c.nA * c.a_bytes + c.nB * c.b_bytes + c.epi_warps * c.out_bufs * stage + 1024 +
                                   64 * kMaxRing);
         return true;
@@ -1242,7 +1234,7 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
                        CU_TENSOR_MAP_INTERLEAVE_NONE, c.bk == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
         };
-        if (!make(&mp.wexp, c.a_rows) || (c.dup && c.nbt > 1 && !make(&mp.wexp_dup, kBlockRows >> c.dup)))
+        if (!make(&mp.wexp, c.a_rows) || (c.dup && c.nbt > 1 && !make(&mp.wexp_dup, kBlockRows / 2)))
             return RMSMP_ERR_CUDA;
     }
 
