@@ -810,9 +810,12 @@ bool stream_build_table(const Problem* probs, int count, int sms, uint8_t* h_tab
     H->nB = H->nAst;                                               // activation slot s goes with A stage s (one commit frees both)
     H->nS = (int)std::min<int64_t>(kRingMax, (avail - (int64_t)H->nB * H->b_bytes) / H->stage_bytes);
     // The two expander sets take alternate stages.  With an even ring each set keeps to its own slots; with an odd one it sees every
-    // other phase of a slot's barrier, which its parity tells from the one two phases earlier only while the set cannot be that far
-    // ahead of the copies: a set is at most nAst + 2 stages ahead of the MMAs.
-    if (H->nS < H->nAst + 2) H->nS &= ~1;
+    // other phase of a slot's barrier, which its parity tells from the one two phases earlier only while the slot's fill before, nS
+    // stages back and the other set's, has landed.  One issuer multiplies the stages in order, and a set that is at a stage has seen
+    // the stage nAst + 2 back multiplied, so from nAst + 2 slots up an odd ring is safe.  Several issuers divide the stages as the
+    // sets do: set and issuer of even stages run ahead of those of odd stages with nothing between them inside an item, so
+    // the ring is even whatever its size.
+    if (H->nch > 1 || H->nS < H->nAst + 2) H->nS &= ~1;
     if (H->nS < 2) return false;
     H->smem_bytes = (uint32_t)(H->nB * H->b_bytes + H->nS * H->stage_bytes + 1024 + 64 * kRingMax);
     // kind::i8: int32 accumulate, signed 8-bit A and B, both K-major, N/8 at bit 17, M/16 at bit 24

@@ -317,20 +317,49 @@ def test_config5_grouped_tensor_launch_matches_oracle(N):
         assert not torch.isnan(y).any()
 
 
-@pytest.mark.parametrize("N", [1, 16, 33, 64, 65, 80, 96, 112, 113, 128])
-def test_grouped_tensor_launch_ring_of_packed_codes(N):
-    """The expander sets take alternate stages and tell a slot's phases apart by parity: the ring has an even number of slots, or
-    enough of them that a set cannot be two of a slot's phases ahead of its copies (header words 5 and 13: slots, A stages)."""
+def _launch_grouped(items, layout=R.OUT_NM):
+    """Plans and launches; returns the plan's table."""
     import torch
-    keep, items, refs = _grouped_case([(384, 512)], N)
+    arr = R.make_gemm_items(items)
+    table = torch.empty(R.rmsmp_grouped_plan_bytes(arr), dtype=torch.uint8, device="cuda")
+    R.rmsmp_gemm_grouped_launch(R.rmsmp_gemm_grouped_prepare(arr, layout, table))
+    torch.cuda.synchronize()
+    return table
+
+
+@pytest.mark.parametrize("N", list(range(16, 129, 16)))
+def test_grouped_tensor_launch_ring_of_packed_codes(N):
+    """The expander sets take alternate stages and tell a slot's phases apart by parity: the ring has an even number of slots, or one
+    issuer, which multiplies the stages in order, and slots enough that a set cannot be two of a slot's phases ahead of its copies (header
+    words 5, 6 and 13: slots, accumulator chains = issuers, A stages)."""
+    import torch
+    _, items, _ = _grouped_case([(384, 512)], N)
     arr = R.make_gemm_items(items)
     table = torch.empty(R.rmsmp_grouped_plan_bytes(arr), dtype=torch.uint8, device="cuda")
     R.rmsmp_gemm_grouped_prepare(arr, R.OUT_NM, table)
     torch.cuda.synchronize()
     header = table[:128].cpu().numpy().view(np.int32)
-    slots, a_stages = int(header[5]), int(header[13])
-    assert a_stages % 2 == 0 and slots >= 2
-    assert slots % 2 == 0 or slots >= a_stages + 2
+    slots, chains, a_stages = int(header[5]), int(header[6]), int(header[13])
+    assert header[4] == N and chains in (1, 2, 4) and a_stages % 2 == 0 and a_stages >= chains and slots >= 2
+    assert slots % 2 == 0 or (chains == 1 and slots >= a_stages + 2)
+
+
+@pytest.mark.parametrize("N", [24, 40, 56, 80, 104])
+def test_grouped_tensor_launch_lists_of_several_laps(N):
+    """Every CTA has several items, long and short ones in turn, of all kinds and an odd number of k-blocks: its stages are several laps
+    of the ring (sixteen, four and three stages an item).  Each layer is in the launch more than once, into outputs of its own."""
+    import torch
+    keep, items, refs = _grouped_case([(1024, 4096), (1000, 1024), (300, 640)], N)
+    all_keep, all_items, all_refs = [], [], []
+    for rep, (k, (layer, d_packed, a, n, ld, step, y, M, acc, nonneg), ref) in [(r, z) for r in range(20) for z in zip(keep, items, refs)]:
+        y2 = torch.full_like(y, float("nan"))
+        acc2 = torch.full_like(y, -5, dtype=torch.int32) if rep % 4 == 0 else None
+        all_keep.append((layer, d_packed, a, y2, acc2))
+        all_items.append((layer, d_packed, a, n, ld, step, y2, M, acc2, nonneg))
+        all_refs.append(ref)
+    header = _launch_grouped(all_items)[:128].cpu().numpy().view(np.int32)
+    assert header[2] > 2 * header[3]                       # items, CTAs
+    _check_grouped(all_keep, all_refs)
 
 
 def test_grouped_tensor_launch_mn_layout_and_single_layer():
