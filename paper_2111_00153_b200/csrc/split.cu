@@ -142,6 +142,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
             uint32_t ph = 0;
             bool ok = true;
             for (int i = 0; i < n_kb; ++i) {
+                if (i == cfg.nst) pdl_wait();                      // (a bounded wait begins when the kernel in front is over)
                 if (i >= cfg.nst && !mbar_wait(empty(s), ph ^ 1, abort_flag)) { ok = false; break; }
                 if (warp == 0) {
                     mbar_arrive_expect_tx(full(s), cfg.tx_b);
@@ -165,6 +166,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         int s = 0, cc = kb0 % cfg.cpt;
         uint32_t ph = 0;
         bool ok = true;
+        pdl_wait();                                       // (the activations come behind it)
         for (int i = 0; i < n_kb; ++i) {
             if (!mbar_wait_step(full(s), ph, abort_flag)) { ok = false; break; }
             tc_fence_after();
@@ -231,7 +233,10 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
             int next_ksteps;
             const uint4* q = fetch_pos(i + 3, next_ksteps);
             const int next_pieces = pieces_of(next_ksteps);
-            if (i >= cfg.nst && !mbar_wait_warp(empty(s), ((i / cfg.nst) & 1) ^ 1, abort_flag)) break;
+            if (i >= cfg.nst) {
+                pdl_wait();                               // (see the producers)
+                if (!mbar_wait_warp(empty(s), ((i / cfg.nst) & 1) ^ 1, abort_flag)) break;
+            }
             const uint32_t dst = sA + s * cfg.a_bytes + row_off;
             if (kGather) {
                 // 32 codes of one tap at a time; a Cp is a multiple of 32, so a step never spans two taps

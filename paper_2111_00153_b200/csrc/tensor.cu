@@ -335,6 +335,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 const int row_a = blk * kBlockRows;
                 int tap = 0, cc = 0, ti = 0, tj = 0;
                 for (int kb = 0; kb < cfg.nkb; ++kb) {
+                    if (pre_a_producer && s == 0 && ph) pdl_wait();              // (a bounded wait begins when the kernel in front is over)
                     if (!mbar_wait(bar_e + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
                     if (pre_b_producer && kTps3) {
                         if (cfg.colshift) {
@@ -382,6 +383,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             uint32_t sa = 0, phA = 0, sb = 0, phB = 0, it = 0;
             const uint64_t desc_a0 = smem_desc_kmajor(sA, cfg.bk), desc_b0 = smem_desc_kmajor(sB, cfg.bk);
             const uint32_t desc_lo0_a = (uint32_t)desc_a0, desc_lo0_b = (uint32_t)desc_b0, desc_hi = (uint32_t)(desc_a0 >> 32);
+            pdl_wait();                                   // (the activations come behind it)
             bool have_a = !kAres || my_tiles == 0 || mbar_wait_step(bar_fullA, 0, abort_flag);
             for (uint32_t tile = first; tile < ntiles && have_a; tile += step, ++it) {
                 // one accumulator per tile, alternating; or (two row blocks per tile) both, every tile
@@ -598,6 +600,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             }
             const bool on = g < total && has_piece();
             const uint32_t piece = piece_of();
+            if (phA == 1) pdl_wait();                     // (see the producers)
             if (!mbar_wait_warp(bar_emptyA + 8 * sa, phA ^ 1, abort_flag)) break;
             const uint32_t dst = sA + sa * cfg.a_bytes;
             auto at = [&](int i) { return dst + (i & 1 ? c_place[i >> 1] >> 16 : c_place[i >> 1] & 0xFFFFu); };

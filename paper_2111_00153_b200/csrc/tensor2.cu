@@ -272,6 +272,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 const HalfPos hp = half_pos(p, cfg, 2 * nt + rank);
                 int cc = 0, tj = 0;
                 for (int st = 0; st < 3 * cfg.cpt; ++st) {
+                    if (warp != 0 && s == 0 && ph) pdl_wait();               // (a bounded wait begins when the kernel in front is over)
                     if (!bar_wait(bar_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
                     const uint32_t fb = lead_full + 8 * s;
                     if (warp == 0) {
@@ -309,6 +310,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 const int nsub = min(kSub2, cfg.nkb - kb);
                 const bool skip = (g & 1u) != mine;
                 if (!skip) {
+                    if (!is_b && ph) pdl_wait();                             // (a bounded wait begins when the kernel in front is over)
                     if (!bar_wait(bar_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
                     // all copies of this stage (up to two k-blocks of two operands in two CTAs) complete on the leader's barrier
                     if (is_b && rank == 0)
@@ -342,6 +344,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
             const uint32_t a_step = a_stage >> 4, b_step = b_stage >> 4;
             const uint32_t row_step = (uint32_t)(p.W * 128) >> 4;                      // (column shift) a tap's rows lie W pixels further on
             uint32_t a_lo = a_lo0, b_lo = b_lo0;
+            pdl_wait();                                                                // (the activations come behind it)
             for (int64_t tile = first; tile < cfg.ntiles; tile += step, ++it) {
                 const uint32_t ab = it & 1;
                 if (!bar_wait_step(bar_tempty + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag)) break;
