@@ -14,10 +14,8 @@
  *     The only memory it obtains by itself is 2 MiB of pinned HOST memory per device, on the first
  *     rmsmp_quantize_pack, used to upload the layer metadata without stalling the stream.
  *   - `stream` is a cudaStream_t passed as void* (0 = default stream).  All device work is
- *     asynchronous on it.  A layer's weights (packed buffer, expanded copy) are read as soon as the
- *     kernel in front on the stream lets its programmatic dependents start: ordinary kernels and copies
- *     that write them are ordered as always; a kernel of the caller's own that writes them must not
- *     trigger its dependents early.
+ *     asynchronous on it, and ordered behind everything in front of it on the stream, kernels that let
+ *     their programmatic dependents start early included (rmsmp_gemm_grouped_launch has a contract of its own).
  *   - Every function returns an rmsmp_status and never throws, aborts or prints.  Everything
  *     that can be validated on the host is validated before anything is launched.
  *   - Device pointers must be 16-byte aligned unless stated otherwise.
@@ -337,8 +335,13 @@ rmsmp_status rmsmp_gemm_grouped(const rmsmp_gemm_item* h_items, int count, rmsmp
  *                               must stay untouched while launches that use it are in flight.  The
  *                               kernels are launched with the programmatic-stream-serialization
  *                               attribute and signal early, so that launches in a row overlap their
- *                               ends and beginnings; what a predecessor may still touch is accessed only
- *                               behind a grid-dependency wait.  Kernels that follow on the stream and
+ *                               ends and beginnings; activations and outputs are accessed only
+ *                               behind a grid-dependency wait.  The table and the layers' packed
+ *                               weights are read ahead of it: a kernel of the caller's own that writes
+ *                               them must not trigger its dependents early (ordinary kernels, copies and
+ *                               this library's calls are ordered as always), and the launch's bounded
+ *                               waits, about a second, begin when that kernel lets its dependents start.
+ *                               Kernels that follow on the stream and
  *                               are launched the ordinary way are ordered as always; one that is itself
  *                               launched with that attribute must call cudaGridDependencySynchronize()
  *                               before it reads the results.
@@ -399,8 +402,8 @@ rmsmp_status rmsmp_conv_implicit_workspace(const rmsmp_layer* layer, const void*
  * RMSMP_ACT_S4 keeps the sign), so the result equals rmsmp_*_workspace followed by
  * rmsmp_quantize_act byte for byte while writing 1 byte per output instead of 4 and saving the
  * quantizer's pass.  [N][M] order only (conv: [B][Ho][Wo][M], ld_codes = M): that is the next
- * layer's input layout.  d_next_codes: device, N * ld_codes bytes; bulk stores are used when it is
- * 16-byte aligned and ld_codes is a multiple of 16.  *h_next_step (host, may be NULL) receives
+ * layer's input layout.  d_next_codes: device, N * ld_codes bytes; sixteen codes a store when it is
+ * 16-byte aligned and ld_codes and M are multiples of 16.  *h_next_step (host, may be NULL) receives
  * next_alpha/15 or next_alpha/7.  Errors: as rmsmp_*_workspace, plus SCALE for a bad next_alpha;
  * VARIANT when the tensor kernel cannot run the problem.
  */

@@ -75,22 +75,26 @@ bool ensure_smem_attr(const void* fn, int bytes, bool* done);
 // Every kernel that a layer call queues is launched as a programmatic dependent of whatever is in front of it on the
 // stream: its CTAs are placed, and its set-up runs, while the kernel in front drains, which takes the launch gap from
 // 1.9 to about 1 us, and such a launch also costs the host less (2.3 against 3 us).  The order of memory accesses is
-// kept by these rules.  (1) pdl_wait() comes before a kernel's first access to what a kernel in front of it may write or read; it
-// returns when those have finished and their writes are visible.  (2) pdl_trigger() (the next kernel may be placed) comes after
-// it, so that a kernel whose successor runs has no unfinished predecessor itself.  Two kernels are exempt, those of the
-// grouped tensor-core launch (stream.cu): act_e4m3_kernel and stream_kernel trigger at once; each of their two waits
-// before it ends, so that neither ends before what is in front of it.  (3) A layer's weights are read ahead of the wait: packed codes,
-// perm, slot, kind, wstep and block table, and the expanded copy, by the contraction kernels, and the launch's table by the
-// grouped launch's.  So whatever writes those must be complete before any kernel behind it can be placed: pack_kernel, the last of
-// the calls that write a packed buffer, and expand_kernel never trigger.  A new writer that triggered would be a race.
-// Activations, the copies of them, outputs and status words stay behind the wait.  (Everything behind the wait: a BERT-base layer of 4096
-// tokens 64.4 us against 62.2, ResNet-18 for one image in codes 108.6 and 105.1, 3x3 256x256 on 6272 pixels without a workspace, whose
-// first codes then arrive beside the activations, 19.6 and 17.7 with its quantizer.)
-// Without a trigger for another reason: tensor_kernel and pair_kernel, because a small kernel whose blocks are placed
-// beside their CTAs has to live with what 200 KB of shared memory leaves of the L1 (the activation quantizer behind a
+// kept by these rules.  (1) pdl_wait() comes before a kernel's first access to global memory; it returns when the kernels in front
+// have finished and their writes are visible.  (2) pdl_trigger() (the next kernel may be placed) comes after it, so that a
+// kernel whose successor runs has no unfinished predecessor itself.  Three kernels read ahead of their wait.  pack_kernel reads the
+// fp32 weights: the kernel in front of it is one of its own call, which triggers by rule 2.  act_e4m3_kernel and stream_kernel, those of
+// the grouped tensor-core launch (stream.cu), trigger at once and read the launch's table (both) and, of every layer, packed
+// codes, perm and wstep (stream_kernel).  Activations, the copies of them, outputs and status words stay behind the wait, and each of
+// the two waits before it ends, so that neither ends before what is in front of it.  (3) So whatever writes a table, packed codes or a
+// packed buffer's metadata must be complete before any kernel behind it can be placed: the last kernel of such a call never
+// triggers (pack_kernel; everything else that writes them is a copy or a kernel in front of pack_kernel), so that its dependents
+// start when all of its blocks have completed.  A new writer that triggered would be a race, and so would be a caller's, which the grouped
+// launch's contract rules out.  (Both fences at the end of pack_kernel besides: 20 layers 260 us without, 270 with.)
+// (Weights read ahead of the wait by every contraction: a BERT-base layer of 4096 tokens 59.5 us against 61.3, ResNet-18 for one image in
+// codes 91.2 and 93.9, 3x3 256x256 on 6272 pixels with its quantizer 16.8 and 18.7.  But a plain call has no contract that says when its weights
+// are settled: behind a kernel that writes them and lets its dependents start before that, it would use the old ones.  Nor is a look ahead
+// that is repeated behind the wait safe: a read-only load behind it may be served from the line that the first one left in the L1.)
+// Without a trigger for another reason: pair_kernel, and tensor_kernel where it takes more than half of the SMs, because a small kernel
+// whose blocks are placed beside their CTAs has to live with what 200 KB of shared memory leaves of the L1 (the activation quantizer behind a
 // convolution: ResNet-18 at batch 256 1168 us with the trigger, 1146 with it just before the end, 1075 without, 1138 with
-// plain launches; split_kernel, for problems that leave SMs free, triggers, and so does tensor_kernel where its grid leaves half of
-// them free: ResNet-18 for one image 96.9 us without, 92.2 so), and the general depthwise form (depthwise.cu).
+// plain launches; with half of the SMs free: ResNet-18 for one image 96.9 us without, 92.2 so), and the general depthwise form
+// (depthwise.cu).
 template <typename... P, typename... A>
 inline cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, const A&... args)
 {

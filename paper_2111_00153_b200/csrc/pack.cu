@@ -243,7 +243,8 @@ cudaError_t launch_unpack(const rmsmp_layer& L, const uint8_t* blob, int8_t* val
 __global__ void __launch_bounds__(256) expand_kernel(const uint8_t* __restrict__ blob, rmsmp_layer L,
                                                      int8_t* __restrict__ wexp)
 {
-    pdl_wait();                                              // and no trigger: see launch_dependent
+    pdl_wait();
+    pdl_trigger();
     blob = pdl_ordered(blob);
     const int chunks = L.Kp >> 5;
     const int64_t total = (int64_t)L.M * chunks;

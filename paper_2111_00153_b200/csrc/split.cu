@@ -113,13 +113,10 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     __syncthreads();
     tc_fence_after();
     if (cfg.S > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");      // this CTA runs: its shared memory may be written
-    // From here on the weights: packed codes, their rows' places and scales, or the expanded copy.  What the kernel in front
-    // writes or reads -- activations, outputs, the status word -- stays behind the waits further down (see launch_dependent).
+    // Every role waits for the kernel in front by itself, behind what it can work out without memory: before its first access to
+    // weights, activations or outputs, and before its first wait for another role.
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
-    const int32_t* const slot_of = p.slot;
-    const float* const wstep = p.wstep;
-    const uint8_t* const kind_of = p.kind;
 
     int b0, h0;
     if (cfg.tiles_per_image) { b0 = nt / cfg.tiles_per_image; h0 = (nt - b0 * cfg.tiles_per_image) * cfg.th; }
@@ -133,16 +130,17 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
             if (warp == 0) {
                 tensormap_prefetch(&maps.act[0]);
                 if (act_parity_split(p)) { tensormap_prefetch(&maps.act[1]); tensormap_prefetch(&maps.act[2]); tensormap_prefetch(&maps.act[3]); }
-                pdl_wait();
-                pdl_trigger();
+            } else {
+                tensormap_prefetch(&maps.wexp);
             }
             int tap = kb0 / cfg.cpt, cc = kb0 - tap * cfg.cpt;
             int ti = tap / p.kw, tj = tap - ti * p.kw;
+            pdl_wait();
+            if (warp == 0) pdl_trigger();
             int s = 0;
             uint32_t ph = 0;
             bool ok = true;
             for (int i = 0; i < n_kb; ++i) {
-                if (i == cfg.nst) pdl_wait();                      // (a bounded wait begins when the kernel in front is over)
                 if (i >= cfg.nst && !mbar_wait(empty(s), ph ^ 1, abort_flag)) { ok = false; break; }
                 if (warp == 0) {
                     mbar_arrive_expect_tx(full(s), cfg.tx_b);
@@ -166,7 +164,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         int s = 0, cc = kb0 % cfg.cpt;
         uint32_t ph = 0;
         bool ok = true;
-        pdl_wait();                                       // (the activations come behind it)
+        pdl_wait();                                       // (a bounded wait begins when the kernel in front is over)
         for (int i = 0; i < n_kb; ++i) {
             if (!mbar_wait_step(full(s), ph, abort_flag)) { ok = false; break; }
             tc_fence_after();
@@ -188,11 +186,14 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         const int row = ((warp - kSplitFirst) & 3) * 32 + lane, m_row = blk * kBlockRows + row;
         int kind = -1;
         const uint8_t* src = p.q4;
+        pdl_wait();
+        if (kGather) pdl_trigger();
         if (m_row < p.M) {
-            kind = p.kind[m_row];
-            const int packed = __ldg(slot_of + m_row);
+            kind = __ldg(pdl_ordered(p.kind) + m_row);
+            const int packed = __ldg(pdl_ordered(p.slot) + m_row);
             src = kind == kFixed8 ? p.q8 + (size_t)(packed - p.nP - p.nF4) * p.Kp : p.q4 + (size_t)packed * (p.Kp >> 1);
         }
+        src = pdl_ordered(src);
         const uint32_t swz = cfg.bk == 128 ? (uint32_t)(row & 7) : (uint32_t)((row >> 1) & 3);
         const uint32_t row_off = (uint32_t)row * (uint32_t)cfg.bk;
         // The codes of a k-block are in registers before its turn comes: the next one's are loaded as soon as this one's
@@ -208,7 +209,7 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
         auto pieces_of = [&](int ksteps) { return kind < 0 ? 0 : (eight ? 2 * ksteps : ksteps); };      // 16-byte pieces of a row
         // this thread's pixel of the tile (kGather): its image, and the input position of its tap (0, 0)
         int px_y = 0, px_x = 0;
-        const int8_t* px_img = p.act;
+        const int8_t* px_img = pdl_ordered(p.act);
         const bool px_ok = kGather && row < cfg.npix && (int64_t)nt * cfg.npix + row < p.N;
         if (px_ok) {
             const uint32_t n = (uint32_t)((int64_t)nt * cfg.npix + row), t = n / (uint32_t)p.Wo, b = t / (uint32_t)p.Ho;
@@ -223,20 +224,12 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
 #pragma unroll
             for (int u = 0; u < 8; ++u) raw[u] = u < pieces ? __ldg(q + u) : make_uint4(0u, 0u, 0u, 0u);
         }
-        if (kGather) {
-            pdl_wait();
-            pdl_trigger();
-            px_img = pdl_ordered(px_img);
-        }
         for (int i = grp; i < n_kb; i += 3) {
             const int s = i % cfg.nst;
             int next_ksteps;
             const uint4* q = fetch_pos(i + 3, next_ksteps);
             const int next_pieces = pieces_of(next_ksteps);
-            if (i >= cfg.nst) {
-                pdl_wait();                               // (see the producers)
-                if (!mbar_wait_warp(empty(s), ((i / cfg.nst) & 1) ^ 1, abort_flag)) break;
-            }
+            if (i >= cfg.nst && !mbar_wait_warp(empty(s), ((i / cfg.nst) & 1) ^ 1, abort_flag)) break;
             const uint32_t dst = sA + s * cfg.a_bytes + row_off;
             if (kGather) {
                 // 32 codes of one tap at a time; a Cp is a multiple of 32, so a step never spans two taps
@@ -317,11 +310,11 @@ split_kernel(const Problem p, const SplitCfg cfg, const __grid_constant__ SplitM
     }
     float scale = 0.0f;
     int shift = 0;
+    pdl_wait();
     if (row_ok) {
-        scale = __fmul_rn(__ldg(wstep + m), p.act_step);
-        shift = (!kPre && __ldg(kind_of + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
+        scale = __fmul_rn(__ldg(pdl_ordered(p.wstep) + m), p.act_step);
+        shift = (!kPre && __ldg(pdl_ordered(p.kind) + m) == kFixed4) ? 4 : 0;         // expanded as 16 * value
     }
-    pdl_wait();                                           // the outputs
     const ActFast rq = act_fast_setup(kRQ ? p.rq_alpha : 1.0f, kRQ ? p.rq_kind : 0);
     const bool out_mn = !kRQ && p.out_mn != 0;
     // the finished sum of this lane's row at column j of the tile

@@ -127,9 +127,10 @@ __device__ __forceinline__ void fill_resident_weights(const Problem& p, const Te
     if (r < rows) {
         const int m = row_first + r;
         const bool have = m < p.M;
-        const int kind = have ? (int)p.kind[m] : kFixed8;
-        const int slot = have ? p.slot[m] : 0;
+        const int kind = have ? (int)__ldg(pdl_ordered(p.kind) + m) : kFixed8;
+        const int slot = have ? __ldg(pdl_ordered(p.slot) + m) : 0;
         const uint8_t* src = (kind == kFixed8) ? p.q8 + (size_t)(have ? slot - n4 : 0) * p.Kp : p.q4 + (size_t)slot * (p.Kp >> 1);
+        src = pdl_ordered(src);
         const uint32_t phase = (cfg.bk == 128) ? (uint32_t)(r & 7) : (uint32_t)((r >> 1) & 3);
         const uint32_t row_base = sA + (uint32_t)r * (uint32_t)cfg.bk;
         const int pieces = cfg.nkb << pshift;
@@ -263,11 +264,10 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // (the weights are read ahead of the wait for the kernel in front, activations and outputs behind it: see launch_dependent)
+    // Every role waits for the kernel in front by itself, behind what it can work out without memory: before its first access to
+    // weights, activations or outputs, and before its first wait for another role.
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
-    const float* const wstep = p.wstep;                   // (weights: read ahead of the wait)
-    const uint8_t* const kind_of = p.kind;
 
     // (tile indices fit 32 bits with a step to spare: checked on the host)
     const uint32_t ntiles = (uint32_t)cfg.ntiles;
@@ -285,6 +285,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     const int64_t my_tiles = (ntiles > first) ? (ntiles - first + step - 1) / step : 0;
 
     if (kAres && cfg.fill && warp != 0) {
+        pdl_wait();
         // every warp but the activation producer's (whose first copies go out meanwhile) expands the row block;
         // one of them then reports the resident weights to the MMA thread
         if (my_tiles > 0) fill_resident_weights(p, cfg, sA, my_blk * kBlockRows, dup, (int)threadIdx.x - 32, kThreads - 32);
@@ -298,6 +299,10 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
     const bool pre_a_producer = kPre && !kAres && warp == 2;
     if (pre_b_producer || pre_a_producer) {
         if (lane == 0) {
+            if (pre_b_producer) tensormap_prefetch(&maps.act[0]);
+            if (kPre && !cfg.fill && (kAres || pre_a_producer)) tensormap_prefetch(kAres && dup && cfg.nbt > 1 ? &maps.wexp_dup : &maps.wexp);
+            pdl_wait();
+            if (pre_b_producer && cfg.trigger) pdl_trigger();
             if (pre_b_producer && kAres && my_tiles > 0 && !cfg.fill) {
                 // resident weights: every k-block's rows, once
                 mbar_arrive_expect_tx(bar_fullA, (uint32_t)cfg.nkb * cfg.a_tx);
@@ -310,11 +315,6 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     if (dup) tma_load_2d(dst + cfg.a_bytes / 2, map, bar_fullA, koff, my_blk * kBlockRows);
                     if (++cc == cfg.cpt) { cc = 0; ++tap; }
                 }
-            }
-            if (pre_b_producer) {
-                tensormap_prefetch(&maps.act[0]);
-                pdl_wait();
-                if (cfg.trigger) pdl_trigger();
             }
             const uint32_t nring = pre_b_producer ? (uint32_t)cfg.nB : (uint32_t)cfg.nA;
             const uint32_t bar_e = pre_b_producer ? bar_emptyB : bar_emptyA;
@@ -335,7 +335,6 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 const int row_a = blk * kBlockRows;
                 int tap = 0, cc = 0, ti = 0, tj = 0;
                 for (int kb = 0; kb < cfg.nkb; ++kb) {
-                    if (pre_a_producer && s == 0 && ph) pdl_wait();              // (a bounded wait begins when the kernel in front is over)
                     if (!mbar_wait(bar_e + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
                     if (pre_b_producer && kTps3) {
                         if (cfg.colshift) {
@@ -383,7 +382,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             uint32_t sa = 0, phA = 0, sb = 0, phB = 0, it = 0;
             const uint64_t desc_a0 = smem_desc_kmajor(sA, cfg.bk), desc_b0 = smem_desc_kmajor(sB, cfg.bk);
             const uint32_t desc_lo0_a = (uint32_t)desc_a0, desc_lo0_b = (uint32_t)desc_b0, desc_hi = (uint32_t)(desc_a0 >> 32);
-            pdl_wait();                                   // (the activations come behind it)
+            pdl_wait();                                   // (a bounded wait begins when the kernel in front is over)
             bool have_a = !kAres || my_tiles == 0 || mbar_wait_step(bar_fullA, 0, abort_flag);
             for (uint32_t tile = first; tile < ntiles && have_a; tile += step, ++it) {
                 // one accumulator per tile, alternating; or (two row blocks per tile) both, every tile
@@ -502,8 +501,9 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         const int64_t total = my_tiles * cfg.nkb;
         const bool rows_change = step % (uint32_t)p.nblocks != 0u;
         // a row block's rows in the packed buffer: first and number of each kind
-        const int32_t* const blocks = p.blocks, *const perm = p.perm;
-        const uint4* const codes = reinterpret_cast<const uint4*>(p.q4);
+        pdl_wait();
+        const int32_t* const blocks = pdl_ordered(p.blocks), *const perm = pdl_ordered(p.perm);
+        const uint4* const codes = reinterpret_cast<const uint4*>(pdl_ordered(p.q4));
         int4 blk_a;
         int2 blk_b;
         int blk_next = 0;
@@ -600,7 +600,6 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
             }
             const bool on = g < total && has_piece();
             const uint32_t piece = piece_of();
-            if (phA == 1) pdl_wait();                     // (see the producers)
             if (!mbar_wait_warp(bar_emptyA + 8 * sa, phA ^ 1, abort_flag)) break;
             const uint32_t dst = sA + sa * cfg.a_bytes;
             auto at = [&](int i) { return dst + (i & 1 ? c_place[i >> 1] >> 16 : c_place[i >> 1] & 0xFFFFu); };
@@ -663,7 +662,7 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
         int scale_blk = -1, shift = 0;
         float scale = 0.f;
         const ActFast rq_fast = act_fast_setup(kRQ ? p.rq_alpha : 1.0f, kRQ ? p.rq_kind : 0);
-        pdl_wait();                                                        // the outputs
+        pdl_wait();
         for (uint32_t tile = first; tile < ntiles && alive; tile += step, ++it) {
           // a tile is one row block (accumulators alternate between tiles), or two (one accumulator each)
           for (int half = 0; half <= kM2; ++half) {
@@ -689,8 +688,8 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                 scale = 0.f;
                 shift = 0;
                 if (row_ok) {
-                    scale = __fmul_rn(__ldg(wstep + m), p.act_step);
-                    shift = (!kPre && __ldg(kind_of + m) == kFixed4) ? 4 : 0;   // expanders store Fixed-4 codes as 16 * value
+                    scale = __fmul_rn(__ldg(pdl_ordered(p.wstep) + m), p.act_step);
+                    shift = (!kPre && __ldg(pdl_ordered(p.kind) + m) == kFixed4) ? 4 : 0;   // expanders store Fixed-4 codes as 16 * value
                 }
             }
             if (!mbar_wait_warp(bar_tfull + 8 * ab, tpar, abort_flag)) { alive = false; break; }

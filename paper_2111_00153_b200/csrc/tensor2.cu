@@ -245,11 +245,10 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     __syncthreads();
     cluster_sync_all();                                   // both CTAs' barriers exist before anyone signals the peer
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // (the weights are read ahead of the wait for the kernel in front, activations and outputs behind it; no trigger: see
-    // launch_dependent)
+    // Every role waits for the kernel in front by itself: before its first access to weights, activations or outputs, and before
+    // its first wait for another role.  No trigger: see launch_dependent.
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     volatile int* abort_flag = &s_abort;
-    const float* const wstep = p.wstep;                   // (weights: read ahead of the wait)
 
     const int64_t first = blockIdx.x >> 1, step = gridDim.x >> 1;      // cluster index, clusters in the grid
     const uint32_t lead_full = map_to_rank(bar_full, 0), lead_tempty = map_to_rank(bar_tempty, 0);
@@ -260,10 +259,8 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
         // the weights of the taps (0, j), (1, j), (2, j).
         if (lane == 0) {
             const int ti = warp - 2;
-            if (warp == 0) {
-                asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.act[0]) : "memory");
-                pdl_wait();
-            }
+            tensormap_prefetch(warp == 0 ? &maps.act[0] : &maps.wexp);
+            pdl_wait();
             uint32_t s = 0, ph = 0;
             bool ok = true;
             for (int64_t tile = first; tile < cfg.ntiles && ok; tile += step) {
@@ -272,7 +269,6 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 const HalfPos hp = half_pos(p, cfg, 2 * nt + rank);
                 int cc = 0, tj = 0;
                 for (int st = 0; st < 3 * cfg.cpt; ++st) {
-                    if (warp != 0 && s == 0 && ph) pdl_wait();               // (a bounded wait begins when the kernel in front is over)
                     if (!bar_wait(bar_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
                     const uint32_t fb = lead_full + 8 * s;
                     if (warp == 0) {
@@ -298,7 +294,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
         // so each operand has two producer threads taking alternate stages.
         const bool is_b = (warp == 0 || warp == 3);
         const uint32_t mine = (warp >= 3) ? 1u : 0u;
-        if (is_b) pdl_wait();
+        pdl_wait();
         uint32_t s = 0, ph = 0, g = 0;
         bool ok = true;
         for (int64_t tile = first; tile < cfg.ntiles && ok; tile += step) {
@@ -310,7 +306,6 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 const int nsub = min(kSub2, cfg.nkb - kb);
                 const bool skip = (g & 1u) != mine;
                 if (!skip) {
-                    if (!is_b && ph) pdl_wait();                             // (a bounded wait begins when the kernel in front is over)
                     if (!bar_wait(bar_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
                     // all copies of this stage (up to two k-blocks of two operands in two CTAs) complete on the leader's barrier
                     if (is_b && rank == 0)
@@ -344,7 +339,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
             const uint32_t a_step = a_stage >> 4, b_step = b_stage >> 4;
             const uint32_t row_step = (uint32_t)(p.W * 128) >> 4;                      // (column shift) a tap's rows lie W pixels further on
             uint32_t a_lo = a_lo0, b_lo = b_lo0;
-            pdl_wait();                                                                // (the activations come behind it)
+            pdl_wait();                                                                // (a bounded wait begins when the kernel in front is over)
             for (int64_t tile = first; tile < cfg.ntiles; tile += step, ++it) {
                 const uint32_t ab = it & 1;
                 if (!bar_wait_step(bar_tempty + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag)) break;
@@ -387,13 +382,13 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
         const int nch = (cfg.img_pix + 31) >> 5;             // 32-pixel chunks per run of pixels
         uint32_t it = 0;
         bool alive = true;
-        pdl_wait();                                          // the outputs
+        pdl_wait();
         for (int64_t tile = first; tile < cfg.ntiles && alive; tile += step, ++it) {
             const uint32_t ab = it & 1;
             const int64_t nt = tile / cfg.nbt;
             const int blk = (int)(tile - nt * cfg.nbt) * 2 + (int)rank;
             const int m = blk * kBlockRows + quarter * 32 + lane;
-            const float scale = (m < p.M) ? __fmul_rn(__ldg(wstep + m), p.act_step) : 0.f;
+            const float scale = (m < p.M) ? __fmul_rn(__ldg(pdl_ordered(p.wstep) + m), p.act_step) : 0.f;
             int64_t n0h[2];
             int nvalid[2];
 #pragma unroll

@@ -144,3 +144,51 @@ def _behind_a_late_kernel(early_trigger, name, ns, part):
 def test_a_call_waits_for_a_long_kernel_in_front(early_trigger, name):
     """Longer than the kernels' bounded waits, which begin when the kernel in front is over."""
     _behind_a_late_kernel(early_trigger, name, 1_500_000_000, part=2)
+
+
+@pytest.mark.parametrize("name", ROUTES)
+def test_a_call_reads_weights_that_the_kernel_in_front_writes_late(early_trigger, name):
+    """Packed codes with their metadata and the expanded copy are as the kernel in front leaves them, not as it finds them."""
+    _behind_a_late_kernel(early_trigger, name, 20_000_000, part=0)
+
+
+def test_weights_packed_and_expanded_again_between_calls():
+    """Two layers in turn, packed into the same buffer, expanded into the same workspace and into the library's scratch, with nothing
+    between the calls: each uses its own weights."""
+    import torch
+    M, K, N = 512, 1024, 200
+    g = synth.rng(151)
+    scheme, bits = O.assign_rows(synth.weights_normal(g, (M, K)), (50, 30, 20))
+    layer = R.rmsmp_layer_init(M, K, 1, 1, scheme, bits)
+    packed = torch.zeros(layer.packed_bytes, dtype=torch.uint8, device="cuda")
+    ws = torch.zeros(R.rmsmp_workspace_bytes(layer), dtype=torch.int8, device="cuda")
+    codes = torch.from_numpy(synth.act_codes_uniform(g, (N, K))).cuda()
+    Ws = [synth.weights_normal(g, (M, K)) for _ in range(2)]
+    alphas = [synth.alpha_rows(W) for W in Ws]
+    refs = [O.layer_linear(W, scheme, bits, a, codes.cpu().numpy(), np.float32(0.25))[-1].reshape(N, M) for W, a in zip(Ws, alphas)]
+    dW = [torch.from_numpy(W).cuda() for W in Ws]
+    outs = torch.full((24, 4, N, M), float("nan"), dtype=torch.float32, device="cuda")
+    n16 = torch.full((24, 16, M), float("nan"), dtype=torch.float32, device="cuda")
+    arrs = [R.make_gemm_items([(layer, packed, codes, 16, K, 0.25, n16[i], M, None, 1)]) for i in range(24)]
+    tables = [torch.empty(R.rmsmp_grouped_plan_bytes(arrs[0]), dtype=torch.uint8, device="cuda") for _ in range(24)]
+    plans = [R.rmsmp_gemm_grouped_prepare(a, R.OUT_NM, t) for a, t in zip(arrs, tables)]
+    torch.cuda.synchronize()
+    for i in range(24):
+        R.rmsmp_quantize_pack(dW[i % 2], R.W_LINEAR, layer, scheme, bits, alphas[i % 2], R.POT_NEAREST, packed)
+        if i % 4 < 2:
+            R.rmsmp_gemm_grouped_launch(plans[i])                       # directly behind the packing
+            R.rmsmp_gemm(layer, packed, codes, N, K, 0.25, outs[i, 0], M, R.OUT_NM)
+        else:
+            R.rmsmp_gemm(layer, packed, codes, N, K, 0.25, outs[i, 0], M, R.OUT_NM)
+            R.rmsmp_gemm_grouped_launch(plans[i])
+        R.rmsmp_expand_weights(layer, packed, ws)
+        R.rmsmp_gemm_workspace(layer, packed, ws, codes, N, K, 0.25, outs[i, 1], M)
+        R.rmsmp_gemm_builtin_scratch(layer, packed, codes, N, K, 0.25, outs[i, 2], M)
+        R.rmsmp_gemm_builtin_scratch(layer, packed, codes, N, K, 0.25, outs[i, 3], M)
+    torch.cuda.synchronize()
+    assert R.rmsmp_last_device_status(packed) == R.OK
+    got, got16 = outs.cpu().numpy(), n16.cpu().numpy()
+    for i in range(24):
+        for k in range(4):
+            assert np.array_equal(got[i, k].view(np.uint32), refs[i % 2].view(np.uint32)), (i, k)
+        assert np.array_equal(got16[i].view(np.uint32), refs[i % 2][:16].view(np.uint32)), i
