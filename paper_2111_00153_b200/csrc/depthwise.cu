@@ -11,9 +11,9 @@
 // 74 us for 56 x 56 x 192 at batch 64).  So the words of four neighbouring columns are transposed (4 x 4
 // bytes, eight permutes), which makes the three taps of a kernel row one dot product; a thread owns a
 // channel quad and four neighbouring columns and walks down a strip of rows, so that every input row is
-// loaded and transposed once for the three output rows that it touches.  Its next four input rows are on their way
-// meanwhile, into words of shared memory of its own (nobody waits for anybody): in registers one row was what there was room for
-// (56 x 56 x 192 at batch 64, launches back to back: 44.2 us so, 41.9 with the ring; two blocks of 128-register threads per SM).
+// loaded and transposed once for the three output rows that it touches, and the next row's loads are in flight
+// meanwhile.  What is left is load latency at two blocks of 128-register threads per SM; down tall strips of stride one the next four input
+// rows are on their way instead, into words of shared memory of the thread's own, where nobody waits for anybody (see launch_depthwise).
 // Other filters: a word is split into four one-channel words, one output per work item.
 #include <algorithm>
 #include "common.cuh"
@@ -25,9 +25,10 @@ namespace {
 constexpr int kDwThreads = 256;
 constexpr int kDwCols = 4;                                 // output columns per thread (3 x 3 path)
 constexpr size_t kDwSmem = 226 * 1024;
-constexpr int kDwAhead = 4;                                // input rows on their way per thread (3 x 3 path)
+constexpr int kDwAhead = 4;                                // input rows on their way per thread (with a ring)
 constexpr uint32_t kDwRingColumn = kDwThreads * 4;         // a column of a ring row: a word per thread
-__host__ __device__ constexpr int dw_ring_bytes(int s) { return (kDwAhead + 1) * (3 * s + 3) * (int)kDwRingColumn; }
+constexpr size_t kDwRing = (kDwAhead + 1) * 6 * (size_t)kDwRingColumn;
+constexpr int kDwRingStrip = 10;                           // strip height from which on the ring pays
 // Sums start from the bits of 1.5 * 2^23: a nine-tap sum of int8 products is below 2^18, so the finished word IS the
 // float 1.5 * 2^23 + sum and one subtraction gives float(sum) exactly.
 constexpr int kDwMagicBits = 0x4B400000;
@@ -105,8 +106,9 @@ __device__ __forceinline__ void dw_store(const Problem& p, uint32_t n, int q, co
 }
 
 // kS = 1, 2: 3 x 3 filters of that stride, strips of `strip` output rows; kS = 0: any filter, one output per item.
-// kAcc: the sums are wanted too (their addresses take registers that the strips need: 5 % of the time).
-template <int kS, bool kAcc>
+// kAcc: the sums are wanted too (their addresses take registers that the strips need: 5 % of the time).  kRing (stride 1): input rows
+// through a ring of the thread's own words.
+template <int kS, bool kAcc, bool kRing>
 __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const Problem given, const int strip)
 {
     extern __shared__ uint32_t s_w[];                     // [tap][quad]: channel 4q+j in byte j
@@ -140,6 +142,7 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
         const uint32_t ncol = (uint32_t)(p.Wo + kDwCols - 1) / kDwCols, nstrip = (uint32_t)(p.Ho + strip - 1) / (uint32_t)strip;
         const uint32_t n_items = (uint32_t)p.B * nstrip * ncol;
         constexpr int kXW = 3 * kS + 3;                                // input columns under four outputs
+        static_assert(!kRing || kXW == 6, "");
         const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_w) + (uint32_t)((taps * C + 15) & ~15) + 4u * threadIdx.x;
         for (int qi = 0; qi < qpt; ++qi) {
             const int q = my_q0 + qi * lanes_q;
@@ -163,17 +166,30 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
 #pragma unroll
                 for (int x = 0; x < kXW; ++x) in_x |= ((unsigned)(x0 + x) < (unsigned)p.W ? 1u : 0u) << x;
                 // behind the last input row of the strip; 0 where the whole strip lies in the padding above the image, so
-                // that the one unsigned comparison in load() rules out rows in front of the image too
+                // that the one unsigned comparison in load() and fetch() rules out rows in front of the image too
                 const int y_end = max(0, min(p.H, (ho0 + rows - 1) * kS - p.pad + 3));
-                // The thread's next input row on its way to its own words of the ring; rows and columns outside the image become zeros.
-                int y = ho0 * kS - p.pad;                              // the input row to fetch next
+                auto load = [&](int y, uint32_t (&a)[kXW]) {           // rows and columns outside the image read as zero
+                    const int8_t* r = src + (int64_t)y * row_pitch;
+                    if ((unsigned)y >= (unsigned)y_end) {
+#pragma unroll
+                        for (int x = 0; x < kXW; ++x) a[x] = 0u;
+                    } else if (in_x == (1u << kXW) - 1u) {             // the usual case, without a predicate per column
+#pragma unroll
+                        for (int x = 0; x < kXW; ++x) a[x] = __ldg(reinterpret_cast<const uint32_t*>(r + (uint32_t)x * pitch));
+                    } else {
+#pragma unroll
+                        for (int x = 0; x < kXW; ++x) a[x] = ((in_x >> x) & 1u) ? __ldg(reinterpret_cast<const uint32_t*>(r + (uint32_t)x * pitch)) : 0u;
+                    }
+                };
+                int y = ho0 * kS - p.pad;                              // the input row to load next
+                // kRing: that row on its way to the thread's own words of the ring; rows and columns outside the image become zeros.
                 uint32_t put = ring, got = ring;                       // where it goes, and where the next one to be used lies
                 auto fetch = [&]() {
                     const int8_t* r = src + (int64_t)y * row_pitch;
                     if ((unsigned)y >= (unsigned)y_end) {
 #pragma unroll
                         for (int x = 0; x < kXW; ++x) dw_copy(put + x * kDwRingColumn, p.act, 0u);
-                    } else if (in_x == (1u << kXW) - 1u) {             // the usual case, without a choice per column
+                    } else if (in_x == (1u << kXW) - 1u) {
 #pragma unroll
                         for (int x = 0; x < kXW; ++x) dw_copy(put + x * kDwRingColumn, r + (uint32_t)x * pitch, 4u);
                     } else {
@@ -217,23 +233,45 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
                 };
                 DwRow<kS> r[3];
                 uint32_t a[kXW];
-                asm volatile("cp.async.wait_group 0;" ::: "memory");   // (what the last item fetched behind its end: zeros)
+                if constexpr (kRing) {
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");           // (what the last item fetched behind its end: zeros)
 #pragma unroll
-                for (int i = 0; i < kDwAhead; ++i) fetch();
-                if constexpr (kS == 1) {
-                    take(a); dw_arrange<1>(a, r[0]);
-                    take(a); dw_arrange<1>(a, r[1]);
+                    for (int i = 0; i < kDwAhead; ++i) fetch();
+                    take(a); dw_arrange<kS>(a, r[0]);
+                    take(a); dw_arrange<kS>(a, r[1]);
                     for (int h = 0; h < rows; h += 3) {
                         // three output rows a turn, so that the rows' places in r[] are fixed
-                        take(a); dw_arrange<1>(a, r[2]); emit(h, r[0], r[1], r[2]);
-                        if (h + 1 < rows) { take(a); dw_arrange<1>(a, r[0]); emit(h + 1, r[1], r[2], r[0]); }
-                        if (h + 2 < rows) { take(a); dw_arrange<1>(a, r[1]); emit(h + 2, r[2], r[0], r[1]); }
+                        take(a); dw_arrange<kS>(a, r[2]); emit(h, r[0], r[1], r[2]);
+                        if (h + 1 < rows) { take(a); dw_arrange<kS>(a, r[0]); emit(h + 1, r[1], r[2], r[0]); }
+                        if (h + 2 < rows) { take(a); dw_arrange<kS>(a, r[1]); emit(h + 2, r[2], r[0], r[1]); }
+                    }
+                } else if constexpr (kS == 1) {
+                    uint32_t nx[kXW];
+                    load(y, a);
+                    load(y + 1, nx);
+                    dw_arrange<1>(a, r[0]);
+                    load(y + 2, a);
+                    dw_arrange<1>(nx, r[1]);
+                    y += 3;
+                    for (int h = 0; h < rows; h += 3) {                // a row's words are loaded while the row in front of it is worked on
+                        load(y, nx); dw_arrange<1>(a, r[2]); emit(h, r[0], r[1], r[2]);
+                        if (h + 1 < rows) { load(y + 1, a); dw_arrange<1>(nx, r[0]); emit(h + 1, r[1], r[2], r[0]); }
+                        if (h + 2 < rows) { load(y + 2, nx); dw_arrange<1>(a, r[1]); emit(h + 2, r[2], r[0], r[1]); }
+#pragma unroll
+                        for (int x = 0; x < kXW; ++x) a[x] = nx[x];
+                        y += 3;
                     }
                 } else {
-                    take(a); dw_arrange<2>(a, r[0]);
+                    uint32_t nx[kXW];
+                    load(y, a);
+                    load(y + 1, nx);
+                    dw_arrange<2>(a, r[0]);
+                    load(y + 2, a);
+                    y += 3;
                     for (int h = 0; h < rows; h += 2) {                // r[0] and r[2] take turns as the shared row
-                        take(a); dw_arrange<2>(a, r[1]); take(a); dw_arrange<2>(a, r[2]); emit(h, r[0], r[1], r[2]);
-                        if (h + 1 < rows) { take(a); dw_arrange<2>(a, r[1]); take(a); dw_arrange<2>(a, r[0]); emit(h + 1, r[2], r[1], r[0]); }
+                        dw_arrange<2>(nx, r[1]); load(y, nx); dw_arrange<2>(a, r[2]); load(y + 1, a); emit(h, r[0], r[1], r[2]);
+                        if (h + 1 < rows) { dw_arrange<2>(nx, r[1]); load(y + 2, nx); dw_arrange<2>(a, r[0]); load(y + 3, a); emit(h + 1, r[2], r[1], r[0]); }
+                        y += 4;
                     }
                 }
             }
@@ -280,18 +318,17 @@ bool depthwise_supported(const Problem& p)
 
 cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
 {
-    const size_t table = (size_t)p.kh * p.kw * p.M, with_ring = ((table + 15) & ~(size_t)15) + dw_ring_bytes(p.stride);
-    const int variant = (p.kh == 3 && p.kw == 3 && (p.stride == 1 || p.stride == 2) && with_ring <= kDwSmem) ? p.stride : 0;
-    const size_t smem = variant ? with_ring : table;
+    const size_t table = (size_t)p.kh * p.kw * p.M, with_ring = ((table + 15) & ~(size_t)15) + kDwRing;
+    const int variant = (p.kh == 3 && p.kw == 3 && (p.stride == 1 || p.stride == 2)) ? p.stride : 0;
     const bool acc = variant != 0 && p.acc;
-    static bool attr_set[3][2][kMaxDevices] = {};
-    void (*const kernel)(const Problem, const int) = variant == 1 ? (acc ? depthwise_kernel<1, true> : depthwise_kernel<1, false>)
-                                                   : variant == 2 ? (acc ? depthwise_kernel<2, true> : depthwise_kernel<2, false>)
-                                                                  : depthwise_kernel<0, false>;
-    const void* fn = reinterpret_cast<const void*>(kernel);
-    if (smem > 48 * 1024 && !ensure_smem_attr(fn, (int)kDwSmem, attr_set[variant][acc])) return cudaErrorUnknown;
+    static bool attr_set[4][2][kMaxDevices] = {};
+    typedef void (*Kernel)(const Problem, const int);
+    Kernel kernel = variant == 1 ? (acc ? depthwise_kernel<1, true, false> : depthwise_kernel<1, false, false>)
+                  : variant == 2 ? (acc ? depthwise_kernel<2, true, false> : depthwise_kernel<2, false, false>)
+                                 : depthwise_kernel<0, false, false>;
+    if (table > 48 * 1024 && !ensure_smem_attr(reinterpret_cast<const void*>(kernel), (int)kDwSmem, attr_set[variant][acc])) return cudaErrorUnknown;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kDwThreads, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, reinterpret_cast<const void*>(kernel), kDwThreads, table);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     const int quads = p.M >> 2;
@@ -320,7 +357,17 @@ cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
     }
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    return launch_dependent(kernel, (unsigned)blocks, kDwThreads, smem, st, p, strip);
+    // Tall strips of stride one through the ring, where as many blocks fit beside each other with it.  (Launches back to back, registers
+    // against ring: 576 channels, 64 images of 14 x 14, strips of 14 rows 24.8 us and 21.2; 192, 64 of 56 x 56, 19 rows 48.4 and 44.9; 192, 64 of
+    // 28 x 28, 10 rows 17.0 and 16.6; 384, 64 of 14 x 14, 7 rows 14.8 and 14.7; 960, 64 of 7 x 7, 4 rows 20.2 and 20.7; 144, 8 of 56 x 56, 4 rows
+    // 9.4 and 10.2.  With sums 192, 64 of 56 x 56 72.7 and 76.2.  Stride two, whose rows are nine words: 192, 64 of 56 x 56 25.3 and 26.4, 192, 64 of 28 x 28
+    // 10.0 and 11.4, 8, 70 of 100 x 100 9.5 and 12.4.)
+    if (variant == 1 && !acc && strip >= kDwRingStrip && (with_ring + 1024) * (size_t)per_sm <= 228 * 1024) {
+        const Kernel ringed = depthwise_kernel<1, false, true>;
+        if (with_ring > 48 * 1024 && !ensure_smem_attr(reinterpret_cast<const void*>(ringed), (int)kDwSmem, attr_set[3][0])) return cudaErrorUnknown;
+        return launch_dependent(ringed, (unsigned)blocks, kDwThreads, with_ring, st, p, strip);
+    }
+    return launch_dependent(kernel, (unsigned)blocks, kDwThreads, table, st, p, strip);
 }
 
 }  // namespace rmsmp

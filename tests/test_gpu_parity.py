@@ -1363,3 +1363,31 @@ def test_depthwise_threads_that_take_several_strips(stride, B):
     R.rmsmp_conv_depthwise(layer, d_packed, torch.from_numpy(codes).cuda(), B, H, H, stride, 1, 0.5, y)
     torch.cuda.synchronize()
     assert np.array_equal(y.cpu().numpy().view(np.uint32), O.epilogue(acc_ref, wstep, np.float32(0.5)).view(np.uint32))
+
+
+@pytest.mark.parametrize("C,H,W,B,stride,with_acc", [
+    (96, 32, 1, 1528, 1, False),        # strips of eleven rows through the ring, two for some threads
+    (28, 32, 5, 2697, 1, False),
+    (1028, 11, 1, 446, 1, False),       # several channel quads a thread
+    (100, 29, 6, 64, 1, False),         # strips of fewer rows, in registers
+    (20000, 11, 1, 100, 1, False),      # the ring beside a filter table of 180 KB
+    (22752, 11, 1, 100, 1, False),      # no room for it beside the widest table
+    (22752, 5, 3, 1, 1, True), (22752, 5, 4, 2, 2, False), (20604, 5, 3, 2, 2, False), (22752, 5, 3, 1, 2, True),
+])
+def test_depthwise_strips_with_and_without_a_ring(C, H, W, B, stride, with_acc):
+    import torch
+    g = synth.rng(145, C + H + B)
+    Wt = synth.weights_kaiming(g, C, 1, 3, 3)
+    scheme, bits = O.assign_rows(Wt, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    codes = g.integers(-128, 128, size=(B, H, W, C), dtype=np.int8)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    v_ref, wstep = O.quantize_rows(Wt.reshape(C, -1), scheme, bits, alpha)
+    acc_ref = O.conv_depthwise(v_ref.reshape(C, 3, 3), codes, stride, 1)
+    y = torch.full(acc_ref.shape, float("nan"), dtype=torch.float32, device="cuda")
+    acc = torch.full(acc_ref.shape, -5, dtype=torch.int32, device="cuda")
+    R.rmsmp_conv_depthwise(layer, d_packed, torch.from_numpy(codes).cuda(), B, H, W, stride, 1, 0.5, y, acc if with_acc else None)
+    torch.cuda.synchronize()
+    if with_acc:
+        assert np.array_equal(acc.cpu().numpy(), acc_ref)
+    assert np.array_equal(y.cpu().numpy().view(np.uint32), O.epilogue(acc_ref, wstep, np.float32(0.5)).view(np.uint32))
