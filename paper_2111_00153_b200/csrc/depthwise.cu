@@ -276,6 +276,7 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
                 }
             }
         }
+        if constexpr (kRing) asm volatile("cp.async.wait_group 0;" ::: "memory");      // (the block's shared memory is its own until it ends)
         return;
     } else {
     const uint32_t N = (uint32_t)p.N, hw = (uint32_t)(p.Ho * p.Wo);
