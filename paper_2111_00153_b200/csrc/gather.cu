@@ -371,10 +371,14 @@ cudaError_t launch_im2col(const int8_t* act, int B, int H, int W, int C, int64_t
     if (ra.tile < Wo && ra.tile >= 32) ra.tile &= ~31;
     const size_t smem = ((size_t)ra.tile * ld_cols + (size_t)kh * ra.rowb + 31) / 32 * 32 + 32 + sizeof(Piece) * (size_t)(a.units + kh);
     if (C == 3 && pix_pitch == 3 && kh == kw && (kw == 3 || kw == 5 || kw == 7) && ld_cols == (3 * kw * kw + 15) / 16 * 16 && stride <= 4) {
-        const int rows = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)Ho, 256 / Wo, 8}));
+        // As many rows a pass as leave every SM one: im2col_rows_kernel, here with about 256 pixels a pass whatever their number, and so: 7x7 of step
+        // two, one image of 112x112 2.7, 3.4 and 2.7 us, 25 of 37x77 4.1, 3.9 and 3.4; twice as many passes: 256 of 32x32 at step four 4.4, now 3.4.
+        // Few passes of several rows are too few at step four (7x7, 8 of 224x224 4.0, 4.0 and 4.4; 64 of 64x64 4.0, 3.4 and 3.3).
+        const int64_t per_sm = (int64_t)B * Ho / sm_count();
+        const int rows = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)Ho, 256 / Wo, 8, per_sm}));
         const size_t bytes = (size_t)rows * Wo * ld_cols + ((size_t)(rows - 1) * stride + kh) * ra.rowb;
         const int64_t items = (int64_t)B * ((Ho + rows - 1) / rows);
-        if (bytes <= 46 * 1024 && items < (1ll << 31)) {
+        if (bytes <= 46 * 1024 && items < (1ll << 31) && (stride < 4 || rows == 1 || per_sm >= 6)) {
             // (five blocks an SM at most, as below)
             const size_t smem3 = std::max<size_t>(bytes, 40 * 1024);
             auto* const kernel = kw == 3 ? im2col_rgb_kernel<3> : kw == 5 ? im2col_rgb_kernel<5> : im2col_rgb_kernel<7>;

@@ -1391,3 +1391,28 @@ def test_depthwise_strips_with_and_without_a_ring(C, H, W, B, stride, with_acc):
     if with_acc:
         assert np.array_equal(acc.cpu().numpy(), acc_ref)
     assert np.array_equal(y.cpu().numpy().view(np.uint32), O.epilogue(acc_ref, wstep, np.float32(0.5)).view(np.uint32))
+
+
+@pytest.mark.parametrize("k,stride,pad,B,H,W,offset", [
+    (7, 2, 3, 64, 37, 64, 0),      # eight output rows a pass, the last one of an image has three
+    (7, 2, 3, 40, 9, 223, 1),      # a pass of two rows, or one
+    (3, 2, 1, 200, 31, 31, 0),     # more rows a pass than pixels would need
+    (3, 1, 4, 100, 5, 6, 2),       # padding wider than the filter
+    (5, 2, 2, 30, 33, 47, 7),      # three rows a pass: as many as leave every SM a pass
+    (5, 4, 2, 300, 17, 40, 3),     # a step of four: passes enough
+    (5, 4, 2, 100, 17, 40, 3),     # too few
+])
+def test_patch_matrix_of_three_channels_and_many_rows(k, stride, pad, B, H, W, offset):
+    import torch
+    g = synth.rng(146, k + H + W)
+    act = g.integers(-128, 128, size=(B, H, W, 3), dtype=np.int8)
+    raw = torch.full((offset + act.size,), 77, dtype=torch.int8, device="cuda")
+    raw[offset:] = torch.from_numpy(act.reshape(-1)).cuda()
+    ld = (3 * k * k + 15) // 16 * 16
+    ref = O.im2col(act, k, k, stride, pad, ld)
+    out = torch.full((ref.size + 256,), 99, dtype=torch.int8, device="cuda")
+    R.rmsmp_im2col_codes(raw[offset:], B, H, W, 3, 3, k, k, stride, pad, out[128:], ld)
+    torch.cuda.synchronize()
+    got = out.cpu().numpy()
+    assert np.array_equal(got[128:-128].reshape(ref.shape), ref)
+    assert (got[:128] == 99).all() and (got[-128:] == 99).all()
