@@ -12,7 +12,7 @@
 // bytes, eight permutes), which makes the three taps of a kernel row one dot product; a thread owns a
 // channel quad and four neighbouring columns and walks down a strip of rows, so that every input row is
 // loaded and transposed once for the three output rows that it touches, and the next row's loads are in flight
-// meanwhile.  What is left is load latency at two blocks of 128-register threads per SM; down tall strips of stride one the next four input
+// meanwhile.  What is left is load latency at two blocks of 128-register threads per SM; down tall strips the next four input
 // rows are on their way instead, into words of shared memory of the thread's own, where nobody waits for anybody (see launch_depthwise).
 // Other filters: a word is split into four one-channel words, one output per work item.
 #include <algorithm>
@@ -27,8 +27,7 @@ constexpr int kDwCols = 4;                                 // output columns per
 constexpr size_t kDwSmem = 226 * 1024;
 constexpr int kDwAhead = 4;                                // input rows on their way per thread (with a ring)
 constexpr uint32_t kDwRingColumn = kDwThreads * 4;         // a column of a ring row: a word per thread
-constexpr size_t kDwRing = (kDwAhead + 1) * 6 * (size_t)kDwRingColumn;
-constexpr int kDwRingStrip = 10;                           // strip height from which on the ring pays
+__host__ __device__ constexpr size_t dw_ring(int s) { return (kDwAhead + 1) * (3 * s + 3) * (size_t)kDwRingColumn; }
 // Sums start from the bits of 1.5 * 2^23: a nine-tap sum of int8 products is below 2^18, so the finished word IS the
 // float 1.5 * 2^23 + sum and one subtraction gives float(sum) exactly.
 constexpr int kDwMagicBits = 0x4B400000;
@@ -106,8 +105,8 @@ __device__ __forceinline__ void dw_store(const Problem& p, uint32_t n, int q, co
 }
 
 // kS = 1, 2: 3 x 3 filters of that stride, strips of `strip` output rows; kS = 0: any filter, one output per item.
-// kAcc: the sums are wanted too (their addresses take registers that the strips need: 5 % of the time).  kRing (stride 1): input rows
-// through a ring of the thread's own words.
+// kAcc: the sums are wanted too (their addresses take registers that the strips need: 5 % of the time).  kRing: input rows through
+// a ring of the thread's own words.
 template <int kS, bool kAcc, bool kRing>
 __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const Problem given, const int strip)
 {
@@ -142,7 +141,6 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
         const uint32_t ncol = (uint32_t)(p.Wo + kDwCols - 1) / kDwCols, nstrip = (uint32_t)(p.Ho + strip - 1) / (uint32_t)strip;
         const uint32_t n_items = (uint32_t)p.B * nstrip * ncol;
         constexpr int kXW = 3 * kS + 3;                                // input columns under four outputs
-        static_assert(!kRing || kXW == 6, "");
         const uint32_t ring = (uint32_t)__cvta_generic_to_shared(s_w) + (uint32_t)((taps * C + 15) & ~15) + 4u * threadIdx.x;
         for (int qi = 0; qi < qpt; ++qi) {
             const int q = my_q0 + qi * lanes_q;
@@ -238,12 +236,19 @@ __global__ void __launch_bounds__(kDwThreads, kS ? 2 : 4) depthwise_kernel(const
 #pragma unroll
                     for (int i = 0; i < kDwAhead; ++i) fetch();
                     take(a); dw_arrange<kS>(a, r[0]);
-                    take(a); dw_arrange<kS>(a, r[1]);
-                    for (int h = 0; h < rows; h += 3) {
-                        // three output rows a turn, so that the rows' places in r[] are fixed
-                        take(a); dw_arrange<kS>(a, r[2]); emit(h, r[0], r[1], r[2]);
-                        if (h + 1 < rows) { take(a); dw_arrange<kS>(a, r[0]); emit(h + 1, r[1], r[2], r[0]); }
-                        if (h + 2 < rows) { take(a); dw_arrange<kS>(a, r[1]); emit(h + 2, r[2], r[0], r[1]); }
+                    if constexpr (kS == 1) {
+                        take(a); dw_arrange<kS>(a, r[1]);
+                        for (int h = 0; h < rows; h += 3) {
+                            // three output rows a turn, so that the rows' places in r[] are fixed
+                            take(a); dw_arrange<kS>(a, r[2]); emit(h, r[0], r[1], r[2]);
+                            if (h + 1 < rows) { take(a); dw_arrange<kS>(a, r[0]); emit(h + 1, r[1], r[2], r[0]); }
+                            if (h + 2 < rows) { take(a); dw_arrange<kS>(a, r[1]); emit(h + 2, r[2], r[0], r[1]); }
+                        }
+                    } else {
+                        for (int h = 0; h < rows; h += 2) {            // r[0] and r[2] take turns as the shared row
+                            take(a); dw_arrange<kS>(a, r[1]); take(a); dw_arrange<kS>(a, r[2]); emit(h, r[0], r[1], r[2]);
+                            if (h + 1 < rows) { take(a); dw_arrange<kS>(a, r[1]); take(a); dw_arrange<kS>(a, r[0]); emit(h + 1, r[2], r[1], r[0]); }
+                        }
                     }
                 } else if constexpr (kS == 1) {
                     uint32_t nx[kXW];
@@ -319,10 +324,10 @@ bool depthwise_supported(const Problem& p)
 
 cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
 {
-    const size_t table = (size_t)p.kh * p.kw * p.M, with_ring = ((table + 15) & ~(size_t)15) + kDwRing;
+    const size_t table = (size_t)p.kh * p.kw * p.M, with_ring = ((table + 15) & ~(size_t)15) + dw_ring(p.stride);
     const int variant = (p.kh == 3 && p.kw == 3 && (p.stride == 1 || p.stride == 2)) ? p.stride : 0;
     const bool acc = variant != 0 && p.acc;
-    static bool attr_set[4][2][kMaxDevices] = {};
+    static bool attr_set[5][2][kMaxDevices] = {};
     typedef void (*Kernel)(const Problem, const int);
     Kernel kernel = variant == 1 ? (acc ? depthwise_kernel<1, true, false> : depthwise_kernel<1, false, false>)
                   : variant == 2 ? (acc ? depthwise_kernel<2, true, false> : depthwise_kernel<2, false, false>)
@@ -358,14 +363,16 @@ cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
     }
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    // Tall strips of stride one through the ring, where as many blocks fit beside each other with it.  (Launches back to back, registers
-    // against ring: 576 channels, 64 images of 14 x 14, strips of 14 rows 24.8 us and 21.2; 192, 64 of 56 x 56, 19 rows 48.4 and 44.9; 192, 64 of
-    // 28 x 28, 10 rows 17.0 and 16.6; 384, 64 of 14 x 14, 7 rows 14.8 and 14.7; 960, 64 of 7 x 7, 4 rows 20.2 and 20.7; 144, 8 of 56 x 56, 4 rows
-    // 9.4 and 10.2.  With sums 192, 64 of 56 x 56 72.7 and 76.2.  Stride two, whose rows are nine words: 192, 64 of 56 x 56 25.3 and 26.4, 192, 64 of 28 x 28
-    // 10.0 and 11.4, 8, 70 of 100 x 100 9.5 and 12.4.)
-    if (variant == 1 && !acc && strip >= kDwRingStrip && (with_ring + 1024) * (size_t)per_sm <= 228 * 1024) {
-        const Kernel ringed = depthwise_kernel<1, false, true>;
-        if (with_ring > 48 * 1024 && !ensure_smem_attr(reinterpret_cast<const void*>(ringed), (int)kDwSmem, attr_set[3][0])) return cudaErrorUnknown;
+    // Tall strips through the ring, where as many blocks fit beside each other with it; of stride two, whose rows are nine words, where a
+    // quarter of a block's threads has no item.  (Launches back to back, registers against ring: 576 channels, 64 images of 14 x 14, strips of 14
+    // rows 24.8 us and 21.2; 192, 64 of 56 x 56, 19 rows 48.4 and 44.9; 192, 64 of 28 x 28, 10 rows 17.0 and 16.6; 384, 64 of 14 x 14, 7 rows 14.8
+    // and 14.7; 960, 64 of 7 x 7, 4 rows 20.2 and 20.7; 144, 8 of 56 x 56, 4 rows 9.4 and 10.2.  With sums 192, 64 of 56 x 56 72.7 and 76.2.  Stride two:
+    // 576, 64 of 28 x 28, 14 rows, 144 threads 34.5 and 28.9; 384, 64 of 28 x 28, 7 rows, 192 threads 21.4 and 20.4; 576, 64 of 14 x 14, 4 rows 17.1 and 17.6;
+    // 192, 64 of 56 x 56, 10 rows, 240 threads 25.3 and 26.4.)
+    const bool tall = variant == 1 ? strip >= 10 : variant == 2 && strip >= 7 && 4 * ipg * std::min(quads, kDwThreads) <= 3 * kDwThreads;
+    if (tall && !acc && with_ring <= kDwSmem && (with_ring + 1024) * (size_t)per_sm <= 228 * 1024) {
+        const Kernel ringed = variant == 1 ? depthwise_kernel<1, false, true> : depthwise_kernel<2, false, true>;
+        if (with_ring > 48 * 1024 && !ensure_smem_attr(reinterpret_cast<const void*>(ringed), (int)kDwSmem, attr_set[2 + variant][0])) return cudaErrorUnknown;
         return launch_dependent(ringed, (unsigned)blocks, kDwThreads, with_ring, st, p, strip);
     }
     return launch_dependent(kernel, (unsigned)blocks, kDwThreads, table, st, p, strip);

@@ -1372,6 +1372,10 @@ def test_depthwise_threads_that_take_several_strips(stride, B):
     (100, 29, 6, 64, 1, False),         # strips of fewer rows, in registers
     (20000, 11, 1, 100, 1, False),      # the ring beside a filter table of 180 KB
     (22752, 11, 1, 100, 1, False),      # no room for it beside the widest table
+    (22260, 11, 1, 100, 1, False), (22300, 11, 1, 100, 1, False), (22340, 11, 1, 100, 1, False), (22416, 11, 1, 100, 1, False),      # the last tables with room, and the next
+    (528, 14, 1, 464, 2, False),        # of stride two, two strips for some threads
+    (516, 13, 4, 488, 2, False),
+    (20604, 13, 1, 40, 2, False), (18000, 13, 1, 100, 2, False),      # most threads have an item: registers
     (22752, 5, 3, 1, 1, True), (22752, 5, 4, 2, 2, False), (20604, 5, 3, 2, 2, False), (22752, 5, 3, 1, 2, True),
 ])
 def test_depthwise_strips_with_and_without_a_ring(C, H, W, B, stride, with_acc):
