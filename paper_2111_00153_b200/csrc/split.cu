@@ -35,7 +35,6 @@ constexpr int kSplitThreads = 448;
 constexpr int kSplitFirst = 2;                   // first of the twelve working warps
 constexpr int kSplitRing = 8;
 constexpr int kSplitSmem = 200 * 1024;
-constexpr int kSplitHalf = 112 * 1024;
 
 struct SplitCfg {
     int tb, th, npix;        // images / output rows / pixels per tile (the last tile of an image or batch may have fewer)
@@ -503,9 +502,6 @@ bool plan_split(const Problem& p, SplitCfg& best, double* us = nullptr, bool gat
             c.cpo = S > 1 ? (c.n_pad / 8 + S - 1) / S : 0;
             const int red = S * c.cpo * 8 * 512;
             c.nst = std::min(std::min(kpc, kSplitRing), (kSplitSmem - 2048 - red) / (c.a_bytes + c.b_bytes));
-            // (half of the shared memory where four stages fit in it: the next launch's CTAs, with their weights, beside these)
-            const int half = (kSplitHalf - 2048 - red) / (c.a_bytes + c.b_bytes);
-            if (c.pre && half >= 4) c.nst = std::min(c.nst, half);
             // fewer than three stages are not enough for the three expander groups: a group may run ahead of the others by
             // two of its own k-blocks, and a stage's barrier tells only neighbouring phases apart
             if (c.nst < 3 && c.nst < kpc) continue;
