@@ -40,11 +40,13 @@ constexpr int kNumEpiWarps = 4;
 constexpr int kPreWarps = 2 + 8 + kNumEpiWarps;  // warps of the forms that have no expanders
 constexpr int kGroups = 2;                       // expander groups taking alternate k-blocks
 constexpr int kNumExpWarps = 4 * kGroups;
-// Codes out: a chunk is some 250 instructions, most of them waiting for the one in front, and its bytes are few: more warps with
-// one set of registers each, not twelve with two (192x32 on 200,704 pixels 25.5 us with twelve, 23.9 so; 256x256 3x3 on 256 images
-// of 14x14 30.9 and 30.4).
+// Codes out on resident weights: a chunk is some 250 instructions, most of them waiting for the one in front, and its bytes are few:
+// more warps, with one set of registers each (192x32 on 200,704 pixels 25.5 us with twelve, 23.9 so).  Through the rings a tile takes longer and
+// more warps that wait for it are in its way, unless the codes have to leave one by one: 160x192 3x3 on 64 images of 28x28 43.4 us with nineteen,
+// 36.7 with eleven, 768x3072 N=4096 13.3 and 11.8, 32x32 7x7 of step two on 145 of 11x11 19.5 and 16.1, 64x32 7x7 on 64 of 28x28 41.5 and 42.7; but
+// 332x384 3x3 on 234 of 7x7 19.0 and 22.8.
 constexpr int kRqWarps = 22;
-__host__ __device__ constexpr int warps_of(int mode, int rq) { return mode ? (rq ? kRqWarps : kPreWarps) : 2 + kNumExpWarps + kNumEpiWarps; }
+__host__ __device__ constexpr int warps_of(int mode, bool many) { return mode ? (many ? kRqWarps : kPreWarps) : 2 + kNumExpWarps + kNumEpiWarps; }
 constexpr int kWarpStage = 32 * 32 * 4;          // 4 KB: 32 pixels x 32 rows of fp32/int32
 constexpr int kRqStage = 2 * 32 * 32;            // two buffers of 32 pixels x 32 codes
 constexpr int kWideEpi = 8;                      // epilogue warps of the form with 144 KB of resident weights (codes out: twice as many)
@@ -217,13 +219,13 @@ __device__ __forceinline__ void tmem_ld_four(uint32_t taddr, uint32_t (&v)[4])
 //        shared memory; 1 expanded weights from a workspace through the ring; 2 the same, weights resident in
 //        shared memory; 3 resident weights and three taps per activation stage.  A compile-time constant so that
 //        an instantiation carries only the code of its own form.
-// kOut:  1 when the output is fp32 [N][M] through bulk stores without an accumulator dump (the common case): the
-//        epilogue then carries only that path; 0 decides at run time.
+// kOut:  1 when the output is fp32 [N][M] through bulk stores without an accumulator dump (the common case), or codes through the
+//        rings by 16-byte stores: the epilogue then carries only that path; 0 decides at run time.
 template <int kM2, int kRQ, int kMode, int kOut>
-__global__ void __launch_bounds__(32 * warps_of(kMode, kRQ), 1)
+__global__ void __launch_bounds__(32 * warps_of(kMode, kRQ && !kOut), 1)
 tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps maps)
 {
-    constexpr int kThreads = 32 * warps_of(kMode, kRQ);
+    constexpr int kThreads = 32 * warps_of(kMode, kRQ && !kOut);
     constexpr bool kPre = kMode != 0, kAres = kMode >= 2, kTps3 = kMode == 3;
     const bool use_tma_store = kOut ? true : (cfg.tma_store != 0);
     const bool out_mn = kOut ? false : (p.out_mn != 0);
@@ -1060,13 +1062,15 @@ bool plan(const Problem& p, TensorCfg& c)
     c.cta_full = 0;
     c.epi_warps = kNumEpiWarps;
     const int stage = p.rq_codes ? kRqStage : kWarpStage;
+    // (a row count that is not a multiple of 16 would spill into the padding columns)
+    if (p.rq_codes && p.M % 16 == 0 && p.ld_codes % 16 == 0 && (reinterpret_cast<uintptr_t>(p.rq_codes) & 15) == 0) c.tma_store = 1;
     if (c.pre) {
         c.nA = (c.bk == 64) ? 6 : 3; c.nB = (c.bk == 64) ? 8 : 4; c.out_bufs = 1;
-        c.epi_warps = warps_of(1, p.rq_codes != nullptr) - 3;   // warp 2 fetches the weights (unless they are resident)
+        c.epi_warps = warps_of(1, p.rq_codes && !c.tma_store) - 3;   // warp 2 fetches the weights (unless they are resident)
         c.dup = (p.M <= 64) ? 1 : 0;
         if (resident) {
             c.ares = 1;
-            c.epi_warps = wide ? (p.rq_codes ? 2 * kWideEpi : kWideEpi) : warps_of(1, p.rq_codes != nullptr) - 2;
+            c.epi_warps = wide ? (p.rq_codes ? 2 * kWideEpi : kWideEpi) : warps_of(2, p.rq_codes) - 2;
             c.nA = c.nkb;
             const int64_t left = kSmemLimit - (1024 + 64 * kMaxRing) - (int64_t)c.nkb * c.a_bytes -
                                  (int64_t)c.epi_warps * stage;
@@ -1245,8 +1249,6 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
     if (p.rq_codes) {
         // re-quantized output: [N][ld_codes] code bytes, sixteen rows of a pixel a store
         if (!c.pre || p.out_mn) return RMSMP_ERR_VARIANT;
-        // (a row count that is not a multiple of 16 would spill into the padding columns)
-        if (p.M % 16 == 0 && p.ld_codes % 16 == 0 && (reinterpret_cast<uintptr_t>(p.rq_codes) & 15) == 0) c.tma_store = 1;
     }
     // ([row][pixel]: a bulk store starts at a pixel that is a multiple of four)
     if (ld_ok && (!p.out_mn || (c.tail_rows == 0 && (c.tiles_per_image == 0 || p.Ho % c.th == 0)))) {
@@ -1273,21 +1275,22 @@ rmsmp_status launch_tensor(const Problem& p, cudaStream_t st)
 
     c.trigger = 2 * grid <= p.sms;
 
-    // the kernel's form (see tensor_kernel): [mode][two row blocks][1: re-quantizing epilogue, 2: plain fp32 [N][M] bulk-store output]
+    // the kernel's form (see tensor_kernel): [mode][two row blocks][1: re-quantizing epilogue, 2: plain fp32 [N][M] bulk-store output,
+    // 3: codes through the rings by 16-byte stores]
     typedef void (*KernelFn)(const Problem, const TensorCfg, const Maps);
-    static const KernelFn table[4][2][3] = {
-        {{tensor_kernel<0, 0, 0, 0>, nullptr, tensor_kernel<0, 0, 0, 1>}, {nullptr, nullptr, nullptr}},
-        {{tensor_kernel<0, 0, 1, 0>, tensor_kernel<0, 1, 1, 0>, tensor_kernel<0, 0, 1, 1>},
-         {tensor_kernel<1, 0, 1, 0>, tensor_kernel<1, 1, 1, 0>, tensor_kernel<1, 0, 1, 1>}},
-        {{tensor_kernel<0, 0, 2, 0>, tensor_kernel<0, 1, 2, 0>, tensor_kernel<0, 0, 2, 1>}, {nullptr, nullptr, nullptr}},
-        {{tensor_kernel<0, 0, 3, 0>, tensor_kernel<0, 1, 3, 0>, tensor_kernel<0, 0, 3, 1>}, {nullptr, nullptr, nullptr}},
+    static const KernelFn table[4][2][4] = {
+        {{tensor_kernel<0, 0, 0, 0>, nullptr, tensor_kernel<0, 0, 0, 1>}, {}},
+        {{tensor_kernel<0, 0, 1, 0>, tensor_kernel<0, 1, 1, 0>, tensor_kernel<0, 0, 1, 1>, tensor_kernel<0, 1, 1, 1>},
+         {tensor_kernel<1, 0, 1, 0>, tensor_kernel<1, 1, 1, 0>, tensor_kernel<1, 0, 1, 1>, tensor_kernel<1, 1, 1, 1>}},
+        {{tensor_kernel<0, 0, 2, 0>, tensor_kernel<0, 1, 2, 0>, tensor_kernel<0, 0, 2, 1>}, {}},
+        {{tensor_kernel<0, 0, 3, 0>, tensor_kernel<0, 1, 3, 0>, tensor_kernel<0, 0, 3, 1>}, {}},
     };
     const int mode = !c.pre ? 0 : (!c.ares ? 1 : (c.tps > 1 ? 3 : 2));
     const int i2 = c.m2 ? 1 : 0;
-    const int io = p.rq_codes ? 1 : ((c.tma_store && !p.out_mn && !p.acc) ? 2 : 0);
+    const int io = p.rq_codes ? (mode == 1 && c.tma_store ? 3 : 1) : ((c.tma_store && !p.out_mn && !p.acc) ? 2 : 0);
     const KernelFn fn = table[mode][i2][io];
     if (!fn) return RMSMP_ERR_VARIANT;
-    static bool attr_set[4][2][3][kMaxDevices] = {};
+    static bool attr_set[4][2][4][kMaxDevices] = {};
     if (!ensure_smem_attr(reinterpret_cast<const void*>(fn), kSmemLimit, attr_set[mode][i2][io])) return RMSMP_ERR_CUDA;
     if (launch_dependent(fn, (unsigned)grid, 32 * warps_of(mode, io == 1), c.smem_bytes, st, p, c, mp) != cudaSuccess) {
         cudaGetLastError();

@@ -1420,3 +1420,34 @@ def test_patch_matrix_of_three_channels_and_many_rows(k, stride, pad, B, H, W, o
     got = out.cpu().numpy()
     assert np.array_equal(got[128:-128].reshape(ref.shape), ref)
     assert (got[:128] == 99).all() and (got[-128:] == 99).all()
+
+
+@pytest.mark.parametrize("M,Cin,k,stride,B,H", [
+    (32, 32, 7, 2, 145, 11),       # through the rings, sixteen codes a store
+    (144, 80, 5, 1, 9, 17),        # two row blocks, the second of sixteen rows
+    (256, 1040, 1, 1, 40, 13),     # 1x1 with a last chunk of sixteen channels
+    (68, 96, 5, 1, 9, 17),         # codes one by one
+    (20, 144, 3, 1, 30, 15),       # the same with duplicated rows
+    (332, 384, 3, 1, 70, 7),
+])
+def test_requantized_codes_of_long_tiles(M, Cin, k, stride, B, H):
+    import torch
+    g = synth.rng(147, M + Cin)
+    Wt = synth.weights_kaiming(g, M, Cin, k, k)
+    scheme, bits = _mixed_map(M, M, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    act = synth.act_codes_uniform(g, (B, H, H, Cin))
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    ws = torch.empty(R.rmsmp_workspace_bytes(layer), dtype=torch.int8, device="cuda")
+    R.rmsmp_expand_weights(layer, d_packed, ws)
+    images = sorted({0, B // 2, B - 1})
+    _, _, _, y_ref = O.layer_conv(Wt, scheme, bits, alpha, np.ascontiguousarray(act[images]), np.float32(0.125), stride, k // 2)
+    na = _next_alpha(y_ref)
+    Ho = (H + 2 * (k // 2) - k) // stride + 1
+    for kind in (R.ACT_U4, R.ACT_S4):
+        want, _ = O.quantize_act(y_ref.reshape(len(images), Ho * Ho, M), na, kind)
+        out = torch.full((B * Ho * Ho, M), 99, dtype=torch.int8, device="cuda")
+        R.rmsmp_conv_implicit_workspace_requant(layer, d_packed, ws, torch.from_numpy(act).cuda(), B, H, H, stride, k // 2, 0.125, na, kind, out)
+        torch.cuda.synchronize()
+        assert R.rmsmp_last_device_status(d_packed) == R.OK
+        assert np.array_equal(out.cpu().numpy().reshape(B, Ho * Ho, M)[images], want)
