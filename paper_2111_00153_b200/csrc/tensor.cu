@@ -40,11 +40,13 @@ constexpr int kNumEpiWarps = 4;
 constexpr int kPreWarps = 2 + 8 + kNumEpiWarps;  // warps of the forms that have no expanders
 constexpr int kGroups = 2;                       // expander groups taking alternate k-blocks
 constexpr int kNumExpWarps = 4 * kGroups;
-// Codes out on resident weights: a chunk is some 250 instructions, most of them waiting for the one in front, and its bytes are few:
-// more warps, with one set of registers each (192x32 on 200,704 pixels 25.5 us with twelve, 23.9 so).  Through the rings a tile takes longer and
-// more warps that wait for it are in its way, unless the codes have to leave one by one: 160x192 3x3 on 64 images of 28x28 43.4 us with nineteen,
-// 36.7 with eleven, 768x3072 N=4096 13.3 and 11.8, 32x32 7x7 of step two on 145 of 11x11 19.5 and 16.1, 64x32 7x7 on 64 of 28x28 41.5 and 42.7; but
-// 332x384 3x3 on 234 of 7x7 19.0 and 22.8.
+// Codes out: a chunk is some 250 instructions, most of them waiting for the one in front, and its bytes are few: many warps, with one
+// set of registers each, where nothing else bounds the tile (plan(): tiles of one k-block on resident weights, four rounds of them and
+// more: 192x32 on 200,704 pixels 23.8 us with twenty, 24.2 with twelve, 512x64 on 50,000 16.6 and 16.9) or where the codes have to leave one by one
+// (332x384 3x3 on 234 images of 7x7 19.0 and 22.8).  Elsewhere warps that wait for a tile are in the way of its copies and products: 128x64 3x3 of
+// step two on 256 of 56x56 26.7 with twenty, 23.5 with twelve, 288x288 1x1 of step two on 36 of 72x72 18.4 and 15.8, 64x64 1x1 on 2 of 96x96 4.9 and 4.5;
+// through the rings 160x192 3x3 on 64 of 28x28 43.4 with nineteen, 36.7 with eleven, 768x3072 N=4096 13.3 and 11.8, 32x32 7x7 of step two on 145 of
+// 11x11 19.5 and 16.1, 64x32 7x7 on 64 of 28x28 41.5 and 42.7.
 constexpr int kRqWarps = 22;
 __host__ __device__ constexpr int warps_of(int mode, bool many) { return mode ? (many ? kRqWarps : kPreWarps) : 2 + kNumExpWarps + kNumEpiWarps; }
 constexpr int kWarpStage = 32 * 32 * 4;          // 4 KB: 32 pixels x 32 rows of fp32/int32
@@ -1070,7 +1072,8 @@ bool plan(const Problem& p, TensorCfg& c)
         c.dup = (p.M <= 64) ? 1 : 0;
         if (resident) {
             c.ares = 1;
-            c.epi_warps = wide ? (p.rq_codes ? 2 * kWideEpi : kWideEpi) : warps_of(2, p.rq_codes) - 2;
+            const bool many = p.rq_codes && (!c.tma_store || (c.nkb == 1 && c.ntiles >= 4 * (int64_t)p.sms));
+            c.epi_warps = wide ? (p.rq_codes ? 2 * kWideEpi : kWideEpi) : warps_of(2, many) - 2;
             c.nA = c.nkb;
             const int64_t left = kSmemLimit - (1024 + 64 * kMaxRing) - (int64_t)c.nkb * c.a_bytes -
                                  (int64_t)c.epi_warps * stage;

@@ -1429,8 +1429,11 @@ def test_patch_matrix_of_three_channels_and_many_rows(k, stride, pad, B, H, W, o
     (68, 96, 5, 1, 9, 17),         # codes one by one
     (20, 144, 3, 1, 30, 15),       # the same with duplicated rows
     (332, 384, 3, 1, 70, 7),
+    (288, 288, 1, 2, 21, 50),      # resident weights of five k-blocks
+    (144, 32, 1, 1, 75, 32),       # of one, and four rounds of tiles
+    (148, 32, 1, 1, 75, 32),       # the same one by one
 ])
-def test_requantized_codes_of_long_tiles(M, Cin, k, stride, B, H):
+def test_requantized_codes_of_long_and_of_short_tiles(M, Cin, k, stride, B, H):
     import torch
     g = synth.rng(147, M + Cin)
     Wt = synth.weights_kaiming(g, M, Cin, k, k)
