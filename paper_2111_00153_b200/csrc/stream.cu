@@ -466,15 +466,14 @@ stream_kernel(const uint8_t* __restrict__ table)
                 last_status = v.P->status;
                 const int nst = (int)same((uint32_t)v.nst), nkb = (int)same((uint32_t)v.nkb), kind = (int)same((uint32_t)v.kind);
                 const uint32_t ab = n & (buffers - 1u), lap = n >> (buffers == 4u ? 2 : 1);      // nAcc is 2 or 4
-                bool have_acc = false;                    // this issuer has made sure the item's accumulator buffer is free
+                // The buffer's previous item is out, and with it everybody's report on that one in.  Every issuer waits, whether or not a
+                // stage of the item is its own: with two buffers and four issuers one that had none in two items could
+                // otherwise be two of a buffer's phases ahead of the epilogue, which a parity does not tell from none.
+                if (!mbar_wait_parked_step(bar_tempty + 8 * ab, (lap & 1) ^ 1, abort_flag)) break;
                 // its own stages only: those whose index over the whole list is me modulo nch (1, 2 or 4); the A stage
                 // advances by nch with them (nch <= nAst)
                 for (int st = (int)(((uint32_t)me - t) & (chains - 1u)); st < nst; st += (int)chains) {
                     {
-                        if (!have_acc) {
-                            if (!mbar_wait_parked_step(bar_tempty + 8 * ab, (lap & 1) ^ 1, abort_flag)) { ok = false; break; }
-                            have_acc = true;
-                        }
                         if (!mbar_wait_parked_step(bar_fullB + 8 * sa, phA, abort_flag) || !mbar_wait_parked_step(bar_fullA + 8 * sa, phA, abort_flag)) { ok = false; break; }
                         tc_fence_after();
                         {
@@ -500,11 +499,7 @@ stream_kernel(const uint8_t* __restrict__ table)
                 }
                 t += (uint32_t)nst;
                 if (!ok) break;
-                // Every issuer reports once per item, whether or not a stage of it was its own.  An issuer without
-                // stages in short items can be items ahead of the others: before it reports on this buffer again
-                // it makes sure that the buffer's previous item has everybody's report (one arrival per phase).
-                if (lap >= 1 && !mbar_wait_parked_step(bar_tfull + 8 * ab, (lap - 1) & 1, abort_flag)) break;
-                mma_commit_step(bar_tfull + 8 * ab);
+                mma_commit_step(bar_tfull + 8 * ab);       // every issuer reports once per item, whether or not a stage of it was its own
             }
         }
     } else if (warp < kFirstEpi) {

@@ -344,22 +344,40 @@ def test_grouped_tensor_launch_ring_of_packed_codes(N):
     assert slots % 2 == 0 or (chains == 1 and slots >= a_stages + 2)
 
 
+def _several_times(shapes, N, times):
+    """A grouped case whose layers are in the launch `times` times each, into outputs of their own."""
+    import torch
+    keep, items, refs = _grouped_case(shapes, N)
+    all_keep, all_items, all_refs = [], [], []
+    for rep in range(times):
+        for (layer, d_packed, a, n, ld, step, y, M, acc, nonneg), ref in zip(items, refs):
+            y2 = torch.full_like(y, float("nan"))
+            acc2 = torch.full_like(y, -5, dtype=torch.int32) if rep % 4 == 0 else None
+            all_keep.append((layer, d_packed, a, y2, acc2))
+            all_items.append((layer, d_packed, a, n, ld, step, y2, M, acc2, nonneg))
+            all_refs.append(ref)
+    return all_keep, all_items, all_refs
+
+
 @pytest.mark.parametrize("N", [24, 40, 56, 80, 104])
 def test_grouped_tensor_launch_lists_of_several_laps(N):
     """Every CTA has several items, long and short ones in turn, of all kinds and an odd number of k-blocks: its stages are several laps
-    of the ring (sixteen, four and three stages an item).  Each layer is in the launch more than once, into outputs of its own."""
-    import torch
-    keep, items, refs = _grouped_case([(1024, 4096), (1000, 1024), (300, 640)], N)
-    all_keep, all_items, all_refs = [], [], []
-    for rep, (k, (layer, d_packed, a, n, ld, step, y, M, acc, nonneg), ref) in [(r, z) for r in range(20) for z in zip(keep, items, refs)]:
-        y2 = torch.full_like(y, float("nan"))
-        acc2 = torch.full_like(y, -5, dtype=torch.int32) if rep % 4 == 0 else None
-        all_keep.append((layer, d_packed, a, y2, acc2))
-        all_items.append((layer, d_packed, a, n, ld, step, y2, M, acc2, nonneg))
-        all_refs.append(ref)
-    header = _launch_grouped(all_items)[:128].cpu().numpy().view(np.int32)
+    of the ring (sixteen, four and three stages an item)."""
+    keep, items, refs = _several_times([(1024, 4096), (1000, 1024), (300, 640)], N, 20)
+    header = _launch_grouped(items)[:128].cpu().numpy().view(np.int32)
     assert header[2] > 2 * header[3]                       # items, CTAs
-    _check_grouped(all_keep, all_refs)
+    _check_grouped(keep, refs)
+
+
+@pytest.mark.parametrize("times", [60, 900])
+@pytest.mark.parametrize("N", [4, 17, 32, 48, 128])
+def test_grouped_tensor_launch_lists_of_short_items(N, times):
+    """Items of one and two stages: an issuer has no stage in most of them, and the epilogue is what takes the time.  At 17 to 32 tokens four
+    issuers share two accumulator buffers.  (The longer lists do not fit into shared memory.)"""
+    keep, items, refs = _several_times([(512, 256), (300, 512), (384, 128)], N, times)
+    header = _launch_grouped(items)[:128].cpu().numpy().view(np.int32)
+    assert header[2] > (5 if times == 60 else 64) * header[3]
+    _check_grouped(keep, refs)
 
 
 def test_grouped_tensor_launch_mn_layout_and_single_layer():
