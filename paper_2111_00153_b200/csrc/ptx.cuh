@@ -182,22 +182,7 @@ __device__ __forceinline__ uint64_t smem_desc_kmajor(uint32_t addr, int row_byte
     d |= (uint64_t)(row_bytes == 128 ? 2 : 4) << 61;     // 128-byte / 64-byte swizzle
     return d;
 }
-// One MMA, the descriptors given as 32-bit halves.  The MMA thread runs alone at a few cycles
-// per instruction, and its per-k-block instruction count shows directly in the kernel time, so
-// it keeps only the low words (address field) moving and leaves the high words constant.
-__device__ __forceinline__ void mma_i8_halves(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
-                                              uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "mov.b64 da, {%1, %3};\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %4, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// The MMAs of a warp in step: all lanes take part, the elected one issues.  What a warp can issue is what bounds tiles of fewer
+// The MMAs of a warp in step, the descriptors given as 32-bit halves of which the low one moves: all lanes take part, the elected one issues.  What a warp can issue is what bounds tiles of fewer
 // than 256 columns: measured with one wait and one commit to every four MMAs, lane 0 in a branch of its own takes 124 cycles an
 // MMA whatever its size; each MMA behind an election of its own 101; four behind one election 63 to 69 up to 128 columns
 // and, from 160, the N / 2 that the tensor pipe takes.  (The branch, and a flag in a register as the predicate, leave the compiler in
@@ -258,11 +243,6 @@ __device__ __forceinline__ void mma_commit_step(uint32_t bar)
 {
     asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
                  "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
 }
 // Issue a 32-column accumulator load; the registers are valid only after tmem_ld_wait(v).
 __device__ __forceinline__ void tmem_ld_issue(uint32_t taddr, uint32_t (&v)[32])

@@ -72,7 +72,7 @@ constexpr int kAStageCols = 64;                                       // 256 cod
 constexpr int kMaxTokens = 128;                                       // accumulator columns of one chain at most
 constexpr int kRingMax = 12;
 constexpr int kStreamMaxK = 16384;                                    // reduction length up to which the fp32 sums of PoT tiles are exact
-constexpr int kLocalItems = 64;                                        // items of a CTA's list kept in shared memory
+constexpr int kLocalItems = 64;                                        // items of a CTA's list kept in shared memory (with 96, lists of 89 took 1 % less)
 constexpr int kStreamSmem = 232448 - 64 - kLocalItems * 16;            // (for 128 tokens just enough for six slots of packed codes)
 constexpr uint32_t kPlanMagic = 0x53545247u;                          // "STRG"
 
@@ -111,12 +111,12 @@ struct StreamHeader {               // first 128 bytes of the table
     int32_t n_pad, nS, nch, nB;               // tokens rounded up to 16, slots of the packed-code ring, accumulator chains (1, 2 or 4), slots of the activation ring
     uint32_t stage_bytes, b_bytes, idesc, smem_bytes;   // one slot of the packed-code ring / of the activation ring
     int32_t acc_cols, nAst;                   // tensor memory: columns of one accumulator buffer (nch * n_pad); A stages behind the two buffers
-    uint32_t off_first, off_items, off_probs, bytes;
+    uint32_t off_probs, bytes;
     uint32_t idesc_fp;                        // instruction descriptor of PoT tiles (E3M2 x E4M3 -> fp32)
     uint32_t off_act, n_fp;                   // scratch of the E4M3 activation copies; layers that have one
     uint32_t conv_grid_x;                     // blocks per layer of the kernel that writes them
     int32_t nAcc;                             // accumulator buffers in tensor memory (2 or 4): items in flight between issuers and epilogue
-    uint32_t pad[9];
+    uint32_t pad[11];
 };
 static_assert(sizeof(StreamHeader) == 128, "header is 128 bytes");
 // Behind it: the first item of every CTA's list (and the end of the last one's), then the lists.
@@ -473,27 +473,23 @@ stream_kernel(const uint8_t* __restrict__ table)
                 // its own stages only: those whose index over the whole list is me modulo nch (1, 2 or 4); the A stage
                 // advances by nch with them (nch <= nAst)
                 for (int st = (int)(((uint32_t)me - t) & (chains - 1u)); st < nst; st += (int)chains) {
-                    {
-                        if (!mbar_wait_parked_step(bar_fullB + 8 * sa, phA, abort_flag) || !mbar_wait_parked_step(bar_fullA + 8 * sa, phA, abort_flag)) { ok = false; break; }
-                        tc_fence_after();
-                        {
-                            const uint32_t chain = (uint32_t)st & (chains - 1u);
-                            const uint32_t d_tmem = tmem + ab * buffer_cols + chain * chain_cols;
-                            const uint32_t a_t = acc_base + sa * kAStageCols, b_lo = b_lo0 + sa * b_step;
-                            // a 32-code step is 8 columns of A and 32 bytes (two 16-byte units) of a B row; the first
-                            // instruction into a chain in this item overwrites it
-                            const bool both = 2 * st + 1 < nkb;             // (an odd number of k-blocks: the last stage has one)
-                            const uint32_t first = st < (int)chains ? 0u : 1u, b_lo2 = b_lo + b_half;
-                            if (kind == kPoT4) {
-                                mma_tmem_a_step<true>(d_tmem, a_t, b_lo, desc_hi, desc_fp, first);
-                                if (both) mma_tmem_a_step<true>(d_tmem, a_t + 32, b_lo2, desc_hi, desc_fp, 1u);
-                            } else {
-                                mma_tmem_a_step<false>(d_tmem, a_t, b_lo, desc_hi, desc_i8, first);
-                                if (both) mma_tmem_a_step<false>(d_tmem, a_t + 32, b_lo2, desc_hi, desc_i8, 1u);
-                            }
-                            mma_commit_step(bar_emptyA + 8 * sa);
-                        }
+                    if (!mbar_wait_parked_step(bar_fullB + 8 * sa, phA, abort_flag) || !mbar_wait_parked_step(bar_fullA + 8 * sa, phA, abort_flag)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t chain = (uint32_t)st & (chains - 1u);
+                    const uint32_t d_tmem = tmem + ab * buffer_cols + chain * chain_cols;
+                    const uint32_t a_t = acc_base + sa * kAStageCols, b_lo = b_lo0 + sa * b_step;
+                    // a 32-code step is 8 columns of A and 32 bytes (two 16-byte units) of a B row; the first
+                    // instruction into a chain in this item overwrites it
+                    const bool both = 2 * st + 1 < nkb;             // (an odd number of k-blocks: the last stage has one)
+                    const uint32_t first = st < (int)chains ? 0u : 1u, b_lo2 = b_lo + b_half;
+                    if (kind == kPoT4) {
+                        mma_tmem_a_step<true>(d_tmem, a_t, b_lo, desc_hi, desc_fp, first);
+                        if (both) mma_tmem_a_step<true>(d_tmem, a_t + 32, b_lo2, desc_hi, desc_fp, 1u);
+                    } else {
+                        mma_tmem_a_step<false>(d_tmem, a_t, b_lo, desc_hi, desc_i8, first);
+                        if (both) mma_tmem_a_step<false>(d_tmem, a_t + 32, b_lo2, desc_hi, desc_i8, 1u);
                     }
+                    mma_commit_step(bar_emptyA + 8 * sa);
                     sa += chains;
                     if (sa >= stages) { sa -= stages; phA ^= 1; }
                 }
@@ -817,8 +813,7 @@ bool stream_build_table(const Problem* probs, int count, int sms, uint8_t* h_tab
     H->idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(H->n_pad >> 3) << 17) | ((uint32_t)(kBlockRows >> 4) << 24);
     // kind::f8f6f4: fp32 accumulate (1 at bit 4), A = E3M2 (4 at bit 7), B = E4M3 (0 at bit 10)
     H->idesc_fp = (1u << 4) | (4u << 7) | (0u << 10) | ((uint32_t)(H->n_pad >> 3) << 17) | ((uint32_t)(kBlockRows >> 4) << 24);
-    H->off_first = (uint32_t)L.off_first; H->off_items = (uint32_t)L.off_items; H->off_probs = (uint32_t)L.off_probs;
-    H->bytes = (uint32_t)L.bytes;
+    H->off_probs = (uint32_t)L.off_probs; H->bytes = (uint32_t)L.bytes;
     H->off_act = (uint32_t)L.off_act;
 
     // problems and their tensor maps

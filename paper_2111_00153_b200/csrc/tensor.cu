@@ -15,10 +15,10 @@
 //               index, so accumulator lanes are in original row order and the output needs no
 //               scatter through the permutation.
 //   last four   epilogue, one per tensor-memory quarter (in workspace mode the expander warps
-//               have nothing to expand and join the epilogue, three warps per quarter): tcgen05.ld (next chunk in flight while
-//               the current one is processed), undo the x16 of Fixed-4 rows, convert, scale by
-//               wstep*act_step, stage 32 pixels x 32 rows in a private double buffer and write it
-//               with a bulk tensor store.
+//               have nothing to expand and join the epilogue, about three warps per quarter, five where codes leave; see
+//               warps_of): tcgen05.ld (of fp32 outputs the next chunk is in flight while the current one is processed), undo the x16 of
+//               Fixed-4 rows, convert, scale by wstep*act_step, stage 32 pixels x 32 rows in buffers of the warp's own and write them
+//               with a bulk tensor store (codes: sixteen bytes a store).
 // Every wait on an mbarrier is bounded; when one runs out the kernel records
 // RMSMP_ERR_TIMEOUT in the packed buffer's status word, all roles leave their loops, tensor
 // memory is freed and the kernel returns.
@@ -411,18 +411,16 @@ tensor_kernel(const Problem p, const TensorCfg cfg, const __grid_constant__ Maps
                     for (int kb = 0; kb < cfg.nkb; kb += 3) {
                         if (!mbar_wait_step(bar_fullB + 8 * sb, phB, abort_flag)) { ok = false; break; }
                         tc_fence_after();
-                        {
-                            if (two) {
-                                mma_i8_step<2>(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
-                                mma_i8_step<2>(d_tmem, a_lo + a_t, b_lo + t_step, desc_hi, cfg.idesc, 1u);
-                                mma_i8_step<2>(d_tmem, a_lo + 2 * a_t, b_lo + 2 * t_step, desc_hi, cfg.idesc, 1u);
-                            } else {
-                                mma_i8_step<1>(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
-                                mma_i8_step<1>(d_tmem, a_lo + a_t, b_lo + t_step, desc_hi, cfg.idesc, 1u);
-                                mma_i8_step<1>(d_tmem, a_lo + 2 * a_t, b_lo + 2 * t_step, desc_hi, cfg.idesc, 1u);
-                            }
-                            mma_commit_step(bar_emptyB + 8 * sb);
+                        if (two) {
+                            mma_i8_step<2>(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
+                            mma_i8_step<2>(d_tmem, a_lo + a_t, b_lo + t_step, desc_hi, cfg.idesc, 1u);
+                            mma_i8_step<2>(d_tmem, a_lo + 2 * a_t, b_lo + 2 * t_step, desc_hi, cfg.idesc, 1u);
+                        } else {
+                            mma_i8_step<1>(d_tmem, a_lo, b_lo, desc_hi, cfg.idesc, kb ? 1u : 0u);
+                            mma_i8_step<1>(d_tmem, a_lo + a_t, b_lo + t_step, desc_hi, cfg.idesc, 1u);
+                            mma_i8_step<1>(d_tmem, a_lo + 2 * a_t, b_lo + 2 * t_step, desc_hi, cfg.idesc, 1u);
                         }
+                        mma_commit_step(bar_emptyB + 8 * sb);
                         a_lo += a_adv;
                         b_lo += b_step;
                         if (cfg.cpt > 1) two = !two || two_last;

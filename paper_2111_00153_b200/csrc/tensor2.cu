@@ -40,7 +40,6 @@ constexpr int kRing2 = 3;                       // stages; a stage holds TWO k-b
 constexpr int kSub2 = 2;
 constexpr int kPairSmem = 232448 - 1024;         // 227 KB per CTA less room for the static variables
 constexpr int kPairRest = kEpiWarps2 * kWarpStage2 + 1024 + 64 * 2 * kRing2;      // all but the stages
-constexpr long long kWaitCycles2 = 2000000000LL;
 
 struct PairCfg {
     int tb, th;              // images / output rows per half
@@ -68,7 +67,6 @@ struct PairMaps {
     CUtensorMap act[4], wexp, out_full, out_tail;      // act: one map, or one per parity sub-grid (stride 2)
 };
 
-__device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t cluster_rank()
 {
     uint32_t r;
@@ -87,54 +85,10 @@ __device__ __forceinline__ void cluster_sync_all()
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
 // arrivals on a barrier given by its shared::cluster address (own or peer CTA)
 __device__ __forceinline__ void bar_arrive_cluster(uint32_t cbar)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cbar) : "memory");
-}
-__device__ __forceinline__ bool bar_try_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag)
-{
-    if (bar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 64; ++i)
-            if (bar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > kWaitCycles2) { *abort_flag = 1; return false; }
-    }
-}
-// (a warp that walks its loop in step: the verdict is a vote)
-__device__ __forceinline__ bool bar_wait_step(uint32_t bar, uint32_t parity, volatile int* abort_flag)
-{
-    if (__all_sync(0xffffffffu, bar_try_wait(bar, parity))) return true;
-    const long long t0 = clock64();
-    for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 64; ++i)
-            if (__all_sync(0xffffffffu, bar_try_wait(bar, parity))) return true;
-        if (__any_sync(0xffffffffu, *abort_flag != 0 || clock64() - t0 > kWaitCycles2)) { *abort_flag = 1; return false; }
-    }
-}
-__device__ __forceinline__ bool bar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
-{
-    bool ok = true;
-    if ((threadIdx.x & 31) == 0) ok = bar_wait(bar, parity, abort_flag);
-    return __all_sync(0xffffffffu, ok);
 }
 // TMA loads of a CTA pair: data into this CTA's shared memory, completion on a barrier that may
 // live in the peer CTA (cta_group::2 form; no multicast).
@@ -150,39 +104,12 @@ __device__ __forceinline__ void pair_load_2d(uint32_t dst, const CUtensorMap* ma
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(dst), "l"(map), "r"(cbar), "r"(c0), "r"(c1) : "memory");
 }
-__device__ __forceinline__ void store_2d(const CUtensorMap* map, uint32_t src, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
-                 ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
 // Arrive (once all MMAs issued so far have finished) on the barrier at this shared-memory offset in BOTH CTAs.
 __device__ __forceinline__ void pair_commit(uint32_t bar)
 {
     asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
                  "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
                  ::"r"(bar), "h"((uint16_t)3) : "memory");
-}
-__device__ __forceinline__ void ld_issue(uint32_t taddr, uint32_t (&v)[32])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void ld_wait(uint32_t (&v)[32])
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
-                   "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
-                   "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
-                 :: "memory");
 }
 
 // First pixel and geometry of half `hf` (global half index): image / row coordinates for the TMA
@@ -209,7 +136,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
 pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps maps)
 {
     extern __shared__ uint8_t smem_raw[];
-    const uint32_t smem_base = (s32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sA = smem_base;
     const int ring = kShift ? cfg.ring : kRing2;
     const uint32_t a_stage = kShift ? 3 * kStageA : kSub2 * kStageA, b_stage = kShift ? (uint32_t)cfg.b_stage : kSub2 * kStageB;
@@ -226,25 +153,25 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kRing2; ++s) {               // (a ring has no more stages than that)
-            bar_init(bar_full + 8 * s, 1);       // the leader's activation producer announces all four copies' bytes; leader only
-            bar_init(bar_empty + 8 * s, 1);      // the leader's commit, delivered to both CTAs
+            mbar_init(bar_full + 8 * s, 1);       // the leader's activation producer announces all four copies' bytes; leader only
+            mbar_init(bar_empty + 8 * s, 1);      // the leader's commit, delivered to both CTAs
         }
         for (int b = 0; b < 2; ++b) {
-            bar_init(bar_tfull + 8 * b, 1);                    // the leader's commit, delivered to both CTAs
-            bar_init(bar_tempty + 8 * b, 2 * kEpiWarps2);      // every epilogue warp of both CTAs; used in the leader only
+            mbar_init(bar_tfull + 8 * b, 1);                    // the leader's commit, delivered to both CTAs
+            mbar_init(bar_tempty + 8 * b, 2 * kEpiWarps2);      // every epilogue warp of both CTAs; used in the leader only
         }
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
         // one warp of EACH CTA of the pair takes part in the allocation
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s32(&s_tmem_base)) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem_base)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
     cluster_sync_all();                                   // both CTAs' barriers exist before anyone signals the peer
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc_fence_after();
     // Every role waits for the kernel in front by itself: before its first access to weights, activations or outputs, and before
     // its first wait for another role.  No trigger: see launch_dependent.
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
@@ -269,7 +196,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 const HalfPos hp = half_pos(p, cfg, 2 * nt + rank);
                 int cc = 0, tj = 0;
                 for (int st = 0; st < 3 * cfg.cpt; ++st) {
-                    if (!bar_wait(bar_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
+                    if (!mbar_wait(bar_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
                     const uint32_t fb = lead_full + 8 * s;
                     if (warp == 0) {
                         if (rank == 0)
@@ -306,7 +233,7 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 const int nsub = min(kSub2, cfg.nkb - kb);
                 const bool skip = (g & 1u) != mine;
                 if (!skip) {
-                    if (!bar_wait(bar_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
+                    if (!mbar_wait(bar_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
                     // all copies of this stage (up to two k-blocks of two operands in two CTAs) complete on the leader's barrier
                     if (is_b && rank == 0)
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
@@ -342,22 +269,20 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
             pdl_wait();                                                                // (a bounded wait begins when the kernel in front is over)
             for (int64_t tile = first; tile < cfg.ntiles; tile += step, ++it) {
                 const uint32_t ab = it & 1;
-                if (!bar_wait_step(bar_tempty + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (!mbar_wait_step(bar_tempty + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag)) break;
+                tc_fence_after();
                 const uint32_t d_tmem = tmem_base + ab * 256;
                 bool ok = true;
                 for (int kb = 0; kb < cfg.nkb; kb += kShift ? 3 : kSub2) {
-                    if (!bar_wait_step(bar_full + 8 * s, ph, abort_flag)) { ok = false; break; }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    if (!mbar_wait_step(bar_full + 8 * s, ph, abort_flag)) { ok = false; break; }
+                    tc_fence_after();
                     if (kShift) {
-                        {
 #pragma unroll
-                            for (int i = 0; i < 3; ++i) {
-                                const uint32_t a1 = a_lo + i * (kStageA >> 4), b1 = b_lo + i * row_step;
-                                mma_i8_pair_step(d_tmem, a1, b1, hi, cfg.idesc, (kb | i) ? 1u : 0u);
-                            }
-                            pair_commit(bar_empty + 8 * s);
+                        for (int i = 0; i < 3; ++i) {
+                            const uint32_t a1 = a_lo + i * (kStageA >> 4), b1 = b_lo + i * row_step;
+                            mma_i8_pair_step(d_tmem, a1, b1, hi, cfg.idesc, (kb | i) ? 1u : 0u);
                         }
+                        pair_commit(bar_empty + 8 * s);
                     } else {
                         mma_i8_pair_step(d_tmem, a_lo, b_lo, hi, cfg.idesc, kb ? 1u : 0u);
                         if (kb + 1 < cfg.nkb) mma_i8_pair_step(d_tmem, a_lo + (kStageA >> 4), b_lo + (kStageB >> 4), hi, cfg.idesc, 1u);
@@ -397,8 +322,8 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 n0h[h] = hp.n0;
                 nvalid[h] = (int)max((int64_t)0, min((int64_t)cfg.npix_h, p.N - hp.n0));
             }
-            if (!bar_wait_warp(bar_tfull + 8 * ab, (it >> 1) & 1, abort_flag)) { alive = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (!mbar_wait_warp(bar_tfull + 8 * ab, (it >> 1) & 1, abort_flag)) { alive = false; break; }
+            tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + ab * 256;
             const bool rows_ok = blk * kBlockRows + quarter * 32 < p.M;
             // chunk index i = (h * runs + e) * nch + c; this warp takes i = my_rank, my_rank + cstride, ...
@@ -408,8 +333,8 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                 const int h = i >= per_half, u = i - h * per_half, e = kShift ? u / nch : 0, c = u - e * nch;
                 const int at = e * cfg.img_pix + c * 32;                 // the chunk's first pixel in its half
                 if (!rows_ok || at >= nvalid[h]) continue;
-                ld_issue(taddr + h * cfg.nh_pad + e * cfg.img_cols + c * 32, v);
-                ld_wait(v);
+                tmem_ld_issue(taddr + h * cfg.nh_pad + e * cfg.img_cols + c * 32, v);
+                tmem_ld_wait(v);
                 if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 __syncwarp();
                 const uint32_t a0 = my_stage + lane * 4;
@@ -418,15 +343,15 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
                     const uint32_t w = __float_as_uint(__fmul_rn(__int2float_rn((int)v[j]), scale));
                     asm volatile("st.shared.b32 [%0], %1;" ::"r"(a0 + j * 128), "r"(w) : "memory");
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
                     const bool tail = cfg.tail_rows && (c == (cfg.img_pix >> 5));
-                    store_2d(tail ? &maps.out_tail : &maps.out_full, my_stage, blk * kBlockRows + quarter * 32, (int)(n0h[h] + at));
+                    tma_store_2d(tail ? &maps.out_tail : &maps.out_full, my_stage, blk * kBlockRows + quarter * 32, (int)(n0h[h] + at));
                 }
             }
             // accumulators of this tile are out of tensor memory: tell the leader
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            tc_fence_before();
             __syncwarp();
             if (lane == 0) bar_arrive_cluster(lead_tempty + 8 * ab);
         }
@@ -434,11 +359,11 @@ pair_kernel(const Problem p, const PairCfg cfg, const __grid_constant__ PairMaps
     }
 
     // ---------------------------------------------------------- teardown
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
     cluster_sync_all();                                   // nobody signals a CTA that has left
     if (warp == 1) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
     }
     if (threadIdx.x == 0 && s_abort) atomicMax(p.status, (uint32_t)RMSMP_ERR_TIMEOUT);

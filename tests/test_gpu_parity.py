@@ -1264,6 +1264,23 @@ def test_column_shift_stages_of_any_width(M, Cin, B, H, W):
         _check_some_images(Wt, scheme, bits, alpha, act, 1, 1, y, acc, images)
 
 
+@pytest.mark.parametrize("want_acc", [True, False])
+@pytest.mark.parametrize("M,Cin,B,H,W", [
+    (128, 80, 150, 29, 9),        # the output turned in shared memory
+    (20, 128, 150, 29, 9),
+    (128, 128, 300, 16, 16),      # by bulk stores
+])
+def test_wide_column_shift_stages_into_rows_of_pixels(M, Cin, B, H, W, want_acc):
+    g = synth.rng(148, M + Cin + W)
+    Wt = synth.weights_kaiming(g, M, Cin, 3, 3)
+    scheme, bits = _mixed_map(M, 13, (50, 30, 20))
+    alpha = synth.alpha_rows(Wt)
+    layer, d_packed = Hn.pack_layer(Wt, scheme, bits, alpha)
+    act = g.integers(-16, 17, size=(B, H, W, Cin)).astype(np.int8)
+    y, acc = Hn.conv(layer, d_packed, act, 1, 1, 0.25, Hn.WORKSPACE, R.OUT_MN, want_acc=want_acc)
+    _check_some_images(Wt, scheme, bits, alpha, act, 1, 1, y, acc, sorted({0, 1, B // 2, B - 1}))
+
+
 @pytest.mark.parametrize("Cin,B,H,W", [
     (256, 387, 7, 7),             # two images a half with staged rows between them, the last half has one
     (256, 200, 11, 13),           # halves of six rows, the last of an image repeats one
