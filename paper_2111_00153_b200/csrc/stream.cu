@@ -466,13 +466,16 @@ stream_kernel(const uint8_t* __restrict__ table)
                 last_status = v.P->status;
                 const int nst = (int)same((uint32_t)v.nst), nkb = (int)same((uint32_t)v.nkb), kind = (int)same((uint32_t)v.kind);
                 const uint32_t ab = n & (buffers - 1u), lap = n >> (buffers == 4u ? 2 : 1);      // nAcc is 2 or 4
-                // The buffer's previous item is out, and with it everybody's report on that one in.  Every issuer waits, whether or not a
-                // stage of the item is its own: with two buffers and four issuers one that had none in two items could
-                // otherwise be two of a buffer's phases ahead of the epilogue, which a parity does not tell from none.
-                if (!mbar_wait_parked_step(bar_tempty + 8 * ab, (lap & 1) ^ 1, abort_flag)) break;
+                // Every issuer waits for the buffer's previous item to be out (and everybody's report on it is in then), before its first
+                // stage of the item or, if none is its own, before it reports: with two buffers and four issuers one that had no stage in
+                // two items could otherwise be two of a buffer's phases ahead of the epilogue, which a parity does not tell from none.
+                // (Before it looks at the item's stages: one token 0.3 us more.)
+                auto buffer_free = [&]() { return mbar_wait_parked_step(bar_tempty + 8 * ab, (lap & 1) ^ 1, abort_flag); };
+                bool have_acc = false;
                 // its own stages only: those whose index over the whole list is me modulo nch (1, 2 or 4); the A stage
                 // advances by nch with them (nch <= nAst)
                 for (int st = (int)(((uint32_t)me - t) & (chains - 1u)); st < nst; st += (int)chains) {
+                    if (!have_acc && !(have_acc = buffer_free())) { ok = false; break; }
                     if (!mbar_wait_parked_step(bar_fullB + 8 * sa, phA, abort_flag) || !mbar_wait_parked_step(bar_fullA + 8 * sa, phA, abort_flag)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t chain = (uint32_t)st & (chains - 1u);
@@ -494,7 +497,7 @@ stream_kernel(const uint8_t* __restrict__ table)
                     if (sa >= stages) { sa -= stages; phA ^= 1; }
                 }
                 t += (uint32_t)nst;
-                if (!ok) break;
+                if (!ok || (!have_acc && !buffer_free())) break;
                 mma_commit_step(bar_tfull + 8 * ab);       // every issuer reports once per item, whether or not a stage of it was its own
             }
         }
