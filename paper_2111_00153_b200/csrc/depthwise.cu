@@ -361,15 +361,16 @@ cudaError_t launch_depthwise(const Problem& p, cudaStream_t st)
         const int64_t sms = sm_count();
         if (blocks > sms) blocks = (blocks + sms - 1) / sms * sms;
     }
+    const int64_t rounds = (blocks + cap - 1) / cap;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     // Tall strips through the ring, where as many blocks fit beside each other with it; of stride two, whose rows are nine words, where a
-    // quarter of a block's threads has no item.  (Launches back to back, registers against ring: 576 channels, 64 images of 14 x 14, strips of 14
+    // quarter of a block's threads has no item and a thread with one walks seven rows and more.  (Launches back to back, registers against ring: 576 channels, 64 images of 14 x 14, strips of 14
     // rows 24.8 us and 21.2; 192, 64 of 56 x 56, 19 rows 48.4 and 44.9; 192, 64 of 28 x 28, 10 rows 17.0 and 16.6; 384, 64 of 14 x 14, 7 rows 14.8
     // and 14.7; 960, 64 of 7 x 7, 4 rows 20.2 and 20.7; 144, 8 of 56 x 56, 4 rows 9.4 and 10.2.  With sums 192, 64 of 56 x 56 72.7 and 76.2.  Stride two:
-    // 576, 64 of 28 x 28, 14 rows, 144 threads 34.5 and 28.9; 384, 64 of 28 x 28, 7 rows, 192 threads 21.4 and 20.4; 576, 64 of 14 x 14, 4 rows 17.1 and 17.6;
-    // 192, 64 of 56 x 56, 10 rows, 240 threads 25.3 and 26.4.)
-    const bool tall = variant == 1 ? strip >= 10 : variant == 2 && strip >= 7 && 4 * ipg * std::min(quads, kDwThreads) <= 3 * kDwThreads;
+    // 576, 64 of 28 x 28, 14 rows, 144 threads 34.5 and 28.9; 384, 64 of 28 x 28, 7 rows, 192 threads 21.4 and 20.4; 576, 64 of 14 x 14, 4 rows 17.1 and 17.6,
+    // 43 of 30 x 30, 5 rows twice 29.5 and 25.8; 516, 9 of 43 x 43, 6 rows 17.1 and 17.8; 192, 64 of 56 x 56, 10 rows, 240 threads 25.3 and 26.4.)
+    const bool tall = variant == 1 ? strip >= 10 : variant == 2 && strip * rounds >= 7 && 4 * ipg * std::min(quads, kDwThreads) <= 3 * kDwThreads;
     if (tall && !acc && with_ring <= kDwSmem && (with_ring + 1024) * (size_t)per_sm <= 228 * 1024) {
         const Kernel ringed = variant == 1 ? depthwise_kernel<1, false, true> : depthwise_kernel<2, false, true>;
         if (with_ring > 48 * 1024 && !ensure_smem_attr(reinterpret_cast<const void*>(ringed), (int)kDwSmem, attr_set[2 + variant][0])) return cudaErrorUnknown;

@@ -1392,6 +1392,8 @@ def test_depthwise_threads_that_take_several_strips(stride, B):
     (22260, 11, 1, 100, 1, False), (22300, 11, 1, 100, 1, False), (22340, 11, 1, 100, 1, False), (22416, 11, 1, 100, 1, False),      # the last tables with room, and the next
     (528, 14, 1, 464, 2, False),        # of stride two, two strips for some threads
     (516, 13, 4, 488, 2, False),
+    (576, 30, 30, 43, 2, False),        # five rows twice, and six once
+    (516, 43, 43, 9, 2, False),
     (20604, 13, 1, 40, 2, False), (18000, 13, 1, 100, 2, False),      # most threads have an item: registers
     (22752, 5, 3, 1, 1, True), (22752, 5, 4, 2, 2, False), (20604, 5, 3, 2, 2, False), (22752, 5, 3, 1, 2, True),
 ])
