@@ -807,8 +807,8 @@ bool stream_build_table(const Problem* probs, int count, int sms, uint8_t* h_tab
     // other phase of a slot's barrier, which its parity tells from the one two phases earlier only while the slot's fill before, nS
     // stages back and the other set's, has landed.  One issuer multiplies the stages in order, and a set that is at a stage has seen
     // the stage nAst + 2 back multiplied, so from nAst + 2 slots up an odd ring is safe.  Several issuers divide the stages as the
-    // sets do: set and issuer of even stages run ahead of those of odd stages with nothing between them inside an item, so
-    // the ring is even whatever its size.
+    // sets do, and set and issuer of even stages are held to those of odd ones by nothing but the order of the activation tiles, nAst stages
+    // further on: 2 nAst + 3 slots would do, and nine with two issuers do not (a model of the barriers); the ring is even whatever its size.
     if (H->nch > 1 || H->nS < H->nAst + 2) H->nS &= ~1;
     if (H->nS < 2) return false;
     H->smem_bytes = (uint32_t)(H->nB * H->b_bytes + H->nS * H->stage_bytes + 1024 + 64 * kRingMax);
